@@ -815,9 +815,9 @@ static int make_map(CUtensorMap* m, const void* ptr, int64_t T, int H, int d, in
     return BF1_OK;
 }
 
-// O [T, Hq, d] bf16 for the epilogue's TMA stores: box = 32 elements (64 bytes) x 1 head x 32 tokens,
+// O (or dQ) [T, Hq, d] bf16 for an epilogue's TMA stores: box = 32 elements (64 bytes) x 1 head x 32 tokens,
 // 64-byte swizzle.
-static int make_store_map(CUtensorMap* m, void* ptr, int64_t T, int H, int d) {
+int make_store_map(CUtensorMap* m, void* ptr, int64_t T, int H, int d) {
     const MapKey key{ptr, T, H, d, 1, 32, 1};
     if (const CUtensorMap* hit = g_map_cache.find(key)) {
         *m = *hit;

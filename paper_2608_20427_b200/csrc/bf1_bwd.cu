@@ -5,31 +5,34 @@
 // 4.2).  With P = exp(S - LSE) recomputed from the saved LSE and D_i = <dO_i, O_i>:
 //     dV_p += P^T dO,   dP = dO V_p^T,   dS = P o (dP - D) * scale,   dQ += dS K_p,   dK_p += dS^T Q.
 // dQ of a query block sums over the KV blocks of its list; dK / dV of a KV block sum over the query
-// blocks that read it.  So there are two kernels, each walking the route in the direction in which its
-// output stays put, and nothing is ever added in global memory (no atomics, no fp32 gradient buffers,
-// the same bits on every run):
+// blocks that read it.  Nothing is ever added in global memory (no atomics, no fp32 gradient buffers, the same
+// bits on every run).  One call is three launches:
 //
-//   bwd_dq_kernel    unit = (query block, KV head, pair of query heads), as in the forward pass: the two
-//                    heads are the 128 rows of every MMA.  Per list entry p:
+//   bwd_prep_kernel  D_i for every row (one pass over dO and O), and beside it, in one CTA, the INVERSE route:
+//                    the readers of every KV block, derived from the lists on every call (any lists: the
+//                    planner's or the caller's).
+//   bwd_dkv_kernel   unit = (KV block p, KV head, a run of the query blocks that read p).  Per reader j and pair
+//                    of query heads (the two heads are the 128 rows of every MMA):
 //                        S  = Q  K_p^T   (128 x 64 x d)    A, B K-major from shared memory
 //                        dP = dO V_p^T   (128 x 64 x d)
-//                        dQ += dS K_p    (128 x d x 64)    A = dS (bf16, written over S in tensor memory by
-//                                                          the threads), B = K_p MN-major; accumulates in TMEM
-//                    It also leaves D_i in the workspace for the second kernel.
-//   bwd_dkv_kernel   unit = (KV block p, KV head, a run of the query blocks that read p): the INVERSE
-//                    route, which a few small kernels derive from the lists on every call (any lists: the
-//                    planner's or the caller's).  Per reader j (and pair of heads), S and dP as above, then
 //                        dV^T += dO^T P  (d x 64 x 128)    A = dO MN-major, B = P MN-major ([q][kv] tile)
 //                        dK^T += Q^T  dS (d x 64 x 128)    A = Q MN-major,  B = dS MN-major
 //                    accumulating in tensor memory across all readers (head dimension on the lanes), and
 //                    one store at the end.  A block with very many readers (block 0: every query block)
-//                    is cut into runs of `chunk` readers handled by different CTAs; their fp32 partial
-//                    sums are added in run order by bwd_combine_kernel.
+//                    is cut into runs of `chunk` readers handled by different CTAs that leave fp32 partial sums.
+//                    The dS tiles (bf16, 16 KB each) also go to the workspace, one per list entry.
+//   bwd_dq_kernel    unit = (query block, KV head, pair of query heads): dQ += dS K_p over the list, dS as the
+//                    dK/dV kernel left it; and, in warps of their own, the partial sums added up in run order.
 //
-// Both compute kernels are persistent: one CTA of 16 warps per SM that takes all of tensor memory (two S/dP
-// buffers and two accumulator buffers) and walks through its share of the units, with warps for copies, for
-// issuing MMAs, for the arithmetic on S and dP and for reading finished sums out, so that copies, MMAs and
-// arithmetic of neighbouring entries and units overlap (see the comment in front of each kernel).  P is rounded
+// Keeping dS costs 32 KB of traffic per list entry, KV head and pair; computing it again costs two more MMA passes (S and
+// dP), the exponentials and the V tiles.  Measured (recomputed -> kept,
+// inverse route and D_i included): 0.135 -> 0.115 ms for forward and backward of 4K tokens (16 query heads, d = 128),
+// 1.02 -> 0.944 ms at 32K.
+// A route whose dS would not fit (kDsMost for one KV head) is run by bwd_dq_recompute_kernel instead.
+//
+// The compute kernels are persistent: one CTA of 10 to 16 warps per SM that walks through its share of the units, with
+// warps for copies, for issuing MMAs, for the arithmetic on S and dP and for reading finished sums out, so that copies,
+// MMAs and arithmetic of neighbouring entries and units overlap (see the comment in front of each kernel).  P is rounded
 // to bf16 before the MMAs, as in the forward.  With d = 64 the transposed products still run as M = 128 MMAs:
 // tensor-memory lanes 64..127 then hold nothing of value and are not read.
 #include <cuda.h>
@@ -42,14 +45,18 @@ namespace bf1 {
 
 constexpr int kBlock64 = 64;     // b: tokens per block
 constexpr int kMinChunk = 16;    // readers per dK/dV unit, at least
+constexpr int kDsTile = 128 * 64 * 2;          // bytes of one dS tile: [128 q rows][64 kv], 128-byte rows, swizzled
+constexpr int64_t kDsGroup = 1LL << 30;        // dS kept at a time: as many KV heads as fit this (at least one)
+constexpr int64_t kDsMost = 8LL << 30;         // one KV head's dS larger than this is not kept but computed again
 
 // The inverse route and the units of bwd_dkv_kernel, all inside the caller's workspace.
 struct InvPlan {
     int32_t* count;       // [cap] readers of KV slot g (with multiplicity)
     int32_t* start;       // [cap + 1] first reader of slot g in `readers`
+    int32_t* unit0;       // [cap + 1] first unit of slot g
     int32_t* chunks;      // [cap] runs the slot's readers are cut into
     int32_t* part0;       // [cap] first partial-sum slot of a slot with more than one run, else -1
-    int32_t* readers;     // [cap * max_degree] query slots, ascending per KV slot
+    int32_t* readers;     // [cap * max_degree] list entries (query slot * max_degree + place), ascending per KV slot
     int32_t* unit_slot;   // [max_units] KV slot of the unit
     int32_t* unit_begin;  // [max_units] its readers: readers[begin .. end)
     int32_t* unit_end;
@@ -69,13 +76,15 @@ struct BwdArgs {
     const int32_t* num_qblocks;
     const int32_t* order;      // may be null
     int32_t max_degree, capacity, total_tokens, hq, hkv, group;
+    int32_t head0, nheads; // KV heads this launch works on: head0 .. head0 + nheads - 1
     int32_t interleave;    // 1: units of all KV heads interleaved (longest first over all heads); 0: KV head by KV head
     int32_t* status;
     float scale, scale_log2;
     const __nv_bfloat16* o;
     const __nv_bfloat16* d_o;
     const float* lse;
-    float* delta;          // [hq, T] D_i = <dO_i, O_i>: written by the dQ kernel, read by the dK/dV kernel
+    float* delta;          // [hq, T] D_i = <dO_i, O_i>
+    __nv_bfloat16* ds;     // [nheads][pairs][cap * max_degree] dS tiles of kDsTile bytes, or null: not kept
     __nv_bfloat16* dq;
     __nv_bfloat16* dk;
     __nv_bfloat16* dv;
@@ -83,12 +92,14 @@ struct BwdArgs {
     InvPlan inv;
 };
 
+__device__ __forceinline__ int safe_entry(int p, int e, int cnt, int j) {
+    if (p < 0 || p > j || (e == cnt - 1) != (p == j)) p = (e == cnt - 1) ? j : 0;
+    return p;
+}
 // Entry e of a list as every kernel of this library uses it: kept inside [0, j], the last entry the
 // query block itself, whatever the array holds (a caller's route may be wrong; the forward flags it).
 __device__ __forceinline__ int list_entry(const int32_t* list, int e, int cnt, int j) {
-    int p = list[e];
-    if (p < 0 || p > j || (e == cnt - 1) != (p == j)) p = (e == cnt - 1) ? j : 0;
-    return p;
+    return safe_entry(list[e], e, cnt, j);
 }
 
 // ---- pieces shared by the two compute kernels ------------------------------------------------------------------
@@ -174,42 +185,38 @@ __device__ __forceinline__ void load_q_tile(uint32_t dst, const CUtensorMap* tm,
     }
 }
 
-__device__ __forceinline__ void ld_shared_v4(uint32_t addr, uint32_t (&w)[4]) {
-    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(addr));
-}
-
-// ---- dQ --------------------------------------------------------------------------------------------------------
+// ---- dQ from recomputed dS ---------------------------------------------------------------------------------------
+//
+// For routes whose dS tiles would not fit the workspace.
 //
 // One persistent CTA of 16 warps per SM.  Units (query block, KV head, pair of heads) are dealt out statically, in
 // the route's longest-list-first order KV head by KV head, back and forth over the CTAs so that each gets the same
 // mix.  Everything a unit needs travels through rings whose next entry is under way while the current one is in
 // use, across unit boundaries as well:
 //     warp 0    copies Q of every unit (two buffers) and the K tile of every list entry (ring of kStages)
-//     warp 1    copies dO of every unit, its O tile (into a whole ring stage, ahead of the unit's K/V tiles) and
-//               the V tiles
+//     warp 1    copies dO of every unit and the V tiles
 //     warp 2    issues S and dP of every entry into one of two S/dP buffers in tensor memory, as soon as the K / V
 //               tiles are there and the dQ MMAs that read the buffer's last dS are done
 //     warp 3    issues the dQ MMAs of every entry; dQ accumulates in one of two buffers
 //     warps 4-11   the arithmetic on S and dP, two threads per tile row (32 key columns each); dS (bf16) goes back
 //               into tensor memory over S, from where the dQ MMAs read it as their A operand
-//     warps 12-15   per unit: D_i = <dO_i, O_i> and the LSE of every row into shared memory (and D_i into the
-//               workspace, for the dK/dV kernel) one unit ahead; then the finished dQ tile of the unit before,
-//               from tensor memory to global memory
+//     warps 12-15   per unit: D_i and the LSE of every row into shared memory one unit ahead; then the finished dQ
+//               tile of the unit before, from tensor memory to global memory
 // Every wait of a role is on a barrier it waits on once per phase, in phase order: a parity wait is only
 // meaningful one phase ahead.
-constexpr int kDqThreads = 512;
+constexpr int kDqrThreads = 512;
 constexpr int kStages = 3;
 // Q / dO buffer (and barrier) of unit n, and the parity of its n-th use
 __device__ __forceinline__ int qbuf(int n) { return n & 1; }
 __device__ __forceinline__ uint32_t qpar(int n) { return (n >> 1) & 1; }
 
 template <int D>
-struct DqSmem {
+struct DqrSmem {
     static constexpr int kQBytes = 128 * D * 2;      // Q / dO / O tile [D / 64 chunks][128 rows][128 B]
     static constexpr int kKVBytes = 64 * D * 2;      // K / V tile      [D / 64 chunks][64 rows][128 B]
     static constexpr int kQ = 0;                     // [2]
     static constexpr int kDO = kQ + 2 * kQBytes;     // [2]
-    static constexpr int kRing = kDO + 2 * kQBytes;  // [kStages] of K | V (or one O tile)
+    static constexpr int kRing = kDO + 2 * kQBytes;  // [kStages] of K | V
     static constexpr int kRow = kRing + kStages * 2 * kKVBytes;   // D_i [2][128], LSE [2][128] (fp32)
     static constexpr int kBar = kRow + 2048;
     static constexpr int kUsed = kBar + 512;
@@ -224,7 +231,7 @@ struct DqUnit {
 // Unit n of this CTA (see above for the order).
 __device__ __forceinline__ DqUnit dq_unit(const BwdArgs& a, int n, int nqb, int pairs) {
     DqUnit u;
-    const int per_head = nqb * pairs, total = per_head * a.hkv;
+    const int per_head = nqb * pairs, total = per_head * a.nheads;
     const int G = gridDim.x;
     const int i = n * G + ((n & 1) ? G - 1 - (int)blockIdx.x : (int)blockIdx.x);
     u.ok = i < total;
@@ -234,7 +241,7 @@ __device__ __forceinline__ DqUnit dq_unit(const BwdArgs& a, int n, int nqb, int 
     if (u.ok) {
         int rank;
         if (a.interleave) {          // rank-major: the longest lists of all heads first
-            const int per_rank = pairs * a.hkv;
+            const int per_rank = pairs * a.nheads;
             rank = i / per_rank;
             const int rem = i - rank * per_rank;
             u.kvh = rem / pairs;
@@ -245,6 +252,7 @@ __device__ __forceinline__ DqUnit dq_unit(const BwdArgs& a, int n, int nqb, int 
             rank = rem / pairs;
             u.pair = rem - rank * pairs;
         }
+        u.kvh += a.head0;
         int slot = a.order ? a.order[rank] : rank;
         slot = min(max(slot, 0), nqb - 1);
         u.slot = slot;
@@ -263,13 +271,12 @@ __device__ __forceinline__ void named_sync(int id, int threads) {
 }
 
 template <int D>
-__global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_constant__ CUtensorMap tm_q,
-                                                            const __grid_constant__ CUtensorMap tm_k,
-                                                            const __grid_constant__ CUtensorMap tm_v,
-                                                            const __grid_constant__ CUtensorMap tm_do,
-                                                            const __grid_constant__ CUtensorMap tm_o,
-                                                            const BwdArgs a) {
-    using L = DqSmem<D>;
+__global__ void __launch_bounds__(kDqrThreads, 1) bwd_dq_recompute_kernel(const __grid_constant__ CUtensorMap tm_q,
+                                                                       const __grid_constant__ CUtensorMap tm_k,
+                                                                       const __grid_constant__ CUtensorMap tm_v,
+                                                                       const __grid_constant__ CUtensorMap tm_do,
+                                                                       const BwdArgs a) {
+    using L = DqrSmem<D>;
     extern __shared__ __align__(1024) uint8_t smem[];
     uint32_t& s_tmem = *reinterpret_cast<uint32_t*>(smem + L::kBar + 496);
     int& s_abort = *reinterpret_cast<int*>(smem + L::kBar + 500);
@@ -284,9 +291,8 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
     const uint32_t bars = base + L::kBar;
     // barriers (8 bytes each)
     const uint32_t qdo_full = bars;                          // [2] Q and dO of a unit landed (both copy warps announce bytes)
-    const uint32_t qdo_free = qdo_full + 16;                 // [2] the unit's MMAs are done and its D_i computed
-    const uint32_t o_full = qdo_free + 16;                   // [2] the unit's O tile landed
-    const uint32_t row_full = o_full + 16;                   // [2] D_i and LSE of the unit's rows are in shared memory
+    const uint32_t qdo_free = qdo_full + 16;                 // [2] the unit's MMAs are done
+    const uint32_t row_full = qdo_free + 16;                 // [2] D_i and LSE of the unit's rows are in shared memory
     const uint32_t row_free = row_full + 16;                 // [2] ... and have been read by both arithmetic groups (8 warps)
     const uint32_t sdp_full = row_free + 16;                 // [2] S and dP of an entry computed
     const uint32_t ds_ready = sdp_full + 16;                 // [2] dS written (8 warps)
@@ -294,15 +300,14 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
     const uint32_t dq_free = dq_full + 16;                   // [2] ... and has been read out of tensor memory
     const uint32_t dq_done = dq_free + 16;                   // [2] the dQ MMAs that read dS from an S / dP buffer are done
     const uint32_t kv_full = dq_done + 16;                   // [kStages] a K and a V tile landed (both copy warps announce bytes)
-    const uint32_t ring_free = kv_full + 8 * kStages;        // [kStages] the stage's tiles (or O tile) have been used
-    static_assert(160 + 16 * kStages <= 496, "barriers overlap the words behind them");
+    const uint32_t ring_free = kv_full + 8 * kStages;        // [kStages] the stage's tiles have been used
+    static_assert(144 + 16 * kStages <= 496, "barriers overlap the words behind them");
     if (tid == 0) {
         s_abort = (base & 1023u) ? 1 : 0;
         if (s_abort && a.status) atomicOr(a.status, BF1_DEV_WAIT_TIMEOUT);
         for (int b = 0; b < 2; ++b) {
             mbar_init(qdo_full + 8 * b, 2);
-            mbar_init(qdo_free + 8 * b, 2);
-            mbar_init(o_full + 8 * b, 1);
+            mbar_init(qdo_free + 8 * b, 1);
             mbar_init(row_full + 8 * b, 1);
             mbar_init(row_free + 8 * b, 8);
             mbar_init(sdp_full + 8 * b, 1);
@@ -323,8 +328,8 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
         tmem_relinquish();
     }
     if (a.group == 1) {   // one head per KV head: rows 64..127 of the Q / dO buffers are never written by a copy
-        clear_idle_rows<D>(base + L::kQ, base + L::kDO, tid, kDqThreads);
-        clear_idle_rows<D>(base + L::kQ + L::kQBytes, base + L::kDO + L::kQBytes, tid, kDqThreads);
+        clear_idle_rows<D>(base + L::kQ, base + L::kDO, tid, kDqrThreads);
+        clear_idle_rows<D>(base + L::kQ + L::kQBytes, base + L::kDO + L::kQBytes, tid, kDqrThreads);
     }
     tc_fence_before();
     __syncthreads();
@@ -358,7 +363,7 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
         DqUnit u = dq_unit(a, 0, nqb, pairs);
         for (int n = 0; u.ok; ++n) {
             const DqUnit un = dq_unit(a, n + 1, nqb, pairs);
-            const int b = n & 1, head0 = u.kvh * a.group + u.pair * 2;
+            const int head0 = u.kvh * a.group + u.pair * 2;
             const int32_t* list = a.kv_idx + (size_t)u.slot * a.max_degree;
             const int qb = qbuf(n);
             if (n >= 2) mbar_wait(qdo_free + 8 * qb, qpar(n - 2), abort_flag, a.status);
@@ -368,16 +373,6 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
                 else load_q_tile<D>(base + L::kDO + qb * L::kQBytes, &tm_do, u.tok0, head0, a.group, qdo_full + 8 * qb);
             }
             __syncwarp();
-            // the O tile's ring entry
-            if (!first) {
-                ring_wait_free();
-                if (elect_one()) {
-                    mbar_expect_tx(o_full + 8 * b, q_tx);
-                    load_q_tile<D>(stage_k(rs), &tm_o, u.tok0, head0, a.group, o_full + 8 * b);
-                }
-                __syncwarp();
-            }
-            ring_next();
             for (int it = 0; it < u.cnt; ++it) {
                 const int p = list_entry(list, it, u.cnt, u.j);
                 ring_wait_free();
@@ -398,7 +393,7 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
         constexpr uint32_t kHi = desc_hi_sw128(1024);
         constexpr uint32_t kIdQ = idesc_bf16_f32(D, true);             // dQ: 128 x d, A from tensor memory, B (K tile) MN-major
         DqUnit u = dq_unit(a, 0, nqb, pairs);
-        int t = 0, rs = 1 % kStages;       // entries so far; ring stage of the entry (entry 0 of the ring is unit 0's O tile)
+        int t = 0, rs = 0;                 // entries so far; ring stage of the entry
         uint32_t kv_phase = 0;             // per stage: parity of the K / V tiles put into it so far
         for (int n = 0; u.ok; ++n) {
             const DqUnit un = dq_unit(a, n + 1, nqb, pairs);
@@ -449,7 +444,6 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
                 ++t;
                 if (++rs == kStages) rs = 0;
             }
-            if (++rs == kStages) rs = 0;   // the next unit's O tile
             u = un;
         }
     } else if (warp >= 4 && warp < 12) {
@@ -486,42 +480,20 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
         // ---- per unit: D_i and LSE one unit ahead; the finished dQ tile of the unit before ----
         const uint32_t t_lane = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
         const int row = tid & 127, hl = row >> 6, tl = row & 63;
-        int r = 0;   // ring entry of the current unit's O tile
         auto prologue = [&](const DqUnit& u, int n) {
             const int b = n & 1;
             const int h = u.kvh * a.group + u.pair * 2 + hl, tok = u.tok0 + tl;
             const bool row_ok = tl < u.rows_valid && u.pair * 2 + hl < a.group;   // G = 1: rows 64..127 belong to no head
             float lse2 = INFINITY, Drow = 0.f;
-            if (row_ok) lse2 = a.lse[(size_t)h * a.total_tokens + tok] * 1.4426950408889634f;
-            mbar_wait(qdo_full + 8 * qbuf(n), qpar(n), abort_flag, a.status);
-            mbar_wait(o_full + 8 * b, (n >> 1) & 1, abort_flag, a.status);
-            if (n >= 2) mbar_wait(row_free + 8 * b, ((n >> 1) - 1) & 1, abort_flag, a.status);
-            const int rs = r % kStages;
             if (row_ok) {
-                const uint32_t sO = stage_k(rs), sDO = base + L::kDO + qbuf(n) * L::kQBytes;
-#pragma unroll
-                for (int c = 0; c < D / 8; ++c) {   // 16-byte pieces of the row: chunk c / 8 of 64 columns, piece c % 8
-                    const uint32_t off = (c >> 3) * 16384 + row * 128 + (((c & 7) ^ (row & 7)) << 4);
-                    uint32_t ow[4], gw[4];
-                    ld_shared_v4(sO + off, ow);
-                    ld_shared_v4(sDO + off, gw);
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        Drow = fmaf(__uint_as_float(ow[e] << 16), __uint_as_float(gw[e] << 16), Drow);
-                        Drow = fmaf(__uint_as_float(ow[e] & 0xffff0000u), __uint_as_float(gw[e] & 0xffff0000u), Drow);
-                    }
-                }
-                a.delta[(size_t)h * a.total_tokens + tok] = Drow;   // for the dK/dV kernel
+                lse2 = a.lse[(size_t)h * a.total_tokens + tok] * 1.4426950408889634f;
+                Drow = a.delta[(size_t)h * a.total_tokens + tok];
             }
+            if (n >= 2) mbar_wait(row_free + 8 * b, ((n >> 1) - 1) & 1, abort_flag, a.status);
             s_drow[b * 128 + row] = Drow;
             s_lse[b * 128 + row] = lse2;
             named_sync(1, 128);
-            if ((tid & 127) == 0) {
-                mbar_arrive(ring_free + 8 * rs);
-                mbar_arrive(qdo_free + 8 * qbuf(n));
-                mbar_arrive(row_full + 8 * b);
-            }
-            r += u.cnt + 1;
+            if ((tid & 127) == 0) mbar_arrive(row_full + 8 * b);
         };
         DqUnit u = dq_unit(a, 0, nqb, pairs);
         if (u.ok) prologue(u, 0);
@@ -564,8 +536,8 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
 
 // ---- the inverse route -----------------------------------------------------------------------------------------
 
-// The readers of KV slot gp are the query slots of the same sequence whose list names its block (with multiplicity,
-// should a caller's list name a block twice).  Transposing the lists is a counting sort by KV slot, linear in the
+// The readers of KV slot gp are the list entries of the same sequence that name its block (an entry is its query slot
+// times max_degree plus its place in the list).  Transposing the lists is a counting sort by KV slot, linear in the
 // number of list entries: count (one thread per entry), scan (inverse_units_kernel), fill in whatever order the
 // atomics give, then sort every slot's readers ascending -- the order in which the dK/dV kernel adds is thereby the
 // same on every run.
@@ -590,8 +562,18 @@ __global__ void __launch_bounds__(256) inverse_route_kernel(const BwdArgs a) {
         int g, kv;
         if (!inverse_entry(a, nqb, f, g, kv)) continue;
         if (!kFill) atomicAdd(a.inv.count + kv, 1);
-        else a.inv.readers[a.inv.start[kv] + atomicSub(a.inv.count + kv, 1) - 1] = g;
+        else a.inv.readers[a.inv.start[kv] + atomicSub(a.inv.count + kv, 1) - 1] = f;
     }
+}
+
+// Ascending sort of c <= 32 values, one per lane.
+__device__ __forceinline__ int rank_in_warp(int v, int c, int lane) {
+    int rank = 0;
+    for (int j = 0; j < c; ++j) {
+        const int vj = __shfl_sync(0xffffffffu, v, j);
+        rank += (vj < v) || (vj == v && j < lane);
+    }
+    return rank;
 }
 
 // One CTA per KV slot: its readers ascending.  Up to 32 by ranking inside a warp; more by a bitonic network whose
@@ -608,11 +590,7 @@ __global__ void __launch_bounds__(256) inverse_sort_kernel(const BwdArgs a) {
     if (c <= 32) {
         if (tid >= 32) return;
         const int v = lane < c ? r[lane] : 0x7fffffff;
-        int rank = 0;
-        for (int j = 0; j < c; ++j) {
-            const int vj = __shfl_sync(0xffffffffu, v, j);
-            rank += (vj < v) || (vj == v && j < lane);
-        }
+        const int rank = rank_in_warp(v, c, lane);
         if (lane < c) r[rank] = v;
         return;
     }
@@ -638,125 +616,228 @@ __global__ void __launch_bounds__(256) inverse_sort_kernel(const BwdArgs a) {
     }
 }
 
-// One CTA: offsets of the reader lists, the run length, and the units of the dK/dV kernel.  kAll: the counting and the
-// filling of the readers as well (few list entries: one launch instead of four).
+// One CTA of 1024 threads: offsets of the reader lists, the run length, and the units of the dK/dV kernel.  kAll: the
+// counting, filling and sorting of the readers as well, in shared memory: `smem` then holds inverse_words() words.
+// (Otherwise inverse_route_kernel has counted the readers in the workspace and will fill them in.)
+__host__ __device__ inline int64_t inverse_words(int64_t cap, int64_t max_degree) { return 3 * cap + 2 + 2 * cap * max_degree; }
+
 template <bool kAll>
-__global__ void __launch_bounds__(1024, 1) inverse_units_kernel(const BwdArgs a) {
-    __shared__ int32_t s_warp[32];
-    __shared__ int32_t s_carry[5];
-    __shared__ int32_t s_chunk;
+__device__ __forceinline__ void inverse_units(const BwdArgs& a, int32_t* smem) {
+    __shared__ unsigned long long s_warp[32];
+    __shared__ int32_t s_bin[1024];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nqb = min(*a.num_qblocks, a.capacity);
     const InvPlan& v = a.inv;
-    // exclusive scan of x over the CTA, with a running carry in s_carry[which]
-    auto scan = [&](int x, int which, int& excl) {
-        int incl = x;
+    int32_t* count = kAll ? smem : v.count;
+    int32_t* start = kAll ? count + a.capacity : v.start;           // [nqb + 1] first reader of a slot
+    int32_t* unit0 = kAll ? start + a.capacity + 1 : v.unit0;       // [nqb + 1] first unit of a slot
+    int32_t* kv_of = kAll ? unit0 + a.capacity + 1 : nullptr;       // per entry: the KV slot it names, or -1
+    int32_t* readers = kAll ? kv_of + a.capacity * a.max_degree : nullptr;
+    // inclusive scan of x over the CTA
+    auto scan = [&](unsigned long long x, unsigned long long& total) {
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
-            const int up = __shfl_up_sync(0xffffffffu, incl, off);
-            if (lane >= off) incl += up;
+            const unsigned long long up = __shfl_up_sync(0xffffffffu, x, off);
+            if (lane >= off) x += up;
         }
-        if (lane == 31) s_warp[warp] = incl;
+        if (lane == 31) s_warp[warp] = x;
         __syncthreads();
-        if (warp == 0) {
-            int w = s_warp[lane];
+        unsigned long long w = s_warp[lane];
 #pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const int up = __shfl_up_sync(0xffffffffu, w, off);
-                if (lane >= off) w += up;
-            }
-            s_warp[lane] = w;
+        for (int off = 1; off < 32; off <<= 1) {
+            const unsigned long long up = __shfl_up_sync(0xffffffffu, w, off);
+            if (lane >= off) w += up;
         }
+        total = __shfl_sync(0xffffffffu, w, 31);
+        const unsigned long long before = __shfl_sync(0xffffffffu, w, (warp - 1) & 31);
         __syncthreads();
-        const int before = (warp > 0 ? s_warp[warp - 1] : 0) + s_carry[which];
-        excl = before + incl - x;
-        const int chunk_total = s_warp[31];
-        __syncthreads();
-        if (tid == 0) s_carry[which] += chunk_total;
-        __syncthreads();
+        return x + (warp > 0 ? before : 0ull);
     };
-    if (tid < 5) s_carry[tid] = 0;
+    auto count_of = [&](int g) { return kAll ? count[g] : __ldcg(count + g); };   // (written by atomics: read where they were performed)
+    s_bin[tid] = 0;
     if (kAll) {
-        for (int g = tid; g < nqb; g += 1024) v.count[g] = 0;
+        for (int g = tid; g < nqb; g += 1024) count[g] = 0;
         __syncthreads();
-        for (int f = tid; f < nqb * a.max_degree; f += 1024) {
-            int g, kv;
-            if (inverse_entry(a, nqb, f, g, kv)) atomicAdd(v.count + kv, 1);
+        constexpr int kAtOnce = 4;      // entries a thread reads together: each is three loads
+        for (int f0 = tid; f0 < nqb * a.max_degree; f0 += kAtOnce * 1024) {
+            int c[kAtOnce], j[kAtOnce], p[kAtOnce];
+#pragma unroll
+            for (int i = 0; i < kAtOnce; ++i) {
+                const int f = min(f0 + i * 1024, nqb * a.max_degree - 1), g = f / a.max_degree;
+                c[i] = a.kv_count[g], j[i] = a.qb_block[g], p[i] = a.kv_idx[f];
+            }
+#pragma unroll
+            for (int i = 0; i < kAtOnce; ++i) {
+                const int f = f0 + i * 1024, g = f / a.max_degree, e = f - g * a.max_degree;
+                const int cnt = min(max(c[i], 1), a.max_degree);
+                if (f >= nqb * a.max_degree) continue;
+                int kv = -1;
+                if (e < cnt) {
+                    kv = g - j[i] + safe_entry(p[i], e, cnt, j[i]);
+                    atomicAdd(count + kv, 1);
+                }
+                kv_of[f] = kv;
+            }
         }
+        __syncthreads();
     }
-    __syncthreads();
     // pass 1: where each slot's readers start; the total decides the run length
+    int readers_total = 0;
     for (int b0 = 0; b0 < nqb; b0 += 1024) {
         const int g = b0 + tid;
-        const int c = g < nqb ? __ldcg(v.count + g) : 0;   // (written by atomics: read where they were performed)
-        int excl;
-        scan(c, 0, excl);
-        if (g < nqb) v.start[g] = excl;
+        const int c = g < nqb ? count_of(g) : 0;
+        unsigned long long total;
+        const int incl = (int)scan((unsigned long long)c, total);
+        if (g < nqb) start[g] = readers_total + incl - c;
+        readers_total += (int)total;
     }
-    if (tid == 0) {
-        const int total = s_carry[0];
-        v.start[nqb] = total;
-        // runs of at least kMinChunk readers, and long enough that the slots with more than one run cannot need
-        // more than `cap` partial-sum slots between them (such a slot has fewer than 2 * count / chunk runs)
-        s_chunk = max(kMinChunk, (2 * total + max(v.cap, 1) - 1) / max(v.cap, 1));
-    }
-    __syncthreads();
-    const int chunk = s_chunk;
-    // pass 2: runs per slot -> unit numbers and partial-sum slots
+    if (tid == 0) start[nqb] = readers_total;
+    // runs of at least kMinChunk readers, and long enough that the slots with more than one run cannot need
+    // more than `cap` partial-sum slots between them (such a slot has fewer than 2 * count / chunk runs)
+    const int chunk = max(kMinChunk, (2 * readers_total + max(v.cap, 1) - 1) / max(v.cap, 1));
+    // pass 2: runs per slot -> unit numbers, partial-sum slots and places in `multi`: one scan, 21 bits each
+    int units = 0, parts = 0, multis = 0;
     for (int b0 = 0; b0 < nqb; b0 += 1024) {
         const int g = b0 + tid;
-        const int c = g < nqb ? __ldcg(v.count + g) : 0;   // (written by atomics: read where they were performed)
-        const int runs = (c + chunk - 1) / chunk;
-        int u0, q0, m0;
-        scan(runs, 1, u0);
-        scan(runs > 1 ? runs : 0, 2, q0);
-        scan(runs > 1 ? 1 : 0, 3, m0);
+        const int c = g < nqb ? count_of(g) : 0;
+        const int runs = (c + chunk - 1) / chunk, split = runs > 1 ? runs : 0;
+        const unsigned long long x = (unsigned long long)runs | (unsigned long long)split << 21 | (unsigned long long)(runs > 1) << 42;
+        unsigned long long total;
+        const unsigned long long excl = scan(x, total) - x;
+        const int q0 = parts + (int)(excl >> 21 & 0x1fffff), m0 = multis + (int)(excl >> 42);
         if (g < nqb) {
+            unit0[g] = units + (int)(excl & 0x1fffff);
             if (runs > 1) v.multi[m0] = g;
             v.chunks[g] = runs;
             v.part0[g] = runs > 1 ? q0 : -1;
-            const int first = v.start[g];
-            for (int r = 0; r < runs; ++r) {
-                if (u0 + r >= v.max_units) break;
-                v.unit_slot[u0 + r] = g;
-                v.unit_begin[u0 + r] = first + r * chunk;
-                v.unit_end[u0 + r] = min(first + c, first + (r + 1) * chunk);
-                v.unit_part[u0 + r] = runs > 1 ? q0 + r : -1;
-            }
+        }
+        units += (int)(total & 0x1fffff), parts += (int)(total >> 21 & 0x1fffff), multis += (int)(total >> 42);
+    }
+    const bool fits = units <= v.max_units && parts <= v.cap;
+    if (tid == 0) {
+        unit0[nqb] = units;
+        if (!fits && a.status) atomicOr(a.status, BF1_DEV_CAPACITY);
+        v.scalars[0] = fits ? units : 0;
+        v.scalars[1] = readers_total;
+        v.scalars[2] = chunk;
+        v.scalars[3] = parts;
+        v.scalars[4] = fits ? multis : 0;
+    }
+    __syncthreads();
+    // the units, a thread each: the slot by binary search
+    auto unit_of = [&](int un, int& g, int& begin, int& end) {
+        int lo = 0, hi = nqb;     // unit0[lo] <= un < unit0[hi]  (a slot without readers has no unit)
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (unit0[mid] <= un) lo = mid; else hi = mid;
+        }
+        g = lo;
+        begin = start[g] + (un - unit0[g]) * chunk;
+        end = min(begin + chunk, start[g + 1]);
+    };
+    auto bin_of = [](int len) { return 1023 - min(len, 1023); };
+    if (fits) {
+        for (int un = tid; un < units; un += 1024) {
+            int g, begin, end;
+            unit_of(un, g, begin, end);
+            v.unit_slot[un] = g;
+            v.unit_begin[un] = begin;
+            v.unit_end[un] = end;
+            const bool split = unit0[g + 1] - unit0[g] > 1;
+            v.unit_part[un] = split ? v.part0[g] + un - unit0[g] : -1;
+            atomicAdd(&s_bin[bin_of(end - begin)], 1);
         }
     }
+    __syncthreads();
     // units by descending length (a counting sort; which of two equally long units comes first does not matter: the
     // order only decides which CTA works on which unit)
-    __shared__ int32_t s_bin[1024];
-    s_bin[tid] = 0;
-    __syncthreads();
-    const int n_units = min(s_carry[1], v.max_units);
-    for (int un = tid; un < n_units; un += 1024) atomicAdd(&s_bin[1023 - min(v.unit_end[un] - v.unit_begin[un], 1023)], 1);
-    __syncthreads();
     {
         const int c = s_bin[tid];
-        int excl;
-        scan(c, 4, excl);
-        s_bin[tid] = excl;           // where the units of this length start
+        unsigned long long total;
+        const int incl = (int)scan((unsigned long long)c, total);
+        s_bin[tid] = incl - c;       // where the units of this length start
     }
     __syncthreads();
-    for (int un = tid; un < n_units; un += 1024)
-        v.unit_order[atomicAdd(&s_bin[1023 - min(v.unit_end[un] - v.unit_begin[un], 1023)], 1)] = un;
-    if (tid == 0) {
-        const bool fits = s_carry[1] <= v.max_units && s_carry[2] <= v.cap;
-        if (!fits && a.status) atomicOr(a.status, BF1_DEV_CAPACITY);
-        v.scalars[0] = fits ? s_carry[1] : 0;
-        v.scalars[1] = s_carry[0];
-        v.scalars[2] = chunk;
-        v.scalars[3] = s_carry[2];
-        v.scalars[4] = fits ? s_carry[3] : 0;
+    if (fits) {
+        for (int un = tid; un < units; un += 1024) {
+            int g, begin, end;
+            unit_of(un, g, begin, end);
+            v.unit_order[atomicAdd(&s_bin[bin_of(end - begin)], 1)] = un;
+        }
     }
     if (kAll) {
-        __syncthreads();
         for (int f = tid; f < nqb * a.max_degree; f += 1024) {
-            int g, kv;
-            if (inverse_entry(a, nqb, f, g, kv)) v.readers[v.start[kv] + atomicSub(v.count + kv, 1) - 1] = g;
+            const int kv = kv_of[f];
+            if (kv >= 0) readers[start[kv] + atomicSub(count + kv, 1) - 1] = f;
         }
+        __syncthreads();
+        // an entry's place among its slot's readers is the number of smaller ones (they are distinct)
+        for (int i = tid; i < readers_total; i += 1024) {
+            const int f = readers[i], kv = kv_of[f], s0 = start[kv], s1 = start[kv + 1];
+            int rank = 0;
+#pragma unroll 4
+            for (int k = s0; k < s1; ++k) rank += readers[k] < f;
+            v.readers[s0 + rank] = f;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(1024, 1) inverse_units_kernel(const BwdArgs a) {
+    inverse_units<false>(a, nullptr);
+}
+
+// D_i = <dO_i, O_i> of every row, and (kInverse) in the first CTA the whole inverse route: a chain of a few
+// microseconds on one SM that is hidden behind the pass over dO and O on the others.  kInverse is chosen while the
+// entries fit shared memory beside the counters (kInvInts words): up to about 64K tokens with the
+// paper's route; beyond, several launches share the work.
+// Measured: 8.3 us at 4K tokens (16 query heads, d = 128) and 56 us at 32K, where the pass over dO and O alone takes 48;
+// the inverse route alone 7 and 25.  (As launches of their own: 12 and 28 us, with D_i in the dQ kernel.)
+constexpr int kInvInts = 24576;
+template <int D, bool kInverse>
+__global__ void __launch_bounds__(1024, 1) bwd_prep_kernel(const BwdArgs a) {
+    extern __shared__ int32_t s_inv[];
+    if (a.status && (*a.status & BF1_DEV_WAIT_TIMEOUT)) return;
+    int cta = blockIdx.x, ctas = gridDim.x;
+    if (kInverse) {
+        if (cta == 0) {
+            inverse_units<true>(a, s_inv);
+            return;
+        }
+        --cta, --ctas;
+    }
+    // a warp takes 16 tokens of one head; a row is read by D / 8 lanes, 16 bytes each
+    constexpr int kLanes = D / 8, kRowsAtOnce = 32 / kLanes, kTokens = 16;
+    const int lane = threadIdx.x & 31, sub = lane % kLanes, r0 = lane / kLanes;
+    const int items = ((a.total_tokens + kTokens - 1) / kTokens) * a.hq;
+    for (int item = cta * 32 + (threadIdx.x >> 5); item < items; item += ctas * 32) {
+        const int h = item % a.hq, t0 = (item / a.hq) * kTokens;
+        float mine = 0.f;
+#pragma unroll
+        for (int it0 = 0; it0 < kTokens / kRowsAtOnce; it0 += 4) {   // 4 rows' loads in flight at once
+            uint4 x[4], g[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int tok = min(t0 + (it0 + i) * kRowsAtOnce + r0, a.total_tokens - 1);
+                const size_t at = ((size_t)tok * a.hq + h) * D + sub * 8;
+                x[i] = *reinterpret_cast<const uint4*>(a.o + at);
+                g[i] = *reinterpret_cast<const uint4*>(a.d_o + at);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t xw[4] = {x[i].x, x[i].y, x[i].z, x[i].w}, gw[4] = {g[i].x, g[i].y, g[i].z, g[i].w};
+                float sum = 0.f;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    sum = fmaf(__uint_as_float(xw[e] << 16), __uint_as_float(gw[e] << 16), sum);
+                    sum = fmaf(__uint_as_float(xw[e] & 0xffff0000u), __uint_as_float(gw[e] & 0xffff0000u), sum);
+                }
+#pragma unroll
+                for (int off = kLanes / 2; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+                if (sub == it0 + i) mine = sum;
+            }
+        }
+        const int tok = t0 + sub * kRowsAtOnce + r0;
+        if (sub < kTokens / kRowsAtOnce && tok < a.total_tokens) a.delta[(size_t)h * a.total_tokens + tok] = mine;
     }
 }
 
@@ -769,7 +850,8 @@ __global__ void __launch_bounds__(1024, 1) inverse_units_kernel(const BwdArgs a)
 //     warp 0    copies K of every unit and Q of every step;  warp 1: V and dO
 //     warp 2    issues S = Q K^T and dP = dO V^T of every step into one of two S/dP buffers in tensor memory
 //     warp 3    issues dV^T += dO^T P and dK^T += Q^T dS of every step; the sums stay in one of two accumulator
-//               buffers in tensor memory across all steps of the unit
+//               buffers in tensor memory across all steps of the unit.  It also starts the copy of every dS tile to
+//               the workspace, as it lies in shared memory: its own MMAs read the tile at the same time
 //     warps 4-11   the arithmetic on S and dP (two threads per tile row), P and dS as bf16 tiles to shared memory
 //     warps 12-15  the finished sums of the unit before, from tensor memory to global memory
 constexpr int kDkvThreads = 512;
@@ -797,7 +879,7 @@ struct DkvUnit {
 // Unit n of this CTA.
 __device__ __forceinline__ DkvUnit dkv_unit(const BwdArgs& a, int n, int n_units, int pairs) {
     DkvUnit u;
-    const int total = n_units * a.hkv;
+    const int total = n_units * a.nheads;
     const int G = gridDim.x;
     const int i = n * G + ((n & 1) ? G - 1 - (int)blockIdx.x : (int)blockIdx.x);
     u.ok = i < total;
@@ -807,12 +889,13 @@ __device__ __forceinline__ DkvUnit dkv_unit(const BwdArgs& a, int n, int n_units
     if (u.ok) {
         int ui;
         if (a.interleave) {
-            ui = i / a.hkv;
-            u.kvh = i - ui * a.hkv;
+            ui = i / a.nheads;
+            u.kvh = i - ui * a.nheads;
         } else {
             u.kvh = i / n_units;
             ui = i - u.kvh * n_units;
         }
+        u.kvh += a.head0;
         const int unit = a.inv.unit_order[ui];
         u.gp = a.inv.unit_slot[unit];
         u.r_begin = a.inv.unit_begin[unit];
@@ -852,7 +935,7 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
     const uint32_t do_free = q_free + 16;          //     next can then start while its dO is still travelling); [2] its dV^T MMAs
     const uint32_t sdp_full = do_free + 16;        // [2] S and dP of a step computed
     const uint32_t pds_ready = sdp_full + 16;      // [2] P and dS of a step are in shared memory (8 warps); S / dP have been read
-    const uint32_t pds_free = pds_ready + 16;      // [1] the MMAs that read P and dS are done
+    const uint32_t pds_free = pds_ready + 16;      // [1] the MMAs that read P and dS, and the copy of dS, are done
     const uint32_t acc_full = pds_free + 8;        // [2] the unit's sums are complete
     const uint32_t acc_free = acc_full + 16;       // [2] ... and have been read out of tensor memory
     if (tid == 0) {
@@ -870,7 +953,7 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
             mbar_init(acc_full + 8 * b, 1);
             mbar_init(acc_free + 8 * b, 1);
         }
-        mbar_init(pds_free, 1);
+        mbar_init(pds_free, 2);
         fence_mbar_init();
     }
     __syncwarp();
@@ -913,10 +996,10 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
                 else tma_load_4d(base + L::kV + b * L::kKVBytes, &tm_v, 0, u.seq0 + u.p * kBlock64, u.kvh, 0, kv_full + 8 * b);
             }
             __syncwarp();
-            int jq = u.steps > 0 ? a.qb_block[a.inv.readers[u.r_begin]] : 0;
+            int jq = u.steps > 0 ? a.qb_block[a.inv.readers[u.r_begin] / a.max_degree] : 0;
             for (int step = 0; step < u.steps; ++step, ++s) {
                 int jq_next = 0;
-                if (step + 1 < u.steps) jq_next = a.qb_block[a.inv.readers[u.r_begin + (step + 1) / pairs]];
+                if (step + 1 < u.steps) jq_next = a.qb_block[a.inv.readers[u.r_begin + (step + 1) / pairs] / a.max_degree];
                 const int sb = s & 1;
                 const uint32_t full = (first ? q_full : do_full) + 8 * sb;
                 if (s >= 2) mbar_wait((first ? q_free : do_free) + 8 * sb, ((s >> 1) - 1) & 1, abort_flag, a.status);
@@ -935,11 +1018,13 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
         // ---- MMAs: warp 2 issues S and dP of every step, warp 3 the two transposed products ----
         constexpr uint32_t kHi = desc_hi_sw128(1024);
         constexpr uint32_t kIdT = idesc_bf16_f32_ab(64, true, true);   // dV^T, dK^T: A and B MN-major
+        const size_t tiles = (size_t)a.capacity * a.max_degree;
         int s = 0;
         DkvUnit u = dkv_unit(a, 0, n_units, pairs);
         for (int n = 0; u.ok; ++n) {
             const DkvUnit un = dkv_unit(a, n + 1, n_units, pairs);
             const int b = n & 1;
+            char* ds_head = reinterpret_cast<char*>(a.ds) + (size_t)(u.kvh - a.head0) * pairs * tiles * kDsTile;
             if (warp == 2) mbar_wait(kv_full + 8 * b, (n >> 1) & 1, abort_flag, a.status);
             else if (n >= 2) mbar_wait(acc_free + 8 * b, ((n >> 1) - 1) & 1, abort_flag, a.status);
             for (int step = 0; step < u.steps; ++step, ++s) {
@@ -960,9 +1045,14 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
                     }
                     __syncwarp();
                 } else {
+                    const int entry = a.inv.readers[u.r_begin + step / pairs];
                     mbar_wait(pds_ready + 8 * sb, (s >> 1) & 1, abort_flag, a.status);
                     tc_fence_after();
                     if (elect_one()) {
+                        if (a.ds) {
+                            bulk_store(ds_head + ((step % pairs) * tiles + entry) * kDsTile, sDS, kDsTile);
+                            bulk_commit_group();
+                        }
                         // dK^T += Q^T dS, then dV^T += dO^T P: A = Q / dO MN-major (M = d: 64 per 128-byte row, next 64 at
                         // +16 KB; K = q rows, 16 per step = 2048 bytes), B = P / dS MN-major (N = 64 kv per row)
                         const uint32_t t_acc = tmem + kColAcc + b * 128;
@@ -990,12 +1080,15 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
                         mma_commit(do_free + 8 * sb);
                         mma_commit(pds_free);
                         if (step == u.steps - 1) mma_commit(acc_full + 8 * b);
+                        bulk_wait_read0();               // the copy has read the dS tile
+                        mbar_arrive(pds_free);
                     }
                     __syncwarp();
                 }
             }
             u = un;
         }
+        bulk_wait0();   // (this thread's copies of dS have landed; nothing to wait for in the other lanes and warp 2)
     } else if (warp < 12) {
         // ---- arithmetic on S and dP: two threads per tile row (head hl, token tl of the reader), warps 4-7 on key
         // columns 0..31 and warps 8-11 on columns 32..63 ----
@@ -1009,7 +1102,7 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
             // the reader of a step, its block index, the row's LSE (log2 domain) and D_i are fetched one step ahead:
             // dependent global loads that would otherwise sit between the MMAs and the arithmetic
             auto fetch = [&](int step, int& g, float& lse2, float& drow) {
-                g = a.inv.readers[u.r_begin + step / pairs];
+                g = a.inv.readers[u.r_begin + step / pairs] / a.max_degree;
                 const int jq = a.qb_block[g], pr = step % pairs;
                 const int rows_valid = min(kBlock64, u.seqlen - jq * kBlock64);
                 lse2 = INFINITY;
@@ -1089,35 +1182,233 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
     if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-// KV blocks whose readers were cut into several runs: add the runs' partial sums in run order.  Few blocks
-// need it (block 0 of a sequence, with the paper's route); the work items are (such a block, KV head, one of
-// its key rows), taken round robin by however many CTAs were launched; a thread adds one element of dK or dV.
+// KV blocks whose readers were cut into several runs: add the runs' partial sums in run order.  Few blocks need it
+// (block 0 of a sequence, with the paper's route); a work item is (such a block, KV head, one of its key rows, dK or dV),
+// one warp each.
 template <int D>
-__global__ void __launch_bounds__(2 * D) bwd_combine_kernel(const BwdArgs a) {
-    const int items = a.inv.scalars[4] * a.hkv * kBlock64;
-    const int which = threadIdx.x / D, col = threadIdx.x % D;   // 0: dK, 1: dV
-    for (int item = blockIdx.x; item < items; item += gridDim.x) {
-        const int row = item % kBlock64, kvh = (item / kBlock64) % a.hkv;
-        const int gp = a.inv.multi[item / (kBlock64 * a.hkv)];
+__device__ __forceinline__ void combine_runs(const BwdArgs& a, int worker, int workers) {
+    constexpr int kVec = D / 32;
+    const int lane = threadIdx.x & 31;
+    const int items = a.inv.scalars[4] * a.nheads * kBlock64 * 2;
+    for (int item = worker; item < items; item += workers) {
+        const int which = item & 1, row = (item >> 1) % kBlock64;   // which = 0: dK, 1: dV
+        const int hm = item / (2 * kBlock64), kvh = a.head0 + hm % a.nheads;
+        const int gp = a.inv.multi[hm / a.nheads];
         const int runs = a.inv.chunks[gp], q0 = a.inv.part0[gp];
         const int seq = a.qb_seq[gp], p = a.qb_block[gp];
         const int seq0 = a.cu_seqlens[seq];
         if (row >= a.cu_seqlens[seq + 1] - seq0 - p * kBlock64) continue;   // key row outside the sequence
-        const float* pk = a.partial + (((size_t)q0 * a.hkv + kvh) * 2 + which) * (kBlock64 * D) + row * D + col;
+        const float* pk = a.partial + (((size_t)q0 * a.hkv + kvh) * 2 + which) * (kBlock64 * D) + row * D + lane * kVec;
         const size_t run_stride = (size_t)a.hkv * 2 * kBlock64 * D;
-        float sum = 0.f;
+        float sum[kVec] = {};
 #pragma unroll 8
-        for (int r = 0; r < runs; ++r) sum += pk[r * run_stride];
-        const size_t o = ((size_t)(seq0 + p * kBlock64 + row) * a.hkv + kvh) * D + col;
-        (which ? a.dv : a.dk)[o] = __float2bfloat16_rn(sum);
+        for (int r = 0; r < runs; ++r) {
+#pragma unroll
+            for (int e = 0; e < kVec; ++e) sum[e] += pk[r * run_stride + e];
+        }
+        uint32_t* out = reinterpret_cast<uint32_t*>((which ? a.dv : a.dk) + ((size_t)(seq0 + p * kBlock64 + row) * a.hkv + kvh) * D + lane * kVec);
+#pragma unroll
+        for (int e = 0; e < kVec; e += 2) out[e / 2] = pack_bf16x2(sum[e], sum[e + 1]);
     }
+}
+template <int D>
+__global__ void __launch_bounds__(256) bwd_combine_kernel(const BwdArgs a) {
+    combine_runs<D>(a, blockIdx.x * 8 + (threadIdx.x >> 5), gridDim.x * 8);
+}
+
+// ---- dQ --------------------------------------------------------------------------------------------------------
+//
+// dQ += dS K_p over the list of a query block: 4 MMAs of 128 x d x 16 per entry.  Per entry the SM takes in 16 KB of dS
+// and 16 KB of K (d = 128) and the MMAs read as much, 512 cycles of shared-memory bandwidth; the dS tiles come from HBM once
+// they outgrow L2, which is then the bound (0.67 GB at 32K tokens, 16 query heads).
+// Measured: 19 us at 4K tokens and 155 us at 32K (recomputing S and dP: 35 and 303).
+// One persistent CTA of 10 warps per SM, units dealt out as above:
+//     warp 0    copies: the dS tile (as the dK/dV kernel left it: the K-major layout of an A operand) and the K tile of
+//               every list entry, through a ring of kDqStages
+//     warp 1    issues the MMAs; dQ accumulates in one of two buffers in tensor memory
+//     warps 2-5  the finished dQ tile of a unit, through shared memory and TMA stores
+//     warps 6-9  KV blocks whose readers were cut into several runs: the runs' partial sums of dK and dV, in run order
+constexpr int kDqThreads = 320;
+constexpr int kDqStages = 6;
+
+template <int D>
+struct DqSmem {
+    static constexpr int kKBytes = 64 * D * 2;
+    static constexpr int kStage = kDsTile + kKBytes;
+    static constexpr int kOut = kDqStages * kStage;          // 4 warps x 2 buffers x 32 rows x 64 B
+    static constexpr int kBar = kOut + 4 * 2 * 2048;
+    static constexpr int kTotal = kBar + 256;
+};
+
+template <int D>
+__global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_constant__ CUtensorMap tm_k,
+                                                            const __grid_constant__ CUtensorMap tm_dq, const BwdArgs a) {
+    using L = DqSmem<D>;
+    extern __shared__ __align__(1024) uint8_t smem[];
+    uint32_t& s_tmem = *reinterpret_cast<uint32_t*>(smem + L::kBar + 240);
+    int& s_abort = *reinterpret_cast<int*>(smem + L::kBar + 244);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (a.status && (*a.status & BF1_DEV_WAIT_TIMEOUT)) return;
+    const int nqb = min(*a.num_qblocks, a.capacity);
+    const int pairs = a.group == 4 ? 2 : 1;
+    const uint32_t base = smem_u32(smem), bars = base + L::kBar;
+    const uint32_t full = bars;                              // [kDqStages] the entry's tiles landed
+    const uint32_t free_ = full + 8 * kDqStages;             // [kDqStages] ... and have been used
+    const uint32_t acc_full = free_ + 8 * kDqStages;         // [2] the unit's dQ is complete
+    const uint32_t acc_free = acc_full + 16;                 // [2] ... and has been read out of tensor memory (4 warps)
+    static_assert(16 * kDqStages + 32 <= 240, "barriers overlap the words behind them");
+    if (tid == 0) {
+        s_abort = (base & 1023u) ? 1 : 0;
+        if (s_abort && a.status) atomicOr(a.status, BF1_DEV_WAIT_TIMEOUT);
+        for (int s = 0; s < kDqStages; ++s) {
+            mbar_init(full + 8 * s, 1);
+            mbar_init(free_ + 8 * s, 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(acc_full + 8 * b, 1);
+            mbar_init(acc_free + 8 * b, 4);
+        }
+        fence_mbar_init();
+    }
+    __syncwarp();
+    if (warp == 0) {
+        tmem_alloc(smem_u32(&s_tmem), 256);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = s_tmem;
+    volatile int* abort_flag = &s_abort;
+    if (s_abort) {   // (uniform over the CTA)
+        __syncthreads();
+        if (warp == 0) tmem_dealloc(tmem, 256);
+        return;
+    }
+    if (warp == 0) {
+        // ---- copies ----
+        const size_t tiles = (size_t)a.capacity * a.max_degree;
+        int r = 0, rs = 0, rk = 0;      // entries so far, as (stage, turn of the ring)
+        DqUnit u = dq_unit(a, 0, nqb, pairs);
+        for (int n = 0; u.ok; ++n) {
+            const DqUnit un = dq_unit(a, n + 1, nqb, pairs);
+            const int32_t* list = a.kv_idx + (size_t)u.slot * a.max_degree;
+            const char* ds = reinterpret_cast<const char*>(a.ds) +
+                             (((size_t)(u.kvh - a.head0) * pairs + u.pair) * tiles + (size_t)u.slot * a.max_degree) * kDsTile;
+            for (int it = 0; it < u.cnt; ++it) {
+                const int p = list_entry(list, it, u.cnt, u.j);
+                if (r >= kDqStages) mbar_wait(free_ + 8 * rs, (rk - 1) & 1, abort_flag, a.status);
+                if (elect_one()) {
+                    const uint32_t dst = base + rs * L::kStage;
+                    mbar_expect_tx(full + 8 * rs, L::kStage);
+                    bulk_load(dst, ds + (size_t)it * kDsTile, kDsTile, full + 8 * rs);
+                    tma_load_4d(dst + kDsTile, &tm_k, 0, u.seq0 + p * kBlock64, u.kvh, 0, full + 8 * rs);
+                }
+                __syncwarp();
+                ++r;
+                if (++rs == kDqStages) { rs = 0; ++rk; }
+            }
+            u = un;
+        }
+    } else if (warp == 1) {
+        // ---- MMAs: A = dS [128 q][64 kv] K-major (16 kv = 32 bytes per step), B = K tile MN-major (16 kv rows = 2048
+        // bytes per step, next 64 d columns 8 KB away) ----
+        constexpr uint32_t kHi = desc_hi_sw128(1024);
+        constexpr uint32_t kIdQ = idesc_bf16_f32(D, true);
+        int rs = 0;
+        uint32_t phase = 0;
+        DqUnit u = dq_unit(a, 0, nqb, pairs);
+        for (int n = 0; u.ok; ++n) {
+            const DqUnit un = dq_unit(a, n + 1, nqb, pairs);
+            const int b = n & 1;
+            if (n >= 2) mbar_wait(acc_free + 8 * b, ((n >> 1) - 1) & 1, abort_flag, a.status);
+            for (int it = 0; it < u.cnt; ++it) {
+                mbar_wait(full + 8 * rs, phase, abort_flag, a.status);
+                tc_fence_after();
+                if (elect_one()) {
+                    const uint32_t alo = desc_lo_sw128(base + rs * L::kStage, 16);
+                    const uint32_t blo = desc_lo_sw128(base + rs * L::kStage + kDsTile, 8192);
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk) {
+                        if (kk == 0 && it == 0) mma_ss_lohi<false>(tmem + b * 128, alo, blo, kHi, kIdQ);
+                        else mma_ss_lohi<true>(tmem + b * 128, alo + ((kk * 32) >> 4), blo + ((kk * 2048) >> 4), kHi, kIdQ);
+                    }
+                    mma_commit(free_ + 8 * rs);
+                    if (it == u.cnt - 1) mma_commit(acc_full + 8 * b);
+                }
+                __syncwarp();
+                if (++rs == kDqStages) { rs = 0; phase ^= 1; }
+            }
+            u = un;
+        }
+    } else if (warp < 6) {
+        // ---- finished dQ tiles: one thread per row ----
+        const int quarter = warp & 3, row = quarter * 32 + lane, hl = row >> 6, tl = row & 63;
+        const uint32_t t_lane = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
+        const uint32_t stage_w = base + L::kOut + quarter * 4096;
+        DqUnit u = dq_unit(a, 0, nqb, pairs);
+        for (int n = 0; u.ok; ++n) {
+            const DqUnit un = dq_unit(a, n + 1, nqb, pairs);
+            const int b = n & 1;
+            const int h = u.kvh * a.group + u.pair * 2 + hl;
+            const bool head_ok = u.pair * 2 + hl < a.group;   // G = 1: rows 64..127 belong to no head (warp-uniform)
+            mbar_wait(acc_full + 8 * b, (n >> 1) & 1, abort_flag, a.status);
+            tc_fence_after();
+            uint32_t pk[D / 2];
+#pragma unroll
+            for (int c = 0; c < D / 32; ++c) {
+                uint32_t v[32];
+                tmem_ld32(t_lane + b * 128 + c * 32, v);
+                tmem_wait_ld();
+#pragma unroll
+                for (int e = 0; e < 16; ++e) pk[c * 16 + e] = pack_bf16x2(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1]));
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_free + 8 * b);
+            if (head_ok && (tl | 31) < u.rows_valid) {        // all 32 rows of the warp lie in the sequence (warp-uniform)
+                const uint32_t sw = (lane >> 1) & 3;          // 64-byte swizzle: chunk ^= (row / 2) % 4
+#pragma unroll
+                for (int c = 0; c < D / 32; ++c) {            // 32 columns at a time, two staging tiles in turn
+                    const uint32_t tile = stage_w + (c & 1) * 2048;
+                    if (lane == 0) bulk_wait_read1();         // the store before the last has read its tile
+                    __syncwarp();
+#pragma unroll
+                    for (int ch = 0; ch < 4; ++ch)
+                        st_shared_v4(tile + lane * 64 + ((ch ^ sw) << 4), pk[c * 16 + ch * 4], pk[c * 16 + ch * 4 + 1],
+                                     pk[c * 16 + ch * 4 + 2], pk[c * 16 + ch * 4 + 3]);
+                    fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) {
+                        tma_store_3d(&tm_dq, c * 32, h, u.tok0 + (tl & 32), tile);
+                        bulk_commit_group();
+                    }
+                }
+            } else if (head_ok && tl < u.rows_valid) {        // the rows after these belong to someone else
+                __nv_bfloat16* dqrow = a.dq + ((size_t)(u.tok0 + tl) * a.hq + h) * D;
+#pragma unroll
+                for (int c = 0; c < D / 8; ++c)
+                    *reinterpret_cast<uint4*>(dqrow + c * 8) = make_uint4(pk[c * 4], pk[c * 4 + 1], pk[c * 4 + 2], pk[c * 4 + 3]);
+            }
+            u = un;
+        }
+        if (lane == 0) bulk_wait0();
+        __syncwarp();
+    } else {
+        combine_runs<D>(a, blockIdx.x * 4 + (warp - 6), gridDim.x * 4);
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tmem, 256);
 }
 
 int make_map_4d(CUtensorMap* m, const void* ptr, int64_t T, int H, int d, int heads_per_box, int chunks_per_box);   // bf1_attn.cu
+int make_store_map(CUtensorMap* m, void* ptr, int64_t T, int H, int d);                                             // bf1_attn.cu
 
 // Where everything lives in the caller's workspace (256-byte aligned sections).
 struct BwdLayout {
-    size_t delta, ints, partial, total;
+    size_t delta, ints, partial, ds, total;
+    int ds_heads;   // KV heads whose dS is kept at a time; 0: dS is computed again
     size_t n_count, n_start, n_chunks, n_part0, n_readers, n_units, n_multi;   // (n_units: also unit_order)
     BwdLayout(int64_t T, int hq, int hkv, int d, int cap, int max_degree) {
         auto up = [](size_t x) { return (x + 255) / 256 * 256; };
@@ -1130,9 +1421,12 @@ struct BwdLayout {
         n_multi = (size_t)cap;
         delta = 0;
         ints = up((size_t)T * hq * sizeof(float));
-        const size_t n_ints = n_count + n_start + n_chunks + n_part0 + n_readers + 5 * n_units + n_multi + 8;
+        const size_t n_ints = n_count + 2 * n_start + n_chunks + n_part0 + n_readers + 5 * n_units + n_multi + 8;
         partial = ints + up(n_ints * sizeof(int32_t));
-        total = partial + up((size_t)cap * hkv * 2 * kBlock64 * d * sizeof(float));
+        ds = partial + up((size_t)cap * hkv * 2 * kBlock64 * d * sizeof(float));
+        const int64_t per_head = (int64_t)cap * max_degree * (hq / hkv == 4 ? 2 : 1) * kDsTile;
+        ds_heads = per_head > kDsMost ? 0 : (int)std::max<int64_t>(1, std::min<int64_t>(hkv, kDsGroup / per_head));
+        total = ds + up((size_t)ds_heads * per_head);
     }
 };
 
@@ -1177,23 +1471,23 @@ extern "C" int bf1_attn_bwd(const void* q, const void* k, const void* v, const v
     static bool configured[64] = {};
     if (dev < 0 || dev >= 64) return fail(BF1_ERR_NO_DEVICE, "device ordinal %d out of range", dev);
     if (!configured[dev]) {
-        // two CTAs per SM need the whole shared-memory carve-out
+        const int kInvBytes = kInvInts * (int)sizeof(int32_t);
+        BF1_CUDA_CHECK(cudaFuncSetAttribute(bwd_prep_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kInvBytes));
+        BF1_CUDA_CHECK(cudaFuncSetAttribute(bwd_prep_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kInvBytes));
         BF1_CUDA_CHECK(cudaFuncSetAttribute(bwd_dq_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, DqSmem<128>::kTotal));
         BF1_CUDA_CHECK(cudaFuncSetAttribute(bwd_dq_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, DqSmem<64>::kTotal));
+        BF1_CUDA_CHECK(cudaFuncSetAttribute(bwd_dq_recompute_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, DqrSmem<128>::kTotal));
+        BF1_CUDA_CHECK(cudaFuncSetAttribute(bwd_dq_recompute_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, DqrSmem<64>::kTotal));
         BF1_CUDA_CHECK(cudaFuncSetAttribute(bwd_dkv_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, DkvSmem<128>::kTotal));
         BF1_CUDA_CHECK(cudaFuncSetAttribute(bwd_dkv_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, DkvSmem<64>::kTotal));
-        BF1_CUDA_CHECK(cudaFuncSetAttribute(bwd_dq_kernel<128>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
-        BF1_CUDA_CHECK(cudaFuncSetAttribute(bwd_dq_kernel<64>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
-        BF1_CUDA_CHECK(cudaFuncSetAttribute(bwd_dkv_kernel<128>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
-        BF1_CUDA_CHECK(cudaFuncSetAttribute(bwd_dkv_kernel<64>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
         configured[dev] = true;
     }
-    CUtensorMap tq, tk, tv, tg, to;
+    CUtensorMap tq, tk, tv, tg, tdq;
     // Q and dO: two heads and all column chunks per copy; with one head per KV head, one head and one chunk
     const int q_heads = group == 1 ? 1 : 2, q_chunks = group == 1 ? 1 : d / 64;
     if (int rc = make_map_4d(&tq, q, total_tokens, hq, d, q_heads, q_chunks)) return rc;
     if (int rc = make_map_4d(&tg, d_o, total_tokens, hq, d, q_heads, q_chunks)) return rc;
-    if (int rc = make_map_4d(&to, o, total_tokens, hq, d, q_heads, q_chunks)) return rc;
+    if (int rc = make_store_map(&tdq, dq, total_tokens, hq, d)) return rc;
     if (int rc = make_map_4d(&tk, k, total_tokens, hkv, d, 1, d / 64)) return rc;
     if (int rc = make_map_4d(&tv, v, total_tokens, hkv, d, 1, d / 64)) return rc;
     const int cap = route->capacity_qblocks;
@@ -1230,6 +1524,7 @@ extern "C" int bf1_attn_bwd(const void* q, const void* k, const void* v, const v
     int32_t* ip = (int32_t*)(ws + lay.ints);
     a.inv.count = ip;            ip += lay.n_count;
     a.inv.start = ip;            ip += lay.n_start;
+    a.inv.unit0 = ip;            ip += lay.n_start;
     a.inv.chunks = ip;           ip += lay.n_chunks;
     a.inv.part0 = ip;            ip += lay.n_part0;
     a.inv.readers = ip;          ip += lay.n_readers;
@@ -1245,29 +1540,49 @@ extern "C" int bf1_attn_bwd(const void* q, const void* k, const void* v, const v
     cudaStream_t st = (cudaStream_t)stream;
     int sms = 0;
     BF1_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    // the inverse route (readers of every KV block, cut into units) ...
-    if ((int64_t)cap * route->max_degree <= 4096) {
-        inverse_units_kernel<true><<<1, 1024, 0, st>>>(a);   // few entries: count, scan and fill in one CTA
-    } else {
+    // D_i of every row, and the inverse route (readers of every KV block, cut into units)
+    const bool one_cta = inverse_words(cap, route->max_degree) <= kInvInts;
+    const int prep_ctas = (int)std::min<int64_t>(sms, ((total_tokens + 15) / 16 * hq + 31) / 32);
+    if (!one_cta) {
         BF1_CUDA_CHECK(cudaMemsetAsync(a.inv.count, 0, lay.n_count * sizeof(int32_t), st));
         const int grid_inv = (int)std::min<int64_t>(((int64_t)cap * route->max_degree + 255) / 256, 4 * (int64_t)sms);
         inverse_route_kernel<false><<<grid_inv, 256, 0, st>>>(a);
-        inverse_units_kernel<false><<<1, 1024, 0, st>>>(a);
+        inverse_units_kernel<<<1, 1024, 0, st>>>(a);
         inverse_route_kernel<true><<<grid_inv, 256, 0, st>>>(a);
-    }
-    inverse_sort_kernel<<<cap, 256, 0, st>>>(a);
-    BF1_CUDA_CHECK(cudaGetLastError());
-    // ... dQ (and D_i) along the route, dK / dV along its inverse
-    const int grid_q = (int)std::min<int64_t>(sms, (int64_t)cap * hkv * (group == 4 ? 2 : 1));   // persistent: one CTA per SM
-    const int grid_kv = (int)std::min<int64_t>(sms, (int64_t)lay.n_units * hkv);
-    if (d == 128) {
-        bwd_dq_kernel<128><<<grid_q, kDqThreads, DqSmem<128>::kTotal, st>>>(tq, tk, tv, tg, to, a);
-        bwd_dkv_kernel<128><<<grid_kv, kDkvThreads, DkvSmem<128>::kTotal, st>>>(tq, tk, tv, tg, a);
-        bwd_combine_kernel<128><<<4 * sms, 256, 0, st>>>(a);
+        inverse_sort_kernel<<<cap, 256, 0, st>>>(a);
+        if (d == 128) bwd_prep_kernel<128, false><<<prep_ctas, 1024, 0, st>>>(a);
+        else bwd_prep_kernel<64, false><<<prep_ctas, 1024, 0, st>>>(a);
     } else {
-        bwd_dq_kernel<64><<<grid_q, kDqThreads, DqSmem<64>::kTotal, st>>>(tq, tk, tv, tg, to, a);
-        bwd_dkv_kernel<64><<<grid_kv, kDkvThreads, DkvSmem<64>::kTotal, st>>>(tq, tk, tv, tg, a);
-        bwd_combine_kernel<64><<<4 * sms, 128, 0, st>>>(a);
+        const int inv_bytes = (int)inverse_words(cap, route->max_degree) * (int)sizeof(int32_t);
+        if (d == 128) bwd_prep_kernel<128, true><<<prep_ctas + 1, 1024, inv_bytes, st>>>(a);
+        else bwd_prep_kernel<64, true><<<prep_ctas + 1, 1024, inv_bytes, st>>>(a);
+    }
+    BF1_CUDA_CHECK(cudaGetLastError());
+    // dK / dV along the inverse route, then dQ along the route, for as many KV heads at a time as the dS buffer holds
+    const int step = lay.ds_heads ? lay.ds_heads : hkv;
+    a.ds = lay.ds_heads ? (__nv_bfloat16*)(ws + lay.ds) : nullptr;
+    for (int h0 = 0; h0 < hkv; h0 += step) {
+        a.head0 = h0;
+        a.nheads = std::min(step, hkv - h0);
+        const int grid_q = (int)std::min<int64_t>(sms, (int64_t)cap * a.nheads * (group == 4 ? 2 : 1));   // persistent: one CTA per SM
+        const int grid_kv = (int)std::min<int64_t>(sms, (int64_t)lay.n_units * a.nheads);
+        if (d == 128) {
+            bwd_dkv_kernel<128><<<grid_kv, kDkvThreads, DkvSmem<128>::kTotal, st>>>(tq, tk, tv, tg, a);
+            if (a.ds) {
+                bwd_dq_kernel<128><<<grid_q, kDqThreads, DqSmem<128>::kTotal, st>>>(tk, tdq, a);
+            } else {
+                bwd_dq_recompute_kernel<128><<<grid_q, kDqrThreads, DqrSmem<128>::kTotal, st>>>(tq, tk, tv, tg, a);
+                bwd_combine_kernel<128><<<4 * sms, 256, 0, st>>>(a);
+            }
+        } else {
+            bwd_dkv_kernel<64><<<grid_kv, kDkvThreads, DkvSmem<64>::kTotal, st>>>(tq, tk, tv, tg, a);
+            if (a.ds) {
+                bwd_dq_kernel<64><<<grid_q, kDqThreads, DqSmem<64>::kTotal, st>>>(tk, tdq, a);
+            } else {
+                bwd_dq_recompute_kernel<64><<<grid_q, kDqrThreads, DqrSmem<64>::kTotal, st>>>(tq, tk, tv, tg, a);
+                bwd_combine_kernel<64><<<4 * sms, 256, 0, st>>>(a);
+            }
+        }
     }
     BF1_CUDA_CHECK(cudaGetLastError());
     return BF1_OK;

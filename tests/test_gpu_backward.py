@@ -216,3 +216,38 @@ def test_backward_rejects_what_it_does_not_support():
                           cu.data_ptr(), 1, 128, 128, 2, 1, 96, 0.0, route.c, q.data_ptr(), q.data_ptr(), q.data_ptr(),
                           q.data_ptr(), None)
     assert rc == -2 and b"dimension" in lib.bf1_last_error()  # d = 96
+
+
+@pytest.mark.parametrize("hq,hkv,d", [(4, 2, 128), (8, 2, 64), (2, 2, 128)], ids=["G2-d128", "G4-d64", "G1-d128"])
+@pytest.mark.parametrize("tiles_bytes", [300 << 20, 700 << 20, 9 << 30], ids=["several-launches", "head-by-head", "recompute"])
+def test_backward_does_not_depend_on_the_row_pitch_of_the_lists(hq, hkv, d, tiles_bytes):
+    """The pitch of the lists sizes the workspace, and its size chooses how dS is kept (all heads, head by head, not at
+    all) and how the inverse route is made (one CTA or several launches).  A pitch far wider than the lists takes a
+    small problem through each choice; the gradients are those of the ordinary pitch.  Recomputed dS has the same bits
+    (same MMAs, same D), only its sum runs through other instructions: fp32 sums of at most 448 products of O(1) in
+    another order differ by 448 * 2^-24 relative to the sum of magnitudes, far below a bf16 step (2^-8), so an element
+    moves by one step at most."""
+    dev = torch.device("cuda:0")
+    w = I.custom([897, 130], hq=hq, hkv=hkv, d=d, seed=6900 + d + hq)
+    q, k, v = (t.to(dev) for t in I.draw_qkv(w))
+    d_o = torch.randn(q.shape, generator=torch.Generator().manual_seed(10)).to(torch.bfloat16).to(dev)
+    cu = bf1.cu_seqlens_tensor(w.seqlens, dev)
+
+    def grads(pitch):
+        cap, deg = bf1.route_capacity(len(w.seqlens), w.total_tokens, w.max_seqlen)
+        route = bf1.plan_route(cu, w.max_seqlen, route=bf1.Route.empty(cap, pitch or deg, dev))
+        o, lse = bf1.attn_fwd(q, k, v, cu, w.max_seqlen, route)
+        out = bf1.attn_bwd(q, k, v, o, lse, d_o, cu, w.max_seqlen, route)
+        torch.cuda.synchronize()
+        route.check_status()
+        return out
+
+    cap, _ = bf1.route_capacity(len(w.seqlens), w.total_tokens, w.max_seqlen)
+    pairs = 2 if hq == 4 * hkv else 1
+    base, wide = grads(None), grads(tiles_bytes // (cap * pairs * 16384))
+    for name, x, y in zip(("dq", "dk", "dv"), base, wide):
+        if tiles_bytes > 8 << 30 and name == "dq":
+            diff = (x.float() - y.float()).abs()
+            assert bool((diff <= 2.0 ** -7 * x.float().abs() + 1e-6).all()), float(diff.max())
+        else:
+            assert torch.equal(x, y), name
