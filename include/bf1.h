@@ -236,8 +236,10 @@ int bf1_decode_fwd(const void *q, const void *k_pages, const void *v_pages, int3
  * at a time over the query blocks that read it), which the call derives from the lists itself: no
  * floating-point atomics anywhere, so all three gradients come out bit-identical on every run.
  * `workspace` (bf1_attn_bwd_workspace_bytes() bytes, 256-byte aligned, contents irrelevant on entry)
- * holds the row terms <d_o, o>, the inverse route and the partial sums of KV blocks with very many
- * readers.  Geometry limits as bf1_attn_fwd.  `route` must be the forward's (host struct; only its
+ * holds the row terms <d_o, o>, the inverse route, the partial sums of KV blocks with very many readers
+ * and, 16 KB per list entry and pair of query heads, the terms dS that dk, dv and dq share (for as many KV
+ * heads at a time as fit 1 GiB, at least one; none when one alone would take more than 8 GiB: they are
+ * then computed twice).  Geometry limits as bf1_attn_fwd.  `route` must be the forward's (host struct; only its
  * capacities are used by the size helper). */
 int64_t bf1_attn_bwd_workspace_bytes(const bf1_route *route /* host */, int64_t total_tokens,
                                      int32_t hq, int32_t hkv, int32_t d);

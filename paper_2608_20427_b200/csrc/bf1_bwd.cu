@@ -57,11 +57,9 @@ struct InvPlan {
     int32_t* chunks;      // [cap] runs the slot's readers are cut into
     int32_t* part0;       // [cap] first partial-sum slot of a slot with more than one run, else -1
     int32_t* readers;     // [cap * max_degree] list entries (query slot * max_degree + place), ascending per KV slot
-    int32_t* unit_slot;   // [max_units] KV slot of the unit
-    int32_t* unit_begin;  // [max_units] its readers: readers[begin .. end)
-    int32_t* unit_end;
-    int32_t* unit_part;   // [max_units] partial-sum slot it writes, or -1: it writes the final bf16 rows
-    int32_t* unit_order;  // [max_units] units, longest first: the order in which the dK/dV kernel deals them out
+    int4* units;          // [max_units][2] longest first: {KV slot, first reader, readers, partial-sum slot or -1 (it
+                          // writes the final bf16 rows)}, {first token of the sequence, block, tokens of the sequence, -}
+    int32_t* tickets;     // [hkv] hand-out counters of the dK/dV launches, by first KV head
     int32_t* multi;       // [cap] the KV slots whose readers were cut into more than one run
     int32_t* scalars;     // [8] number of units, total readers, chunk, partial slots, slots in `multi`
     int32_t cap, max_units;
@@ -655,6 +653,7 @@ __device__ __forceinline__ void inverse_units(const BwdArgs& a, int32_t* smem) {
     };
     auto count_of = [&](int g) { return kAll ? count[g] : __ldcg(count + g); };   // (written by atomics: read where they were performed)
     s_bin[tid] = 0;
+    for (int i = tid; i < a.hkv; i += 1024) v.tickets[i] = 0;
     if (kAll) {
         for (int g = tid; g < nqb; g += 1024) count[g] = 0;
         __syncthreads();
@@ -740,11 +739,6 @@ __device__ __forceinline__ void inverse_units(const BwdArgs& a, int32_t* smem) {
         for (int un = tid; un < units; un += 1024) {
             int g, begin, end;
             unit_of(un, g, begin, end);
-            v.unit_slot[un] = g;
-            v.unit_begin[un] = begin;
-            v.unit_end[un] = end;
-            const bool split = unit0[g + 1] - unit0[g] > 1;
-            v.unit_part[un] = split ? v.part0[g] + un - unit0[g] : -1;
             atomicAdd(&s_bin[bin_of(end - begin)], 1);
         }
     }
@@ -762,7 +756,11 @@ __device__ __forceinline__ void inverse_units(const BwdArgs& a, int32_t* smem) {
         for (int un = tid; un < units; un += 1024) {
             int g, begin, end;
             unit_of(un, g, begin, end);
-            v.unit_order[atomicAdd(&s_bin[bin_of(end - begin)], 1)] = un;
+            const int at = atomicAdd(&s_bin[bin_of(end - begin)], 1), seq = a.qb_seq[g];
+            const bool split = unit0[g + 1] - unit0[g] > 1;
+            const int seq0 = a.cu_seqlens[seq];
+            v.units[2 * at] = make_int4(g, begin, end - begin, split ? v.part0[g] + un - unit0[g] : -1);
+            v.units[2 * at + 1] = make_int4(seq0, a.qb_block[g], a.cu_seqlens[seq + 1] - seq0, 0);
         }
     }
     if (kAll) {
@@ -844,17 +842,35 @@ __global__ void __launch_bounds__(1024, 1) bwd_prep_kernel(const BwdArgs a) {
 // ---- dK, dV ----------------------------------------------------------------------------------------------------
 //
 // One persistent CTA of 16 warps per SM.  A unit is (KV block, KV head, run of the block's readers); units are
-// dealt out statically KV head by KV head, back and forth over the CTAs.  K and V of a unit stay in shared memory
-// (two buffers: the next unit's arrive early), Q and dO of every step (a reader and a pair of its heads) travel
-// through a ring of two stages:
-//     warp 0    copies K of every unit and Q of every step;  warp 1: V and dO
+// handed out through a counter, longest first (KV head by KV head, or all heads together: BwdArgs::interleave).  K and V
+// of a unit stay in shared memory (two buffers: the next unit's arrive early), Q and dO of every step (a reader and a
+// pair of its heads) travel through a ring of two stages:
+//     warp 0    takes the units and describes them to the other roles; copies K of every unit and Q of every step;
+//               brings every step's LSE into shared memory
+//     warp 1    copies V and dO; brings D_i into shared memory
 //     warp 2    issues S = Q K^T and dP = dO V^T of every step into one of two S/dP buffers in tensor memory
 //     warp 3    issues dV^T += dO^T P and dK^T += Q^T dS of every step; the sums stay in one of two accumulator
 //               buffers in tensor memory across all steps of the unit.  It also starts the copy of every dS tile to
 //               the workspace, as it lies in shared memory: its own MMAs read the tile at the same time
 //     warps 4-11   the arithmetic on S and dP (two threads per tile row), P and dS as bf16 tiles to shared memory
 //     warps 12-15  the finished sums of the unit before, from tensor memory to global memory
+// A step moves 304 KB through shared memory (192 KB of MMA operands, 64 KB in, P and dS written, dS read again):
+// 2375 cycles at 128 bytes per cycle, which is the bound.
+// Units described through shared memory, LSE and D_i brought there a step ahead and dynamic hand-out: 55 -> 46 us at 4K
+// tokens, 96 -> 76 us for 16K tokens in 12 sequences (four heads per KV head), 544 -> 483 us at 32K.  (Every role read the
+// unit and the rows' LSE from global memory itself before: 940 of 2900 cycles of a step in the arithmetic warps; and
+// the static deal left the busiest CTA 23 %, 35 % and 9 % above the mean.)
 constexpr int kDkvThreads = 512;
+
+// What warp 0 tells the other roles about a unit.
+struct DkvUnit {
+    int steps;                      // 0: no more units
+    int kvh, part, gp, p, seq0, seqlen, r_begin;
+    int first[32];                  // its first 32 readers (list entries)
+};
+struct DkvStep {
+    int entry, diag;                // the reader, and whether it is the unit's own block
+};
 
 template <int D>
 struct DkvSmem {
@@ -866,49 +882,15 @@ struct DkvSmem {
     static constexpr int kV = kK + 2 * kKVBytes;     // [2]
     static constexpr int kP = kV + 2 * kKVBytes;     // P  [128 q rows][64 kv] bf16, 128-byte rows, swizzled
     static constexpr int kDS = kP + 16384;           // dS likewise
-    static constexpr int kBar = kDS + 16384;
-    static constexpr int kUsed = kBar + 512;
+    static constexpr int kRow = kDS + 16384;         // LSE (log2 domain) [2][128], D_i [2][128]
+    static constexpr int kUnit = kRow + 4 * 512;     // DkvUnit [2]
+    static constexpr int kStep = kUnit + 2 * (int)sizeof(DkvUnit);   // DkvStep [2]
+    static constexpr int kBar = kStep + 2 * (int)sizeof(DkvStep);
+    static constexpr int kUsed = kBar + 8 * 25 + 8;
     // at least this much is requested so that a second CTA never fits an SM: each allocates all of tensor memory
     static constexpr int kTotal = kUsed > 120 * 1024 ? kUsed : 120 * 1024;
 };
-
-struct DkvUnit {
-    int ok, gp, kvh, r_begin, steps, part, seq0, seqlen, p, kv_valid;
-};
-
-// Unit n of this CTA.
-__device__ __forceinline__ DkvUnit dkv_unit(const BwdArgs& a, int n, int n_units, int pairs) {
-    DkvUnit u;
-    const int total = n_units * a.nheads;
-    const int G = gridDim.x;
-    const int i = n * G + ((n & 1) ? G - 1 - (int)blockIdx.x : (int)blockIdx.x);
-    u.ok = i < total;
-    u.gp = u.kvh = u.r_begin = u.seq0 = u.seqlen = u.p = u.kv_valid = 0;
-    u.steps = 0;
-    u.part = -1;
-    if (u.ok) {
-        int ui;
-        if (a.interleave) {
-            ui = i / a.nheads;
-            u.kvh = i - ui * a.nheads;
-        } else {
-            u.kvh = i / n_units;
-            ui = i - u.kvh * n_units;
-        }
-        u.kvh += a.head0;
-        const int unit = a.inv.unit_order[ui];
-        u.gp = a.inv.unit_slot[unit];
-        u.r_begin = a.inv.unit_begin[unit];
-        u.steps = (a.inv.unit_end[unit] - u.r_begin) * pairs;
-        u.part = a.inv.unit_part[unit];
-        const int seq = a.qb_seq[u.gp];
-        u.p = a.qb_block[u.gp];
-        u.seq0 = a.cu_seqlens[seq];
-        u.seqlen = a.cu_seqlens[seq + 1] - u.seq0;
-        u.kv_valid = min(kBlock64, u.seqlen - u.p * kBlock64);      // key rows of this block inside the sequence
-    }
-    return u;
-}
+static_assert(DkvSmem<128>::kTotal <= 227 * 1024, "shared memory of an SM");
 
 template <int D>
 __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_constant__ CUtensorMap tm_q,
@@ -918,8 +900,12 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
                                                               const BwdArgs a) {
     using L = DkvSmem<D>;
     extern __shared__ __align__(1024) uint8_t smem[];
-    uint32_t& s_tmem = *reinterpret_cast<uint32_t*>(smem + L::kBar + 496);
-    int& s_abort = *reinterpret_cast<int*>(smem + L::kBar + 500);
+    uint32_t& s_tmem = *reinterpret_cast<uint32_t*>(smem + L::kBar + 8 * 25);
+    int& s_abort = *reinterpret_cast<int*>(smem + L::kBar + 8 * 25 + 4);
+    volatile DkvUnit* s_unit = reinterpret_cast<volatile DkvUnit*>(smem + L::kUnit);
+    volatile DkvStep* s_step = reinterpret_cast<volatile DkvStep*>(smem + L::kStep);
+    volatile float* s_lse = reinterpret_cast<volatile float*>(smem + L::kRow);
+    volatile float* s_delta = s_lse + 256;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (a.status && (*a.status & BF1_DEV_WAIT_TIMEOUT)) return;
     const int n_units = a.inv.scalars[0];
@@ -929,29 +915,33 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
     const uint32_t bars = base + L::kBar;
     const uint32_t kv_full = bars;                 // [2] K and V of a unit landed (both copy warps announce bytes)
     const uint32_t kv_free = kv_full + 16;         // [2] the unit's S / dP MMAs are done
-    const uint32_t q_full = kv_free + 16;          // [2] Q of a step landed
-    const uint32_t do_full = q_full + 16;          // [2] dO of a step landed
+    const uint32_t q_full = kv_free + 16;          // [2] Q of a step landed; its LSE and DkvStep are written
+    const uint32_t do_full = q_full + 16;          // [2] dO of a step landed; its D_i are written
     const uint32_t q_free = do_full + 16;          // [2] the step's dK^T MMAs are done (they come first: S of the step after
     const uint32_t do_free = q_free + 16;          //     next can then start while its dO is still travelling); [2] its dV^T MMAs
     const uint32_t sdp_full = do_free + 16;        // [2] S and dP of a step computed
     const uint32_t pds_ready = sdp_full + 16;      // [2] P and dS of a step are in shared memory (8 warps); S / dP have been read
-    const uint32_t pds_free = pds_ready + 16;      // [1] the MMAs that read P and dS, and the copy of dS, are done
-    const uint32_t acc_full = pds_free + 8;        // [2] the unit's sums are complete
+    const uint32_t acc_full = pds_ready + 16;      // [2] the unit's sums are complete
     const uint32_t acc_free = acc_full + 16;       // [2] ... and have been read out of tensor memory
+    const uint32_t unit_full = acc_free + 16;      // [2] the unit is described
+    const uint32_t unit_free = unit_full + 16;     // [2] ... and every other warp has read the description
+    const uint32_t pds_free = unit_free + 16;      // [1] the MMAs that read P and dS, and the copy of dS, are done
     if (tid == 0) {
         s_abort = (base & 1023u) ? 1 : 0;
         if (s_abort && a.status) atomicOr(a.status, BF1_DEV_WAIT_TIMEOUT);
         for (int b = 0; b < 2; ++b) {
             mbar_init(kv_full + 8 * b, 2);
             mbar_init(kv_free + 8 * b, 1);
-            mbar_init(q_full + 8 * b, 1);
-            mbar_init(do_full + 8 * b, 1);
+            mbar_init(q_full + 8 * b, 2);
+            mbar_init(do_full + 8 * b, 2);
             mbar_init(q_free + 8 * b, 1);
             mbar_init(do_free + 8 * b, 1);
             mbar_init(sdp_full + 8 * b, 1);
             mbar_init(pds_ready + 8 * b, 8);
             mbar_init(acc_full + 8 * b, 1);
             mbar_init(acc_free + 8 * b, 1);
+            mbar_init(unit_full + 8 * b, 1);
+            mbar_init(unit_free + 8 * b, 15);
         }
         mbar_init(pds_free, 2);
         fence_mbar_init();
@@ -980,39 +970,119 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
     constexpr uint32_t kColDP = 64, kColAcc = 256, kColDKt = 64;
     const uint32_t q_tx = a.group > 1 ? L::kQBytes : L::kQBytes / 2;   // one head per KV head: half a tile per copy set
     const uint32_t sP = base + L::kP, sDS = base + L::kDS;
+    // the description of unit n; a warp that is done with it says so
+    auto wait_unit = [&](int n) -> volatile DkvUnit& {
+        mbar_wait(unit_full + 8 * (n & 1), (n >> 1) & 1, abort_flag, a.status);
+        return s_unit[n & 1];
+    };
+    auto free_unit = [&](int n) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(unit_free + 8 * (n & 1));
+    };
+    auto unit_steps = [&](volatile DkvUnit& u) { return *abort_flag ? 0 : u.steps; };
 
     if (warp == 0 || warp == 1) {
-        // ---- copies ----
+        // ---- copies (and, in warp 0, the units) ----
         const bool first = warp == 0;
+        const uint32_t full = first ? q_full : do_full, free_ = first ? q_free : do_free;
+        const float* rows = first ? a.lse : a.delta;
+        volatile float* s_row = first ? s_lse : s_delta;
+        // warp 0's next unit, taken and read a few steps before it is needed: ticket, then description, then readers
+        const int total = n_units * a.nheads;
+        int next_i = blockIdx.x, next_kvh = 0, next_f = 0;
+        int4 next_a = make_int4(0, 0, 0, -1), next_b = make_int4(0, 0, 0, 0);
+        auto take = [&]() { if (lane == 0) next_i = (int)gridDim.x + atomicAdd(a.inv.tickets + a.head0, 1); };
+        auto describe = [&]() {
+            next_i = __shfl_sync(0xffffffffu, next_i, 0);
+            next_a.z = 0;
+            if (next_i < total) {
+                int ui;
+                if (a.interleave) {
+                    ui = next_i / a.nheads;
+                    next_kvh = next_i - ui * a.nheads;
+                } else {
+                    next_kvh = next_i / n_units;
+                    ui = next_i - next_kvh * n_units;
+                }
+                next_kvh += a.head0;
+                next_a = a.inv.units[2 * ui];
+                next_b = a.inv.units[2 * ui + 1];
+            }
+        };
+        auto read_readers = [&]() { next_f = lane < next_a.z ? a.inv.readers[next_a.y + lane] : 0; };
+        if (first) {
+            describe();
+            read_readers();
+        }
         int s = 0;   // steps so far
-        DkvUnit u = dkv_unit(a, 0, n_units, pairs);
-        for (int n = 0; u.ok; ++n) {
-            const DkvUnit un = dkv_unit(a, n + 1, n_units, pairs);
+        for (int n = 0;; ++n) {
             const int b = n & 1;
+            if (first) {
+                if (n >= 2) mbar_wait(unit_free + 8 * b, ((n >> 1) - 1) & 1, abort_flag, a.status);
+                volatile DkvUnit& d = s_unit[b];
+                d.first[lane] = next_f;
+                if (lane == 0) {
+                    d.steps = next_a.z * pairs;
+                    d.kvh = next_kvh;
+                    d.part = next_a.w;
+                    d.gp = next_a.x;
+                    d.p = next_b.y;
+                    d.seq0 = next_b.x;
+                    d.seqlen = next_b.z;
+                    d.r_begin = next_a.y;
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(unit_full + 8 * b);
+            }
+            volatile DkvUnit& u = wait_unit(n);
+            const int steps = unit_steps(u), kvh = u.kvh, gp = u.gp, p = u.p, seq0 = u.seq0, seqlen = u.seqlen, r_begin = u.r_begin;
+            int my_f = u.first[lane];
+            if (!first) free_unit(n);
+            if (steps == 0) break;
             if (n >= 2) mbar_wait(kv_free + 8 * b, ((n >> 1) - 1) & 1, abort_flag, a.status);
             if (elect_one()) {
                 mbar_expect_tx(kv_full + 8 * b, L::kKVBytes);
-                if (first) tma_load_4d(base + L::kK + b * L::kKVBytes, &tm_k, 0, u.seq0 + u.p * kBlock64, u.kvh, 0, kv_full + 8 * b);
-                else tma_load_4d(base + L::kV + b * L::kKVBytes, &tm_v, 0, u.seq0 + u.p * kBlock64, u.kvh, 0, kv_full + 8 * b);
+                if (first) tma_load_4d(base + L::kK + b * L::kKVBytes, &tm_k, 0, seq0 + p * kBlock64, kvh, 0, kv_full + 8 * b);
+                else tma_load_4d(base + L::kV + b * L::kKVBytes, &tm_v, 0, seq0 + p * kBlock64, kvh, 0, kv_full + 8 * b);
             }
             __syncwarp();
-            int jq = u.steps > 0 ? a.qb_block[a.inv.readers[u.r_begin] / a.max_degree] : 0;
-            for (int step = 0; step < u.steps; ++step, ++s) {
-                int jq_next = 0;
-                if (step + 1 < u.steps) jq_next = a.qb_block[a.inv.readers[u.r_begin + (step + 1) / pairs] / a.max_degree];
-                const int sb = s & 1;
-                const uint32_t full = (first ? q_full : do_full) + 8 * sb;
-                if (s >= 2) mbar_wait((first ? q_free : do_free) + 8 * sb, ((s >> 1) - 1) & 1, abort_flag, a.status);
+            for (int step = 0; step < steps; ++step, ++s) {
+                const int sb = s & 1, idx = step / pairs, pr = step % pairs;
+                if (idx >= 32 && (idx & 31) == 0 && pr == 0)        // runs longer than a warp: the next 32 readers
+                    my_f = r_begin + idx + lane < r_begin + steps / pairs ? a.inv.readers[r_begin + idx + lane] : 0;
+                const int f = __shfl_sync(0xffffffffu, my_f, idx & 31), g = f / a.max_degree;
+                const int jq = g - gp + p;                          // slots of a sequence are consecutive
+                const int head0 = kvh * a.group + pr * 2, rows_valid = min(kBlock64, seqlen - jq * kBlock64);
+                // this step's LSE / D_i, four rows a lane: asked for now, put into shared memory behind the copy
+                float v[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int row = i * 32 + lane, hl = row >> 6, tl = row & 63;
+                    v[i] = first ? INFINITY : 0.f;                  // rows outside: P = 0
+                    if (tl < rows_valid && pr * 2 + hl < a.group)
+                        v[i] = rows[(size_t)(head0 + hl) * a.total_tokens + seq0 + jq * kBlock64 + tl];
+                }
+                if (s >= 2) mbar_wait(free_ + 8 * sb, ((s >> 1) - 1) & 1, abort_flag, a.status);
                 if (elect_one()) {
-                    mbar_expect_tx(full, q_tx);
-                    const int head0 = u.kvh * a.group + (step % pairs) * 2;
-                    if (first) load_q_tile<D>(base + L::kQ + sb * L::kQBytes, &tm_q, u.seq0 + jq * kBlock64, head0, a.group, full);
-                    else load_q_tile<D>(base + L::kDO + sb * L::kQBytes, &tm_do, u.seq0 + jq * kBlock64, head0, a.group, full);
+                    mbar_expect_tx(full + 8 * sb, q_tx);
+                    if (first) load_q_tile<D>(base + L::kQ + sb * L::kQBytes, &tm_q, seq0 + jq * kBlock64, head0, a.group, full + 8 * sb);
+                    else load_q_tile<D>(base + L::kDO + sb * L::kQBytes, &tm_do, seq0 + jq * kBlock64, head0, a.group, full + 8 * sb);
                 }
                 __syncwarp();
-                jq = jq_next;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) s_row[sb * 128 + i * 32 + lane] = first ? v[i] * 1.4426950408889634f : v[i];
+                if (first && lane == 0) {
+                    s_step[sb].entry = f;
+                    s_step[sb].diag = g == gp;
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(full + 8 * sb);
+                if (first) {
+                    if (step == max(steps - 3, 0)) take();
+                    if (step == max(steps - 2, 0)) describe();
+                    if (step == steps - 1) read_readers();
+                }
             }
-            u = un;
         }
     } else if (warp == 2 || warp == 3) {
         // ---- MMAs: warp 2 issues S and dP of every step, warp 3 the two transposed products ----
@@ -1020,14 +1090,16 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
         constexpr uint32_t kIdT = idesc_bf16_f32_ab(64, true, true);   // dV^T, dK^T: A and B MN-major
         const size_t tiles = (size_t)a.capacity * a.max_degree;
         int s = 0;
-        DkvUnit u = dkv_unit(a, 0, n_units, pairs);
-        for (int n = 0; u.ok; ++n) {
-            const DkvUnit un = dkv_unit(a, n + 1, n_units, pairs);
+        for (int n = 0;; ++n) {
+            volatile DkvUnit& u = wait_unit(n);
+            const int steps = unit_steps(u), kvh = u.kvh;
+            free_unit(n);
+            if (steps == 0) break;
             const int b = n & 1;
-            char* ds_head = reinterpret_cast<char*>(a.ds) + (size_t)(u.kvh - a.head0) * pairs * tiles * kDsTile;
+            char* ds_head = reinterpret_cast<char*>(a.ds) + (size_t)(kvh - a.head0) * pairs * tiles * kDsTile;
             if (warp == 2) mbar_wait(kv_full + 8 * b, (n >> 1) & 1, abort_flag, a.status);
             else if (n >= 2) mbar_wait(acc_free + 8 * b, ((n >> 1) - 1) & 1, abort_flag, a.status);
-            for (int step = 0; step < u.steps; ++step, ++s) {
+            for (int step = 0; step < steps; ++step, ++s) {
                 const int sb = s & 1;
                 const uint32_t sQ = base + L::kQ + sb * L::kQBytes, sDO = base + L::kDO + sb * L::kQBytes;
                 if (warp == 2) {
@@ -1041,11 +1113,12 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
                     if (elect_one()) {
                         issue_qk<D>(tmem + sb * 128 + kColDP, sDO, base + L::kV + b * L::kKVBytes);
                         mma_commit(sdp_full + 8 * sb);
-                        if (step == u.steps - 1) mma_commit(kv_free + 8 * b);
+                        if (step == steps - 1) mma_commit(kv_free + 8 * b);
                     }
                     __syncwarp();
                 } else {
-                    const int entry = a.inv.readers[u.r_begin + step / pairs];
+                    mbar_wait(q_full + 8 * sb, (s >> 1) & 1, abort_flag, a.status);   // (DkvStep)
+                    const int entry = s_step[sb].entry;
                     mbar_wait(pds_ready + 8 * sb, (s >> 1) & 1, abort_flag, a.status);
                     tc_fence_after();
                     if (elect_one()) {
@@ -1079,14 +1152,13 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
                         }
                         mma_commit(do_free + 8 * sb);
                         mma_commit(pds_free);
-                        if (step == u.steps - 1) mma_commit(acc_full + 8 * b);
+                        if (step == steps - 1) mma_commit(acc_full + 8 * b);
                         bulk_wait_read0();               // the copy has read the dS tile
                         mbar_arrive(pds_free);
                     }
                     __syncwarp();
                 }
             }
-            u = un;
         }
         bulk_wait0();   // (this thread's copies of dS have landed; nothing to wait for in the other lanes and warp 2)
     } else if (warp < 12) {
@@ -1094,35 +1166,23 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
         // columns 0..31 and warps 8-11 on columns 32..63 ----
         const int half = (warp - 4) >> 2;
         const uint32_t t_lane = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
-        const int row = tid & 127, hl = row >> 6, tl = row & 63;
+        const int row = tid & 127, tl = row & 63;
         int s = 0;
-        DkvUnit u = dkv_unit(a, 0, n_units, pairs);
-        for (int n = 0; u.ok; ++n) {
-            const DkvUnit un = dkv_unit(a, n + 1, n_units, pairs);
-            // the reader of a step, its block index, the row's LSE (log2 domain) and D_i are fetched one step ahead:
-            // dependent global loads that would otherwise sit between the MMAs and the arithmetic
-            auto fetch = [&](int step, int& g, float& lse2, float& drow) {
-                g = a.inv.readers[u.r_begin + step / pairs] / a.max_degree;
-                const int jq = a.qb_block[g], pr = step % pairs;
-                const int rows_valid = min(kBlock64, u.seqlen - jq * kBlock64);
-                lse2 = INFINITY;
-                drow = 0.f;
-                if (tl < rows_valid && pr * 2 + hl < a.group) {
-                    const size_t at = (size_t)(u.kvh * a.group + pr * 2 + hl) * a.total_tokens + u.seq0 + jq * kBlock64 + tl;
-                    lse2 = a.lse[at] * 1.4426950408889634f;
-                    drow = a.delta[at];
-                }
-            };
-            int g = 0, g_next = 0;
-            float lse2 = INFINITY, drow = 0.f, lse2_next = INFINITY, drow_next = 0.f;
-            if (u.steps > 0) fetch(0, g, lse2, drow);
-            for (int step = 0; step < u.steps; ++step, ++s) {
-                if (step + 1 < u.steps) fetch(step + 1, g_next, lse2_next, drow_next);
+        for (int n = 0;; ++n) {
+            volatile DkvUnit& u = wait_unit(n);
+            const int steps = unit_steps(u);
+            free_unit(n);
+            if (steps == 0) break;
+            for (int step = 0; step < steps; ++step, ++s) {
                 const int sb = s & 1;
+                mbar_wait(q_full + 8 * sb, (s >> 1) & 1, abort_flag, a.status);
+                mbar_wait(do_full + 8 * sb, (s >> 1) & 1, abort_flag, a.status);
+                const float lse2 = s_lse[sb * 128 + row], drow = s_delta[sb * 128 + row];
+                const bool diag = s_step[sb].diag;
                 mbar_wait(sdp_full + 8 * sb, (s >> 1) & 1, abort_flag, a.status);
                 tc_fence_after();
                 uint32_t pw[16], dw[16];
-                p_and_ds(t_lane + sb * 128, t_lane + sb * 128 + kColDP, half, tl, g == u.gp, lse2, drow, a.scale, a.scale_log2, pw, dw);
+                p_and_ds(t_lane + sb * 128, t_lane + sb * 128 + kColDP, half, tl, diag, lse2, drow, a.scale, a.scale_log2, pw, dw);
                 if (s >= 1) mbar_wait(pds_free, (s - 1) & 1, abort_flag, a.status);   // the MMAs of the step before have read P and dS
                 store_row_piece(sP + row * 128, row, half, pw);
                 store_row_piece(sDS + row * 128, row, half, dw);
@@ -1130,51 +1190,49 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(pds_ready + 8 * sb);
-                g = g_next, lse2 = lse2_next, drow = drow_next;
             }
-            u = un;
         }
     } else {
         // ---- the finished dV^T / dK^T of a unit: lane = head-dimension index, 64 key rows along the columns ----
         const uint32_t t_lane = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
         const int row = tid & 127;
-        DkvUnit u = dkv_unit(a, 0, n_units, pairs);
-        for (int n = 0; u.ok; ++n) {
-            const DkvUnit un = dkv_unit(a, n + 1, n_units, pairs);
+        for (int n = 0;; ++n) {
+            volatile DkvUnit& u = wait_unit(n);
+            const int steps = unit_steps(u), kvh = u.kvh, part = u.part, tok0 = u.seq0 + u.p * kBlock64;
+            const int kv_valid = min(kBlock64, u.seqlen - u.p * kBlock64);      // key rows of this block inside the sequence
+            free_unit(n);
+            if (steps == 0) break;
             const int b = n & 1;
-            if (u.steps > 0) {
-                mbar_wait(acc_full + 8 * b, (n >> 1) & 1, abort_flag, a.status);
-                tc_fence_after();
-                if (row < D) {   // d = 64: lanes 64..127 hold nothing (warp-uniform)
-                    const size_t rstride = (size_t)a.hkv * D;
-                    const size_t row0 = ((size_t)(u.seq0 + u.p * kBlock64) * a.hkv + u.kvh) * D + row;
-                    float* pk = u.part >= 0 ? a.partial + (((size_t)u.part * a.hkv + u.kvh) * 2) * (kBlock64 * D) + row : nullptr;
+            mbar_wait(acc_full + 8 * b, (n >> 1) & 1, abort_flag, a.status);
+            tc_fence_after();
+            if (row < D) {   // d = 64: lanes 64..127 hold nothing (warp-uniform)
+                const size_t rstride = (size_t)a.hkv * D;
+                const size_t row0 = ((size_t)tok0 * a.hkv + kvh) * D + row;
+                float* pk = part >= 0 ? a.partial + (((size_t)part * a.hkv + kvh) * 2) * (kBlock64 * D) + row : nullptr;
 #pragma unroll 1
-                    for (int hh = 0; hh < 2; ++hh) {
-                        uint32_t vr[32], kr[32];
-                        tmem_ld32(t_lane + kColAcc + b * 128 + hh * 32, vr);
-                        tmem_ld32(t_lane + kColAcc + b * 128 + kColDKt + hh * 32, kr);
-                        tmem_wait_ld();
+                for (int hh = 0; hh < 2; ++hh) {
+                    uint32_t vr[32], kr[32];
+                    tmem_ld32(t_lane + kColAcc + b * 128 + hh * 32, vr);
+                    tmem_ld32(t_lane + kColAcc + b * 128 + kColDKt + hh * 32, kr);
+                    tmem_wait_ld();
 #pragma unroll
-                        for (int c = 0; c < 32; ++c) {
-                            const int kvr = hh * 32 + c;
-                            if (kvr < u.kv_valid) {
-                                if (u.part < 0) {
-                                    a.dv[row0 + kvr * rstride] = __float2bfloat16_rn(__uint_as_float(vr[c]));
-                                    a.dk[row0 + kvr * rstride] = __float2bfloat16_rn(__uint_as_float(kr[c]));
-                                } else {
-                                    pk[kvr * D] = __uint_as_float(kr[c]);
-                                    pk[kBlock64 * D + kvr * D] = __uint_as_float(vr[c]);
-                                }
+                    for (int c = 0; c < 32; ++c) {
+                        const int kvr = hh * 32 + c;
+                        if (kvr < kv_valid) {
+                            if (part < 0) {
+                                a.dv[row0 + kvr * rstride] = __float2bfloat16_rn(__uint_as_float(vr[c]));
+                                a.dk[row0 + kvr * rstride] = __float2bfloat16_rn(__uint_as_float(kr[c]));
+                            } else {
+                                pk[kvr * D] = __uint_as_float(kr[c]);
+                                pk[kBlock64 * D + kvr * D] = __uint_as_float(vr[c]);
                             }
                         }
                     }
                 }
-                tc_fence_before();
-                named_sync(1, 128);
-                if ((tid & 127) == 0) mbar_arrive(acc_free + 8 * b);
             }
-            u = un;
+            tc_fence_before();
+            named_sync(1, 128);
+            if ((tid & 127) == 0) mbar_arrive(acc_free + 8 * b);
         }
     }
     tc_fence_before();
@@ -1409,7 +1467,7 @@ int make_store_map(CUtensorMap* m, void* ptr, int64_t T, int H, int d);         
 struct BwdLayout {
     size_t delta, ints, partial, ds, total;
     int ds_heads;   // KV heads whose dS is kept at a time; 0: dS is computed again
-    size_t n_count, n_start, n_chunks, n_part0, n_readers, n_units, n_multi;   // (n_units: also unit_order)
+    size_t n_count, n_start, n_chunks, n_part0, n_readers, n_units, n_multi;
     BwdLayout(int64_t T, int hq, int hkv, int d, int cap, int max_degree) {
         auto up = [](size_t x) { return (x + 255) / 256 * 256; };
         n_count = (size_t)cap;
@@ -1421,7 +1479,7 @@ struct BwdLayout {
         n_multi = (size_t)cap;
         delta = 0;
         ints = up((size_t)T * hq * sizeof(float));
-        const size_t n_ints = n_count + 2 * n_start + n_chunks + n_part0 + n_readers + 5 * n_units + n_multi + 8;
+        const size_t n_ints = n_count + 2 * n_start + n_chunks + n_part0 + n_readers + 8 * n_units + (size_t)hkv + n_multi + 8;
         partial = ints + up(n_ints * sizeof(int32_t));
         ds = partial + up((size_t)cap * hkv * 2 * kBlock64 * d * sizeof(float));
         const int64_t per_head = (int64_t)cap * max_degree * (hq / hkv == 4 ? 2 : 1) * kDsTile;
@@ -1521,18 +1579,15 @@ extern "C" int bf1_attn_bwd(const void* q, const void* k, const void* v, const v
     a.dk = (__nv_bfloat16*)dk;
     a.dv = (__nv_bfloat16*)dv;
     a.partial = (float*)(ws + lay.partial);
-    int32_t* ip = (int32_t*)(ws + lay.ints);
+    a.inv.units = (int4*)(ws + lay.ints);   // (16-byte entries first)
+    int32_t* ip = (int32_t*)(ws + lay.ints) + 8 * lay.n_units;
     a.inv.count = ip;            ip += lay.n_count;
     a.inv.start = ip;            ip += lay.n_start;
     a.inv.unit0 = ip;            ip += lay.n_start;
     a.inv.chunks = ip;           ip += lay.n_chunks;
     a.inv.part0 = ip;            ip += lay.n_part0;
     a.inv.readers = ip;          ip += lay.n_readers;
-    a.inv.unit_slot = ip;        ip += lay.n_units;
-    a.inv.unit_begin = ip;       ip += lay.n_units;
-    a.inv.unit_end = ip;         ip += lay.n_units;
-    a.inv.unit_part = ip;        ip += lay.n_units;
-    a.inv.unit_order = ip;       ip += lay.n_units;
+    a.inv.tickets = ip;          ip += hkv;
     a.inv.multi = ip;            ip += lay.n_multi;
     a.inv.scalars = ip;
     a.inv.cap = cap;
