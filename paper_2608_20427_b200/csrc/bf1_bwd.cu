@@ -794,6 +794,7 @@ constexpr int kInvInts = 24576;
 template <int D, bool kInverse>
 __global__ void __launch_bounds__(1024, 1) bwd_prep_kernel(const BwdArgs a) {
     extern __shared__ int32_t s_inv[];
+    pdl_wait();
     if (a.status && (*a.status & BF1_DEV_WAIT_TIMEOUT)) return;
     int cta = blockIdx.x, ctas = gridDim.x;
     if (kInverse) {
@@ -907,8 +908,6 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
     volatile float* s_lse = reinterpret_cast<volatile float*>(smem + L::kRow);
     volatile float* s_delta = s_lse + 256;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (a.status && (*a.status & BF1_DEV_WAIT_TIMEOUT)) return;
-    const int n_units = a.inv.scalars[0];
     const int pairs = a.group == 4 ? 2 : 1;
 
     const uint32_t base = smem_u32(smem);
@@ -928,7 +927,6 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
     const uint32_t pds_free = unit_free + 16;      // [1] the MMAs that read P and dS, and the copy of dS, are done
     if (tid == 0) {
         s_abort = (base & 1023u) ? 1 : 0;
-        if (s_abort && a.status) atomicOr(a.status, BF1_DEV_WAIT_TIMEOUT);
         for (int b = 0; b < 2; ++b) {
             mbar_init(kv_full + 8 * b, 2);
             mbar_init(kv_free + 8 * b, 1);
@@ -955,6 +953,11 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
         clear_idle_rows<D>(base + L::kQ, base + L::kDO, tid, kDkvThreads);
         clear_idle_rows<D>(base + L::kQ + L::kQBytes, base + L::kDO + L::kQBytes, tid, kDkvThreads);
     }
+    pdl_wait();
+    if (tid == 0 && a.status) {
+        if (s_abort) atomicOr(a.status, BF1_DEV_WAIT_TIMEOUT);
+        if (*a.status & BF1_DEV_WAIT_TIMEOUT) s_abort = 1;
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -965,6 +968,7 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
         if (warp == 0) tmem_dealloc(tmem, 512);
         return;
     }
+    const int n_units = a.inv.scalars[0];
     // tensor memory: S | dP of buffer b at columns 128 b; dV^T | dK^T (64 columns each: head dimension on the lanes,
     // the block's 64 key rows along the columns) of buffer b at 256 + 128 b
     constexpr uint32_t kColDP = 64, kColAcc = 256, kColDKt = 64;
@@ -1306,8 +1310,6 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
     uint32_t& s_tmem = *reinterpret_cast<uint32_t*>(smem + L::kBar + 240);
     int& s_abort = *reinterpret_cast<int*>(smem + L::kBar + 244);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (a.status && (*a.status & BF1_DEV_WAIT_TIMEOUT)) return;
-    const int nqb = min(*a.num_qblocks, a.capacity);
     const int pairs = a.group == 4 ? 2 : 1;
     const uint32_t base = smem_u32(smem), bars = base + L::kBar;
     const uint32_t full = bars;                              // [kDqStages] the entry's tiles landed
@@ -1317,7 +1319,6 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
     static_assert(16 * kDqStages + 32 <= 240, "barriers overlap the words behind them");
     if (tid == 0) {
         s_abort = (base & 1023u) ? 1 : 0;
-        if (s_abort && a.status) atomicOr(a.status, BF1_DEV_WAIT_TIMEOUT);
         for (int s = 0; s < kDqStages; ++s) {
             mbar_init(full + 8 * s, 1);
             mbar_init(free_ + 8 * s, 1);
@@ -1333,6 +1334,11 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
         tmem_alloc(smem_u32(&s_tmem), 256);
         tmem_relinquish();
     }
+    pdl_wait();
+    if (tid == 0 && a.status) {
+        if (s_abort) atomicOr(a.status, BF1_DEV_WAIT_TIMEOUT);
+        if (*a.status & BF1_DEV_WAIT_TIMEOUT) s_abort = 1;
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -1343,6 +1349,7 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
         if (warp == 0) tmem_dealloc(tmem, 256);
         return;
     }
+    const int nqb = min(*a.num_qblocks, a.capacity);
     if (warp == 0) {
         // ---- copies ----
         const size_t tiles = (size_t)a.capacity * a.max_degree;
@@ -1605,12 +1612,11 @@ extern "C" int bf1_attn_bwd(const void* q, const void* k, const void* v, const v
         inverse_units_kernel<<<1, 1024, 0, st>>>(a);
         inverse_route_kernel<true><<<grid_inv, 256, 0, st>>>(a);
         inverse_sort_kernel<<<cap, 256, 0, st>>>(a);
-        if (d == 128) bwd_prep_kernel<128, false><<<prep_ctas, 1024, 0, st>>>(a);
-        else bwd_prep_kernel<64, false><<<prep_ctas, 1024, 0, st>>>(a);
+        BF1_CUDA_CHECK(launch_pdl(d == 128 ? bwd_prep_kernel<128, false> : bwd_prep_kernel<64, false>, prep_ctas, 1024, 0, st, a));
     } else {
         const int inv_bytes = (int)inverse_words(cap, route->max_degree) * (int)sizeof(int32_t);
-        if (d == 128) bwd_prep_kernel<128, true><<<prep_ctas + 1, 1024, inv_bytes, st>>>(a);
-        else bwd_prep_kernel<64, true><<<prep_ctas + 1, 1024, inv_bytes, st>>>(a);
+        BF1_CUDA_CHECK(launch_pdl(d == 128 ? bwd_prep_kernel<128, true> : bwd_prep_kernel<64, true>, prep_ctas + 1, 1024,
+                                  inv_bytes, st, a));
     }
     BF1_CUDA_CHECK(cudaGetLastError());
     // dK / dV along the inverse route, then dQ along the route, for as many KV heads at a time as the dS buffer holds
@@ -1622,17 +1628,17 @@ extern "C" int bf1_attn_bwd(const void* q, const void* k, const void* v, const v
         const int grid_q = (int)std::min<int64_t>(sms, (int64_t)cap * a.nheads * (group == 4 ? 2 : 1));   // persistent: one CTA per SM
         const int grid_kv = (int)std::min<int64_t>(sms, (int64_t)lay.n_units * a.nheads);
         if (d == 128) {
-            bwd_dkv_kernel<128><<<grid_kv, kDkvThreads, DkvSmem<128>::kTotal, st>>>(tq, tk, tv, tg, a);
+            BF1_CUDA_CHECK(launch_pdl(bwd_dkv_kernel<128>, grid_kv, kDkvThreads, DkvSmem<128>::kTotal, st, tq, tk, tv, tg, a));
             if (a.ds) {
-                bwd_dq_kernel<128><<<grid_q, kDqThreads, DqSmem<128>::kTotal, st>>>(tk, tdq, a);
+                BF1_CUDA_CHECK(launch_pdl(bwd_dq_kernel<128>, grid_q, kDqThreads, DqSmem<128>::kTotal, st, tk, tdq, a));
             } else {
                 bwd_dq_recompute_kernel<128><<<grid_q, kDqrThreads, DqrSmem<128>::kTotal, st>>>(tq, tk, tv, tg, a);
                 bwd_combine_kernel<128><<<4 * sms, 256, 0, st>>>(a);
             }
         } else {
-            bwd_dkv_kernel<64><<<grid_kv, kDkvThreads, DkvSmem<64>::kTotal, st>>>(tq, tk, tv, tg, a);
+            BF1_CUDA_CHECK(launch_pdl(bwd_dkv_kernel<64>, grid_kv, kDkvThreads, DkvSmem<64>::kTotal, st, tq, tk, tv, tg, a));
             if (a.ds) {
-                bwd_dq_kernel<64><<<grid_q, kDqThreads, DqSmem<64>::kTotal, st>>>(tk, tdq, a);
+                BF1_CUDA_CHECK(launch_pdl(bwd_dq_kernel<64>, grid_q, kDqThreads, DqSmem<64>::kTotal, st, tk, tdq, a));
             } else {
                 bwd_dq_recompute_kernel<64><<<grid_q, kDqrThreads, DqrSmem<64>::kTotal, st>>>(tq, tk, tv, tg, a);
                 bwd_combine_kernel<64><<<4 * sms, 256, 0, st>>>(a);

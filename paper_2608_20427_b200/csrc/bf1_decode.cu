@@ -101,6 +101,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_fused_kernel(const DecodeA
     const int warp = tid >> 5, lane = tid & 31, gid = lane >> 2, tig = lane & 3;
     // The page list is fetched together with the plan's count and the length (independent loads in flight at
     // once), not after them: at small batch the kernel is one chain of dependent memory round trips.
+    pdl_wait();
     if (tid < a.max_degree) sPages[tid] = a.page[(size_t)s * a.max_degree + tid];
     const int cnt = a.count[s];
     const int n = a.seqlens[s];
@@ -312,6 +313,7 @@ __global__ void plan_decode_kernel(const int32_t* seqlens, const int32_t* page_t
     // One CTA walks the batch: error bits are collected in shared memory and the status word is
     // WRITTEN once at the end, so no thread's bit can be lost to another thread's clearing store.
     __shared__ int s_bad;
+    pdl_wait();
     if (threadIdx.x == 0) s_bad = 0;
     __syncthreads();
     for (int s = threadIdx.x; s < batch; s += blockDim.x) {
@@ -389,9 +391,8 @@ extern "C" int bf1_plan_decode(const int32_t* seqlens_dev, const int32_t* page_t
                     need, max_pages_per_seq);
     if (batch == 0) return BF1_OK;
     const int threads = batch >= 1024 ? 1024 : ((batch + 31) / 32) * 32;
-    plan_decode_kernel<<<1, threads, 0, (cudaStream_t)stream>>>(seqlens_dev, page_table_dev,
-                                                                               max_pages_per_seq, batch, *cfg, *out);
-    BF1_CUDA_CHECK(cudaGetLastError());
+    BF1_CUDA_CHECK(launch_pdl(plan_decode_kernel, 1, threads, 0, (cudaStream_t)stream, seqlens_dev, page_table_dev,
+                              max_pages_per_seq, batch, *cfg, *out));
     return BF1_OK;
 }
 
@@ -454,8 +455,8 @@ extern "C" int bf1_decode_fwd(const void* q, const void* k_pages, const void* v_
         // enough (sequence, KV head) pairs to fill the GPU: one CTA walks a whole list
         a.nsplit = 1;
         dim3 grid(hkv * pairs, batch);
-        if (d == 128) decode_fused_kernel<128, false><<<grid, kDecThreads, kSmem128, (cudaStream_t)stream>>>(a);
-        else decode_fused_kernel<64, false><<<grid, kDecThreads, kSmem64, (cudaStream_t)stream>>>(a);
+        BF1_CUDA_CHECK(launch_pdl(d == 128 ? decode_fused_kernel<128, false> : decode_fused_kernel<64, false>, grid, kDecThreads,
+                                  d == 128 ? kSmem128 : kSmem64, (cudaStream_t)stream, a));
     } else {
         // few lists: every list is cut into runs of pages, one CTA each (about two CTAs per SM in all, down to one
         // page per CTA), and the last CTA of a list to finish adds the runs' partial results up
@@ -465,9 +466,8 @@ extern "C" int bf1_decode_fwd(const void* q, const void* k_pages, const void* v_
         const int per_max = (plan->max_degree + a.nsplit - 1) / a.nsplit;
         const int stages = std::min(per_max, kDecStages);
         dim3 grid(hkv * pairs, batch, a.nsplit);
-        if (d == 128) decode_fused_kernel<128, true><<<grid, kDecThreads, kSmem128 / kDecStages * stages, (cudaStream_t)stream>>>(a);
-        else decode_fused_kernel<64, true><<<grid, kDecThreads, kSmem64 / kDecStages * stages, (cudaStream_t)stream>>>(a);
+        BF1_CUDA_CHECK(launch_pdl(d == 128 ? decode_fused_kernel<128, true> : decode_fused_kernel<64, true>, grid, kDecThreads,
+                                  (d == 128 ? kSmem128 : kSmem64) / kDecStages * stages, (cudaStream_t)stream, a));
     }
-    BF1_CUDA_CHECK(cudaGetLastError());
     return BF1_OK;
 }

@@ -89,6 +89,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) plan_kernel(const PlanArgs ar
         s_start[0] = 0;
         s_hist_base = batch + 1;
     }
+    pdl_wait();
     __syncthreads();
 
     // ---- phase 1: validate cu_seqlens, blocks per sequence, exclusive scan -> s_start
@@ -309,8 +310,7 @@ extern "C" int bf1_plan_route(const int32_t* cu_seqlens_dev, int32_t batch, int6
     args.max_seqlen = max_seqlen;
     args.cfg = *cfg;
     args.route = *out;
-    plan_kernel<<<1, kPlanThreads, smem, (cudaStream_t)stream>>>(args);
-    BF1_CUDA_CHECK(cudaGetLastError());
+    BF1_CUDA_CHECK(launch_pdl(plan_kernel, 1, kPlanThreads, smem, (cudaStream_t)stream, args));
     return BF1_OK;
 }
 
