@@ -21,6 +21,45 @@ int fail(int code, const char* fmt, ...);
             return ::bf1::fail(BF1_ERR_CUDA, "%s failed: %s", #expr, cudaGetErrorString(e__)); \
     } while (0)
 
+// ---- Eq. 1, entry by entry ---------------------------------------------------------------------------------------
+// The ascending list of route block j is [0] (if the global block is not among the rest), then the dyadic predecessors
+// beyond the window, j - 2^kmax .. j - 2^k0 with 2^k0 the first power of two above W, then the window j - W .. j.  Every
+// entry can be written down from its place alone, so that a planner needs no merge of candidate streams.
+struct ListShape {
+    int j, window, dyadic, kmax, global, count;   // window: predecessors in it; dyadic, global: entries before it
+};
+__host__ __device__ inline int floor_log2(int x) {
+#ifdef __CUDA_ARCH__
+    return 31 - __clz(x);
+#else
+    return 31 - __builtin_clz((unsigned)x);
+#endif
+}
+__host__ __device__ inline ListShape list_shape(const bf1_route_cfg& c, int j) {
+    ListShape s;
+    s.j = j;
+    s.window = c.local_blocks < j ? c.local_blocks : j;
+    s.kmax = j > 0 ? floor_log2(j) : -1;
+    const int k0 = c.local_blocks > 0 ? floor_log2(c.local_blocks) + 1 : 0;
+    s.dyadic = c.dyadic && s.kmax >= k0 ? s.kmax - k0 + 1 : 0;
+    const bool dyadic_is_0 = s.dyadic > 0 && (1 << s.kmax) == j;
+    s.global = c.global_first && j > c.local_blocks && !dyadic_is_0 ? 1 : 0;
+    s.count = s.global + s.dyadic + s.window + 1;
+    return s;
+}
+__host__ __device__ inline int list_block(const ListShape& s, int e) {   // entry e of the list
+    if (e < s.global) return 0;
+    e -= s.global;
+    return e < s.dyadic ? s.j - (1 << (s.kmax - e)) : s.j - s.window + (e - s.dyadic);
+}
+// The same in tiles of 64 tokens, f tiles to a route block: tile t reads every tile of the earlier blocks of its block's
+// list, then the tiles of its own block up to itself.
+__host__ __device__ inline int list_tiles(const ListShape& s, int f, int t) { return (s.count - 1) * f + (t - s.j * f + 1); }
+__host__ __device__ inline int list_tile(const ListShape& s, int f, int e) {
+    const int before = (s.count - 1) * f;
+    return e < before ? list_block(s, e / f) * f + e % f : s.j * f + (e - before);
+}
+
 // ---- programmatic dependent launch ---------------------------------------------------------------------------
 // The kernels of a call (and of consecutive calls on a stream) are short, and each begins with a set-up that needs
 // nothing from the one in front: barriers, tensor memory, tensor maps.  They are launched so that their start and this

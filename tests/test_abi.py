@@ -65,3 +65,16 @@ def test_bad_arguments_are_rejected_on_the_host():
     # empty batch: OK without touching a device
     rc = lib.bf1_dense_causal_fwd(fake, fake, fake, fake, 0, 0, 0, 2, 1, 64, 0.0, fake, fake, None, None)
     assert rc == 0
+
+
+@pytest.mark.parametrize("kw", [dict(), dict(local_blocks=0), dict(local_blocks=1), dict(local_blocks=3, global_first=0),
+                                dict(local_blocks=4), dict(local_blocks=9, dyadic=0), dict(local_blocks=70)],
+                         ids=lambda k: ",".join("%s=%s" % i for i in k.items()) or "paper")
+def test_route_capacity_is_the_longest_list(kw):
+    """The helper looks at the last three blocks only; powers of two are where the list lengths are not monotone."""
+    from oracle import bf1_oracle as O
+    longest = 0
+    _, count, _, _ = O.route(O.cfg(**kw), 64 * 300)
+    for nblk in range(1, 301):
+        longest = max(longest, int(count[nblk - 1]))
+        assert bf1.route_capacity(1, 64 * nblk, 64 * nblk, bf1.RouteCfg(**kw))[1] == longest, nblk

@@ -88,3 +88,33 @@ def test_planner_flags_bad_sequence_lengths_without_faulting():
     route = bf1.plan_route(cu, 1000)
     torch.cuda.synchronize()
     assert int(route.status.item()) == 0 and int(route.num_qblocks.item()) == 16
+
+
+@pytest.mark.parametrize("seqlens,kw", [([1] * 9000, dict()),                                   # more slots than one sweep of the list CTAs
+                                        ([64 * 1100, 65], dict(local_blocks=2000)),             # lists longer than a CTA has threads
+                                        ([64 * 257 + 1, 64 * 127], dict(local_blocks=4))],      # window and dyadic predecessors overlap
+                         ids=["many-slots", "long-lists", "overlap"])
+def test_planner_at_the_edges_of_its_work_split(seqlens, kw):
+    test_planner_matches_oracle_bit_exact(seqlens, kw)
+
+
+@pytest.mark.parametrize("batch", [1, 7, 8, 9, 40])
+def test_decode_planner_at_the_edges_of_its_work_split(batch):
+    """A warp per sequence, eight to a CTA; one bad length anywhere flags the batch and empties that sequence only."""
+    dev = torch.device("cuda:0")
+    rng = np.random.default_rng(batch)
+    lens = [int(x) for x in rng.integers(0, 64 * 70, size=batch)]
+    lens[-1] = 64 * 70
+    table = torch.from_numpy(rng.permutation(batch * 70).astype(np.int32).reshape(batch, 70)).to(dev)
+    for bad in (False, True):
+        if bad:
+            lens[-1] += 1
+        plan = bf1.plan_decode(torch.tensor(lens, dtype=torch.int32, device=dev), table)
+        torch.cuda.synchronize()
+        assert int(plan.status.item()) == (1 if bad else 0)
+        for s, n in enumerate(lens):
+            want = []
+            if n > 0 and not (bad and s == batch - 1):
+                idx, cnt, _, _ = O.route(O.cfg(), n, plan.max_degree)
+                want = table[s].cpu().numpy()[idx[-1, :cnt[-1]]].tolist()
+            assert plan.count[s].item() == len(want) and plan.page[s].tolist() == want + [-1] * (plan.max_degree - len(want))
