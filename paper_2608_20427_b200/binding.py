@@ -3,6 +3,9 @@
 Every step of the operator runs in the library's CUDA kernels.  PyTorch is used for device
 memory, streams and nothing else.  There is no CPU or PyTorch fallback: if the shared
 library cannot be built or loaded, importing callers get an exception.
+
+The calls that launch kernels go through the extension module `_host` (csrc/bf1_host.cpp), which takes the
+tensors apart and calls the C ABI; what only computes sizes on the host uses ctypes.
 """
 from __future__ import annotations
 
@@ -107,14 +110,33 @@ def load():
     return L
 
 
+_host_module = None
+
+
+def _host():
+    """The extension module of the call path (built first if needed)."""
+    global _host_module
+    if _host_module is None:
+        load()
+        _build.build_host()
+        from . import _host as module
+        module.set_error(Bf1Error)
+        _host_module = module
+    return _host_module
+
+
 def _check(rc: int):
     if rc != BF1_OK:
         raise Bf1Error(rc, load().bf1_last_error().decode())
 
 
-def _stream_ptr(stream: Optional[torch.cuda.Stream]) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+def _stream_ptr(stream: Optional[torch.cuda.Stream]) -> Optional[int]:
+    """None stands for the current stream of the current device."""
+    return None if stream is None else int(stream.cuda_stream)
+
+
+def _raw_stream(stream: Optional[torch.cuda.Stream]) -> int:
+    return int((stream if stream is not None else torch.cuda.current_stream()).cuda_stream)
 
 
 def route_capacity(batch: int, total_tokens: int, max_seqlen: int, cfg: Optional[RouteCfg] = None):
@@ -188,58 +210,29 @@ def plan_route(cu_seqlens: torch.Tensor, max_seqlen: int, cfg: Optional[RouteCfg
                route: Optional[Route] = None, stream=None) -> Route:
     """bf1_plan_route: Eq. 1 lists for every query block of the packed batch."""
     cfg = cfg or RouteCfg()
-    assert cu_seqlens.is_cuda and cu_seqlens.dtype == torch.int32 and cu_seqlens.is_contiguous()
-    batch = cu_seqlens.numel() - 1
     total = getattr(cu_seqlens, "_bf1_total", None)
     if total is None:
         total = int(cu_seqlens[-1].item())
     if route is None:
-        cap, deg = route_capacity(batch, total, max_seqlen, cfg)
+        cap, deg = route_capacity(cu_seqlens.numel() - 1, total, max_seqlen, cfg)
         route = Route.empty(cap, deg, cu_seqlens.device, cfg)
-    _check(load().bf1_plan_route(cu_seqlens.data_ptr(), batch, total, max_seqlen, ctypes.byref(cfg),
-                                 ctypes.byref(route.c), _stream_ptr(stream)))
+    _host().plan_route(cu_seqlens, total, max_seqlen, ctypes.addressof(cfg), ctypes.addressof(route.c), _stream_ptr(stream))
     route.cfg = cfg
     return route
-
-
-def _check_qkv(q, k, v):
-    for t in (q, k, v):
-        assert t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous() and t.dim() == 3
-    T, hq, d = q.shape
-    assert k.shape == v.shape and k.shape[0] == T and k.shape[2] == d
-    return T, hq, k.shape[1], d
 
 
 def attn_fwd(q, k, v, cu_seqlens, max_seqlen: int, route: Route, scale: Optional[float] = None,
              out=None, lse=None, stream=None):
     """bf1_attn_fwd.  q [T, hq, d], k/v [T, hkv, d] bf16 CUDA -> (o [T, hq, d] bf16, lse [hq, T] fp32)."""
-    T, hq, hkv, d = _check_qkv(q, k, v)
-    if out is None:
-        out = torch.empty_like(q)
-    if lse is None:
-        lse = torch.empty((hq, T), dtype=torch.float32, device=q.device)
-    _check(load().bf1_attn_fwd(q.data_ptr(), k.data_ptr(), v.data_ptr(), cu_seqlens.data_ptr(),
-                               cu_seqlens.numel() - 1, T, max_seqlen, hq, hkv, d,
-                               float(scale) if scale else 0.0, ctypes.byref(route.c), out.data_ptr(),
-                               lse.data_ptr(), _stream_ptr(stream)))
-    return out, lse
+    return _host().forward(0, q, k, v, cu_seqlens, max_seqlen, scale, out, lse, _stream_ptr(stream),
+                           ctypes.addressof(route.c), None, None)
 
 
 def dense_causal_fwd(q, k, v, cu_seqlens, max_seqlen: int, scale: Optional[float] = None, out=None,
                      lse=None, work=None, stream=None):
     """bf1_dense_causal_fwd: plain causal attention through the same kernel.  `work`: optional
     zero-initialised int32[4] CUDA tensor (word 0 = device status, words 1..2 = hand-out counters)."""
-    T, hq, hkv, d = _check_qkv(q, k, v)
-    if out is None:
-        out = torch.empty_like(q)
-    if lse is None:
-        lse = torch.empty((hq, T), dtype=torch.float32, device=q.device)
-    _check(load().bf1_dense_causal_fwd(q.data_ptr(), k.data_ptr(), v.data_ptr(), cu_seqlens.data_ptr(),
-                                       cu_seqlens.numel() - 1, T, max_seqlen, hq, hkv, d,
-                                       float(scale) if scale else 0.0, out.data_ptr(), lse.data_ptr(),
-                                       work.data_ptr() if work is not None else None,
-                                       _stream_ptr(stream)))
-    return out, lse
+    return _host().forward(1, q, k, v, cu_seqlens, max_seqlen, scale, out, lse, _stream_ptr(stream), work, None, None)
 
 
 def attn_fwd_noalloc(q, k, v, cu_seqlens, max_seqlen: int, out, lse, cfg: Optional[RouteCfg] = None,
@@ -249,15 +242,9 @@ def attn_fwd_noalloc(q, k, v, cu_seqlens, max_seqlen: int, out, lse, cfg: Option
     For callers that must not allocate device memory, so `out` and `lse` are required here and
     the call itself allocates nothing (neither through torch nor through CUDA).  Up to 4096
     query blocks per batch; calls sharing a GPU must not overlap in time."""
-    T, hq, hkv, d = _check_qkv(q, k, v)
     cfg = cfg or RouteCfg()
-    total = getattr(cu_seqlens, "_bf1_total", T)
-    _check(load().bf1_attn_fwd_noalloc(q.data_ptr(), k.data_ptr(), v.data_ptr(), cu_seqlens.data_ptr(),
-                                       cu_seqlens.numel() - 1, total, max_seqlen, hq, hkv, d,
-                                       float(scale) if scale else 0.0, ctypes.byref(cfg), out.data_ptr(),
-                                       lse.data_ptr(), status.data_ptr() if status is not None else None,
-                                       _stream_ptr(stream)))
-    return out, lse
+    return _host().forward(2, q, k, v, cu_seqlens, max_seqlen, scale, out, lse, _stream_ptr(stream),
+                           getattr(cu_seqlens, "_bf1_total", None), ctypes.addressof(cfg), status)
 
 
 @dataclass
@@ -283,13 +270,11 @@ def plan_decode(seqlens: torch.Tensor, page_table: torch.Tensor, cfg: Optional[R
                 plan: Optional[DecodePlan] = None, stream=None) -> DecodePlan:
     """bf1_plan_decode: page list of the newest token's block for every sequence."""
     cfg = cfg or RouteCfg()
-    assert seqlens.is_cuda and seqlens.dtype == torch.int32 and page_table.dtype == torch.int32
-    batch, max_pages = page_table.shape
     if plan is None:
+        batch, max_pages = page_table.shape
         _, deg = route_capacity(1, max_pages * 64, max_pages * 64, cfg)
         plan = DecodePlan.empty(batch, deg, seqlens.device)
-    _check(load().bf1_plan_decode(seqlens.data_ptr(), page_table.data_ptr(), max_pages, batch, ctypes.byref(cfg),
-                                  ctypes.byref(plan.c), _stream_ptr(stream)))
+    _host().plan_decode(seqlens, page_table, ctypes.addressof(cfg), ctypes.addressof(plan.c), _stream_ptr(stream))
     return plan
 
 
@@ -302,17 +287,7 @@ def decode_workspace(batch: int, hq: int, hkv: int, max_degree: int, d: int, dev
 def decode_fwd(q, k_pages, v_pages, seqlens, plan: DecodePlan, workspace, scale: Optional[float] = None,
                out=None, lse=None, stream=None):
     """bf1_decode_fwd.  q [batch, hq, d]; k_pages / v_pages [pages, 64, hkv, d] bf16 CUDA."""
-    batch, hq, d = q.shape
-    num_pages, page, hkv, d2 = k_pages.shape
-    assert page == 64 and d2 == d and v_pages.shape == k_pages.shape
-    if out is None:
-        out = torch.empty_like(q)
-    if lse is None:
-        lse = torch.empty((hq, batch), dtype=torch.float32, device=q.device)
-    _check(load().bf1_decode_fwd(q.data_ptr(), k_pages.data_ptr(), v_pages.data_ptr(), num_pages, seqlens.data_ptr(),
-                                 batch, hq, hkv, d, float(scale) if scale else 0.0, ctypes.byref(plan.c),
-                                 workspace.data_ptr(), out.data_ptr(), lse.data_ptr(), _stream_ptr(stream)))
-    return out, lse
+    return _host().decode(q, k_pages, v_pages, seqlens, ctypes.addressof(plan.c), workspace, scale, out, lse, _stream_ptr(stream))
 
 
 def bwd_workspace(route: Route, total_tokens: int, hq: int, hkv: int, d: int, device) -> torch.Tensor:
@@ -323,17 +298,11 @@ def bwd_workspace(route: Route, total_tokens: int, hq: int, hkv: int, d: int, de
 
 def attn_bwd(q, k, v, o, lse, d_o, cu_seqlens, max_seqlen: int, route: Route, scale: Optional[float] = None,
              workspace=None, stream=None):
-    """bf1_attn_bwd: (dq, dk, dv) in bf16 for the upstream gradient d_o; d = 128 only."""
-    T, hq, hkv, d = _check_qkv(q, k, v)
-    assert d_o.shape == q.shape and d_o.dtype == torch.bfloat16 and d_o.is_contiguous()
+    """bf1_attn_bwd: (dq, dk, dv) in bf16 for the upstream gradient d_o."""
     if workspace is None:
-        workspace = bwd_workspace(route, T, hq, hkv, d, q.device)
-    dq, dk, dv = torch.empty_like(q), torch.empty_like(k), torch.empty_like(v)
-    _check(load().bf1_attn_bwd(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(), d_o.data_ptr(),
-                               cu_seqlens.data_ptr(), cu_seqlens.numel() - 1, T, max_seqlen, hq, hkv, d,
-                               float(scale) if scale else 0.0, ctypes.byref(route.c), workspace.data_ptr(),
-                               dq.data_ptr(), dk.data_ptr(), dv.data_ptr(), _stream_ptr(stream)))
-    return dq, dk, dv
+        workspace = bwd_workspace(route, q.shape[0], q.shape[1], k.shape[1], q.shape[2], q.device)
+    return _host().backward(q, k, v, o, lse, d_o, cu_seqlens, max_seqlen, ctypes.addressof(route.c), scale, workspace,
+                            _stream_ptr(stream))
 
 
 def shard_needed_blocks(n_tokens: int, lo_block: int, hi_block: int, cfg: Optional[RouteCfg] = None):
@@ -358,7 +327,7 @@ def plan_route_shard(n_tokens: int, lo_block: int, hi_block: int, needed_blocks:
     cu = torch.zeros(2, dtype=torch.int32, device=needed_blocks.device)
     _check(load().bf1_plan_route_shard(n_tokens, lo_block, hi_block, ctypes.byref(cfg),
                                        needed_blocks.data_ptr() if needed_blocks.numel() else None, needed_blocks.numel(),
-                                       ctypes.byref(route.c), cu.data_ptr(), _stream_ptr(stream)))
+                                       ctypes.byref(route.c), cu.data_ptr(), _raw_stream(stream)))
     own_tokens = min(n_tokens, hi_block * 64) - lo_block * 64
     cu._bf1_total = needed_blocks.numel() * 64 + own_tokens
     route.cfg = cfg
@@ -391,7 +360,7 @@ def plan_route_shard_strided(n_tokens: int, first_block: int, stride: int, num_b
     _check(load().bf1_plan_route_shard_strided(n_tokens, first_block, stride, num_blocks, ctypes.byref(cfg),
                                                needed_blocks.data_ptr() if needed_blocks.numel() else None,
                                                needed_blocks.numel(), ctypes.byref(route.c), cu.data_ptr(),
-                                               _stream_ptr(stream)))
+                                               _raw_stream(stream)))
     last = first_block + (num_blocks - 1) * stride
     own_tokens = (num_blocks - 1) * 64 + min(64, n_tokens - last * 64)
     cu._bf1_total = needed_blocks.numel() * 64 + own_tokens
