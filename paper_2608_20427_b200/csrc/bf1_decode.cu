@@ -13,9 +13,11 @@
 // The work is memory-bound (every selected K/V byte is read once, 2*G MACs per element): one kernel,
 // decode_fused_kernel, in which a CTA serves one KV head and one pair of query heads and walks a page
 // list, or a run of it, with an online softmax over a ring of cp.async page pairs.  With enough lists
-// to fill the GPU a CTA takes a whole list; with fewer, every list is cut into runs (about two CTAs per
-// SM in all, down to one page per CTA), each CTA leaves a partial (max, sum, O) in the workspace and
-// the last CTA of a list to finish (atomic ticket, reset by the kernel) adds the runs up in run order.
+// to fill the GPU a CTA takes a whole list; with fewer, every list is cut into runs, and the CTAs of a list form a
+// thread-block cluster: they leave a partial (max, sum, O) in their shared memory and the first of them adds the runs up,
+// in run order, over distributed shared memory.  Partial results in global memory behind an atomic ticket were a chain
+// of store, fence, atomic and reload at the end of every call: 6.6 -> 4.6 us for one sequence of 32K tokens (16 query / 8
+// KV heads, d = 128), 8.0 -> 6.4 for eight.
 #include <algorithm>
 
 #include "bf1_common.cuh"
@@ -25,7 +27,9 @@ namespace bf1 {
 constexpr int kPage = 64;             // tokens per page = block width b
 constexpr int kDecThreads = 128;
 constexpr int kDecStages = 3;          // page-pair buffers per CTA
-constexpr int kDecCtasPerSm = 2;       // CTAs aimed at when a list is cut into runs (measured: 1 -> 11.4, 2 -> 10.8, 3 -> 11.7, 6 -> 14.5 us at batch 8)
+// CTAs a list is cut over at most: the portable cluster size.  (At 16, one page each for 11 pages, one sequence takes 5.0 us
+// instead of 4.6, and eight 6.7 instead of 6.4; at 4, 5.1 and 6.3.)
+constexpr int kMaxRuns = 8;
 
 struct DecodeArgs {
     const __nv_bfloat16* q;           // [batch, hq, d]
@@ -39,12 +43,10 @@ struct DecodeArgs {
     int32_t max_degree, hq, hkv, num_pages;
     int32_t group, pairs;             // G = hq / hkv (1, 2 or 4) and ceil(G / 2): a CTA serves one pair of query heads
     float scale_log2;
-    float* part;                      // [batch, hkv * pairs, max_degree, 2, d + 2] partial (o[d], m, l)
-    int32_t* ticket;                  // [batch, hkv * pairs], zero before and after every call
     __nv_bfloat16* o;                 // [batch, hq, d]
     float* lse;                       // [hq, batch]
     int32_t batch;
-    int32_t nsplit;                   // decode_fused_kernel: CTAs a page list is cut over (1: no partial results)
+    int32_t nsplit;                   // CTAs (a cluster) a page list is cut over
 };
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
@@ -73,6 +75,18 @@ __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t& r0, u
                  : "r"(addr));
 }
 
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// A float at this address of the shared memory of the cluster's CTA `rank`.
+__device__ __forceinline__ float ld_cluster(const float* p, uint32_t rank) {
+    uint32_t addr;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(smem_u32(p)), "r"(rank));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+    return v;
+}
+
 // One CTA per (sequence, KV head, pair of query heads[, run of the list]).  Pages stream in through a
 // kDecStages-deep cp.async ring with ONE block-wide synchronisation per page; inside a page each of the
 // four warps owns 16 keys and keeps its own online-softmax state (max, sum, O) for both grouped heads,
@@ -90,9 +104,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_fused_kernel(const DecodeA
     extern __shared__ __align__(128) uint8_t dsmem[];
     __shared__ float sM[4][2], sL[4][2];
     __shared__ float sO[4][2][D];
-    __shared__ float sW[2][64];                         // combine: weight of every partial
-    __shared__ float sRed[2][2];
-    __shared__ int sLast;
+    __shared__ float sPart[2][D + 2];                   // this run's O[d], max, sum per head
     __shared__ int sPages[64];                          // the sequence's page list (max_degree <= 64)
 
     const int kvp = blockIdx.x, s = blockIdx.y, tid = threadIdx.x;
@@ -105,9 +117,9 @@ __global__ void __launch_bounds__(kDecThreads) decode_fused_kernel(const DecodeA
     if (tid < a.max_degree) sPages[tid] = a.page[(size_t)s * a.max_degree + tid];
     const int cnt = a.count[s];
     const int n = a.seqlens[s];
-    if (cnt <= 0) return;
+    if (cnt <= 0) return;             // (here and below: every CTA of a cluster takes the same exit)
     const int j = (n - 1) / kPage;
-    if (j != a.block[s]) {            // the plan belongs to another route epoch
+    if (j != a.block[s]) {               // the plan belongs to another route epoch
         if (tid == 0 && kvp == 0) atomicOr(a.status, BF1_DEV_BAD_ROUTE);
         return;
     }
@@ -116,8 +128,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_fused_kernel(const DecodeA
     const int* pages = sPages;
     // the part of the list this CTA walks: all of it, or the z-th run of `per` entries
     const int per = kSplit ? (cnt + a.nsplit - 1) / a.nsplit : cnt;
-    const int e_lo = kSplit ? (int)blockIdx.z * per : 0, e_hi = min(cnt, e_lo + per);
-    if (e_lo >= cnt) return;          // fewer runs than CTAs for this sequence
+    const int e_lo = kSplit ? min((int)blockIdx.z * per, cnt) : 0, e_hi = min(cnt, e_lo + per);   // (fewer runs than CTAs: empty)
     auto issue_page = [&](int e, int stage) {
         int pg = pages[e];
         if (pg < 0 || pg >= a.num_pages) {
@@ -234,11 +245,11 @@ __global__ void __launch_bounds__(kDecThreads) decode_fused_kernel(const DecodeA
     }
     __syncthreads();
     const int h = tid >> 6, r = tid & 63;
-    float m_all = fmaxf(fmaxf(sM[0][h], sM[1][h]), fmaxf(sM[2][h], sM[3][h]));   // warp 0 always has key 0
+    float m_all = fmaxf(fmaxf(sM[0][h], sM[1][h]), fmaxf(sM[2][h], sM[3][h]));   // (warp 0 has key 0 of every page; -inf: empty run)
     float wgt[4], l_all = 0.f;
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
-        wgt[w] = exp2f(sM[w][h] - m_all);                // 0 for a warp that never saw a valid key
+        wgt[w] = m_all == -INFINITY ? 0.f : exp2f(sM[w][h] - m_all);   // 0 for a warp that never saw a valid key
         l_all = fmaf(wgt[w], sL[w][h], l_all);
     }
     constexpr int kColsPerThread = D / 64;
@@ -252,52 +263,39 @@ __global__ void __launch_bounds__(kDecThreads) decode_fused_kernel(const DecodeA
         out[c] = o;
     }
     if (kSplit) {
-        // ---- this run's (max, sum, O) goes to the workspace; the last CTA of the list to finish adds the runs up in
-        //      run order (fixed and data-independent) ------------------------------------------------------------
-        const int runs = (cnt + per - 1) / per;
+        // ---- this run's (max, sum, O) into shared memory; the cluster's first CTA adds the runs up in run order
+        //      (fixed and data-independent)
         const int c0 = r * kColsPerThread;
-        const size_t list_id = (size_t)s * a.hkv * a.pairs + kvp;
-        float* my = a.part + ((list_id * a.max_degree + blockIdx.z) * 2 + h) * (D + 2);
 #pragma unroll
-        for (int c = 0; c < kColsPerThread; ++c) my[c0 + c] = out[c];
-        if (r == 0) { my[D] = m_all; my[D + 1] = l_all; }
-        __threadfence();
-        __syncthreads();
-        if (tid == 0) {
-            const int t = atomicAdd(a.ticket + list_id, 1);
-            sLast = (t == runs - 1);
-            if (sLast) a.ticket[list_id] = 0;            // ready for the next call
+        for (int c = 0; c < kColsPerThread; ++c) sPart[h][c0 + c] = out[c];
+        if (r == 0) { sPart[h][D] = m_all; sPart[h][D + 1] = l_all; }
+        cluster_sync();
+        if (blockIdx.z == 0) {
+            float pm[kMaxRuns], pl[kMaxRuns], po[kMaxRuns][kColsPerThread];
+#pragma unroll
+            for (int i = 0; i < kMaxRuns; ++i) {         // all of it asked for at once
+                const bool on = i < a.nsplit;
+                pm[i] = on ? ld_cluster(&sPart[h][D], i) : -INFINITY;
+                pl[i] = on ? ld_cluster(&sPart[h][D + 1], i) : 0.f;
+#pragma unroll
+                for (int c = 0; c < kColsPerThread; ++c) po[i][c] = on ? ld_cluster(&sPart[h][c0 + c], i) : 0.f;
+            }
+            m_all = pm[0];                               // run 0 has a page: finite
+#pragma unroll
+            for (int i = 1; i < kMaxRuns; ++i) m_all = fmaxf(m_all, pm[i]);
+            l_all = 0.f;
+#pragma unroll
+            for (int c = 0; c < kColsPerThread; ++c) out[c] = 0.f;
+#pragma unroll
+            for (int i = 0; i < kMaxRuns; ++i) {
+                const float w = exp2f(pm[i] - m_all);
+                l_all = fmaf(w, pl[i], l_all);
+#pragma unroll
+                for (int c = 0; c < kColsPerThread; ++c) out[c] = fmaf(w, po[i][c], out[c]);
+            }
         }
-        __syncthreads();
-        if (!sLast) return;
-        __threadfence();
-        const float* base = a.part + (list_id * a.max_degree * 2 + h) * (D + 2);
-        const size_t estride = 2 * (D + 2);
-        if (r < runs) sW[h][r] = base[r * estride + D];  // every run's max is fetched by its own thread
-        __syncthreads();
-        m_all = -INFINITY;
-        for (int i = 0; i < runs && i < 64; ++i) m_all = fmaxf(m_all, sW[h][i]);
-        float w_mine = 0.f, lpart = 0.f;
-        if (r < runs) {
-            w_mine = exp2f(sW[h][r] - m_all);
-            lpart = w_mine * base[r * estride + D + 1];
-        }
-        __syncthreads();
-        if (r < runs) sW[h][r] = w_mine;
-        l_all = lpart;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) l_all += __shfl_xor_sync(0xffffffffu, l_all, off);
-        if ((tid & 31) == 0) sRed[h][(tid >> 5) & 1] = l_all;
-        __syncthreads();
-        l_all = sRed[h][0] + sRed[h][1];
-#pragma unroll
-        for (int c = 0; c < kColsPerThread; ++c) out[c] = 0.f;
-#pragma unroll 4
-        for (int i = 0; i < runs; ++i) {
-            const float w = sW[h][i];
-#pragma unroll
-            for (int c = 0; c < kColsPerThread; ++c) out[c] = fmaf(w, base[i * estride + c0 + c], out[c]);
-        }
+        cluster_sync();                                  // the partials have been read: their CTAs may leave
+        if (blockIdx.z != 0) return;
     }
     if (h >= nheads) return;                             // G = 1: the second head of the pair does not exist
     const float inv = 1.f / l_all;
@@ -416,42 +414,51 @@ extern "C" int bf1_decode_fwd(const void* q, const void* k_pages, const void* v_
     a.pairs = pairs;
     const float scale = softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)d);
     a.scale_log2 = scale * 1.4426950408889634f;
-    a.part = (float*)workspace;
-    const int64_t part = (int64_t)batch * hkv * pairs * plan->max_degree * 2 * (d + 2) * (int64_t)sizeof(float);
-    a.ticket = (int32_t*)((char*)workspace + ((part + 255) / 256) * 256);
     a.o = (__nv_bfloat16*)o;
     a.lse = lse;
     a.batch = batch;
-    static int sm_count[64] = {};
+    static bool configured[64] = {};
+    static int slots[64][2][kDecStages + 1];   // CTAs of the split kernel the GPU holds at once, by d and ring stages
     int dev = 0;
     BF1_CUDA_CHECK(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return fail(BF1_ERR_NO_DEVICE, "device ordinal %d out of range", dev);
     constexpr int kSmem128 = kDecStages * 2 * 64 * 128 * 2, kSmem64 = kDecStages * 2 * 64 * 64 * 2;
-    if (!sm_count[dev]) {
+    if (!configured[dev]) {
+        int sms = 0;
+        BF1_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         BF1_CUDA_CHECK(cudaFuncSetAttribute(decode_fused_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem128));
         BF1_CUDA_CHECK(cudaFuncSetAttribute(decode_fused_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem128));
         BF1_CUDA_CHECK(cudaFuncSetAttribute(decode_fused_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem64));
         BF1_CUDA_CHECK(cudaFuncSetAttribute(decode_fused_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem64));
-        BF1_CUDA_CHECK(cudaDeviceGetAttribute(&sm_count[dev], cudaDevAttrMultiProcessorCount, dev));
+        for (int st = 1; st <= kDecStages; ++st) {
+            int n = 0;
+            BF1_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, decode_fused_kernel<128, true>, kDecThreads, kSmem128 / kDecStages * st));
+            slots[dev][1][st] = n * sms;
+            BF1_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, decode_fused_kernel<64, true>, kDecThreads, kSmem64 / kDecStages * st));
+            slots[dev][0][st] = n * sms;
+        }
+        configured[dev] = true;
     }
     const int64_t lists = (int64_t)batch * hkv * pairs;
-    if (lists >= sm_count[dev]) {
-        // enough (sequence, KV head) pairs to fill the GPU: one CTA walks a whole list
-        a.nsplit = 1;
-        dim3 grid(hkv * pairs, batch);
-        BF1_CUDA_CHECK(launch_pdl(d == 128 ? decode_fused_kernel<128, false> : decode_fused_kernel<64, false>, grid, kDecThreads,
-                                  d == 128 ? kSmem128 : kSmem64, (cudaStream_t)stream, a));
+    const int page_smem = d == 128 ? kSmem128 / kDecStages : kSmem64 / kDecStages;
+    // A list is cut into as many runs as still make one wave of CTAs, none of them idle (a run of fewer pages than the ring
+    // has stages needs that much less shared memory).
+    int runs = std::min(kMaxRuns, plan->max_degree), stages = kDecStages;
+    for (; runs >= 1; --runs) {
+        const int per = (plan->max_degree + runs - 1) / runs;
+        stages = std::min(per, kDecStages);
+        runs = (plan->max_degree + per - 1) / per;
+        if (runs == 1 || lists * runs <= slots[dev][d == 128][stages]) break;
+    }
+    a.nsplit = runs;
+    const size_t smem = (size_t)page_smem * stages;
+    if (runs == 1) {
+        BF1_CUDA_CHECK(launch_pdl(d == 128 ? decode_fused_kernel<128, false> : decode_fused_kernel<64, false>,
+                                  dim3(hkv * pairs, batch), kDecThreads, smem, (cudaStream_t)stream, a));
     } else {
-        // few lists: every list is cut into runs of pages, one CTA each (about two CTAs per SM in all, down to one
-        // page per CTA), and the last CTA of a list to finish adds the runs' partial results up
-        const int64_t want = (kDecCtasPerSm * (int64_t)sm_count[dev] + lists - 1) / lists;
-        a.nsplit = (int)std::min<int64_t>(std::min<int64_t>(want, plan->max_degree), 64);
-        // a run of fewer pages than the ring has stages needs that much less shared memory (more CTAs per SM)
-        const int per_max = (plan->max_degree + a.nsplit - 1) / a.nsplit;
-        const int stages = std::min(per_max, kDecStages);
-        dim3 grid(hkv * pairs, batch, a.nsplit);
-        BF1_CUDA_CHECK(launch_pdl(d == 128 ? decode_fused_kernel<128, true> : decode_fused_kernel<64, true>, grid, kDecThreads,
-                                  (d == 128 ? kSmem128 : kSmem64) / kDecStages * stages, (cudaStream_t)stream, a));
+        BF1_CUDA_CHECK(launch_pdl_cluster(d == 128 ? decode_fused_kernel<128, true> : decode_fused_kernel<64, true>,
+                                          dim3(hkv * pairs, batch, runs), dim3(1, 1, runs), kDecThreads, smem,
+                                          (cudaStream_t)stream, a));
     }
     return BF1_OK;
 }

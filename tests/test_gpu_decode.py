@@ -202,3 +202,29 @@ def test_decode_with_four_and_with_one_query_head_per_kv_head(hq, hkv, batch_kin
     out, lse, plan, last = run_decode(w, q, k_pages, v_pages, table)
     assert int(plan.status.item()) == 0
     check(w, q, k, v, out, lse, last)
+
+
+@pytest.mark.parametrize("hq,hkv,d", [(16, 8, 128), (8, 2, 64), (3, 3, 128)], ids=["G2-d128", "G4-d64", "G1-d128"])
+@pytest.mark.parametrize("batch", [1, 5, 19, 40])
+@pytest.mark.parametrize("local_blocks", [2, 40], ids=["short-lists", "long-lists"])
+def test_decode_however_a_list_is_cut_into_runs(hq, hkv, d, batch, local_blocks):
+    """Few lists: clusters of up to eight CTAs, with runs of one page up to more pages than a CTA's ring holds, and CTAs
+    without a run (short sequences beside long ones, an empty sequence); many lists: a CTA for a list."""
+    rng = np.random.default_rng(batch + d)
+    lens = [int(x) for x in rng.integers(1, 64 * 60, size=batch)]
+    lens[0] = 64 * 59 + 1
+    if batch > 1:
+        lens[1:5] = [0, 1, 64, 65]
+    w = I.custom(lens, hq=hq, hkv=hkv, d=d, seed=3900 + batch + d, local_blocks=local_blocks)
+    q, k, v = I.draw_qkv(w)
+    k_pages, v_pages, table = paged_cache(w, k, v, seed=9)
+    dev = torch.device(DEV)
+    plan = bf1.plan_decode(torch.tensor(lens, dtype=torch.int32, device=dev), table.to(dev), bf1.RouteCfg(64, local_blocks, 1, 1))
+    out, lse, plan, last = run_decode(w, q, k_pages, v_pages, table, plan=plan)
+    assert int(plan.status.item()) == 0
+    rows = [r for r, n in zip(last, lens) if n > 0]
+    live = [s for s, n in enumerate(lens) if n > 0]
+    o_ref, lse_ref = O.attn_route(O.cfg(local_blocks=local_blocks), q, k, v, w.cu_seqlens(), rows=rows)
+    assert np.abs(out[live] - o_ref[rows]).max() <= O_MAX_ABS
+    assert np.abs(lse[:, live] - lse_ref[:, rows]).max() <= LSE_ABS
+    assert np.isnan(out[[s for s in range(batch) if lens[s] == 0]]).all()
