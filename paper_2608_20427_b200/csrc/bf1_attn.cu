@@ -111,45 +111,49 @@ struct Cfg {
 
 struct Unit {
     int seq0, j, cnt, rows_valid, kvh, tok0, slot;
-    const int32_t* list;
 };
 
-// Unit u of the hand-out order -> what to compute.  KV-head-major (so that the K/V of one head stay hot
-// in L2 while its query blocks are processed), inside a head longest list first, then a tail of short units.
-// With G = 4 the 128 tile rows are 4 heads x 32 tokens, so a 64-token query block is two units
-// (adjacent in the order: they read the same K/V blocks).  `kvh` carries the unit's token offset
-// inside its query block in its upper half.
-__device__ __forceinline__ void decode_unit(const AttnArgs& a, int nqb, int u, Unit& un) {
+// Unit u of the hand-out order -> place in the order of the slots, KV head and token offset.  KV-head-major (so that the
+// K/V of one head stay hot in L2 while its query blocks are processed), inside a head longest list first, then a tail of
+// short units.  With G = 4 the 128 tile rows are 4 heads x 32 tokens, so a 64-token query block is two units
+// (adjacent in the order: they read the same K/V blocks).
+struct Place {
+    int idx, head, tok_off;
+};
+__device__ __forceinline__ Place unit_place(const AttnArgs& a, int nqb, int u) {
+    Place p;
     const int halves = kBlock >> a.r_shift;
-    const int tok_off = (u % halves) << a.r_shift;
+    p.tok_off = (u % halves) << a.r_shift;
     const int uq = u / halves;
     // Body: KV head by KV head, the longer lists of a head first.  Tail: the shortest lists of ALL heads,
     // longest first across heads, so that the units handed out last are small ones and the CTAs finish
-    // together.  The host makes everything tail (tail_div = 1) when K and V fit the L2 cache anyway.
-    const int tail_n = nqb / a.tail_div, body_n = nqb - tail_n;
-    int idx, head;
+    // together.  The host makes everything tail (tail_div = 1: nqb does not matter) when K and V fit the L2 cache anyway.
+    const int body_n = a.tail_div == 1 ? 0 : nqb - nqb / a.tail_div;
     if (uq < body_n * a.hkv) {
-        head = uq / body_n;
-        idx = uq - head * body_n;
+        p.head = uq / body_n;
+        p.idx = uq - p.head * body_n;
     } else {
         const int ut = uq - body_n * a.hkv;
-        idx = body_n + ut / a.hkv;
-        head = ut - (ut / a.hkv) * a.hkv;
+        p.idx = body_n + ut / a.hkv;
+        p.head = ut - (ut / a.hkv) * a.hkv;
     }
-    un.kvh = head | (tok_off << 16);
-    int seq, slot;
+    return p;
+}
+// A slot of the route (dense: a query block of the batch) -> the unit.  `kvh` carries the unit's token offset inside its
+// query block in its upper half; p: the first 32 list entries, one per lane, as the route holds them.
+__device__ __forceinline__ void decode_slot(const AttnArgs& a, const Place& pl, int slot, int lane, Unit& un, int& p) {
+    un.kvh = pl.head | (pl.tok_off << 16);
+    un.slot = slot;
+    int seq = 0;
     if (!a.dense) {
-        slot = a.order ? a.order[idx] : idx;
-        seq = a.qb_seq[slot];
+        // one round trip: nothing here waits for the list's length
+        const int32_t* list = a.kv_idx + (size_t)slot * a.max_degree;
+        p = lane < a.max_degree ? list[lane] : 0;
         un.j = a.qb_block[slot];
-        int c = a.kv_count[slot];
-        un.cnt = min(max(c, 1), a.max_degree);
-        un.slot = slot;
-        un.list = a.kv_idx + (size_t)slot * a.max_degree;
+        un.cnt = min(max(a.kv_count[slot], 1), a.max_degree);
+        if (a.batch > 1) seq = a.qb_seq[slot];
     } else {
-        slot = nqb - 1 - idx;
         int acc = 0;
-        seq = 0;
         un.j = 0;
         for (int s = 0; s < a.batch; ++s) {
             const int nb = (a.cu_seqlens[s + 1] - a.cu_seqlens[s] + kBlock - 1) / kBlock;
@@ -157,13 +161,12 @@ __device__ __forceinline__ void decode_unit(const AttnArgs& a, int nqb, int u, U
             acc += nb;
         }
         un.cnt = un.j + 1;
-        un.slot = slot;
-        un.list = nullptr;
+        p = lane;
     }
     un.seq0 = a.cu_seqlens[seq];
     const int seqlen = a.cu_seqlens[seq + 1] - un.seq0;
-    un.rows_valid = max(0, min(1 << a.r_shift, seqlen - un.j * kBlock - tok_off));   // of this unit's R tokens
-    un.tok0 = un.seq0 + un.j * kBlock + tok_off;
+    un.rows_valid = max(0, min(1 << a.r_shift, seqlen - un.j * kBlock - pl.tok_off));   // of this unit's R tokens
+    un.tok0 = un.seq0 + un.j * kBlock + pl.tok_off;
 }
 
 template <int REGS>
@@ -279,11 +282,14 @@ __global__ void __launch_bounds__(kThreads, 2) attn_fwd_kernel(const __grid_cons
     // The scheduler warp decodes this CTA's first unit (unit blockIdx.x; the shared counter hands
     // out the units after the first gridDim.x) while the others set up barriers and tensor memory:
     // the decode is a chain of dependent global loads that would otherwise delay the first copy.
-    auto fetch_unit = [&](int u, int nqb_, Unit& un, int& my_p) {
-        decode_unit(args, nqb_, u, un);
+    auto slot_at = [&](const Place& pl, int nqb_) {
+        return args.dense ? nqb_ - 1 - pl.idx : args.order ? args.order[min(pl.idx, args.capacity - 1)] : pl.idx;
+    };
+    auto fetch_unit = [&](const Place& pl, int slot, Unit& un, int& my_p) {
+        int p;
+        decode_slot(args, pl, slot, lane, un, p);
         my_p = 0;
         if (lane < un.cnt) {   // entries 0..31, one per lane, made safe to use
-            int p = args.dense ? lane : un.list[lane];
             if (p < 0 || p > un.j || (lane == un.cnt - 1) != (p == un.j)) {
                 if (args.status) atomicOr(args.status, BF1_DEV_BAD_ROUTE);
                 p = (lane == un.cnt - 1) ? un.j : 0;
@@ -295,7 +301,13 @@ __global__ void __launch_bounds__(kThreads, 2) attn_fwd_kernel(const __grid_cons
     int my_p0 = 0;
     bool have0 = false;
     if (warp == 2) {
-        int nqb0 = 0;
+        int nqb0 = 0, slot = 0;
+        Place pl = {};
+        const bool early = !args.dense && args.tail_div == 1;   // the place does not depend on the block count
+        if (early) {
+            pl = unit_place(args, 0, blockIdx.x);
+            slot = slot_at(pl, 0);      // (on its way together with the block count)
+        }
         if (!args.dense) {
             nqb0 = min(*args.num_qblocks, args.capacity);
         } else {
@@ -303,7 +315,13 @@ __global__ void __launch_bounds__(kThreads, 2) attn_fwd_kernel(const __grid_cons
                 nqb0 += (args.cu_seqlens[s + 1] - args.cu_seqlens[s] + kBlock - 1) / kBlock;
         }
         have0 = (int)blockIdx.x < nqb0 * args.hkv * (kBlock >> args.r_shift);
-        if (have0) fetch_unit(blockIdx.x, nqb0, un0, my_p0);
+        if (have0) {
+            if (!early) {
+                pl = unit_place(args, nqb0, blockIdx.x);
+                slot = slot_at(pl, nqb0);
+            }
+            fetch_unit(pl, slot, un0, my_p0);
+        }
     }
     if (args.group == 1) {
         // one query head per KV head: the lower half of the 128-row tile is unused; the MMAs still read it, so
@@ -336,7 +354,10 @@ __global__ void __launch_bounds__(kThreads, 2) attn_fwd_kernel(const __grid_cons
                         u = (args.sched ? atomicAdd(args.sched, 1) + (int)gridDim.x : (int)(blockIdx.x + n * gridDim.x));
                     u = __shfl_sync(0xffffffffu, u, 0);
                     have = u < total_units && !*abort_flag;
-                    if (have) fetch_unit(u, nqb, un, my_p);
+                    if (have) {
+                        const Place pl = unit_place(args, nqb, u);
+                        fetch_unit(pl, slot_at(pl, nqb), un, my_p);
+                    }
                 }
                 const int qs = n % kQueue;
                 if (n >= kQueue) mbar_wait(bar_sq_free + 8 * qs, ((n / kQueue) - 1) & 1, abort_flag, args.status);
