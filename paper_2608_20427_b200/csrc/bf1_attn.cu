@@ -775,41 +775,7 @@ static int get_encode_fn(EncodeTiledFn* fn) {
     return BF1_OK;
 }
 
-// Encoding a tensor map costs a driver call of a microsecond or two, and a forward call needs four.
-// A map is a pure function of (pointer, extents, box, swizzle), so each host thread keeps the last
-// few it built; a layer that is called again with the same buffers (every step of a serving loop,
-// every repetition of a benchmark) then launches without touching the driver.
-struct MapKey {
-    const void* ptr;
-    int64_t T;
-    int32_t H, d, heads_per_box, tokens_per_box, kind;
-    bool operator==(const MapKey& o) const {
-        return ptr == o.ptr && T == o.T && H == o.H && d == o.d && heads_per_box == o.heads_per_box &&
-               tokens_per_box == o.tokens_per_box && kind == o.kind;
-    }
-};
-struct MapCache {
-    static constexpr int kEntries = 64;
-    MapKey key[kEntries];
-    CUtensorMap map[kEntries];
-    bool used[kEntries] = {};
-    static uint32_t slot_of(const MapKey& k) {
-        uint64_t h = (uint64_t)(uintptr_t)k.ptr * 0x9E3779B97F4A7C15ull;
-        h ^= (uint64_t)k.T * 0xC2B2AE3D27D4EB4Full + (uint64_t)(k.H * 131 + k.d * 31 + k.heads_per_box * 7 + k.tokens_per_box * 3 + k.kind);
-        return (uint32_t)(h >> 40) % kEntries;
-    }
-    const CUtensorMap* find(const MapKey& k) const {
-        const uint32_t i = slot_of(k);
-        return used[i] && key[i] == k ? &map[i] : nullptr;
-    }
-    void put(const MapKey& k, const CUtensorMap& m) {
-        const uint32_t i = slot_of(k);
-        key[i] = k;
-        map[i] = m;
-        used[i] = true;
-    }
-};
-static thread_local MapCache g_map_cache;
+// (Encoding a tensor map takes 0.05 us: they are made on every call.)
 
 // [T, H, d] bf16 tensor seen as 4-D {64 elements, T tokens, H heads, d/64 column chunks}; box = 64
 // elements (128 bytes) x 64 tokens x `heads_per_box` heads x all chunks, 128-byte swizzle.  In shared
@@ -818,11 +784,6 @@ static thread_local MapCache g_map_cache;
 static int make_map(CUtensorMap* m, const void* ptr, int64_t T, int H, int d, int heads_per_box, int tokens_per_box = kBlock,
                     int chunks_per_box = 0) {
     if (chunks_per_box == 0) chunks_per_box = d / 64;
-    const MapKey key{ptr, T, H, d, heads_per_box, tokens_per_box, chunks_per_box == d / 64 ? 0 : 2};
-    if (const CUtensorMap* hit = g_map_cache.find(key)) {
-        *m = *hit;
-        return BF1_OK;
-    }
     EncodeTiledFn enc;
     if (int rc = get_encode_fn(&enc)) return rc;
     cuuint64_t dims[4] = {64, (cuuint64_t)T, (cuuint64_t)H, (cuuint64_t)(d / 64)};
@@ -833,18 +794,12 @@ static int make_map(CUtensorMap* m, const void* ptr, int64_t T, int H, int d, in
                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return fail(BF1_ERR_CUDA, "cuTensorMapEncodeTiled failed with CUresult %d", (int)r);
-    g_map_cache.put(key, *m);
     return BF1_OK;
 }
 
 // O (or dQ) [T, Hq, d] bf16 for an epilogue's TMA stores: box = 32 elements (64 bytes) x 1 head x 32 tokens,
 // 64-byte swizzle.
 int make_store_map(CUtensorMap* m, void* ptr, int64_t T, int H, int d) {
-    const MapKey key{ptr, T, H, d, 1, 32, 1};
-    if (const CUtensorMap* hit = g_map_cache.find(key)) {
-        *m = *hit;
-        return BF1_OK;
-    }
     EncodeTiledFn enc;
     if (int rc = get_encode_fn(&enc)) return rc;
     cuuint64_t dims[3] = {(cuuint64_t)d, (cuuint64_t)H, (cuuint64_t)T};
@@ -855,7 +810,6 @@ int make_store_map(CUtensorMap* m, void* ptr, int64_t T, int H, int d) {
                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return fail(BF1_ERR_CUDA, "cuTensorMapEncodeTiled (O) failed with CUresult %d", (int)r);
-    g_map_cache.put(key, *m);
     return BF1_OK;
 }
 
