@@ -73,7 +73,7 @@ struct BwdArgs {
     const int32_t* kv_idx;
     const int32_t* num_qblocks;
     const int32_t* order;      // may be null
-    int32_t max_degree, capacity, total_tokens, hq, hkv, group;
+    int32_t batch, max_degree, capacity, total_tokens, hq, hkv, group;
     int32_t head0, nheads; // KV heads this launch works on: head0 .. head0 + nheads - 1
     int32_t interleave;    // 1: units of all KV heads interleaved (longest first over all heads); 0: KV head by KV head
     int32_t* status;
@@ -223,7 +223,7 @@ struct DqrSmem {
 };
 
 struct DqUnit {
-    int ok, slot, kvh, pair, cnt, seq0, j, tok0, rows_valid;
+    int ok, slot, kvh, pair, cnt, seq0, seqlen, j, tok0, rows_valid;
 };
 
 // Unit n of this CTA (see above for the order).
@@ -233,7 +233,7 @@ __device__ __forceinline__ DqUnit dq_unit(const BwdArgs& a, int n, int nqb, int 
     const int G = gridDim.x;
     const int i = n * G + ((n & 1) ? G - 1 - (int)blockIdx.x : (int)blockIdx.x);
     u.ok = i < total;
-    u.slot = u.kvh = u.pair = u.seq0 = u.j = u.tok0 = 0;
+    u.slot = u.kvh = u.pair = u.seq0 = u.seqlen = u.j = u.tok0 = 0;
     u.cnt = 1;
     u.rows_valid = 0;
     if (u.ok) {
@@ -254,11 +254,12 @@ __device__ __forceinline__ DqUnit dq_unit(const BwdArgs& a, int n, int nqb, int 
         int slot = a.order ? a.order[rank] : rank;
         slot = min(max(slot, 0), nqb - 1);
         u.slot = slot;
-        const int seq = a.qb_seq[slot];
+        const int seq = a.batch > 1 ? a.qb_seq[slot] : 0;
         u.j = a.qb_block[slot];
         u.cnt = min(max(a.kv_count[slot], 1), a.max_degree);
         u.seq0 = a.cu_seqlens[seq];
-        u.rows_valid = min(kBlock64, a.cu_seqlens[seq + 1] - u.seq0 - u.j * kBlock64);
+        u.seqlen = a.cu_seqlens[seq + 1] - u.seq0;
+        u.rows_valid = min(kBlock64, u.seqlen - u.j * kBlock64);
         u.tok0 = u.seq0 + u.j * kBlock64;
     }
     return u;
@@ -1283,22 +1284,36 @@ __global__ void __launch_bounds__(256) bwd_combine_kernel(const BwdArgs a) {
 // dQ += dS K_p over the list of a query block: 4 MMAs of 128 x d x 16 per entry.  Per entry the SM takes in 16 KB of dS
 // and 16 KB of K (d = 128) and the MMAs read as much, 512 cycles of shared-memory bandwidth; the dS tiles come from HBM once
 // they outgrow L2, which is then the bound (0.67 GB at 32K tokens, 16 query heads).
-// Measured: 19 us at 4K tokens and 155 us at 32K (recomputing S and dP: 35 and 303).
-// One persistent CTA of 10 warps per SM, units dealt out as above:
+// Measured: 18 us at 4K tokens and 153 us at 32K (recomputing S and dP: 35 and 303): dS and K arrive at 8.7 TB/s in
+// both cases, whether dS lies in L2 or comes from HBM, which is what bounds it now.
+// One persistent CTA of 11 warps per SM; units are dealt out statically, longest list first (KV head by KV head, or all
+// heads together: BwdArgs::interleave), back and forth over the CTAs:
+//     warp 10   describes the units to the other roles.  What it looks up is a chain of four loads; it does so for 32 units
+//               at a time, one per lane.  (With every role looking its units up itself 4K tokens took 0.6 us more.)
 //     warp 0    copies: the dS tile (as the dK/dV kernel left it: the K-major layout of an A operand) and the K tile of
 //               every list entry, through a ring of kDqStages
 //     warp 1    issues the MMAs; dQ accumulates in one of two buffers in tensor memory
 //     warps 2-5  the finished dQ tile of a unit, through shared memory and TMA stores
 //     warps 6-9  KV blocks whose readers were cut into several runs: the runs' partial sums of dK and dV, in run order
-constexpr int kDqThreads = 320;
+constexpr int kDqThreads = 352;
 constexpr int kDqStages = 6;
+constexpr int kDqUnits = 4;      // descriptions of units in shared memory
+
+// What warp 10 tells the other roles about a unit.
+struct DqDesc {
+    int cnt;                     // list entries; 0: no more units
+    int slot, j, seq0;           // query slot, its block, first token of the sequence
+    int kvh, pair, seqlen;       // KV head, pair of query heads, tokens of the sequence
+    int first[32];               // the first 32 list entries, as the route holds them
+};
 
 template <int D>
 struct DqSmem {
     static constexpr int kKBytes = 64 * D * 2;
     static constexpr int kStage = kDsTile + kKBytes;
     static constexpr int kOut = kDqStages * kStage;          // 4 warps x 2 buffers x 32 rows x 64 B
-    static constexpr int kBar = kOut + 4 * 2 * 2048;
+    static constexpr int kUnit = kOut + 4 * 2 * 2048;        // DqDesc [kDqUnits]
+    static constexpr int kBar = kUnit + (kDqUnits * (int)sizeof(DqDesc) + 15) / 16 * 16;
     static constexpr int kTotal = kBar + 256;
 };
 
@@ -1312,11 +1327,14 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int pairs = a.group == 4 ? 2 : 1;
     const uint32_t base = smem_u32(smem), bars = base + L::kBar;
+    volatile DqDesc* s_unit = reinterpret_cast<volatile DqDesc*>(smem + L::kUnit);
     const uint32_t full = bars;                              // [kDqStages] the entry's tiles landed
     const uint32_t free_ = full + 8 * kDqStages;             // [kDqStages] ... and have been used
     const uint32_t acc_full = free_ + 8 * kDqStages;         // [2] the unit's dQ is complete
     const uint32_t acc_free = acc_full + 16;                 // [2] ... and has been read out of tensor memory (4 warps)
-    static_assert(16 * kDqStages + 32 <= 240, "barriers overlap the words behind them");
+    const uint32_t unit_full = acc_free + 16;                // [kDqUnits] the unit is described
+    const uint32_t unit_free = unit_full + 8 * kDqUnits;     // [kDqUnits] ... and has been read (6 warps)
+    static_assert(16 * kDqStages + 32 + 16 * kDqUnits <= 240, "barriers overlap the words behind them");
     if (tid == 0) {
         s_abort = (base & 1023u) ? 1 : 0;
         for (int s = 0; s < kDqStages; ++s) {
@@ -1326,6 +1344,10 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
         for (int b = 0; b < 2; ++b) {
             mbar_init(acc_full + 8 * b, 1);
             mbar_init(acc_free + 8 * b, 4);
+        }
+        for (int u = 0; u < kDqUnits; ++u) {
+            mbar_init(unit_full + 8 * u, 1);
+            mbar_init(unit_free + 8 * u, 6);
         }
         fence_mbar_init();
     }
@@ -1349,31 +1371,73 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
         if (warp == 0) tmem_dealloc(tmem, 256);
         return;
     }
-    const int nqb = min(*a.num_qblocks, a.capacity);
+    auto wait_unit = [&](int n) -> volatile DqDesc& {
+        mbar_wait(unit_full + 8 * (n % kDqUnits), (n / kDqUnits) & 1, abort_flag, a.status);
+        return s_unit[n % kDqUnits];
+    };
+    auto free_unit = [&](int n) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(unit_free + 8 * (n % kDqUnits));
+    };
     if (warp == 0) {
         // ---- copies ----
         const size_t tiles = (size_t)a.capacity * a.max_degree;
         int r = 0, rs = 0, rk = 0;      // entries so far, as (stage, turn of the ring)
-        DqUnit u = dq_unit(a, 0, nqb, pairs);
-        for (int n = 0; u.ok; ++n) {
-            const DqUnit un = dq_unit(a, n + 1, nqb, pairs);
-            const int32_t* list = a.kv_idx + (size_t)u.slot * a.max_degree;
+        for (int n = 0;; ++n) {
+            volatile DqDesc& u = wait_unit(n);
+            const int cnt = u.cnt, slot = u.slot, j = u.j, seq0 = u.seq0, kvh = u.kvh, pair = u.pair;
+            int p = u.first[lane];
+            free_unit(n);
+            if (cnt == 0 || *abort_flag) break;
             const char* ds = reinterpret_cast<const char*>(a.ds) +
-                             (((size_t)(u.kvh - a.head0) * pairs + u.pair) * tiles + (size_t)u.slot * a.max_degree) * kDsTile;
-            for (int it = 0; it < u.cnt; ++it) {
-                const int p = list_entry(list, it, u.cnt, u.j);
+                             (((size_t)(kvh - a.head0) * pairs + pair) * tiles + (size_t)slot * a.max_degree) * kDsTile;
+            for (int it = 0; it < cnt; ++it) {
+                if (it > 0 && (it & 31) == 0)   // lists longer than a warp: the next 32 entries
+                    p = it + lane < cnt ? a.kv_idx[(size_t)slot * a.max_degree + it + lane] : 0;
+                const int kb = safe_entry(__shfl_sync(0xffffffffu, p, it & 31), it, cnt, j);
                 if (r >= kDqStages) mbar_wait(free_ + 8 * rs, (rk - 1) & 1, abort_flag, a.status);
                 if (elect_one()) {
                     const uint32_t dst = base + rs * L::kStage;
                     mbar_expect_tx(full + 8 * rs, L::kStage);
                     bulk_load(dst, ds + (size_t)it * kDsTile, kDsTile, full + 8 * rs);
-                    tma_load_4d(dst + kDsTile, &tm_k, 0, u.seq0 + p * kBlock64, u.kvh, 0, full + 8 * rs);
+                    tma_load_4d(dst + kDsTile, &tm_k, 0, seq0 + kb * kBlock64, kvh, 0, full + 8 * rs);
                 }
                 __syncwarp();
                 ++r;
                 if (++rs == kDqStages) { rs = 0; ++rk; }
             }
-            u = un;
+        }
+    } else if (warp == 10) {
+        // ---- units, 32 at a time ----
+        const int nqb = min(*a.num_qblocks, a.capacity);
+        bool more = true;
+        for (int n0 = 0; more; n0 += 32) {
+            DqUnit u = dq_unit(a, n0 + lane, nqb, pairs);
+            int p_next = 0;
+            auto list_of = [&](int k) {
+                const int slot = __shfl_sync(0xffffffffu, u.slot, k);
+                p_next = lane < a.max_degree ? a.kv_idx[(size_t)slot * a.max_degree + lane] : 0;
+            };
+            list_of(0);
+            for (int k = 0; k < 32 && more; ++k) {
+                const int n = n0 + k, ub = n % kDqUnits, p = p_next;
+                more = __shfl_sync(0xffffffffu, u.ok, k) && !*abort_flag;
+                if (k < 31) list_of(k + 1);            // (on its way while this unit's place is waited for)
+                if (n >= kDqUnits) mbar_wait(unit_free + 8 * ub, (n / kDqUnits - 1) & 1, abort_flag, a.status);
+                volatile DqDesc& d = s_unit[ub];
+                d.first[lane] = p;
+                if (lane == k) {
+                    d.cnt = more ? u.cnt : 0;
+                    d.slot = u.slot;
+                    d.j = u.j;
+                    d.seq0 = u.seq0;
+                    d.kvh = u.kvh;
+                    d.pair = u.pair;
+                    d.seqlen = u.seqlen;
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(unit_full + 8 * ub);
+            }
         }
     } else if (warp == 1) {
         // ---- MMAs: A = dS [128 q][64 kv] K-major (16 kv = 32 bytes per step), B = K tile MN-major (16 kv rows = 2048
@@ -1382,12 +1446,13 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
         constexpr uint32_t kIdQ = idesc_bf16_f32(D, true);
         int rs = 0;
         uint32_t phase = 0;
-        DqUnit u = dq_unit(a, 0, nqb, pairs);
-        for (int n = 0; u.ok; ++n) {
-            const DqUnit un = dq_unit(a, n + 1, nqb, pairs);
+        for (int n = 0;; ++n) {
+            const int cnt = wait_unit(n).cnt;
+            free_unit(n);
+            if (cnt == 0 || *abort_flag) break;
             const int b = n & 1;
             if (n >= 2) mbar_wait(acc_free + 8 * b, ((n >> 1) - 1) & 1, abort_flag, a.status);
-            for (int it = 0; it < u.cnt; ++it) {
+            for (int it = 0; it < cnt; ++it) {
                 mbar_wait(full + 8 * rs, phase, abort_flag, a.status);
                 tc_fence_after();
                 if (elect_one()) {
@@ -1399,24 +1464,25 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
                         else mma_ss_lohi<true>(tmem + b * 128, alo + ((kk * 32) >> 4), blo + ((kk * 2048) >> 4), kHi, kIdQ);
                     }
                     mma_commit(free_ + 8 * rs);
-                    if (it == u.cnt - 1) mma_commit(acc_full + 8 * b);
+                    if (it == cnt - 1) mma_commit(acc_full + 8 * b);
                 }
                 __syncwarp();
                 if (++rs == kDqStages) { rs = 0; phase ^= 1; }
             }
-            u = un;
         }
     } else if (warp < 6) {
         // ---- finished dQ tiles: one thread per row ----
         const int quarter = warp & 3, row = quarter * 32 + lane, hl = row >> 6, tl = row & 63;
         const uint32_t t_lane = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
         const uint32_t stage_w = base + L::kOut + quarter * 4096;
-        DqUnit u = dq_unit(a, 0, nqb, pairs);
-        for (int n = 0; u.ok; ++n) {
-            const DqUnit un = dq_unit(a, n + 1, nqb, pairs);
-            const int b = n & 1;
-            const int h = u.kvh * a.group + u.pair * 2 + hl;
+        for (int n = 0;; ++n) {
+            volatile DqDesc& u = wait_unit(n);
+            const int cnt = u.cnt, h = u.kvh * a.group + u.pair * 2 + hl, tok0 = u.seq0 + u.j * kBlock64;
+            const int rows_valid = min(kBlock64, u.seqlen - u.j * kBlock64);
             const bool head_ok = u.pair * 2 + hl < a.group;   // G = 1: rows 64..127 belong to no head (warp-uniform)
+            free_unit(n);
+            if (cnt == 0 || *abort_flag) break;
+            const int b = n & 1;
             mbar_wait(acc_full + 8 * b, (n >> 1) & 1, abort_flag, a.status);
             tc_fence_after();
             uint32_t pk[D / 2];
@@ -1431,7 +1497,7 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(acc_free + 8 * b);
-            if (head_ok && (tl | 31) < u.rows_valid) {        // all 32 rows of the warp lie in the sequence (warp-uniform)
+            if (head_ok && (tl | 31) < rows_valid) {        // all 32 rows of the warp lie in the sequence (warp-uniform)
                 const uint32_t sw = (lane >> 1) & 3;          // 64-byte swizzle: chunk ^= (row / 2) % 4
 #pragma unroll
                 for (int c = 0; c < D / 32; ++c) {            // 32 columns at a time, two staging tiles in turn
@@ -1445,17 +1511,16 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
                     fence_proxy_async();
                     __syncwarp();
                     if (lane == 0) {
-                        tma_store_3d(&tm_dq, c * 32, h, u.tok0 + (tl & 32), tile);
+                        tma_store_3d(&tm_dq, c * 32, h, tok0 + (tl & 32), tile);
                         bulk_commit_group();
                     }
                 }
-            } else if (head_ok && tl < u.rows_valid) {        // the rows after these belong to someone else
-                __nv_bfloat16* dqrow = a.dq + ((size_t)(u.tok0 + tl) * a.hq + h) * D;
+            } else if (head_ok && tl < rows_valid) {        // the rows after these belong to someone else
+                __nv_bfloat16* dqrow = a.dq + ((size_t)(tok0 + tl) * a.hq + h) * D;
 #pragma unroll
                 for (int c = 0; c < D / 8; ++c)
                     *reinterpret_cast<uint4*>(dqrow + c * 8) = make_uint4(pk[c * 4], pk[c * 4 + 1], pk[c * 4 + 2], pk[c * 4 + 3]);
             }
-            u = un;
         }
         if (lane == 0) bulk_wait0();
         __syncwarp();
@@ -1566,6 +1631,7 @@ extern "C" int bf1_attn_bwd(const void* q, const void* k, const void* v, const v
     a.kv_idx = route->kv_idx;
     a.num_qblocks = route->num_qblocks;
     a.order = route->order;
+    a.batch = batch;
     a.max_degree = route->max_degree;
     a.capacity = cap;
     a.total_tokens = (int32_t)total_tokens;
