@@ -1211,27 +1211,34 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
             mbar_wait(acc_full + 8 * b, (n >> 1) & 1, abort_flag, a.status);
             tc_fence_after();
             if (row < D) {   // d = 64: lanes 64..127 hold nothing (warp-uniform)
-                const size_t rstride = (size_t)a.hkv * D;
-                const size_t row0 = ((size_t)tok0 * a.hkv + kvh) * D + row;
                 float* pk = part >= 0 ? a.partial + (((size_t)part * a.hkv + kvh) * 2) * (kBlock64 * D) + row : nullptr;
 #pragma unroll 1
-                for (int hh = 0; hh < 2; ++hh) {
-                    uint32_t vr[32], kr[32];
-                    tmem_ld32(t_lane + kColAcc + b * 128 + hh * 32, vr);
-                    tmem_ld32(t_lane + kColAcc + b * 128 + kColDKt + hh * 32, kr);
+                for (int hh = 0; hh < 4; ++hh) {                     // dV / dK, key rows 0..31 / 32..63
+                    const int which = hh >> 1, r0 = (hh & 1) * 32;
+                    uint32_t v[32];
+                    tmem_ld32(t_lane + kColAcc + b * 128 + which * kColDKt + r0, v);
                     tmem_wait_ld();
+                    if (part < 0) {
+                        // four lanes hold four neighbouring head-dimension elements of every key row: after exchanging with
+                        // lane ^ 1 and lane ^ 2 a lane has all four of one row in four, 8 bytes to store at once
+                        __nv_bfloat16* out = (which ? a.dk : a.dv) + ((size_t)tok0 * a.hkv + kvh) * D + (row & ~3);
 #pragma unroll
-                    for (int c = 0; c < 32; ++c) {
-                        const int kvr = hh * 32 + c;
-                        if (kvr < kv_valid) {
-                            if (part < 0) {
-                                a.dv[row0 + kvr * rstride] = __float2bfloat16_rn(__uint_as_float(vr[c]));
-                                a.dk[row0 + kvr * rstride] = __float2bfloat16_rn(__uint_as_float(kr[c]));
-                            } else {
-                                pk[kvr * D] = __uint_as_float(kr[c]);
-                                pk[kBlock64 * D + kvr * D] = __uint_as_float(vr[c]);
-                            }
+                        for (int c = 0; c < 32; c += 4) {
+                            const uint32_t w0 = pack_bf16x2(__uint_as_float(v[c]), __uint_as_float(v[c + 1]));
+                            const uint32_t w1 = pack_bf16x2(__uint_as_float(v[c + 2]), __uint_as_float(v[c + 3]));
+                            const uint32_t x0 = __shfl_xor_sync(0xffffffffu, w0, 1), x1 = __shfl_xor_sync(0xffffffffu, w1, 1);
+                            // even lanes: row c (c + 2), elements lane, lane + 1; odd lanes: row c + 1 (c + 3), lane - 1, lane
+                            const uint32_t sel = (lane & 1) ? 0x3276u : 0x5410u;
+                            const uint32_t y0 = __byte_perm(w0, x0, sel), y1 = __byte_perm(w1, x1, sel);
+                            const uint32_t z = __shfl_xor_sync(0xffffffffu, (lane & 2) ? y0 : y1, 2);
+                            const int kvr = r0 + c + (lane & 3);
+                            if (kvr < kv_valid)
+                                *reinterpret_cast<uint2*>(out + (size_t)kvr * a.hkv * D) = (lane & 2) ? make_uint2(z, y1) : make_uint2(y0, z);
                         }
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < 32; ++c)
+                            if (r0 + c < kv_valid) pk[(which ? 0 : kBlock64 * D) + (r0 + c) * D] = __uint_as_float(v[c]);
                     }
                 }
             }
