@@ -969,7 +969,6 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
         if (warp == 0) tmem_dealloc(tmem, 512);
         return;
     }
-    const int n_units = a.inv.scalars[0];
     // tensor memory: S | dP of buffer b at columns 128 b; dV^T | dK^T (64 columns each: head dimension on the lanes,
     // the block's 64 key rows along the columns) of buffer b at 256 + 128 b
     constexpr uint32_t kColDP = 64, kColAcc = 256, kColDKt = 64;
@@ -993,30 +992,35 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
         const float* rows = first ? a.lse : a.delta;
         volatile float* s_row = first ? s_lse : s_delta;
         // warp 0's next unit, taken and read a few steps before it is needed: ticket, then description, then readers
-        const int total = n_units * a.nheads;
+        int n_units = 0;
         int next_i = blockIdx.x, next_kvh = 0, next_f = 0;
         int4 next_a = make_int4(0, 0, 0, -1), next_b = make_int4(0, 0, 0, 0);
         auto take = [&]() { if (lane == 0) next_i = (int)gridDim.x + atomicAdd(a.inv.tickets + a.head0, 1); };
+        auto look_up = [&]() {          // (interleaved heads: no need of the number of units)
+            int ui;
+            if (a.interleave) {
+                ui = next_i / a.nheads;
+                next_kvh = next_i - ui * a.nheads;
+            } else {
+                next_kvh = next_i / max(n_units, 1);
+                ui = next_i - next_kvh * n_units;
+            }
+            next_kvh += a.head0;
+            ui = min(ui, a.inv.max_units - 1);
+            next_a = a.inv.units[2 * ui];
+            next_b = a.inv.units[2 * ui + 1];
+        };
         auto describe = [&]() {
             next_i = __shfl_sync(0xffffffffu, next_i, 0);
             next_a.z = 0;
-            if (next_i < total) {
-                int ui;
-                if (a.interleave) {
-                    ui = next_i / a.nheads;
-                    next_kvh = next_i - ui * a.nheads;
-                } else {
-                    next_kvh = next_i / n_units;
-                    ui = next_i - next_kvh * n_units;
-                }
-                next_kvh += a.head0;
-                next_a = a.inv.units[2 * ui];
-                next_b = a.inv.units[2 * ui + 1];
-            }
+            if (next_i < n_units * a.nheads) look_up();
         };
         auto read_readers = [&]() { next_f = lane < next_a.z ? a.inv.readers[next_a.y + lane] : 0; };
         if (first) {
-            describe();
+            if (a.interleave) look_up();          // (beside the number of units)
+            n_units = a.inv.scalars[0];
+            if (!a.interleave) look_up();
+            if (next_i >= n_units * a.nheads) next_a.z = 0;
             read_readers();
         }
         int s = 0;   // steps so far
