@@ -44,7 +44,11 @@ constexpr int kThreads = 384;         // 12 warps
 // the last CTAs finished 20 us after the first at 32K, and 8K was 7 % slower.
 constexpr int kQueue = 1;
 constexpr int kRegsCtl = 40, kRegsSoftmax = 120, kRegsEpilogue = 80;   // registers per thread of each warpgroup
-static_assert(kRegsCtl + kRegsSoftmax + kRegsEpilogue <= 240, "register budgets must fit the launch allocation");
+// The launch allocates 80 registers a thread (65536 / (2 CTAs x 384 threads), in steps of 8).  setmaxnreg.dec to more than
+// a warp has is an illegal instruction, and an inc beyond what the other warpgroups' dec gave back would wait for ever.
+constexpr int kRegsLaunch = 80;
+static_assert(kRegsCtl <= kRegsLaunch && kRegsEpilogue <= kRegsLaunch && kRegsSoftmax >= kRegsLaunch &&
+              kRegsCtl + kRegsSoftmax + kRegsEpilogue <= 3 * kRegsLaunch, "register budgets must fit the launch allocation");
 constexpr float kSumGuard = 1.152921504606846976e18f;   // 2^60: a tile whose row sum reaches this (or is not finite)
                                                         // is redone against its own maximum
 
