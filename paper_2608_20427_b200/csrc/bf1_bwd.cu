@@ -1681,7 +1681,8 @@ extern "C" int bf1_attn_bwd(const void* q, const void* k, const void* v, const v
     BF1_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     // D_i of every row, and the inverse route (readers of every KV block, cut into units)
     const bool one_cta = inverse_words(cap, route->max_degree) <= kInvInts;
-    const int prep_ctas = (int)std::min<int64_t>(sms, ((total_tokens + 15) / 16 * hq + 31) / 32);
+    // (one CTA fits an SM: with the inverse route's there must not be more than SMs, or the last one runs all by itself)
+    const int prep_ctas = (int)std::max<int64_t>(1, std::min<int64_t>(sms - (one_cta ? 1 : 0), ((total_tokens + 15) / 16 * hq + 31) / 32));
     if (!one_cta) {
         BF1_CUDA_CHECK(cudaMemsetAsync(a.inv.count, 0, lay.n_count * sizeof(int32_t), st));
         const int grid_inv = (int)std::min<int64_t>(((int64_t)cap * route->max_degree + 255) / 256, 4 * (int64_t)sms);
