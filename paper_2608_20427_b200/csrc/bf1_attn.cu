@@ -231,8 +231,30 @@ __global__ void __launch_bounds__(kThreads, 2) attn_fwd_kernel(const __grid_cons
     int* s_abort = reinterpret_cast<int*>(smem + C::kMiscOff + 4);
     int* s_nqb = reinterpret_cast<int*>(smem + C::kMiscOff + 8);
 
+    // The wait for the kernel in front stands before the set-up here: the loads below and the decode of the first unit are
+    // the longest chain in front of the first copy, and the barriers and the tensor memory are set up beside them.  With
+    // barriers and tensor memory in front of the wait instead: dense 8K tokens 260.4 us, 257.6 as it is; 4K tokens routed
+    // 24.7, 24.3; 1K 13.6, 13.5.
+    pdl_wait();
     if (tid == 0) {
-        *s_abort = (base & 1023u) ? 1 : 0;   // the swizzled tiles need a 1024-byte aligned window
+        // The status word and the block count are read together (two independent loads in flight), and no other
+        // warp waits for them before its own set-up.  If an earlier launch on this status word gave up, this one
+        // raises its abort flag: every role then sees an empty queue and the CTA leaves through the normal exit.
+        const int earlier = args.status ? *args.status : 0;
+        int nqb = 0;
+        if (!args.dense) {
+            nqb = min(*args.num_qblocks, args.capacity);
+        }
+        *s_abort = (earlier & BF1_DEV_WAIT_TIMEOUT) ? 1 : 0;
+        if (base & 1023u) {   // the swizzled tiles need a 1024-byte aligned window
+            *s_abort = 1;
+            if (args.status) atomicOr(args.status, BF1_DEV_WAIT_TIMEOUT);
+        }
+        if (args.dense) {
+            for (int s = 0; s < args.batch; ++s)
+                nqb += (args.cu_seqlens[s + 1] - args.cu_seqlens[s] + kBlock - 1) / kBlock;
+        }
+        *s_nqb = nqb;
         s_nqb[1] = 0;
         mbar_init(bar_q_full, 1);
         mbar_init(bar_q_free, 1);
@@ -259,28 +281,6 @@ __global__ void __launch_bounds__(kThreads, 2) attn_fwd_kernel(const __grid_cons
         tma_prefetch_desc(&tm_k);
         tma_prefetch_desc(&tm_v);
         tma_prefetch_desc(&tm_o);
-    }
-    __syncwarp();
-    if (warp == 1) {
-        tmem_alloc(smem_u32(s_tmem_base), C::kTmemCols);
-        tmem_relinquish();
-    }
-    pdl_wait();
-    if (tid == 0) {
-        // The status word and the block count are read together (two independent loads in flight), and no other
-        // warp waits for them before its own set-up.  If an earlier launch on this status word gave up, this one
-        // raises its abort flag: every role then sees an empty queue and the CTA leaves through the normal exit.
-        const int earlier = args.status ? *args.status : 0;
-        int nqb = 0;
-        if (!args.dense) {
-            nqb = min(*args.num_qblocks, args.capacity);
-        } else {
-            for (int s = 0; s < args.batch; ++s)
-                nqb += (args.cu_seqlens[s + 1] - args.cu_seqlens[s] + kBlock - 1) / kBlock;
-        }
-        if (*s_abort && args.status) atomicOr(args.status, BF1_DEV_WAIT_TIMEOUT);
-        if (earlier & BF1_DEV_WAIT_TIMEOUT) *s_abort = 1;
-        *s_nqb = nqb;
     }
     __syncwarp();
     // The scheduler warp decodes this CTA's first unit (unit blockIdx.x; the shared counter hands
@@ -326,6 +326,10 @@ __global__ void __launch_bounds__(kThreads, 2) attn_fwd_kernel(const __grid_cons
             }
             fetch_unit(pl, slot, un0, my_p0);
         }
+    }
+    if (warp == 1) {
+        tmem_alloc(smem_u32(s_tmem_base), C::kTmemCols);
+        tmem_relinquish();
     }
     if (args.group == 1) {
         // one query head per KV head: the lower half of the 128-row tile is unused; the MMAs still read it, so

@@ -65,7 +65,7 @@ __host__ __device__ inline int list_tile(const ListShape& s, int f, int e) {
 // ---- programmatic dependent launch ---------------------------------------------------------------------------
 // The kernels of a call (and of consecutive calls on a stream) are short, and each begins with a set-up that needs
 // nothing from the one in front: barriers, tensor memory, tensor maps.  They are launched so that their start and this
-// set-up overlap the end of the kernel in front.  pdl_wait() stands in front of a kernel's first access to global memory,
+// set-up overlap the end of the kernel in front (the forward waits first and sets up beside its first loads).  pdl_wait() stands in front of a kernel's first access to global memory,
 // reads and writes alike, in every thread that makes one, and on every path out of the kernel: it returns when the kernel
 // in front is complete and its writes are visible, and through that kernel's own wait everything before it.
 // No kernel lets the next one start earlier than at its own end (griddepcontrol.launch_dependents): tried right behind the
