@@ -615,23 +615,21 @@ __global__ void __launch_bounds__(256) inverse_sort_kernel(const BwdArgs a) {
     }
 }
 
-// One CTA of 1024 threads: offsets of the reader lists, the run length, and the units of the dK/dV kernel.  kAll: the
-// counting, filling and sorting of the readers as well, in shared memory: `smem` then holds inverse_words() words.
-// (Otherwise inverse_route_kernel has counted the readers in the workspace and will fill them in.)
-__host__ __device__ inline int64_t inverse_words(int64_t cap, int64_t max_degree) { return 3 * cap + 2 + 2 * cap * max_degree; }
+// Runs of at least kMinChunk readers, and long enough that the slots with more than one run cannot need more than `cap`
+// partial-sum slots between them (such a slot has fewer than 2 * count / chunk runs).
+__device__ __forceinline__ int run_length(const InvPlan& v, int readers_total) {
+    return max(kMinChunk, (2 * readers_total + max(v.cap, 1) - 1) / max(v.cap, 1));
+}
 
-template <bool kAll>
-__device__ __forceinline__ void inverse_units(const BwdArgs& a, int32_t* smem) {
+// One CTA: offsets of the reader lists, the run length, and the units of the dK/dV kernel.  inverse_route_kernel has
+// counted the readers in the workspace and will fill them in.
+__global__ void __launch_bounds__(1024, 1) inverse_units_kernel(const BwdArgs a) {
     __shared__ unsigned long long s_warp[32];
     __shared__ int32_t s_bin[1024];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nqb = min(*a.num_qblocks, a.capacity);
     const InvPlan& v = a.inv;
-    int32_t* count = kAll ? smem : v.count;
-    int32_t* start = kAll ? count + a.capacity : v.start;           // [nqb + 1] first reader of a slot
-    int32_t* unit0 = kAll ? start + a.capacity + 1 : v.unit0;       // [nqb + 1] first unit of a slot
-    int32_t* kv_of = kAll ? unit0 + a.capacity + 1 : nullptr;       // per entry: the KV slot it names, or -1
-    int32_t* readers = kAll ? kv_of + a.capacity * a.max_degree : nullptr;
+    int32_t *start = v.start, *unit0 = v.unit0;
     // inclusive scan of x over the CTA
     auto scan = [&](unsigned long long x, unsigned long long& total) {
 #pragma unroll
@@ -652,35 +650,9 @@ __device__ __forceinline__ void inverse_units(const BwdArgs& a, int32_t* smem) {
         __syncthreads();
         return x + (warp > 0 ? before : 0ull);
     };
-    auto count_of = [&](int g) { return kAll ? count[g] : __ldcg(count + g); };   // (written by atomics: read where they were performed)
+    auto count_of = [&](int g) { return __ldcg(v.count + g); };   // (written by atomics: read where they were performed)
     s_bin[tid] = 0;
     for (int i = tid; i < a.hkv; i += 1024) v.tickets[i] = 0;
-    if (kAll) {
-        for (int g = tid; g < nqb; g += 1024) count[g] = 0;
-        __syncthreads();
-        constexpr int kAtOnce = 4;      // entries a thread reads together: each is three loads
-        for (int f0 = tid; f0 < nqb * a.max_degree; f0 += kAtOnce * 1024) {
-            int c[kAtOnce], j[kAtOnce], p[kAtOnce];
-#pragma unroll
-            for (int i = 0; i < kAtOnce; ++i) {
-                const int f = min(f0 + i * 1024, nqb * a.max_degree - 1), g = f / a.max_degree;
-                c[i] = a.kv_count[g], j[i] = a.qb_block[g], p[i] = a.kv_idx[f];
-            }
-#pragma unroll
-            for (int i = 0; i < kAtOnce; ++i) {
-                const int f = f0 + i * 1024, g = f / a.max_degree, e = f - g * a.max_degree;
-                const int cnt = min(max(c[i], 1), a.max_degree);
-                if (f >= nqb * a.max_degree) continue;
-                int kv = -1;
-                if (e < cnt) {
-                    kv = g - j[i] + safe_entry(p[i], e, cnt, j[i]);
-                    atomicAdd(count + kv, 1);
-                }
-                kv_of[f] = kv;
-            }
-        }
-        __syncthreads();
-    }
     // pass 1: where each slot's readers start; the total decides the run length
     int readers_total = 0;
     for (int b0 = 0; b0 < nqb; b0 += 1024) {
@@ -692,9 +664,7 @@ __device__ __forceinline__ void inverse_units(const BwdArgs& a, int32_t* smem) {
         readers_total += (int)total;
     }
     if (tid == 0) start[nqb] = readers_total;
-    // runs of at least kMinChunk readers, and long enough that the slots with more than one run cannot need
-    // more than `cap` partial-sum slots between them (such a slot has fewer than 2 * count / chunk runs)
-    const int chunk = max(kMinChunk, (2 * readers_total + max(v.cap, 1) - 1) / max(v.cap, 1));
+    const int chunk = run_length(v, readers_total);
     // pass 2: runs per slot -> unit numbers, partial-sum slots and places in `multi`: one scan, 21 bits each
     int units = 0, parts = 0, multis = 0;
     for (int b0 = 0; b0 < nqb; b0 += 1024) {
@@ -764,47 +734,201 @@ __device__ __forceinline__ void inverse_units(const BwdArgs& a, int32_t* smem) {
             v.units[2 * at + 1] = make_int4(seq0, a.qb_block[g], a.cu_seqlens[seq + 1] - seq0, 0);
         }
     }
-    if (kAll) {
-        for (int f = tid; f < nqb * a.max_degree; f += 1024) {
+}
+
+// The whole inverse route by one CTA of 1024 threads, in inverse_words() words of shared memory: the chain that
+// bwd_prep_kernel hides behind the pass over dO and O, and at 4K tokens the longer of the two, so what counts is the number
+// of dependent steps.  Every load whose address is known goes out first (nothing waits for the number of query blocks);
+// the readers are counted in total beside the counts of the slots, so that one prefix sum gives everything; all full runs
+// of a slot have one length, so that a thread counts and places its slot's units with two atomics each; and the units'
+// places are found while the readers are filled in.
+__host__ __device__ inline int64_t inverse_words(int64_t cap, int64_t max_degree) { return 2 * cap + 1 + 2 * cap * max_degree; }
+
+__device__ __forceinline__ void inverse_route_in_cta(const BwdArgs& a, int32_t* smem, int status) {
+    __shared__ int32_t s_bin[1024];     // units of a length, then where they start: longest first
+    __shared__ unsigned long long s_warp[32];
+    __shared__ int32_t s_total;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const InvPlan& v = a.inv;
+    const int entries = a.capacity * a.max_degree;
+    int32_t* count = smem;
+    int32_t* start = count + a.capacity;            // [nqb + 1] first reader of a slot
+    int32_t* kv_of = start + a.capacity + 1;        // per entry: the KV slot it names, or -1
+    int32_t* readers = kv_of + entries;
+    constexpr int kAtOnce = 4;      // entries a thread reads together: each is three loads
+    int c[kAtOnce], j[kAtOnce], p[kAtOnce];
+    auto load = [&](int f0) {
+#pragma unroll
+        for (int i = 0; i < kAtOnce; ++i) {
+            const int f = min(f0 + i * 1024, entries - 1), g = f / a.max_degree;
+            c[i] = a.kv_count[g], j[i] = a.qb_block[g], p[i] = a.kv_idx[f];
+        }
+    };
+    load(tid);
+    const int my_slot = min(tid, a.capacity - 1);
+    const int my_j = a.qb_block[my_slot], my_seq = a.qb_seq[my_slot];
+    const int nqb = min(*a.num_qblocks, a.capacity);
+    if (status & BF1_DEV_WAIT_TIMEOUT) return;
+#pragma unroll 1
+    for (int g = tid; g < a.capacity; g += 1024) count[g] = 0;
+    s_bin[tid] = 0;
+    if (tid == 0) s_total = 0;
+#pragma unroll 1
+    for (int i = tid; i < a.hkv; i += 1024) v.tickets[i] = 0;
+    __syncthreads();
+    // (a slot behind the last one may hold anything)
+    int my_seq0 = 0, my_end = 0;
+    if (tid < nqb) my_seq0 = a.cu_seqlens[my_seq], my_end = a.cu_seqlens[my_seq + 1];
+    int mine = 0;
+#pragma unroll 1
+    for (int f0 = tid; f0 < nqb * a.max_degree; f0 += kAtOnce * 1024) {
+        if (f0 != tid) load(f0);
+#pragma unroll
+        for (int i = 0; i < kAtOnce; ++i) {
+            const int f = f0 + i * 1024, g = f / a.max_degree, e = f - g * a.max_degree;
+            const int cnt = min(max(c[i], 1), a.max_degree);
+            if (f >= nqb * a.max_degree) continue;
+            int kv = -1;
+            if (e < cnt) {
+                kv = g - j[i] + safe_entry(p[i], e, cnt, j[i]);
+                atomicAdd(count + kv, 1);
+                ++mine;
+            }
+            kv_of[f] = kv;
+        }
+    }
+    mine = __reduce_add_sync(0xffffffffu, mine);
+    if (lane == 0) atomicAdd(&s_total, mine);
+    __syncthreads();
+    const int readers_total = s_total, chunk = run_length(v, readers_total);
+    // prefix sums over the slots of the readers, the units, the partial-sum slots and the slots cut into runs, 16 bits each
+    // (there are fewer entries than that); the number of units of every length is counted beside them
+    auto bin_of = [](int len) { return 1023 - min(len, 1023); };
+    unsigned long long carry = 0;
+#pragma unroll 1
+    for (int b0 = 0; b0 < nqb; b0 += 1024) {
+        const int g = b0 + tid, n = g < nqb ? count[g] : 0;
+        // a slot's units: n / chunk of `chunk` readers, and one with the rest
+        const int full = n < chunk ? 0 : n / chunk, rest = n - full * chunk, runs = full + (rest > 0);
+        if (full) atomicAdd(s_bin + bin_of(chunk), full);
+        if (rest) atomicAdd(s_bin + bin_of(rest), 1);
+        const unsigned long long x = (unsigned long long)(n | runs << 16) | (unsigned long long)(runs > 1 ? runs | 1 << 16 : 0) << 32;
+        unsigned long long incl = x;
+        if (b0 + warp * 32 < nqb) {
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const unsigned long long up = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += up;
+            }
+        }
+        if (lane == 31) s_warp[warp] = incl;
+        __syncthreads();
+        unsigned long long w = s_warp[lane];
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const unsigned long long up = __shfl_up_sync(0xffffffffu, w, off);
+            if (lane >= off) w += up;
+        }
+        const unsigned long long before = __shfl_sync(0xffffffffu, w, (warp - 1) & 31);
+        const unsigned long long at = carry + incl - x + (warp > 0 ? before : 0ull);
+        carry += __shfl_sync(0xffffffffu, w, 31);
+        if (g < nqb) {
+            const int part = (int)(at >> 32 & 0xffff);
+            start[g] = (int)(at & 0xffff);
+            v.chunks[g] = runs;
+            v.part0[g] = runs > 1 ? part : -1;
+            if (runs > 1) v.multi[at >> 48] = g;
+        }
+        __syncthreads();
+    }
+    const int units = (int)(carry >> 16 & 0xffff), parts = (int)(carry >> 32 & 0xffff);
+    const bool fits = units > 0 && units <= v.max_units && parts <= v.cap;
+    if (tid == 0) {
+        start[nqb] = readers_total;
+        if (units > 0 && !fits && a.status) atomicOr(a.status, BF1_DEV_CAPACITY);
+        v.scalars[0] = fits ? units : 0;
+        v.scalars[1] = readers_total;
+        v.scalars[2] = chunk;
+        v.scalars[3] = parts;
+        v.scalars[4] = fits ? (int)(carry >> 48) : 0;
+    }
+    if (warp == 0) {        // (no unit is longer than `chunk`)
+        int first = 0;
+#pragma unroll 1
+        for (int b = bin_of(chunk) & ~31; b < 1024; b += 32) {
+            const int x = s_bin[b + lane];
+            int incl = x;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int up = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += up;
+            }
+            s_bin[b + lane] = first + incl - x;
+            first += __shfl_sync(0xffffffffu, incl, 31);
+        }
+    } else {
+#pragma unroll 1
+        for (int f = tid - 32; f < nqb * a.max_degree; f += 1024 - 32) {
             const int kv = kv_of[f];
             if (kv >= 0) readers[start[kv] + atomicSub(count + kv, 1) - 1] = f;
         }
-        __syncthreads();
-        // an entry's place among its slot's readers is the number of smaller ones (they are distinct)
-        for (int i = tid; i < readers_total; i += 1024) {
-            const int f = readers[i], kv = kv_of[f], s0 = start[kv], s1 = start[kv + 1];
-            int rank = 0;
-#pragma unroll 4
-            for (int k = s0; k < s1; ++k) rank += readers[k] < f;
-            v.readers[s0 + rank] = f;
+    }
+    __syncthreads();
+    if (fits) {
+#pragma unroll 1
+        for (int g = tid; g < nqb; g += 1024) {
+            int seq0 = my_seq0, seqlen = my_end - my_seq0, jg = my_j;
+            if (g != tid) {
+                const int seq = a.qb_seq[g];
+                seq0 = a.cu_seqlens[seq], seqlen = a.cu_seqlens[seq + 1] - seq0, jg = a.qb_block[g];
+            }
+            const int s0 = start[g], n = start[g + 1] - s0, full = n < chunk ? 0 : n / chunk, rest = n - full * chunk;
+            const int part = full + (rest > 0) > 1 ? v.part0[g] : -1;
+            const int at_full = full ? atomicAdd(s_bin + bin_of(chunk), full) : 0;
+            const int at_rest = rest ? atomicAdd(s_bin + bin_of(rest), 1) : 0;
+#pragma unroll 1
+            for (int i = 0; i < full + (rest > 0); ++i) {
+                const int at = i < full ? at_full + i : at_rest;
+                v.units[2 * at] = make_int4(g, s0 + i * chunk, i < full ? chunk : rest, part >= 0 ? part + i : -1);
+                v.units[2 * at + 1] = make_int4(seq0, jg, seqlen, 0);
+            }
         }
     }
-}
-
-__global__ void __launch_bounds__(1024, 1) inverse_units_kernel(const BwdArgs a) {
-    inverse_units<false>(a, nullptr);
+    // an entry's place among its slot's readers is the number of smaller ones (they are distinct)
+#pragma unroll 1
+    for (int i = tid; i < readers_total; i += 1024) {
+        const int f = readers[i], kv = kv_of[f], s0 = start[kv], s1 = start[kv + 1];
+        int rank = 0;
+#pragma unroll 4
+        for (int k = s0; k < s1; ++k) rank += readers[k] < f;
+        v.readers[s0 + rank] = f;
+    }
 }
 
 // D_i = <dO_i, O_i> of every row, and (kInverse) in the first CTA the whole inverse route: a chain of a few
 // microseconds on one SM that is hidden behind the pass over dO and O on the others.  kInverse is chosen while the
 // entries fit shared memory beside the counters (kInvInts words): up to about 64K tokens with the
 // paper's route; beyond, several launches share the work.
-// Measured: 8.3 us at 4K tokens (16 query heads, d = 128) and 56 us at 32K, where the pass over dO and O alone takes 48;
-// the inverse route alone 7 and 25.  (As launches of their own: 12 and 28 us, with D_i in the dQ kernel.)
+// Measured: 7 us at 4K tokens (16 query heads, d = 128), of which the pass over dO and O alone takes 5.1 and the inverse
+// route alone 6.9, and 48 us at 32K, where the inverse route alone takes 21.  (With more dependent steps in the
+// inverse route, a scan for each of its sums, a search for every unit and everything behind the number of query blocks: 8.2
+// and 28 us of its own, a forward and backward of 4K tokens 97.6 us, 95.4 as it is; 16K tokens in 12 sequences 163.7 and
+// 162.8.  As launches of their own: 12 and 28 us, with D_i in the dQ kernel.)
 constexpr int kInvInts = 24576;
 template <int D, bool kInverse>
 __global__ void __launch_bounds__(1024, 1) bwd_prep_kernel(const BwdArgs a) {
     extern __shared__ int32_t s_inv[];
     pdl_wait();
-    if (a.status && (*a.status & BF1_DEV_WAIT_TIMEOUT)) return;
+    const int status = a.status ? *a.status : 0;
     int cta = blockIdx.x, ctas = gridDim.x;
     if (kInverse) {
         if (cta == 0) {
-            inverse_units<true>(a, s_inv);
+            inverse_route_in_cta(a, s_inv, status);
             return;
         }
         --cta, --ctas;
     }
+    if (status & BF1_DEV_WAIT_TIMEOUT) return;
     // a warp takes 16 tokens of one head; a row is read by D / 8 lanes, 16 bytes each
     constexpr int kLanes = D / 8, kRowsAtOnce = 32 / kLanes, kTokens = 16;
     const int lane = threadIdx.x & 31, sub = lane % kLanes, r0 = lane / kLanes;

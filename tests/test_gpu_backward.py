@@ -251,3 +251,32 @@ def test_backward_does_not_depend_on_the_row_pitch_of_the_lists(hq, hkv, d, tile
             assert bool((diff <= 2.0 ** -7 * x.float().abs() + 1e-6).all()), float(diff.max())
         else:
             assert torch.equal(x, y), name
+
+
+@pytest.mark.parametrize("lens,spare,route", [([1] * 1100 + [700], 0, dict()),                    # more slots than threads
+                                              ([8192], 0, dict(local_blocks=9)),                 # runs of more than 16 readers, and a rest
+                                              ([64 * 16], 0, dict(local_blocks=16)),             # 16 readers: one full run, no rest
+                                              ([1000, 65], 1500, dict())],                       # nothing behind the last slot is read as a slot
+                         ids=["slots", "runs", "full-run", "spare-capacity"])
+def test_gradients_at_the_edges_of_the_inverse_route(lens, spare, route):
+    dev = torch.device("cuda:0")
+    w = I.custom(lens, hq=2, hkv=1, d=64, seed=7000 + len(lens), **route)
+    q, k, v = I.draw_qkv(w)
+    d_o = torch.randn(q.shape, generator=torch.Generator().manual_seed(11)).to(torch.bfloat16)
+    cu = bf1.cu_seqlens_tensor(w.seqlens, dev)
+    cap, deg = bf1.route_capacity(len(w.seqlens), w.total_tokens, w.max_seqlen, lib_cfg(w))
+    r = bf1.Route.empty(cap + spare, deg, dev, lib_cfg(w))
+    for t in (r.qb_seq, r.qb_block, r.kv_count, r.kv_idx, r.order):
+        t.fill_(0x7f7f7f7f)
+    bf1.plan_route(cu, w.max_seqlen, lib_cfg(w), route=r)
+    qd, kd, vd, gd = q.to(dev), k.to(dev), v.to(dev), d_o.to(dev)
+    o, lse = bf1.attn_fwd(qd, kd, vd, cu, w.max_seqlen, r)
+    grads = bf1.attn_bwd(qd, kd, vd, o, lse, gd, cu, w.max_seqlen, r)
+    torch.cuda.synchronize()
+    r.check_status()
+    ref = O.attn_route_bwd(oracle_cfg(w), q, k, v, d_o.float().numpy().astype(np.float64), w.cu_seqlens())
+    for name, got, want in zip(("dq", "dk", "dv"), grads, ref):
+        diff = got.float().cpu().numpy().astype(np.float64) - want
+        assert np.isfinite(diff).all(), name
+        rms = float(np.sqrt((diff ** 2).mean() / (want ** 2).mean()))
+        assert rms <= REL_RMS and float(np.abs(diff).max()) <= REL_MAX * float(np.abs(want).max()), (name, rms)
