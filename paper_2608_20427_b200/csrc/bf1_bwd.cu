@@ -1078,7 +1078,39 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
         clear_idle_rows<D>(base + L::kQ, base + L::kDO, tid, kDkvThreads);
         clear_idle_rows<D>(base + L::kQ + L::kQBytes, base + L::kDO + L::kQBytes, tid, kDkvThreads);
     }
+    // warp 0's next unit, taken and read a few steps before it is needed: ticket, then description, then readers
+    int n_units = 0;
+    int next_i = blockIdx.x, next_kvh = 0, next_f = 0;
+    int4 next_a = make_int4(0, 0, 0, -1), next_b = make_int4(0, 0, 0, 0);
+    auto take = [&]() { if (lane == 0) next_i = (int)gridDim.x + atomicAdd(a.inv.tickets + a.head0, 1); };
+    auto look_up = [&]() {          // (interleaved heads: no need of the number of units)
+        int ui;
+        if (a.interleave) {
+            ui = next_i / a.nheads;
+            next_kvh = next_i - ui * a.nheads;
+        } else {
+            next_kvh = next_i / max(n_units, 1);
+            ui = next_i - next_kvh * n_units;
+        }
+        next_kvh += a.head0;
+        ui = min(ui, a.inv.max_units - 1);
+        next_a = a.inv.units[2 * ui];
+        next_b = a.inv.units[2 * ui + 1];
+    };
+    auto describe = [&]() {
+        next_i = __shfl_sync(0xffffffffu, next_i, 0);
+        next_a.z = 0;
+        if (next_i < n_units * a.nheads) look_up();
+    };
+    auto read_readers = [&]() { next_f = lane < next_a.z ? a.inv.readers[next_a.y + lane] : 0; };
     pdl_wait();
+    // The first unit is read beside the status word (interleaved heads: where it stands does not depend on the number of
+    // units).  After an earlier launch gave up it may be anything and is not used: its index is in range all the same.
+    // (With the dQ kernel's first units likewise: forward and backward of 4K tokens 96.3 us behind the status word, 95.7 so.)
+    if (warp == 0) {
+        n_units = a.inv.scalars[0];
+        if (a.interleave) look_up();
+    }
     if (tid == 0 && a.status) {
         if (s_abort) atomicOr(a.status, BF1_DEV_WAIT_TIMEOUT);
         if (*a.status & BF1_DEV_WAIT_TIMEOUT) s_abort = 1;
@@ -1115,34 +1147,7 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
         const uint32_t full = first ? q_full : do_full, free_ = first ? q_free : do_free;
         const float* rows = first ? a.lse : a.delta;
         volatile float* s_row = first ? s_lse : s_delta;
-        // warp 0's next unit, taken and read a few steps before it is needed: ticket, then description, then readers
-        int n_units = 0;
-        int next_i = blockIdx.x, next_kvh = 0, next_f = 0;
-        int4 next_a = make_int4(0, 0, 0, -1), next_b = make_int4(0, 0, 0, 0);
-        auto take = [&]() { if (lane == 0) next_i = (int)gridDim.x + atomicAdd(a.inv.tickets + a.head0, 1); };
-        auto look_up = [&]() {          // (interleaved heads: no need of the number of units)
-            int ui;
-            if (a.interleave) {
-                ui = next_i / a.nheads;
-                next_kvh = next_i - ui * a.nheads;
-            } else {
-                next_kvh = next_i / max(n_units, 1);
-                ui = next_i - next_kvh * n_units;
-            }
-            next_kvh += a.head0;
-            ui = min(ui, a.inv.max_units - 1);
-            next_a = a.inv.units[2 * ui];
-            next_b = a.inv.units[2 * ui + 1];
-        };
-        auto describe = [&]() {
-            next_i = __shfl_sync(0xffffffffu, next_i, 0);
-            next_a.z = 0;
-            if (next_i < n_units * a.nheads) look_up();
-        };
-        auto read_readers = [&]() { next_f = lane < next_a.z ? a.inv.readers[next_a.y + lane] : 0; };
         if (first) {
-            if (a.interleave) look_up();          // (beside the number of units)
-            n_units = a.inv.scalars[0];
             if (!a.interleave) look_up();
             if (next_i >= n_units * a.nheads) next_a.z = 0;
             read_readers();
@@ -1492,6 +1497,12 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
         tmem_relinquish();
     }
     pdl_wait();
+    int nqb = 0;
+    DqUnit u;
+    if (warp == 10) {       // its first units, beside the status word
+        nqb = min(*a.num_qblocks, a.capacity);
+        u = dq_unit(a, lane, nqb, pairs);
+    }
     if (tid == 0 && a.status) {
         if (s_abort) atomicOr(a.status, BF1_DEV_WAIT_TIMEOUT);
         if (*a.status & BF1_DEV_WAIT_TIMEOUT) s_abort = 1;
@@ -1544,10 +1555,9 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
         }
     } else if (warp == 10) {
         // ---- units, 32 at a time ----
-        const int nqb = min(*a.num_qblocks, a.capacity);
         bool more = true;
         for (int n0 = 0; more; n0 += 32) {
-            DqUnit u = dq_unit(a, n0 + lane, nqb, pairs);
+            if (n0 > 0) u = dq_unit(a, n0 + lane, nqb, pairs);
             int p_next = 0;
             auto list_of = [&](int k) {
                 const int slot = __shfl_sync(0xffffffffu, u.slot, k);

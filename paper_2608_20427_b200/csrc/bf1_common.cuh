@@ -70,7 +70,8 @@ __host__ __device__ inline int list_tile(const ListShape& s, int f, int e) {
 // in front is complete and its writes are visible, and through that kernel's own wait everything before it.
 // No kernel lets the next one start earlier than at its own end (griddepcontrol.launch_dependents): tried right behind the
 // set-up, the waiting CTAs cost the running ones more than they gained (forward and backward of 4K tokens: 106.8 us
-// without any of this, 106.6 with the early start, 99.3 as it is; 32K tokens: 892, 925, 893), and a kernel that asks for
+// without any of this, 106.6 with the early start, 99.3 as it is; 32K tokens: 892, 925, 893), started as late as a CTA's
+// last unit they gained nothing (forward of 4K tokens 24.6 either way, with the backward 97 and 99), and a kernel that asks for
 // tensor memory could then find it held by one that waits for it.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
