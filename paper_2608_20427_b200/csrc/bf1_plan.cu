@@ -9,7 +9,7 @@
 // write the lists, a thread per entry (an entry follows from its place: list_tile in bf1_common.cuh), kListSlots query
 // blocks to a CTA.  What is left is a chain of launch, one read of cu_seqlens, a few block-wide synchronisations and the
 // stores.
-// Measured: 10.4 -> 7.0 us for four sequences of 40K tokens, 5.0 -> 4.2 for one of 1K (one CTA that merged the candidate
+// Measured: 10.4 -> 5.7 us for four sequences of 40K tokens, 5.0 -> 3.7 for one of 1K (one CTA that merged the candidate
 // streams of a list in one thread before; one CTA with a thread per entry: 13.9, its issue slots are the bound).
 //
 // The attention kernels work on tiles of 64 tokens.  With the route block width b = 128 every slot of
@@ -55,7 +55,6 @@ __global__ void __launch_bounds__(kPlanThreads, 1) plan_kernel(const PlanArgs ar
     __shared__ int32_t s_scan[kPlanThreads];
     __shared__ int32_t s_bad;
     __shared__ unsigned long long s_total;
-    __shared__ int32_t s_hist_base;  // offset of the histogram inside s_mem
 
     const int tid = threadIdx.x;
     const bf1_route& r = args.route;
@@ -65,54 +64,72 @@ __global__ void __launch_bounds__(kPlanThreads, 1) plan_kernel(const PlanArgs ar
         s_bad = 0;
         s_total = 0ull;
         s_start[0] = 0;
-        s_hist_base = batch + 1;
     }
+    int32_t* s_hist = s_mem + batch + 1;  // [max_degree + 1] (the first CTA's)
+    if (blockIdx.x == 0)
+        for (int i = tid; i <= r.max_degree; i += kPlanThreads) s_hist[i] = 0;
     pdl_wait();
-    __syncthreads();
 
     // ---- phase 1: validate cu_seqlens, blocks per sequence, exclusive scan -> s_start
+    auto blocks_of = [&](int s, bool& bad) -> int32_t {
+        const int32_t lo = args.cu_seqlens[s], hi = args.cu_seqlens[s + 1];
+        const int32_t len = hi - lo;
+        bad = lo < 0 || len < 0 || len > args.max_seqlen || (long long)hi > args.total_tokens ||
+              (s == 0 && lo != 0) || (s == batch - 1 && (long long)hi != args.total_tokens);
+        return bad ? 0 : (len + kTile - 1) / kTile;
+    };
     int32_t carry = 0;
-    for (int base = 0; base < batch; base += kPlanThreads) {
-        const int s = base + tid;
-        int32_t nb = 0;
-        if (s < batch) {
-            const int32_t lo = args.cu_seqlens[s], hi = args.cu_seqlens[s + 1];
-            const int32_t len = hi - lo;
-            if (lo < 0 || len < 0 || len > args.max_seqlen || (long long)hi > args.total_tokens ||
-                (s == 0 && lo != 0) || (s == batch - 1 && (long long)hi != args.total_tokens)) {
-                atomicOr(&s_bad, BF1_DEV_BAD_SEQLENS);
-            } else {
-                nb = (len + kTile - 1) / kTile;
-            }
-        }
-        // inclusive scan of nb over the 1024 threads: shuffles inside a warp, then over the 32 warp totals
-        int32_t incl = nb;
+    if (batch <= 32) {
+        // Every warp scans the lengths for itself: one barrier instead of five, and the histogram is cleared
+        // and a slot's list length computed once: plan and forward of 1K tokens 13.0 -> 12.4 us.
+        const int lane = tid & 31;
+        bool bad = false;
+        int32_t incl = lane < batch ? blocks_of(lane, bad) : 0;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
             const int32_t up = __shfl_up_sync(0xffffffffu, incl, off);
-            if ((tid & 31) >= off) incl += up;
+            if (lane >= off) incl += up;
         }
-        if ((tid & 31) == 31) s_scan[tid >> 5] = incl;
+        carry = __shfl_sync(0xffffffffu, incl, 31);
+        const bool any_bad = __any_sync(0xffffffffu, bad);
+        if (tid < batch) s_start[tid + 1] = incl;
+        if (tid == 0) s_bad = (any_bad ? BF1_DEV_BAD_SEQLENS : 0) | (carry > r.capacity_qblocks ? BF1_DEV_CAPACITY : 0);
+    } else {
         __syncthreads();
-        if (tid < 32) {
-            int32_t w = s_scan[tid];
+        for (int base = 0; base < batch; base += kPlanThreads) {
+            const int s = base + tid;
+            bool bad = false;
+            const int32_t nb = s < batch ? blocks_of(s, bad) : 0;
+            if (bad) atomicOr(&s_bad, BF1_DEV_BAD_SEQLENS);
+            // inclusive scan of nb over the 1024 threads: shuffles inside a warp, then over the 32 warp totals
+            int32_t incl = nb;
 #pragma unroll
             for (int off = 1; off < 32; off <<= 1) {
-                const int32_t up = __shfl_up_sync(0xffffffffu, w, off);
-                if (tid >= off) w += up;
+                const int32_t up = __shfl_up_sync(0xffffffffu, incl, off);
+                if ((tid & 31) >= off) incl += up;
             }
-            s_scan[32 + tid] = w;   // inclusive totals of warps 0..tid
+            if ((tid & 31) == 31) s_scan[tid >> 5] = incl;
+            __syncthreads();
+            if (tid < 32) {
+                int32_t w = s_scan[tid];
+#pragma unroll
+                for (int off = 1; off < 32; off <<= 1) {
+                    const int32_t up = __shfl_up_sync(0xffffffffu, w, off);
+                    if (tid >= off) w += up;
+                }
+                s_scan[32 + tid] = w;   // inclusive totals of warps 0..tid
+            }
+            __syncthreads();
+            incl += (tid >= 32) ? s_scan[32 + (tid >> 5) - 1] : 0;
+            const int32_t chunk_total = s_scan[32 + 31];
+            if (s < batch) s_start[s + 1] = carry + incl;
+            carry += chunk_total;
+            __syncthreads();
         }
-        __syncthreads();
-        incl += (tid >= 32) ? s_scan[32 + (tid >> 5) - 1] : 0;
-        const int32_t chunk_total = s_scan[32 + 31];
-        if (s < batch) s_start[s + 1] = carry + incl;
-        carry += chunk_total;
-        __syncthreads();
+        if (tid == 0 && carry > r.capacity_qblocks) atomicOr(&s_bad, BF1_DEV_CAPACITY);
     }
-    const int32_t nqb = carry;
-    if (tid == 0 && nqb > r.capacity_qblocks) atomicOr(&s_bad, BF1_DEV_CAPACITY);
     __syncthreads();
+    const int32_t nqb = carry;
     // sequence of slot g: last s with s_start[s] <= g (empty sequences have equal starts)
     auto seq_of = [&](int g) {
         int lo = 0, hi = batch;  // invariant: s_start[lo] <= g < s_start[hi]
@@ -150,18 +167,17 @@ __global__ void __launch_bounds__(kPlanThreads, 1) plan_kernel(const PlanArgs ar
     }
 
     // ---- phase 2: one thread per slot: where it is, its list's length, its pairs
-    int32_t* s_hist = s_mem + s_hist_base;  // [max_degree + 1]
-    for (int i = tid; i <= r.max_degree; i += kPlanThreads) s_hist[i] = 0;
-    __syncthreads();
-    auto degree_of = [&](int jt) { return min(list_tiles(list_shape(args.cfg, jt / f), f, jt), r.max_degree); };
+    auto tiles_of = [&](int jt) { return list_tiles(list_shape(args.cfg, jt / f), f, jt); };
     unsigned long long my_pairs = 0ull;
+    int first_deg = -1;              // of slot tid
     for (int g = tid; g < nqb; g += kPlanThreads) {
         const int s = seq_of(g);
         const int jt = g - s_start[s];   // tile inside the sequence
         const int32_t len = args.cu_seqlens[s + 1] - args.cu_seqlens[s];
         const int rows = min(kTile, len - jt * kTile);
-        if (list_tiles(list_shape(args.cfg, jt / f), f, jt) > r.max_degree) atomicOr(&s_bad, BF1_DEV_CAPACITY);
-        const int deg = degree_of(jt);
+        const int tiles = tiles_of(jt), deg = min(tiles, r.max_degree);
+        if (tiles > r.max_degree) atomicOr(&s_bad, BF1_DEV_CAPACITY);
+        if (g == tid) first_deg = deg;
         const int32_t pairs = rows * kTile * (deg - 1) + rows * (rows + 1) / 2;
         r.qb_seq[g] = s;
         r.qb_block[g] = jt;
@@ -196,7 +212,8 @@ __global__ void __launch_bounds__(kPlanThreads, 1) plan_kernel(const PlanArgs ar
     __syncthreads();
     for (int g0 = 0; g0 < nqb; g0 += kPlanThreads) {
         const int g = g0 + tid;
-        const int deg = g < nqb ? degree_of(g - s_start[seq_of(g)]) : -1;
+        int deg = first_deg;         // (-1 behind the last slot)
+        if (g0 > 0) deg = g < nqb ? min(tiles_of(g - s_start[seq_of(g)]), r.max_degree) : -1;
         const unsigned same = __match_any_sync(0xffffffffu, deg);    // one atomic per length and warp
         const int leader = __ffs(same) - 1, rank = __popc(same & ((1u << (tid & 31)) - 1));
         int pos = 0;

@@ -118,3 +118,17 @@ def test_decode_planner_at_the_edges_of_its_work_split(batch):
                 idx, cnt, _, _ = O.route(O.cfg(), n, plan.max_degree)
                 want = table[s].cpu().numpy()[idx[-1, :cnt[-1]]].tolist()
             assert plan.count[s].item() == len(want) and plan.page[s].tolist() == want + [-1] * (plan.max_degree - len(want))
+
+
+@pytest.mark.parametrize("batch", [31, 32, 33])
+def test_planner_where_the_scan_of_the_lengths_changes(batch):
+    """Up to 32 sequences every warp scans the lengths, beyond that the CTA does; one bad length flags the batch in both."""
+    lens = [int(x) for x in np.random.default_rng(batch).integers(0, 400, size=batch)]
+    lens[0], lens[-1] = 0, 401
+    test_planner_matches_oracle_bit_exact(lens, dict())
+    cu = bf1.cu_seqlens_tensor(lens, torch.device("cuda:0"))
+    cap, deg = bf1.route_capacity(batch, sum(lens), 401)
+    for bad, slots, longest in ((1, cap, 400), (2, cap // 2, 401)):
+        route = bf1.plan_route(cu, longest, route=bf1.Route.empty(slots, deg, cu.device))
+        torch.cuda.synchronize()
+        assert int(route.status.item()) == bad and int(route.num_qblocks.item()) == 0
