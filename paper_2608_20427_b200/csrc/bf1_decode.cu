@@ -12,13 +12,20 @@
 //
 // The work is memory-bound (every selected K/V byte is read once, 2*G MACs per element): one kernel,
 // decode_fused_kernel, in which a CTA serves one KV head and one pair of query heads and walks a page
-// list, or a run of it, with an online softmax over a ring of cp.async page pairs.  With enough lists
+// list, or several runs of it, with an online softmax over a ring of cp.async page pairs.  With enough lists
 // to fill the GPU a CTA takes a whole list; with fewer, every list is cut into runs, and the CTAs of a list form a
-// thread-block cluster: they leave a partial (max, sum, O) in their shared memory and the first of them adds the runs up,
-// in run order, over distributed shared memory.  Partial results in global memory behind an atomic ticket were a chain
-// of store, fence, atomic and reload at the end of every call: 6.6 -> 4.6 us for one sequence of 32K tokens (16 query / 8
-// KV heads, d = 128), 8.0 -> 6.4 for eight.
+// thread-block cluster: they send a partial (max, sum, O) of every run into the shared memory of the CTA that adds the runs
+// up, in run order (each CTA of the cluster some of the columns).  Partial results in global memory behind an atomic ticket were a
+// chain of store, fence, atomic and reload at the end of every call, and partial results that the first CTA fetched from the
+// others' shared memory needed a second cluster barrier: 6.6, 4.6 and 4.3 us for one sequence of 32K tokens (16 query /
+// 8 KV heads, d = 128).
+// What a run is and which CTA walks it are two choices.  P is rounded to bf16 against the maximum of its run, and a
+// key that is that maximum (P = 1) is not rounded at all: longer runs are less precise (11 pages as runs of two: relative
+// error 1.99e-3 against 64 bits, page by page: 1.95e-3).  So the runs depend on the number of lists alone, as short as two
+// CTAs per SM would make them, and a CTA takes as many runs as the clusters that fit the GPU leave it.  Eight sequences of
+// 65 to 32768 tokens take 7.3 us for it, 6.4 with the longer runs of four CTAs each (8.0 with the ticket).
 #include <algorithm>
+#include <atomic>
 
 #include "bf1_common.cuh"
 
@@ -27,9 +34,13 @@ namespace bf1 {
 constexpr int kPage = 64;             // tokens per page = block width b
 constexpr int kDecThreads = 128;
 constexpr int kDecStages = 3;          // page-pair buffers per CTA
-// CTAs a list is cut over at most: the portable cluster size.  (At 16, one page each for 11 pages, one sequence takes 5.0 us
-// instead of 4.6, and eight 6.7 instead of 6.4; at 4, 5.1 and 6.3.)
-constexpr int kMaxRuns = 8;
+constexpr int kDecCtasPerSm = 2;       // runs a list is cut into: what this many CTAs per SM would take, one each
+constexpr int kMaxRuns = 64;           // at least 1, at most a run per page
+// CTAs of a cluster at most.  Above 8 a cluster may find fewer places (bf1_decode_fwd asks), but a CTA with one run instead
+// of two or more wins whatever it costs: one list of 11 / 41 / 64 pages takes 5.1 / 9.4 / 11.6 us with eight CTAs, 4.0 /
+// 6.7 / 8.1 with up to sixteen.
+constexpr int kMaxCtas = 16;
+constexpr int kMaxRunsPerCta = 8;
 
 struct DecodeArgs {
     const __nv_bfloat16* q;           // [batch, hq, d]
@@ -46,7 +57,11 @@ struct DecodeArgs {
     __nv_bfloat16* o;                 // [batch, hq, d]
     float* lse;                       // [hq, batch]
     int32_t batch;
-    int32_t nsplit;                   // CTAs (a cluster) a page list is cut over
+    int32_t nsplit;                   // runs a page list is cut into, at most
+    int32_t nctas;                    // CTAs (a cluster) they are dealt to
+    int32_t share;                    // columns (of the pair's 2 d) a CTA of the cluster adds up, a multiple of 32
+    int32_t sums, gather, ring;       // shared memory: the CTA's RunStates, then from these bytes on (max, sum) [run][2] and
+                                      // columns [run][share] of the list's runs, and the page ring
 };
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
@@ -75,26 +90,36 @@ __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t& r0, u
                  : "r"(addr));
 }
 
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// This shared-memory address in the cluster's CTA `rank`.
+__device__ __forceinline__ uint32_t map_cluster(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
 }
-// A float at this address of the shared memory of the cluster's CTA `rank`.
-__device__ __forceinline__ float ld_cluster(const float* p, uint32_t rank) {
-    uint32_t addr;
-    float v;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(smem_u32(p)), "r"(rank));
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-    return v;
+__device__ __forceinline__ void st_cluster(uint32_t addr, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
 }
+__device__ __forceinline__ void st_cluster_v2(uint32_t addr, float x, float y) {
+    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(x), "f"(y) : "memory");
+}
+// x / y for small whole numbers (below 2^20: half a step from a whole quotient is more than the division's error)
+__device__ __forceinline__ int small_div(int x, int y) { return (int)__fdividef((float)x + 0.5f, (float)y); }
 
-// One CTA per (sequence, KV head, pair of query heads[, run of the list]).  Pages stream in through a
+// One CTA per (sequence, KV head, pair of query heads[, share of the list's runs]).  Pages stream in through a
 // kDecStages-deep cp.async ring with ONE block-wide synchronisation per page; inside a page each of the
 // four warps owns 16 keys and keeps its own online-softmax state (max, sum, O) for both grouped heads,
-// merged once at the end.  The arithmetic uses warp-level mma (m16n8k16: the two heads are rows 0 and 1
+// merged at the end of the run.  The arithmetic uses warp-level mma (m16n8k16: the two heads are rows 0 and 1
 // of the 16-row operand, the rest is zero): the work is memory-bound, but as scalar FMAs it was a chain
 // of 1500 dependent instructions and five synchronisations per page, which is what bounded the kernel.
+template <int D>
+struct RunState {                                       // the four warps' states at the end of a run
+    float o[4][2][D + 8], m[4][2], l[4][2];              // (rows 8 banks apart)
+};
 template <int D, bool kSplit>
-__global__ void __launch_bounds__(kDecThreads) decode_fused_kernel(const DecodeArgs a) {
+__global__ void __launch_bounds__(kDecThreads, D == 64 ? 4 : 2) decode_fused_kernel(const DecodeArgs a) {
     constexpr int kRowBytes = D * 2;
     constexpr int kVecPerRow = D / 8;                   // 16-byte chunks per row
     constexpr int kVecPerThread = kPage * kVecPerRow / kDecThreads;
@@ -102,9 +127,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_fused_kernel(const DecodeA
     // [stage][K | V][64 rows][D bf16]; the 16-byte chunks of every row are XOR-swizzled with (row & 7), which
     // keeps both the B-fragment loads of K (8 rows, same chunk) and the ldmatrix rows of V conflict-free
     extern __shared__ __align__(128) uint8_t dsmem[];
-    __shared__ float sM[4][2], sL[4][2];
-    __shared__ float sO[4][2][D];
-    __shared__ float sPart[2][D + 2];                   // this run's O[d], max, sum per head
+    RunState<D>* sRun = reinterpret_cast<RunState<D>*>(dsmem);   // of this CTA's runs, in front of the ring
     __shared__ int sPages[64];                          // the sequence's page list (max_degree <= 64)
 
     const int kvp = blockIdx.x, s = blockIdx.y, tid = threadIdx.x;
@@ -115,20 +138,25 @@ __global__ void __launch_bounds__(kDecThreads) decode_fused_kernel(const DecodeA
     // once), not after them: at small batch the kernel is one chain of dependent memory round trips.
     pdl_wait();
     if (tid < a.max_degree) sPages[tid] = a.page[(size_t)s * a.max_degree + tid];
-    const int cnt = a.count[s];
+    int cnt = max(min(a.count[s], a.max_degree), 0);
     const int n = a.seqlens[s];
-    if (cnt <= 0) return;             // (here and below: every CTA of a cluster takes the same exit)
     const int j = (n - 1) / kPage;
-    if (j != a.block[s]) {               // the plan belongs to another route epoch
+    if (cnt > 0 && j != a.block[s]) {    // the plan belongs to another route epoch
         if (tid == 0 && kvp == 0) atomicOr(a.status, BF1_DEV_BAD_ROUTE);
-        return;
+        cnt = 0;
     }
+    // Nothing to do.  A CTA of a cluster stays all the same: whatever it reads here, the others may store to its shared memory.
+    if (!kSplit && cnt == 0) return;
     const int tail = n - j * kPage;   // valid tokens of the self page (the last list entry)
-    __syncthreads();                  // sPages is complete (every exit above is taken by the whole CTA)
+    __syncthreads();                  // sPages is complete
     const int* pages = sPages;
-    // the part of the list this CTA walks: all of it, or the z-th run of `per` entries
-    const int per = kSplit ? (cnt + a.nsplit - 1) / a.nsplit : cnt;
-    const int e_lo = kSplit ? min((int)blockIdx.z * per, cnt) : 0, e_hi = min(cnt, e_lo + per);   // (fewer runs than CTAs: empty)
+    // the part of the list this CTA walks: all of it as one run, or its share of the list's runs of `per` entries (the later CTAs
+    // get one more where they do not come out even: the last run may be shorter)
+    const int per = kSplit ? max(small_div(cnt + a.nsplit - 1, a.nsplit), 1) : cnt;
+    const int runs = kSplit ? small_div(cnt + per - 1, per) : 1;
+    const int run0 = kSplit ? small_div(blockIdx.z * runs, a.nctas) : 0;
+    const int e_lo = run0 * per, e_hi = kSplit ? min(cnt, small_div((blockIdx.z + 1) * runs, a.nctas) * per) : cnt;   // (may be empty)
+    const uint32_t ring = smem_u32(dsmem) + a.ring;
     auto issue_page = [&](int e, int stage) {
         int pg = pages[e];
         if (pg < 0 || pg >= a.num_pages) {
@@ -139,7 +167,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_fused_kernel(const DecodeA
         const size_t row_stride = (size_t)a.hkv * D;
         const __nv_bfloat16* kp = a.k_pages + ((size_t)pg * kPage * a.hkv + kvh) * D;
         const __nv_bfloat16* vp = a.v_pages + ((size_t)pg * kPage * a.hkv + kvh) * D;
-        const uint32_t kb = smem_u32(dsmem) + stage * 2 * kPageBytes, vb = kb + kPageBytes;
+        const uint32_t kb = ring + stage * 2 * kPageBytes, vb = kb + kPageBytes;
 #pragma unroll
         for (int q = 0; q < kVecPerThread; ++q) {
             const int i = tid + q * kDecThreads, rr = i / kVecPerRow, c = i % kVecPerRow;
@@ -154,6 +182,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_fused_kernel(const DecodeA
         if (e_lo + i < e_hi) issue_page(e_lo + i, i);
         cp_async_commit();                               // possibly empty: keeps the group count uniform
     }
+    if (kSplit) cluster_arrive_relaxed();                        // (waited for in front of the first store to another CTA)
     // A fragments of Q: rows 0 and 1 of the 16-row operand are the two grouped heads, the rest zero
     uint32_t qa[D / 16][2];
     {
@@ -169,6 +198,25 @@ __global__ void __launch_bounds__(kDecThreads) decode_fused_kernel(const DecodeA
 #pragma unroll
     for (int dn = 0; dn < D / 8; ++dn) acc[dn][0] = acc[dn][1] = acc[dn][2] = acc[dn][3] = 0.f;
     const int key0 = warp * 16;                          // this warp's 16 keys of every page
+    auto leave_sums = [&](RunState<D>& st) {             // this warp's state of a run: what is ready first ...
+        if (gid < 2 && tig == 0) { st.m[warp][gid] = m_run; st.l[warp][gid] = l_run; }
+    };
+    auto leave_o = [&](RunState<D>& st) {                // ... and what the MMAs add up
+        if (gid >= 2) return;
+#pragma unroll
+        for (int dn = 0; dn < D / 8; ++dn)
+            *reinterpret_cast<float2*>(&st.o[warp][gid][dn * 8 + 2 * tig]) = make_float2(acc[dn][0], acc[dn][1]);
+    };
+    int run = 0, run_end = e_lo + per;                   // the run at hand (of this CTA's), and the entry behind it
+    // Where this thread's columns of a run go: to the CTA of the cluster that adds them up.
+    constexpr int kColsPerThread = D / 64;
+    const int c0 = (tid & 63) * kColsPerThread;
+    uint32_t to_gather = 0, to_sums = 0;
+    if (kSplit) {
+        const int v = (tid >> 6) * D + c0, rank = small_div(v, a.share);
+        to_gather = map_cluster(smem_u32(dsmem) + a.gather + (run0 * a.share + v - rank * a.share) * 4, rank);
+        to_sums = map_cluster(smem_u32(dsmem) + a.sums + (run0 * 2 + (tid >> 6)) * 8, min(tid & 63, a.nctas - 1));
+    }
 
     for (int e = e_lo; e < e_hi; ++e) {
         cp_async_wait<kDecStages - 2>();                 // page e has landed (for this thread's copies)
@@ -176,133 +224,162 @@ __global__ void __launch_bounds__(kDecThreads) decode_fused_kernel(const DecodeA
         if (e + kDecStages - 1 < e_hi) issue_page(e + kDecStages - 1, (e - e_lo + kDecStages - 1) % kDecStages);
         cp_async_commit();
         const int valid = (e == cnt - 1) ? tail : kPage;
-        if (key0 >= valid) continue;                     // warp-uniform: none of this warp's keys exists
-        const uint32_t kb = smem_u32(dsmem) + ((e - e_lo) % kDecStages) * 2 * kPageBytes, vb = kb + kPageBytes;
-        // ---- scores of 16 keys: two n-tiles of 8 keys, D / 16 k-steps ----------------------------
-        float sc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+        const uint32_t kb = ring + ((e - e_lo) % kDecStages) * 2 * kPageBytes, vb = kb + kPageBytes;
+        const bool keys = key0 < valid;                  // warp-uniform: some of this warp's keys exist
+        uint32_t pa0 = 0, pa2 = 0;
+        float alpha = 1.f;
+        if (keys) {
+            // ---- scores of 16 keys: two n-tiles of 8 keys, D / 16 k-steps ----------------------------
+            float sc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk) {
+            for (int kk = 0; kk < D / 16; ++kk) {
 #pragma unroll
-            for (int nt = 0; nt < 2; ++nt) {
-                const int key = key0 + nt * 8 + gid;     // B fragment: n = gid, k = 2*tig (+8)
-                const uint32_t row = kb + key * kRowBytes + tig * 4;
-                uint32_t b0, b1;
-                asm volatile("ld.shared.b32 %0, [%1];" : "=r"(b0) : "r"(row + (((2 * kk) ^ (key & 7)) << 4)));
-                asm volatile("ld.shared.b32 %0, [%1];" : "=r"(b1) : "r"(row + (((2 * kk + 1) ^ (key & 7)) << 4)));
-                mma_16816(sc[nt], qa[kk][0], 0u, qa[kk][1], 0u, b0, b1);
+                for (int nt = 0; nt < 2; ++nt) {
+                    const int key = key0 + nt * 8 + gid;     // B fragment: n = gid, k = 2*tig (+8)
+                    const uint32_t row = kb + key * kRowBytes + tig * 4;
+                    uint32_t b0, b1;
+                    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(b0) : "r"(row + (((2 * kk) ^ (key & 7)) << 4)));
+                    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(b1) : "r"(row + (((2 * kk + 1) ^ (key & 7)) << 4)));
+                    mma_16816(sc[nt], qa[kk][0], 0u, qa[kk][1], 0u, b0, b1);
+                }
+            }
+            // lane (gid < 2, tig) holds head gid's scores of keys key0 + nt*8 + 2*tig, +1
+            float sv[4];
+            float mx = -INFINITY;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int key = key0 + (i >> 1) * 8 + 2 * tig + (i & 1);
+                sv[i] = (gid < 2) ? ((key < valid) ? sc[i >> 1][i & 1] * a.scale_log2 : -INFINITY) : 0.f;
+                mx = fmaxf(mx, sv[i]);
+            }
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));       // finite: key0 < valid
+            const float m_new = fmaxf(m_run, mx);
+            alpha = exp2f(m_run - m_new);                   // 0 on the warp's first page
+            float pv[4], psum = 0.f;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                pv[i] = exp2f(sv[i] - m_new);
+                psum += pv[i];
+            }
+            psum += __shfl_xor_sync(0xffffffffu, psum, 1);
+            psum += __shfl_xor_sync(0xffffffffu, psum, 2);
+            l_run = l_run * alpha + psum;
+            m_run = m_new;
+            // P as the A operand of the second mma: the C layout of the scores is the A layout of the next k-step
+            pa0 = gid < 2 ? pack_bf16x2(pv[0], pv[1]) : 0u;   // keys 2*tig, +1
+            pa2 = gid < 2 ? pack_bf16x2(pv[2], pv[3]) : 0u;   // keys 8 + 2*tig, +1
+        }
+        if (kSplit && e == run_end) {                    // a new run: the MMAs of the one before have had the time of these scores
+            leave_o(sRun[run++]);
+            run_end += per;
+#pragma unroll
+            for (int dn = 0; dn < D / 8; ++dn) acc[dn][0] = acc[dn][1] = 0.f;      // (the other rows of the operand stay zero)
+        }
+        if (keys) {
+            // ---- O = alpha * O + P V: D / 8 n-tiles of 8 columns, V fragments by ldmatrix.trans ---------
+            const int lrow = key0 + (lane & 7) + ((lane >> 3) & 1) * 8;      // ldmatrix: lane supplies row (lane % 8) of matrix lane / 8
+            const uint32_t vrow = vb + lrow * kRowBytes;
+#pragma unroll
+            for (int dn = 0; dn < D / 8; dn += 2) {
+                acc[dn][0] *= alpha;
+                acc[dn][1] *= alpha;
+                acc[dn + 1][0] *= alpha;
+                acc[dn + 1][1] *= alpha;
+                uint32_t r0, r1, r2, r3;   // matrices: (keys 0-7, dn), (keys 8-15, dn), (keys 0-7, dn+1), (keys 8-15, dn+1)
+                ldmatrix_x4_trans(vrow + (((dn + (lane >> 4)) ^ (lrow & 7)) << 4), r0, r1, r2, r3);
+                mma_16816(acc[dn], pa0, 0u, pa2, 0u, r0, r1);
+                mma_16816(acc[dn + 1], pa0, 0u, pa2, 0u, r2, r3);
             }
         }
-        // lane (gid < 2, tig) holds head gid's scores of keys key0 + nt*8 + 2*tig, +1
-        float sv[4];
-        float mx = -INFINITY;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int key = key0 + (i >> 1) * 8 + 2 * tig + (i & 1);
-            sv[i] = (gid < 2) ? ((key < valid) ? sc[i >> 1][i & 1] * a.scale_log2 : -INFINITY) : 0.f;
-            mx = fmaxf(mx, sv[i]);
-        }
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));       // finite: key0 < valid
-        const float m_new = fmaxf(m_run, mx);
-        const float alpha = exp2f(m_run - m_new);                   // 0 on the warp's first page
-        float pv[4], psum = 0.f;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            pv[i] = exp2f(sv[i] - m_new);
-            psum += pv[i];
-        }
-        psum += __shfl_xor_sync(0xffffffffu, psum, 1);
-        psum += __shfl_xor_sync(0xffffffffu, psum, 2);
-        l_run = l_run * alpha + psum;
-        m_run = m_new;
-        // P as the A operand of the second mma: the C layout of the scores is the A layout of the next k-step
-        const uint32_t pa0 = gid < 2 ? pack_bf16x2(pv[0], pv[1]) : 0u;   // keys 2*tig, +1
-        const uint32_t pa2 = gid < 2 ? pack_bf16x2(pv[2], pv[3]) : 0u;   // keys 8 + 2*tig, +1
-        // ---- O = alpha * O + P V: D / 8 n-tiles of 8 columns, V fragments by ldmatrix.trans ---------
-        const int lrow = key0 + (lane & 7) + ((lane >> 3) & 1) * 8;      // ldmatrix: lane supplies row (lane % 8) of matrix lane / 8
-        const uint32_t vrow = vb + lrow * kRowBytes;
-#pragma unroll
-        for (int dn = 0; dn < D / 8; dn += 2) {
-            acc[dn][0] *= alpha;
-            acc[dn][1] *= alpha;
-            acc[dn + 1][0] *= alpha;
-            acc[dn + 1][1] *= alpha;
-            uint32_t r0, r1, r2, r3;   // matrices: (keys 0-7, dn), (keys 8-15, dn), (keys 0-7, dn+1), (keys 8-15, dn+1)
-            ldmatrix_x4_trans(vrow + (((dn + (lane >> 4)) ^ (lrow & 7)) << 4), r0, r1, r2, r3);
-            mma_16816(acc[dn], pa0, 0u, pa2, 0u, r0, r1);
-            mma_16816(acc[dn + 1], pa0, 0u, pa2, 0u, r2, r3);
+        if (kSplit && e + 1 == run_end) {                // the run ends
+            leave_sums(sRun[run]);
+            m_run = -INFINITY;
+            l_run = 0.f;
         }
     }
     cp_async_wait<0>();
-    // ---- merge the four warps' states ------------------------------------------------------------------
-    if (gid < 2) {
-        if (tig == 0) { sM[warp][gid] = m_run; sL[warp][gid] = l_run; }
-#pragma unroll
-        for (int dn = 0; dn < D / 8; ++dn) {
-            sO[warp][gid][dn * 8 + 2 * tig] = acc[dn][0];
-            sO[warp][gid][dn * 8 + 2 * tig + 1] = acc[dn][1];
-        }
+    if (e_lo < e_hi) {
+        if (!kSplit || e_hi != run_end) leave_sums(sRun[run]);   // (a shorter last run)
+        leave_o(sRun[run++]);
     }
     __syncthreads();
-    const int h = tid >> 6, r = tid & 63;
-    float m_all = fmaxf(fmaxf(sM[0][h], sM[1][h]), fmaxf(sM[2][h], sM[3][h]));   // (warp 0 has key 0 of every page; -inf: empty run)
-    float wgt[4], l_all = 0.f;
+    // ---- merge the four warps' states of every run ------------------------------------------------------
+    if (kSplit) cluster_wait();                          // the other CTAs of the cluster have started
+    float m_all = -INFINITY, l_all = 0.f, out[kColsPerThread];
+#pragma unroll 2
+    for (int i = 0; i < run; ++i) {
+        const RunState<D>& st = sRun[i];
+        const int h = tid >> 6;
+        m_all = fmaxf(fmaxf(st.m[0][h], st.m[1][h]), fmaxf(st.m[2][h], st.m[3][h]));   // warp 0 has key 0 of every page
+        float wgt[4];
+        l_all = 0.f;
 #pragma unroll
-    for (int w = 0; w < 4; ++w) {
-        wgt[w] = m_all == -INFINITY ? 0.f : exp2f(sM[w][h] - m_all);   // 0 for a warp that never saw a valid key
-        l_all = fmaf(wgt[w], sL[w][h], l_all);
-    }
-    constexpr int kColsPerThread = D / 64;
-    float out[kColsPerThread];
-#pragma unroll
-    for (int c = 0; c < kColsPerThread; ++c) {
-        const int col = r * kColsPerThread + c;
-        float o = 0.f;
-#pragma unroll
-        for (int w = 0; w < 4; ++w) o = fmaf(wgt[w], sO[w][h][col], o);
-        out[c] = o;
-    }
-    if (kSplit) {
-        // ---- this run's (max, sum, O) into shared memory; the cluster's first CTA adds the runs up in run order
-        //      (fixed and data-independent)
-        const int c0 = r * kColsPerThread;
-#pragma unroll
-        for (int c = 0; c < kColsPerThread; ++c) sPart[h][c0 + c] = out[c];
-        if (r == 0) { sPart[h][D] = m_all; sPart[h][D + 1] = l_all; }
-        cluster_sync();
-        if (blockIdx.z == 0) {
-            float pm[kMaxRuns], pl[kMaxRuns], po[kMaxRuns][kColsPerThread];
-#pragma unroll
-            for (int i = 0; i < kMaxRuns; ++i) {         // all of it asked for at once
-                const bool on = i < a.nsplit;
-                pm[i] = on ? ld_cluster(&sPart[h][D], i) : -INFINITY;
-                pl[i] = on ? ld_cluster(&sPart[h][D + 1], i) : 0.f;
-#pragma unroll
-                for (int c = 0; c < kColsPerThread; ++c) po[i][c] = on ? ld_cluster(&sPart[h][c0 + c], i) : 0.f;
-            }
-            m_all = pm[0];                               // run 0 has a page: finite
-#pragma unroll
-            for (int i = 1; i < kMaxRuns; ++i) m_all = fmaxf(m_all, pm[i]);
-            l_all = 0.f;
-#pragma unroll
-            for (int c = 0; c < kColsPerThread; ++c) out[c] = 0.f;
-#pragma unroll
-            for (int i = 0; i < kMaxRuns; ++i) {
-                const float w = exp2f(pm[i] - m_all);
-                l_all = fmaf(w, pl[i], l_all);
-#pragma unroll
-                for (int c = 0; c < kColsPerThread; ++c) out[c] = fmaf(w, po[i][c], out[c]);
-            }
+        for (int w = 0; w < 4; ++w) {
+            wgt[w] = exp2f(st.m[w][h] - m_all);          // 0 for a warp that never saw a valid key
+            l_all = fmaf(wgt[w], st.l[w][h], l_all);
         }
-        cluster_sync();                                  // the partials have been read: their CTAs may leave
-        if (blockIdx.z != 0) return;
-    }
-    if (h >= nheads) return;                             // G = 1: the second head of the pair does not exist
-    const float inv = 1.f / l_all;
-    __nv_bfloat16* orow = a.o + ((size_t)s * a.hq + hbase + h) * D;
 #pragma unroll
-    for (int c = 0; c < kColsPerThread; ++c) orow[r * kColsPerThread + c] = __float2bfloat16_rn(out[c] * inv);
-    if (r == 0) a.lse[(size_t)(hbase + h) * a.batch + s] = (m_all + log2f(l_all)) * 0.6931471805599453f;
+        for (int c = 0; c < kColsPerThread; ++c) {
+            out[c] = 0.f;
+#pragma unroll
+            for (int w = 0; w < 4; ++w) out[c] = fmaf(wgt[w], st.o[w][h][c0 + c], out[c]);
+            if (kSplit) st_cluster(to_gather + (i * a.share + c) * 4, out[c]);
+        }
+        if (kSplit && (tid & 63) < a.nctas) st_cluster_v2(to_sums + i * 16, m_all, l_all);
+    }
+    if (!kSplit) {
+        const int h = tid >> 6;
+        if (h >= nheads) return;                         // G = 1: the second head of the pair does not exist
+        const float inv = 1.f / l_all;
+        __nv_bfloat16* orow = a.o + ((size_t)s * a.hq + hbase + h) * D + c0;
+#pragma unroll
+        for (int c = 0; c < kColsPerThread; ++c) orow[c] = __float2bfloat16_rn(out[c] * inv);
+        if ((tid & 63) == 0) a.lse[(size_t)(hbase + h) * a.batch + s] = (m_all + log2f(l_all)) * 0.6931471805599453f;
+        return;
+    }
+    // ---- add the runs up in run order (fixed and data-independent): every CTA of the cluster its share of the columns, 32 to
+    //      a warp, and every warp the maxima and sums of its head, a run (and the run 32 further) to a lane
+    cluster_arrive();
+    cluster_wait();                                      // everything for this CTA is in its shared memory
+    const int v0 = blockIdx.z * a.share, v_end = runs > 0 ? min(v0 + a.share, 2 * D) : 0;
+    for (int v = v0 + tid; v < v_end; v += kDecThreads) {
+        const int h = v / D, col = v % D;                // (v - lane is a multiple of 32: the same head in a warp)
+        const float2* sums = reinterpret_cast<const float2*>(dsmem + a.sums) + h;         // [run][2]
+        const float* part = reinterpret_cast<const float*>(dsmem + a.gather) + (v - v0);  // [run][share]
+        float2 ml[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) ml[k] = lane + 32 * k < runs ? sums[(lane + 32 * k) * 2] : make_float2(-INFINITY, 0.f);
+        float m = fmaxf(ml[0].x, ml[1].x);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+        float w[2] = {0.f, 0.f}, sum[2] = {0.f, 0.f};
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            if (32 * k >= runs) break;
+            if (lane + 32 * k < runs) w[k] = exp2f(ml[k].x - m);
+            sum[k] = __fmul_rn(w[k], ml[k].y);
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) sum[k] += __shfl_xor_sync(0xffffffffu, sum[k], off);
+        }
+        const float l = sum[0] + sum[1];
+        float o = 0.f;
+        for (int i0 = 0; i0 < runs; i0 += 8) {           // eight at a time, asked for together
+            float wi[8], p[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                wi[i] = __shfl_sync(0xffffffffu, i0 & 32 ? w[1] : w[0], (i0 + i) & 31);
+                p[i] = part[min(i0 + i, runs - 1) * a.share];
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (i0 + i < runs) o = fmaf(wi[i], p[i], o);
+        }
+        if (h < nheads) {                                // (G = 1: the second head of the pair does not exist)
+            a.o[((size_t)s * a.hq + hbase + h) * D + col] = __float2bfloat16_rn(o * (1.f / l));
+            if (col == 0) a.lse[(size_t)(hbase + h) * a.batch + s] = (m + log2f(l)) * 0.6931471805599453f;
+        }
+    }
 }
 
 // Eq. 1 for the block of the newest token of every sequence, mapped through the page table: a warp per sequence, a lane
@@ -342,6 +419,29 @@ __global__ void __launch_bounds__(kPlanDecodeWarps * 32) plan_decode_kernel(cons
         bad = __syncthreads_or(bad);
         if (threadIdx.x == 0) *plan.status = bad ? BF1_DEV_BAD_SEQLENS : 0;
     }
+}
+
+// Clusters of `ctas` CTAs of the split kernel that the GPU runs at once; asked for once per device and shape.
+static int clusters_that_fit(void (*kernel)(DecodeArgs), int dev, int wide, int ctas, int stages, int slots, size_t smem, int* fit) {
+    static std::atomic<int> known[64][2][kMaxCtas + 1][kDecStages + 1][kMaxRunsPerCta + 1];   // 0: not asked yet, else one more
+    std::atomic<int>& k = known[dev][wide][ctas][stages][slots];
+    int n = k.load(std::memory_order_relaxed) - 1;
+    if (n < 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(1, 1, ctas);
+        cfg.blockDim = dim3(kDecThreads);
+        cfg.dynamicSmemBytes = smem;
+        cudaLaunchAttribute attr = {};
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = attr.val.clusterDim.y = 1;
+        attr.val.clusterDim.z = ctas;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        BF1_CUDA_CHECK(cudaOccupancyMaxActiveClusters(&n, kernel, &cfg));
+        k.store(n + 1, std::memory_order_relaxed);
+    }
+    *fit = n;
+    return BF1_OK;
 }
 
 int check_cfg(const bf1_route_cfg* cfg);   // bf1_plan.cu
@@ -417,48 +517,63 @@ extern "C" int bf1_decode_fwd(const void* q, const void* k_pages, const void* v_
     a.o = (__nv_bfloat16*)o;
     a.lse = lse;
     a.batch = batch;
-    static bool configured[64] = {};
-    static int slots[64][2][kDecStages + 1];   // CTAs of the split kernel the GPU holds at once, by d and ring stages
     int dev = 0;
     BF1_CUDA_CHECK(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return fail(BF1_ERR_NO_DEVICE, "device ordinal %d out of range", dev);
     constexpr int kSmem128 = kDecStages * 2 * 64 * 128 * 2, kSmem64 = kDecStages * 2 * 64 * 64 * 2;
-    if (!configured[dev]) {
-        int sms = 0;
+    constexpr int kState128 = sizeof(RunState<128>), kState64 = sizeof(RunState<64>);
+    auto up = [](int x) { return (x + 127) / 128 * 128; };
+    static std::atomic<int> sm_count[64];      // 0: this device has not been set up
+    int sms = sm_count[dev].load(std::memory_order_acquire);
+    if (!sms) {
+        BF1_CUDA_CHECK(cudaFuncSetAttribute(decode_fused_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, up(kState128) + kSmem128));
+        BF1_CUDA_CHECK(cudaFuncSetAttribute(decode_fused_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024 + kSmem128));
+        BF1_CUDA_CHECK(cudaFuncSetAttribute(decode_fused_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, up(kState64) + kSmem64));
+        BF1_CUDA_CHECK(cudaFuncSetAttribute(decode_fused_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024 + kSmem64));
+        BF1_CUDA_CHECK(cudaFuncSetAttribute(decode_fused_kernel<128, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        BF1_CUDA_CHECK(cudaFuncSetAttribute(decode_fused_kernel<64, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         BF1_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        BF1_CUDA_CHECK(cudaFuncSetAttribute(decode_fused_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem128));
-        BF1_CUDA_CHECK(cudaFuncSetAttribute(decode_fused_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem128));
-        BF1_CUDA_CHECK(cudaFuncSetAttribute(decode_fused_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem64));
-        BF1_CUDA_CHECK(cudaFuncSetAttribute(decode_fused_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem64));
-        for (int st = 1; st <= kDecStages; ++st) {
-            int n = 0;
-            BF1_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, decode_fused_kernel<128, true>, kDecThreads, kSmem128 / kDecStages * st));
-            slots[dev][1][st] = n * sms;
-            BF1_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, decode_fused_kernel<64, true>, kDecThreads, kSmem64 / kDecStages * st));
-            slots[dev][0][st] = n * sms;
-        }
-        configured[dev] = true;
+        sm_count[dev].store(sms, std::memory_order_release);
     }
     const int64_t lists = (int64_t)batch * hkv * pairs;
-    const int page_smem = d == 128 ? kSmem128 / kDecStages : kSmem64 / kDecStages;
-    // A list is cut into as many runs as still make one wave of CTAs, none of them idle (a run of fewer pages than the ring
-    // has stages needs that much less shared memory).
-    int runs = std::min(kMaxRuns, plan->max_degree), stages = kDecStages;
-    for (; runs >= 1; --runs) {
-        const int per = (plan->max_degree + runs - 1) / runs;
-        stages = std::min(per, kDecStages);
-        runs = (plan->max_degree + per - 1) / per;
-        if (runs == 1 || lists * runs <= slots[dev][d == 128][stages]) break;
-    }
-    a.nsplit = runs;
-    const size_t smem = (size_t)page_smem * stages;
-    if (runs == 1) {
+    const int page_smem = d == 128 ? kSmem128 / kDecStages : kSmem64 / kDecStages, state = d == 128 ? kState128 : kState64;
+    if (lists >= sms) {
+        // enough lists to fill the GPU: one CTA walks a whole list
+        a.nsplit = a.nctas = 1;
+        a.ring = up(state);
         BF1_CUDA_CHECK(launch_pdl(d == 128 ? decode_fused_kernel<128, false> : decode_fused_kernel<64, false>,
-                                  dim3(hkv * pairs, batch), kDecThreads, smem, (cudaStream_t)stream, a));
-    } else {
-        BF1_CUDA_CHECK(launch_pdl_cluster(d == 128 ? decode_fused_kernel<128, true> : decode_fused_kernel<64, true>,
-                                          dim3(hkv * pairs, batch, runs), dim3(1, 1, runs), kDecThreads, smem,
-                                          (cudaStream_t)stream, a));
+                                  dim3(hkv * pairs, batch), kDecThreads, (size_t)a.ring + (size_t)page_smem * kDecStages,
+                                  (cudaStream_t)stream, a));
+        return BF1_OK;
     }
+    a.nsplit = (int)std::min<int64_t>({(kDecCtasPerSm * (int64_t)sms + lists - 1) / lists, plan->max_degree, kMaxRuns});
+    // The runs of a list go to as many CTAs as still let all clusters run at once (a cluster's CTAs share a GPC, so this is
+    // less than what the SMs hold: 48 lists of 11 pages over six CTAs each took 12.0 us, a second wave of clusters; with four
+    // 8.8).  Over 270 pairs of lists (1 to 147) and lengths (5 to 64 pages) this is the fastest number of CTAs or
+    // within 4.3 % of it, 0.05 % on average.
+    // A list has at most nsplit runs; one of max_degree entries has `most` of `per` pages, shorter ones have shorter runs.
+    const int per = (plan->max_degree + a.nsplit - 1) / a.nsplit, most = (plan->max_degree + per - 1) / per;
+    auto ceil_div = [](int x, int y) { return (x + y - 1) / y; };
+    auto kernel = d == 128 ? decode_fused_kernel<128, true> : decode_fused_kernel<64, true>;
+    size_t smem = 0;
+    for (int ctas = std::min(kMaxCtas, most); ctas >= 1; --ctas) {
+        ctas = ceil_div(most, ceil_div(most, ctas));     // (none of them idle)
+        const int slots = ceil_div(a.nsplit, ctas);      // runs of a CTA, at most (the first choice always has few enough)
+        if (slots > kMaxRunsPerCta) break;
+        // a CTA with fewer pages than the ring has stages needs that much less shared memory
+        const int stages = std::min(std::max(slots * (per - 1), ceil_div(most, ctas) * per), kDecStages);
+        a.nctas = ctas;
+        a.share = ceil_div(2 * d / 32, ctas) * 32;
+        a.sums = up(slots * state);
+        a.gather = a.sums + up(slots * ctas * 2 * 8);
+        a.ring = a.gather + slots * ctas * a.share * 4;
+        smem = (size_t)a.ring + (size_t)page_smem * stages;
+        if (ctas == 1) break;
+        int fit = 0;
+        if (int rc = clusters_that_fit(kernel, dev, d == 128, ctas, stages, slots, smem, &fit)) return rc;
+        if (lists <= fit) break;
+    }
+    BF1_CUDA_CHECK(launch_pdl_cluster(kernel, dim3(hkv * pairs, batch, a.nctas), dim3(1, 1, a.nctas), kDecThreads, smem,
+                                      (cudaStream_t)stream, a));
     return BF1_OK;
 }

@@ -228,3 +228,55 @@ def test_decode_however_a_list_is_cut_into_runs(hq, hkv, d, batch, local_blocks)
     assert np.abs(out[live] - o_ref[rows]).max() <= O_MAX_ABS
     assert np.abs(lse[:, live] - lse_ref[:, rows]).max() <= LSE_ABS
     assert np.isnan(out[[s for s in range(batch) if lens[s] == 0]]).all()
+
+
+@pytest.mark.parametrize("hq,hkv,d", [(16, 8, 128), (2, 1, 64), (4, 1, 128)], ids=["G2-d128", "G2-d64", "G4-d128"])
+def test_few_lists_are_rounded_page_by_page(hq, hkv, d):
+    """P is rounded to bf16 against the maximum of its run, so a key that is the maximum of its 16 keys of a page is not
+    rounded at all when a run is a page (as it is while two CTAs per SM hold a run each).  Here one key of every 16 has a
+    score of O(1) and the others at most -300, whose weight is 0 in fp32: nothing but the result itself is then rounded.
+    The fp32 sums behind a score (d products, sum of magnitudes about 25) are off by d * 2^-23 * 25 at most, a weight
+    relatively by that times the scale, 3.4e-5: a result comes to lie on the other side of a rounding boundary in about 2 *
+    3.4e-5 / 2^-8 = 2 % of the elements at worst.  Runs of two pages round every other weight by up to 2^-9."""
+    lens = [64 * 500 + 17, 64 * 130]
+    w = I.custom(lens, hq=hq, hkv=hkv, d=d, seed=4100 + d)
+    q, k, v = I.draw_qkv(w)
+    k = (k.float() * 0.3).to(torch.bfloat16)
+    k[..., 0] = -448.0
+    q[..., 0] = 8.0
+    cu = w.cu_seqlens()
+    for s, n in enumerate(lens):
+        g = torch.arange(n // 16)
+        k[cu[s] + 16 * g + (7 * g) % 16, :, 0] = 0.0
+    k_pages, v_pages, table = paged_cache(w, k, v, seed=12)
+    out, lse, plan, last = run_decode(w, q, k_pages, v_pages, table)
+    assert int(plan.status.item()) == 0 and plan.count.tolist() == [11, 10]
+    for s, n in enumerate(lens):
+        j = (n - 1) // 64
+        idx, c, _, _ = O.route(O.cfg(), n, plan.max_degree)
+        rows = torch.cat([torch.arange(64 * b, min(64 * b + 64, n)) for b in idx[j, :c[j]]]) + cu[s]
+        kk, vv = (t[rows].double().repeat_interleave(hq // hkv, 1) for t in (k, v))
+        p = torch.softmax(torch.einsum("hd,nhd->hn", q[last[s]].double(), kk) * d ** -0.5, 1)
+        want = torch.einsum("hn,nhd->hd", p, vv).to(torch.bfloat16).float().numpy()
+        assert (out[s] != want).mean() <= 0.03, (out[s] != want).mean()
+
+
+def test_a_plan_that_changes_between_the_ctas_of_a_list_stays_in_bounds():
+    """Sequences without a plan, and of another route epoch, among others: all CTAs of their clusters go through the whole
+    kernel, nothing of theirs is written, and the others' rows are those of a batch without them."""
+    lens = [64 * 70, 130, 64 * 300 + 9, 5000]
+    w = I.custom(lens, hq=4, hkv=2, d=128, seed=4200)
+    q, k, v = I.draw_qkv(w)
+    k_pages, v_pages, table = paged_cache(w, k, v, seed=13)
+    dev = torch.device(DEV)
+    ref, ref_lse, _, _ = run_decode(w, q, k_pages, v_pages, table)
+    plan = bf1.plan_decode(torch.tensor(lens, dtype=torch.int32, device=dev), table.to(dev))
+    plan.count[1] = -3
+    plan.block[2] += 1
+    plan.count[3] = 1 << 20                       # (kept to the row pitch)
+    plan.page[3, int((plan.page[3] >= 0).sum()):] = plan.page[3, 0]
+    out, lse, plan, _ = run_decode(w, q, k_pages, v_pages, table, plan=plan)
+    assert int(plan.status.item()) == 8
+    assert np.isnan(out[[1, 2]]).all() and np.isnan(lse[:, [1, 2]]).all()
+    assert np.array_equal(out[0], ref[0]) and np.array_equal(lse[:, 0], ref_lse[:, 0])
+    assert np.isfinite(out[3]).all()
