@@ -239,7 +239,10 @@ int bf1_decode_fwd(const void *q, const void *k_pages, const void *v_pages, int3
  * and, 16 KB per list entry and pair of query heads, the terms dS that dk, dv and dq share (for as many KV
  * heads at a time as fit 1 GiB, at least one; none when one alone would take more than 8 GiB: they are
  * then computed twice).  Geometry limits as bf1_attn_fwd.  `route` must be the forward's (host struct; only its
- * capacities are used by the size helper). */
+ * capacities are used by the size helper), and more is asked of it than by the forward: the block p that an entry of slot
+ * g names (query block j of its sequence) is looked for in slot g - (j - p), where every route of bf1_plan_route has it.
+ * A route with an entry for which that slot does not exist or is another block (a shard's route, slots in another order)
+ * has no backward: BF1_DEV_BAD_ROUTE is set, and dq, dk and dv are left unwritten. */
 int64_t bf1_attn_bwd_workspace_bytes(const bf1_route *route /* host */, int64_t total_tokens,
                                      int32_t hq, int32_t hkv, int32_t d);
 int bf1_attn_bwd(const void *q, const void *k, const void *v, const void *o, const float *lse,

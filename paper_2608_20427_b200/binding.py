@@ -187,7 +187,8 @@ class Route:
     def from_host(qb_seq, qb_block, kv_count, kv_idx, pair_count, order, total_pairs: int, device,
                   cfg: Optional[RouteCfg] = None) -> "Route":
         """Upload a route the caller built on the host (any ascending lists whose last entry is the
-        query block itself; kv_idx [slots, max_degree] padded with -1).  Marshalling only."""
+        query block itself; kv_idx [slots, max_degree] padded with -1).  Marshalling only.  The forward takes the
+        slots in any order; the backward wants the blocks of a sequence in consecutive slots (see bf1_attn_bwd)."""
         kv_idx = torch.as_tensor(kv_idx, dtype=torch.int32)
         slots, max_degree = kv_idx.shape
         r = Route.empty(max(slots, 1), max_degree, device, cfg)

@@ -51,7 +51,8 @@ constexpr int64_t kDsMost = 8LL << 30;         // one KV head's dS larger than t
 
 // The inverse route and the units of bwd_dkv_kernel, all inside the caller's workspace.
 struct InvPlan {
-    int32_t* count;       // [cap] readers of KV slot g (with multiplicity)
+    int32_t* count;       // [cap] readers of KV slot g (with multiplicity); behind them, of the several-launch path, whether some
+                          // list entry names no slot
     int32_t* start;       // [cap + 1] first reader of slot g in `readers`
     int32_t* unit0;       // [cap + 1] first unit of slot g
     int32_t* chunks;      // [cap] runs the slot's readers are cut into
@@ -90,6 +91,8 @@ struct BwdArgs {
     InvPlan inv;
 };
 
+// The sequence of a slot.
+__device__ __forceinline__ int slot_seq(const BwdArgs& a, int g) { return a.batch > 1 ? a.qb_seq[g] : 0; }
 __device__ __forceinline__ int safe_entry(int p, int e, int cnt, int j) {
     if (p < 0 || p > j || (e == cnt - 1) != (p == j)) p = (e == cnt - 1) ? j : 0;
     return p;
@@ -254,7 +257,7 @@ __device__ __forceinline__ DqUnit dq_unit(const BwdArgs& a, int n, int nqb, int 
         int slot = a.order ? a.order[rank] : rank;
         slot = min(max(slot, 0), nqb - 1);
         u.slot = slot;
-        const int seq = a.batch > 1 ? a.qb_seq[slot] : 0;
+        const int seq = slot_seq(a, slot);
         u.j = a.qb_block[slot];
         u.cnt = min(max(a.kv_count[slot], 1), a.max_degree);
         u.seq0 = a.cu_seqlens[seq];
@@ -283,7 +286,7 @@ __global__ void __launch_bounds__(kDqrThreads, 1) bwd_dq_recompute_kernel(const 
     float* s_lse = s_drow + 256;                                       // [2][128]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (a.status && (*a.status & BF1_DEV_WAIT_TIMEOUT)) return;
-    const int nqb = min(*a.num_qblocks, a.capacity);
+    const int nqb = a.inv.scalars[0] ? min(*a.num_qblocks, a.capacity) : 0;   // (no units: no gradients of this route)
     const int pairs = a.group == 4 ? 2 : 1;
 
     const uint32_t base = smem_u32(smem);
@@ -540,26 +543,34 @@ __global__ void __launch_bounds__(kDqrThreads, 1) bwd_dq_recompute_kernel(const 
 // number of list entries: count (one thread per entry), scan (inverse_units_kernel), fill in whatever order the
 // atomics give, then sort every slot's readers ascending -- the order in which the dK/dV kernel adds is thereby the
 // same on every run.
-__device__ __forceinline__ bool inverse_entry(const BwdArgs& a, int nqb, int f, int& g, int& kv) {
-    g = f / a.max_degree;
-    if (g >= nqb) return false;
-    const int e = f - g * a.max_degree;
+// The slot of an entry's block p lies as many slots in front of its query slot g as p blocks in front of j, because the
+// planner numbers the query blocks of a sequence one after the other.  Nothing else needs that (the forward takes a route
+// with its slots in any order, and a shard's, whose first blocks have no slots), so it is checked for every entry: the slot
+// exists, and it is that block of the same sequence.  One entry for which it is not so and the route has no backward.
+__device__ __forceinline__ bool names_slot(int kv, int nqb, int p, int seq, int batch, const int32_t* block, const int32_t* seqs) {
+    return kv >= 0 && kv < nqb && block[kv] == p && seq >= 0 && seq < batch && (batch == 1 || seqs[kv] == seq);
+}
+// 1: an entry and the slot kv it names; 0: no entry; -1: an entry that names no slot.
+__device__ __forceinline__ int inverse_entry(const BwdArgs& a, int nqb, int f, int& kv) {
+    const int g = f / a.max_degree, e = f - g * a.max_degree;
     const int cnt = min(max(a.kv_count[g], 1), a.max_degree);
-    if (e >= cnt) return false;
-    const int j = a.qb_block[g];
-    kv = g - j + list_entry(a.kv_idx + (size_t)g * a.max_degree, e, cnt, j);   // slots of a sequence are consecutive
-    return true;
+    if (e >= cnt) return 0;
+    const int j = a.qb_block[g], p = list_entry(a.kv_idx + (size_t)g * a.max_degree, e, cnt, j);
+    kv = g - j + p;
+    return names_slot(kv, nqb, p, slot_seq(a, g), a.batch, a.qb_block, a.qb_seq) ? 1 : -1;
 }
 
-// kFill = false: count[kv] += 1 (count is zero on entry).  kFill = true: count[kv] is counted down again and hands out
+// kFill = false: count[kv] += 1 (count, and the word behind it, are zero on entry).  kFill = true: count[kv] is counted down again and hands out
 // the places behind start[kv].
 template <bool kFill>
 __global__ void __launch_bounds__(256) inverse_route_kernel(const BwdArgs a) {
     const int nqb = min(*a.num_qblocks, a.capacity);
     const int total = nqb * a.max_degree;
     for (int f = blockIdx.x * 256 + threadIdx.x; f < total; f += gridDim.x * 256) {
-        int g, kv;
-        if (!inverse_entry(a, nqb, f, g, kv)) continue;
+        int kv;
+        const int is = inverse_entry(a, nqb, f, kv);
+        if (!kFill && is < 0) a.inv.count[a.inv.cap] = 1;
+        if (is <= 0) continue;
         if (!kFill) atomicAdd(a.inv.count + kv, 1);
         else a.inv.readers[a.inv.start[kv] + atomicSub(a.inv.count + kv, 1) - 1] = f;
     }
@@ -683,10 +694,10 @@ __global__ void __launch_bounds__(1024, 1) inverse_units_kernel(const BwdArgs a)
         }
         units += (int)(total & 0x1fffff), parts += (int)(total >> 21 & 0x1fffff), multis += (int)(total >> 42);
     }
-    const bool fits = units <= v.max_units && parts <= v.cap;
+    const bool sound = __ldcg(v.count + v.cap) == 0, fits = sound && units <= v.max_units && parts <= v.cap;
     if (tid == 0) {
         unit0[nqb] = units;
-        if (!fits && a.status) atomicOr(a.status, BF1_DEV_CAPACITY);
+        if (!fits && a.status) atomicOr(a.status, sound ? BF1_DEV_CAPACITY : BF1_DEV_BAD_ROUTE);
         v.scalars[0] = fits ? units : 0;
         v.scalars[1] = readers_total;
         v.scalars[2] = chunk;
@@ -727,7 +738,7 @@ __global__ void __launch_bounds__(1024, 1) inverse_units_kernel(const BwdArgs a)
         for (int un = tid; un < units; un += 1024) {
             int g, begin, end;
             unit_of(un, g, begin, end);
-            const int at = atomicAdd(&s_bin[bin_of(end - begin)], 1), seq = a.qb_seq[g];
+            const int at = atomicAdd(&s_bin[bin_of(end - begin)], 1), seq = slot_seq(a, g);
             const bool split = unit0[g + 1] - unit0[g] > 1;
             const int seq0 = a.cu_seqlens[seq];
             v.units[2 * at] = make_int4(g, begin, end - begin, split ? v.part0[g] + un - unit0[g] : -1);
@@ -747,7 +758,7 @@ __host__ __device__ inline int64_t inverse_words(int64_t cap, int64_t max_degree
 __device__ __forceinline__ void inverse_route_in_cta(const BwdArgs& a, int32_t* smem, int status) {
     __shared__ int32_t s_bin[1024];     // units of a length, then where they start: longest first
     __shared__ unsigned long long s_warp[32];
-    __shared__ int32_t s_total;
+    __shared__ int32_t s_total, s_bad;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const InvPlan& v = a.inv;
     const int entries = a.capacity * a.max_degree;
@@ -766,19 +777,29 @@ __device__ __forceinline__ void inverse_route_in_cta(const BwdArgs& a, int32_t* 
     };
     load(tid);
     const int my_slot = min(tid, a.capacity - 1);
-    const int my_j = a.qb_block[my_slot], my_seq = a.qb_seq[my_slot];
+    const int my_j = a.qb_block[my_slot], my_seq = slot_seq(a, my_slot);
+    // the slots' blocks and sequences, for names_slot(): in the place of the readers until those are filled in (with one
+    // entry to a list there is none to check but the slot itself)
+    int32_t *block = a.max_degree > 1 ? readers : count, *seqs = a.max_degree > 1 ? readers + a.capacity : count;
     const int nqb = min(*a.num_qblocks, a.capacity);
     if (status & BF1_DEV_WAIT_TIMEOUT) return;
+    if (a.max_degree > 1) {
+#pragma unroll 1
+        for (int g = tid; g < a.capacity; g += 1024) {
+            block[g] = g == tid ? my_j : a.qb_block[g];
+            seqs[g] = g == tid ? my_seq : slot_seq(a, g);
+        }
+    }
 #pragma unroll 1
     for (int g = tid; g < a.capacity; g += 1024) count[g] = 0;
     s_bin[tid] = 0;
-    if (tid == 0) s_total = 0;
+    if (tid == 0) s_total = s_bad = 0;
 #pragma unroll 1
     for (int i = tid; i < a.hkv; i += 1024) v.tickets[i] = 0;
     __syncthreads();
     // (a slot behind the last one may hold anything)
     int my_seq0 = 0, my_end = 0;
-    if (tid < nqb) my_seq0 = a.cu_seqlens[my_seq], my_end = a.cu_seqlens[my_seq + 1];
+    if (tid < nqb && my_seq >= 0 && my_seq < a.batch) my_seq0 = a.cu_seqlens[my_seq], my_end = a.cu_seqlens[my_seq + 1];
     int mine = 0;
 #pragma unroll 1
     for (int f0 = tid; f0 < nqb * a.max_degree; f0 += kAtOnce * 1024) {
@@ -790,9 +811,14 @@ __device__ __forceinline__ void inverse_route_in_cta(const BwdArgs& a, int32_t* 
             if (f >= nqb * a.max_degree) continue;
             int kv = -1;
             if (e < cnt) {
-                kv = g - j[i] + safe_entry(p[i], e, cnt, j[i]);
-                atomicAdd(count + kv, 1);
-                ++mine;
+                const int b = safe_entry(p[i], e, cnt, j[i]);
+                kv = g - j[i] + b;
+                if (a.max_degree == 1 || names_slot(kv, nqb, b, seqs[g], a.batch, block, seqs)) {
+                    atomicAdd(count + kv, 1);
+                    ++mine;
+                } else {
+                    s_bad = 1;
+                }
             }
             kv_of[f] = kv;
         }
@@ -800,6 +826,13 @@ __device__ __forceinline__ void inverse_route_in_cta(const BwdArgs& a, int32_t* 
     mine = __reduce_add_sync(0xffffffffu, mine);
     if (lane == 0) atomicAdd(&s_total, mine);
     __syncthreads();
+    if (s_bad) {                     // (uniform over the CTA)
+        if (tid == 0) {
+            if (a.status) atomicOr(a.status, BF1_DEV_BAD_ROUTE);
+            v.scalars[0] = v.scalars[4] = 0;
+        }
+        return;
+    }
     const int readers_total = s_total, chunk = run_length(v, readers_total);
     // prefix sums over the slots of the readers, the units, the partial-sum slots and the slots cut into runs, 16 bits each
     // (there are fewer entries than that); the number of units of every length is counted beside them
@@ -879,7 +912,7 @@ __device__ __forceinline__ void inverse_route_in_cta(const BwdArgs& a, int32_t* 
         for (int g = tid; g < nqb; g += 1024) {
             int seq0 = my_seq0, seqlen = my_end - my_seq0, jg = my_j;
             if (g != tid) {
-                const int seq = a.qb_seq[g];
+                const int seq = slot_seq(a, g);
                 seq0 = a.cu_seqlens[seq], seqlen = a.cu_seqlens[seq + 1] - seq0, jg = a.qb_block[g];
             }
             const int s0 = start[g], n = start[g + 1] - s0, full = n < chunk ? 0 : n / chunk, rest = n - full * chunk;
@@ -1398,7 +1431,7 @@ __device__ __forceinline__ void combine_runs(const BwdArgs& a, int worker, int w
         const int hm = item / (2 * kBlock64), kvh = a.head0 + hm % a.nheads;
         const int gp = a.inv.multi[hm / a.nheads];
         const int runs = a.inv.chunks[gp], q0 = a.inv.part0[gp];
-        const int seq = a.qb_seq[gp], p = a.qb_block[gp];
+        const int seq = slot_seq(a, gp), p = a.qb_block[gp];
         const int seq0 = a.cu_seqlens[seq];
         if (row >= a.cu_seqlens[seq + 1] - seq0 - p * kBlock64) continue;   // key row outside the sequence
         const float* pk = a.partial + (((size_t)q0 * a.hkv + kvh) * 2 + which) * (kBlock64 * D) + row * D + lane * kVec;
@@ -1501,6 +1534,7 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
     DqUnit u;
     if (warp == 10) {       // its first units, beside the status word
         nqb = min(*a.num_qblocks, a.capacity);
+        if (a.inv.scalars[0] == 0) nqb = 0;     // the dK/dV kernel had no units: there is no dS
         u = dq_unit(a, lane, nqb, pairs);
     }
     if (tid == 0 && a.status) {
@@ -1687,7 +1721,7 @@ struct BwdLayout {
     size_t n_count, n_start, n_chunks, n_part0, n_readers, n_units, n_multi;
     BwdLayout(int64_t T, int hq, int hkv, int d, int cap, int max_degree) {
         auto up = [](size_t x) { return (x + 255) / 256 * 256; };
-        n_count = (size_t)cap;
+        n_count = (size_t)cap + 1;
         n_start = (size_t)cap + 1;
         n_chunks = (size_t)cap;
         n_part0 = (size_t)cap;

@@ -280,3 +280,80 @@ def test_gradients_at_the_edges_of_the_inverse_route(lens, spare, route):
         assert np.isfinite(diff).all(), name
         rms = float(np.sqrt((diff ** 2).mean() / (want ** 2).mean()))
         assert rms <= REL_RMS and float(np.abs(diff).max()) <= REL_MAX * float(np.abs(want).max()), (name, rms)
+
+
+def _hand_written(route, slots, pitch, dev):
+    """The planned route with its slots in another order (or some of them only), uploaded as a caller's."""
+    t = {n: getattr(route, n).cpu()[slots] for n in ("qb_seq", "qb_block", "kv_count", "kv_idx", "pair_count")}
+    if pitch:
+        t["kv_idx"] = torch.nn.functional.pad(t["kv_idx"], (0, pitch - t["kv_idx"].shape[1]), value=-1)
+    return bf1.Route.from_host(order=torch.arange(len(slots)), total_pairs=0, device=dev, **t)
+
+
+def _raw_backward(q, k, v, d_o, cu, max_len, route):
+    """Forward, then the C entry point with gradients that hold NaN beforehand; they, and the status words after each."""
+    o, lse = bf1.attn_fwd(q, k, v, cu, max_len, route, out=torch.zeros_like(q), lse=torch.zeros((q.shape[1], q.shape[0]), device=q.device))
+    after_forward = int(route.status.item())
+    ws = bf1.bwd_workspace(route, q.shape[0], q.shape[1], k.shape[1], q.shape[2], q.device)
+    grads = [torch.full_like(t, float("nan")) for t in (q, k, v)]
+    rc = bf1.load().bf1_attn_bwd(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(), d_o.data_ptr(), cu.data_ptr(),
+                                 cu.numel() - 1, q.shape[0], max_len, q.shape[1], k.shape[1], q.shape[2], 0.0, route.c, ws.data_ptr(),
+                                 *(t.data_ptr() for t in grads), torch.cuda.current_stream().cuda_stream)
+    assert rc == 0
+    torch.cuda.synchronize()
+    return grads, after_forward, int(route.status.item())
+
+
+@pytest.mark.parametrize("pitch", [0, 500, 19000], ids=["one-cta", "several-launches", "recompute"])
+def test_routes_whose_blocks_are_not_found_where_the_planner_puts_them(pitch):
+    """The backward looks for block p of an entry as many slots in front of its query slot as p lies in front of the query
+    block.  Routes for which another slot, or none, is there run forward; their backward flags them and writes nothing."""
+    dev = torch.device("cuda:0")
+    w = I.custom([64 * 9 + 5, 64 * 6], hq=4, hkv=2, d=64, seed=7300)
+    q, k, v = (t.to(dev) for t in I.draw_qkv(w))
+    d_o = torch.randn(q.shape, generator=torch.Generator().manual_seed(12)).to(torch.bfloat16).to(dev)
+    cu = bf1.cu_seqlens_tensor(w.seqlens, dev)
+    planned = bf1.plan_route(cu, w.max_seqlen)
+    want, _, st = _raw_backward(q, k, v, d_o, cu, w.max_seqlen, planned)
+    assert st == 0
+    first, second = list(range(10)), list(range(10, 16))
+    # the sequences in the other order: every sequence's slots still follow each other
+    got, st_fwd, st = _raw_backward(q, k, v, d_o, cu, w.max_seqlen, _hand_written(planned, second + first, pitch, dev))
+    assert st_fwd == 0 and st == 0
+    for x, y in zip(got, want):
+        assert pitch > 1000 or torch.equal(x, y)      # (recomputed dS: see the test of the row pitch)
+        assert bool((x.float() - y.float()).abs().max() <= 2.0 ** -7 * y.float().abs().max())
+    for name, slots in (("reversed", first[::-1] + second), ("two swapped", [0, 2, 1] + first[3:] + second), ("no first block", first[1:] + second),
+                        ("a block missing", first[:4] + first[5:] + second), ("interleaved", [x for p in zip(first, second) for x in p])):
+        got, st_fwd, st = _raw_backward(q, k, v, d_o, cu, w.max_seqlen, _hand_written(planned, slots, pitch, dev))
+        assert st_fwd == 0 and st == 8, (name, st_fwd, st)
+        assert all(bool(t.isnan().all()) for t in got), name
+
+
+def test_a_shard_route_has_no_backward_and_a_window_in_mid_sequence_has():
+    dev = torch.device("cuda:0")
+    n = 64 * 20
+    w = I.custom([n], hq=2, hkv=1, d=128, seed=7400)
+    q, k, v = (t.to(dev) for t in I.draw_qkv(w))
+    d_o = torch.randn(q.shape, generator=torch.Generator().manual_seed(13)).to(torch.bfloat16).to(dev)
+    # blocks 12 .. 19 as a shard
+    needed = bf1.shard_needed_blocks(n, 12, 20)
+    route, cu = bf1.plan_route_shard(n, 12, 20, torch.tensor(needed, dtype=torch.int32, device=dev))
+    rows = torch.cat([torch.arange(64 * b, 64 * b + 64) for b in needed + list(range(12, 20))]).to(dev)
+    got, st_fwd, st = _raw_backward(q[rows], k[rows], v[rows], d_o[rows], cu, rows.numel(), route)
+    assert st_fwd == 0 and st == 8 and all(bool(t.isnan().all()) for t in got)
+    # blocks 12 .. 19 with a window of two, those lists cut off at block 12: every block that is named has its slot
+    cfg = bf1.RouteCfg(64, 2, 0, 0)
+    cu = bf1.cu_seqlens_tensor([n], dev)
+    planned = bf1.plan_route(cu, n, cfg)
+    idx = planned.kv_idx.cpu()[12:].clone()
+    count = planned.kv_count.cpu()[12:].clone()
+    idx[0], count[0] = torch.tensor([12, -1, -1]), 1
+    idx[1], count[1] = torch.tensor([12, 13, -1]), 2
+    part = bf1.Route.from_host(torch.zeros(8), torch.arange(12, 20), count, idx, torch.zeros(8), torch.arange(8), 0, dev, cfg)
+    got, st_fwd, st = _raw_backward(q, k, v, d_o, cu, n, part)
+    alone = bf1.cu_seqlens_tensor([64 * 8], dev)
+    want, _, _ = _raw_backward(q[64 * 12:], k[64 * 12:], v[64 * 12:], d_o[64 * 12:], alone, 64 * 8, bf1.plan_route(alone, 64 * 8, cfg))
+    assert st_fwd == 0 and st == 0
+    for x, y in zip(got, want):
+        assert torch.equal(x[64 * 12:], y) and bool(x[:64 * 12].isnan().all())
