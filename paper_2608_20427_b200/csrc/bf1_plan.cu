@@ -20,6 +20,7 @@
 #include <stdarg.h>
 
 #include <algorithm>
+#include <atomic>
 
 #include "bf1_common.cuh"
 
@@ -52,7 +53,7 @@ struct PlanArgs {
 __global__ void __launch_bounds__(kPlanThreads, 1) plan_kernel(const PlanArgs args) {
     extern __shared__ int32_t s_mem[];
     int32_t* s_start = s_mem;  // [batch + 1] first slot of each sequence
-    __shared__ int32_t s_scan[kPlanThreads];
+    __shared__ int32_t s_scan[64];   // totals of the warps, and their sums
     __shared__ int32_t s_bad;
     __shared__ unsigned long long s_total;
 
@@ -292,9 +293,18 @@ extern "C" int bf1_plan_route(const int32_t* cu_seqlens_dev, int32_t batch, int6
         return fail(BF1_ERR_CAPACITY, "route max_degree %d < %d needed for max_seqlen %d", out->max_degree,
                     need_deg, max_seqlen);
     const size_t smem = sizeof(int32_t) * ((size_t)batch + 1 + (size_t)out->max_degree + 1);
-    if (smem > 200 * 1024) return fail(BF1_ERR_UNSUPPORTED, "batch %d or max_degree %d too large for the planner", batch, out->max_degree);
-    if (smem > 48 * 1024)
-        BF1_CUDA_CHECK(cudaFuncSetAttribute(plan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    constexpr int kMostSmem = 200 * 1024;
+    if (smem > kMostSmem) return fail(BF1_ERR_UNSUPPORTED, "batch %d or max_degree %d too large for the planner", batch, out->max_degree);
+    if (smem > 32 * 1024) {   // (48 KB, static shared memory included, need no leave; once per device, so that no call takes back another's)
+        static std::atomic<bool> allowed[64];
+        int dev = 0;
+        BF1_CUDA_CHECK(cudaGetDevice(&dev));
+        if (dev < 0 || dev >= 64) return fail(BF1_ERR_NO_DEVICE, "device ordinal %d out of range", dev);
+        if (!allowed[dev].load(std::memory_order_acquire)) {
+            BF1_CUDA_CHECK(cudaFuncSetAttribute(plan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem));
+            allowed[dev].store(true, std::memory_order_release);
+        }
+    }
     PlanArgs args;
     args.cu_seqlens = cu_seqlens_dev;
     args.batch = batch;

@@ -132,3 +132,9 @@ def test_planner_where_the_scan_of_the_lengths_changes(batch):
         route = bf1.plan_route(cu, longest, route=bf1.Route.empty(slots, deg, cu.device))
         torch.cuda.synchronize()
         assert int(route.status.item()) == bad and int(route.num_qblocks.item()) == 0
+
+
+@pytest.mark.parametrize("batch", [11200, 11800, 12270, 12300, 50000])
+def test_planner_where_its_shared_memory_passes_what_needs_no_leave(batch):
+    """One word for a sequence: 48 KB are passed, together with what the kernel declares itself, at about 12,200 of them."""
+    test_planner_matches_oracle_bit_exact([1] * batch, dict())
