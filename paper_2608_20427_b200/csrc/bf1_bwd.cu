@@ -550,14 +550,15 @@ __global__ void __launch_bounds__(kDqrThreads, 1) bwd_dq_recompute_kernel(const 
 __device__ __forceinline__ bool names_slot(int kv, int nqb, int p, int seq, int batch, const int32_t* block, const int32_t* seqs) {
     return kv >= 0 && kv < nqb && block[kv] == p && seq >= 0 && seq < batch && (batch == 1 || seqs[kv] == seq);
 }
-// 1: an entry and the slot kv it names; 0: no entry; -1: an entry that names no slot.
+// 1: an entry and the slot kv it names; 0: no entry; -1: an entry that names no slot (looked at if kCheck).
+template <bool kCheck>
 __device__ __forceinline__ int inverse_entry(const BwdArgs& a, int nqb, int f, int& kv) {
     const int g = f / a.max_degree, e = f - g * a.max_degree;
     const int cnt = min(max(a.kv_count[g], 1), a.max_degree);
     if (e >= cnt) return 0;
     const int j = a.qb_block[g], p = list_entry(a.kv_idx + (size_t)g * a.max_degree, e, cnt, j);
     kv = g - j + p;
-    return names_slot(kv, nqb, p, slot_seq(a, g), a.batch, a.qb_block, a.qb_seq) ? 1 : -1;
+    return !kCheck || names_slot(kv, nqb, p, slot_seq(a, g), a.batch, a.qb_block, a.qb_seq) ? 1 : -1;
 }
 
 // kFill = false: count[kv] += 1 (count, and the word behind it, are zero on entry).  kFill = true: count[kv] is counted down again and hands out
@@ -566,9 +567,10 @@ template <bool kFill>
 __global__ void __launch_bounds__(256) inverse_route_kernel(const BwdArgs a) {
     const int nqb = min(*a.num_qblocks, a.capacity);
     const int total = nqb * a.max_degree;
+    if (kFill && a.inv.scalars[0] == 0) return;      // (some entry names no slot)
     for (int f = blockIdx.x * 256 + threadIdx.x; f < total; f += gridDim.x * 256) {
         int kv;
-        const int is = inverse_entry(a, nqb, f, kv);
+        const int is = inverse_entry<!kFill>(a, nqb, f, kv);
         if (!kFill && is < 0) a.inv.count[a.inv.cap] = 1;
         if (is <= 0) continue;
         if (!kFill) atomicAdd(a.inv.count + kv, 1);
@@ -753,12 +755,18 @@ __global__ void __launch_bounds__(1024, 1) inverse_units_kernel(const BwdArgs a)
 // the readers are counted in total beside the counts of the slots, so that one prefix sum gives everything; all full runs
 // of a slot have one length, so that a thread counts and places its slot's units with two atomics each; and the units'
 // places are found while the readers are filled in.
+// A slot with many readers (block 0) has a warp go through all entries in order instead of every reader counting the smaller
+// ones, which grows with their square: a backward of 261,000 tokens that read block 0 and their own (4079 readers) takes 236
+// us (2 query heads, d = 64), 592 with the counting alone.  The line lies where the two cost the same at 12,000 entries, the
+// most that fit: 256^2 / 32 steps of the CTA against 12,000 / 32 of one warp, about six times as long each.
+constexpr int kManyReaders = 256;
+constexpr int kInvInts = 24576;     // words of shared memory, at most
 __host__ __device__ inline int64_t inverse_words(int64_t cap, int64_t max_degree) { return 2 * cap + 1 + 2 * cap * max_degree; }
 
 __device__ __forceinline__ void inverse_route_in_cta(const BwdArgs& a, int32_t* smem, int status) {
     __shared__ int32_t s_bin[1024];     // units of a length, then where they start: longest first
     __shared__ unsigned long long s_warp[32];
-    __shared__ int32_t s_total, s_bad;
+    __shared__ int32_t s_total, s_bad, s_nmany, s_many[kInvInts / 2 / kManyReaders];   // (entries take half of the words at most)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const InvPlan& v = a.inv;
     const int entries = a.capacity * a.max_degree;
@@ -793,7 +801,7 @@ __device__ __forceinline__ void inverse_route_in_cta(const BwdArgs& a, int32_t* 
 #pragma unroll 1
     for (int g = tid; g < a.capacity; g += 1024) count[g] = 0;
     s_bin[tid] = 0;
-    if (tid == 0) s_total = s_bad = 0;
+    if (tid == 0) s_total = s_bad = s_nmany = 0;
 #pragma unroll 1
     for (int i = tid; i < a.hkv; i += 1024) v.tickets[i] = 0;
     __syncthreads();
@@ -871,6 +879,7 @@ __device__ __forceinline__ void inverse_route_in_cta(const BwdArgs& a, int32_t* 
             v.chunks[g] = runs;
             v.part0[g] = runs > 1 ? part : -1;
             if (runs > 1) v.multi[at >> 48] = g;
+            if (n > kManyReaders) s_many[atomicAdd(&s_nmany, 1)] = g;
         }
         __syncthreads();
     }
@@ -929,8 +938,21 @@ __device__ __forceinline__ void inverse_route_in_cta(const BwdArgs& a, int32_t* 
     }
     // an entry's place among its slot's readers is the number of smaller ones (they are distinct)
 #pragma unroll 1
+    for (int b = warp; b < s_nmany; b += 32) {
+        const int g = s_many[b];
+        int at = start[g];
+#pragma unroll 4
+        for (int f0 = g * a.max_degree; f0 < nqb * a.max_degree; f0 += 32) {
+            const bool is = f0 + lane < nqb * a.max_degree && kv_of[f0 + lane] == g;
+            const unsigned all = __ballot_sync(0xffffffffu, is);
+            if (is) v.readers[at + __popc(all & ((1u << lane) - 1))] = f0 + lane;
+            at += __popc(all);
+        }
+    }
+#pragma unroll 1
     for (int i = tid; i < readers_total; i += 1024) {
         const int f = readers[i], kv = kv_of[f], s0 = start[kv], s1 = start[kv + 1];
+        if (s1 - s0 > kManyReaders) continue;
         int rank = 0;
 #pragma unroll 4
         for (int k = s0; k < s1; ++k) rank += readers[k] < f;
@@ -947,7 +969,6 @@ __device__ __forceinline__ void inverse_route_in_cta(const BwdArgs& a, int32_t* 
 // inverse route, a scan for each of its sums, a search for every unit and everything behind the number of query blocks: 8.2
 // and 28 us of its own, a forward and backward of 4K tokens 97.6 us, 95.4 as it is; 16K tokens in 12 sequences 163.7 and
 // 162.8.  As launches of their own: 12 and 28 us, with D_i in the dQ kernel.)
-constexpr int kInvInts = 24576;
 template <int D, bool kInverse>
 __global__ void __launch_bounds__(1024, 1) bwd_prep_kernel(const BwdArgs a) {
     extern __shared__ int32_t s_inv[];

@@ -357,3 +357,27 @@ def test_a_shard_route_has_no_backward_and_a_window_in_mid_sequence_has():
     assert st_fwd == 0 and st == 0
     for x, y in zip(got, want):
         assert torch.equal(x[64 * 12:], y) and bool(x[:64 * 12].isnan().all())
+
+
+@pytest.mark.parametrize("lens,kw", [([64 * 257], dict()), ([64 * 700 - 9], dict(local_blocks=0, dyadic=0)),
+                                     ([64 * 300, 64 * 280, 70], dict(local_blocks=1, dyadic=0)), ([64 * 256, 64 * 40], dict())],
+                         ids=["257", "700", "two-of-them", "256"])
+def test_blocks_with_many_readers_are_the_same_however_the_inverse_route_is_made(lens, kw):
+    """Block 0 of a sequence is read by all of its blocks.  In one CTA more than 256 readers are put in order by going
+    through all entries; a pitch too wide for one CTA sorts them in a launch of its own.  The sums run in that order."""
+    dev = torch.device("cuda:0")
+    w = I.custom(lens, hq=2, hkv=1, d=64, seed=7500 + len(lens), **kw)
+    q, k, v = (t.to(dev) for t in I.draw_qkv(w))
+    d_o = torch.randn(q.shape, generator=torch.Generator().manual_seed(14)).to(torch.bfloat16).to(dev)
+    cu = bf1.cu_seqlens_tensor(w.seqlens, dev)
+    cap, deg = bf1.route_capacity(len(lens), w.total_tokens, w.max_seqlen, lib_cfg(w))
+    assert 2 * cap + 1 + 2 * cap * deg <= 24576 < 2 * cap + 1 + 2 * cap * 60
+    grads = []
+    for pitch in (deg, 60):
+        route = bf1.plan_route(cu, w.max_seqlen, lib_cfg(w), route=bf1.Route.empty(cap, pitch, dev, lib_cfg(w)))
+        o, lse = bf1.attn_fwd(q, k, v, cu, w.max_seqlen, route)
+        grads.append(bf1.attn_bwd(q, k, v, o, lse, d_o, cu, w.max_seqlen, route))
+        torch.cuda.synchronize()
+        route.check_status()
+    assert all(torch.equal(x, y) for x, y in zip(*grads))
+    assert all(bool(x.isfinite().all()) for x in grads[0])
