@@ -32,6 +32,8 @@
 // All hand-offs are mbarriers; every wait is bounded (see mbar_wait).
 #include <cuda.h>
 
+#include <atomic>
+
 #include "bf1_common.cuh"
 
 namespace bf1 {
@@ -770,16 +772,16 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 static int get_encode_fn(EncodeTiledFn* fn) {
-    static EncodeTiledFn cached = nullptr;
-    if (!cached) {
+    static std::atomic<EncodeTiledFn> cached{nullptr};
+    if (!cached.load(std::memory_order_relaxed)) {
         void* p = nullptr;
         cudaDriverEntryPointQueryResult qres;
         BF1_CUDA_CHECK(cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &qres));
         if (!p || qres != cudaDriverEntryPointSuccess)
             return fail(BF1_ERR_CUDA, "cuTensorMapEncodeTiled is not available from this driver");
-        cached = reinterpret_cast<EncodeTiledFn>(p);
+        cached.store(reinterpret_cast<EncodeTiledFn>(p), std::memory_order_relaxed);
     }
-    *fn = cached;
+    *fn = cached.load(std::memory_order_relaxed);
     return BF1_OK;
 }
 
@@ -828,17 +830,17 @@ int make_map_4d(CUtensorMap* m, const void* ptr, int64_t T, int H, int d, int he
 
 struct DeviceInfo {
     int sm_count = 0;
-    bool ok = false;
 };
 
 static int device_info(DeviceInfo* out) {
-    static DeviceInfo cache[64];
+    static std::atomic<int> sm_count[64];   // 0: this device has not been set up
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return fail(BF1_ERR_NO_DEVICE, "no CUDA device: %s", cudaGetErrorString(e));
     if (dev < 0 || dev >= 64) return fail(BF1_ERR_NO_DEVICE, "device ordinal %d out of range", dev);
-    if (!cache[dev].ok) {
-        int major = 0, sms = 0;
+    int sms = sm_count[dev].load(std::memory_order_acquire);
+    if (!sms) {
+        int major = 0;
         BF1_CUDA_CHECK(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev));
         if (major != 10) return fail(BF1_ERR_NO_DEVICE, "device compute capability %d.x is not sm_100", major);
         BF1_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -846,10 +848,9 @@ static int device_info(DeviceInfo* out) {
                                             Cfg<128>::kTotal));
         BF1_CUDA_CHECK(cudaFuncSetAttribute(attn_fwd_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             Cfg<64>::kTotal));
-        cache[dev].sm_count = sms;
-        cache[dev].ok = true;
+        sm_count[dev].store(sms, std::memory_order_release);
     }
-    *out = cache[dev];
+    out->sm_count = sms;
     return BF1_OK;
 }
 

@@ -38,6 +38,7 @@
 #include <cuda.h>
 
 #include <algorithm>
+#include <atomic>
 
 #include "bf1_common.cuh"
 
@@ -1798,9 +1799,9 @@ extern "C" int bf1_attn_bwd(const void* q, const void* k, const void* v, const v
     BF1_CUDA_CHECK(cudaGetDevice(&dev));
     BF1_CUDA_CHECK(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev));
     if (major != 10) return fail(BF1_ERR_NO_DEVICE, "device compute capability %d.x is not sm_100", major);
-    static bool configured[64] = {};
+    static std::atomic<bool> configured[64];
     if (dev < 0 || dev >= 64) return fail(BF1_ERR_NO_DEVICE, "device ordinal %d out of range", dev);
-    if (!configured[dev]) {
+    if (!configured[dev].load(std::memory_order_acquire)) {
         const int kInvBytes = kInvInts * (int)sizeof(int32_t);
         BF1_CUDA_CHECK(cudaFuncSetAttribute(bwd_prep_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kInvBytes));
         BF1_CUDA_CHECK(cudaFuncSetAttribute(bwd_prep_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kInvBytes));
@@ -1810,7 +1811,7 @@ extern "C" int bf1_attn_bwd(const void* q, const void* k, const void* v, const v
         BF1_CUDA_CHECK(cudaFuncSetAttribute(bwd_dq_recompute_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, DqrSmem<64>::kTotal));
         BF1_CUDA_CHECK(cudaFuncSetAttribute(bwd_dkv_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, DkvSmem<128>::kTotal));
         BF1_CUDA_CHECK(cudaFuncSetAttribute(bwd_dkv_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, DkvSmem<64>::kTotal));
-        configured[dev] = true;
+        configured[dev].store(true, std::memory_order_release);
     }
     CUtensorMap tq, tk, tv, tg, tdq;
     // Q and dO: two heads and all column chunks per copy; with one head per KV head, one head and one chunk

@@ -23,6 +23,8 @@
 //     rewrites all of it, including the status and hand-out words that must start at zero).
 //     Calls that can overlap on the GPU -- different streams without ordering -- race on it.
 //   - No cudaMalloc, cudaFree or allocating library routine is called.
+#include <atomic>
+
 #include "bf1_common.cuh"
 
 namespace bf1 {
@@ -57,19 +59,19 @@ static __device__ __align__(256) int32_t g_scratch[kScratchWords];
 
 // Device address of g_scratch on the current device, looked up once per device.
 int scratch_address(int32_t** out) {
-    static int32_t* cache[64] = {};
+    static std::atomic<int32_t*> cache[64];
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return bf1::fail(BF1_ERR_NO_DEVICE, "no CUDA device: %s", cudaGetErrorString(e));
     if (dev < 0 || dev >= 64) return bf1::fail(BF1_ERR_NO_DEVICE, "device ordinal %d out of range", dev);
-    if (!cache[dev]) {
+    if (!cache[dev].load(std::memory_order_relaxed)) {
         void* p = nullptr;
         e = cudaGetSymbolAddress(&p, g_scratch);
         if (e != cudaSuccess || !p)
             return bf1::fail(BF1_ERR_CUDA, "cudaGetSymbolAddress(scratch) failed: %s", cudaGetErrorString(e));
-        cache[dev] = static_cast<int32_t*>(p);
+        cache[dev].store(static_cast<int32_t*>(p), std::memory_order_relaxed);
     }
-    *out = cache[dev];
+    *out = cache[dev].load(std::memory_order_relaxed);
     return BF1_OK;
 }
 
