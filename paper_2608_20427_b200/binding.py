@@ -10,6 +10,7 @@ tensors apart and calls the C ABI; what only computes sizes on the host uses cty
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import math
 from dataclasses import dataclass
 from typing import Optional, Sequence
@@ -118,8 +119,10 @@ def _host():
     global _host_module
     if _host_module is None:
         load()
-        _build.build_host()
-        from . import _host as module
+        name = __package__ + "._host"
+        spec = importlib.util.spec_from_file_location(name, _build.build_host())
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
         module.set_error(Bf1Error)
         _host_module = module
     return _host_module

@@ -1,4 +1,4 @@
-"""Builds libbf1.so (the C-ABI library, nvcc for sm_100a) and _host.so (the binding's call path, g++) in-tree."""
+"""Builds libbf1.so (the C-ABI library, nvcc for sm_100a) and the extension module _host (the binding's call path, g++) in-tree."""
 from __future__ import annotations
 
 import os
@@ -9,7 +9,6 @@ import sysconfig
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libbf1.so")
-HOST = os.path.join(HERE, "_host.so")
 HOST_SOURCE = os.path.join(CSRC, "bf1_host.cpp")
 SOURCES = ["bf1_plan.cu", "bf1_attn.cu", "bf1_noalloc.cu", "bf1_decode.cu", "bf1_bwd.cu", "bf1_shard.cu"]
 HEADERS = ["bf1_common.cuh", os.path.join("..", "..", "include", "bf1.h")]
@@ -52,16 +51,24 @@ def build(force: bool = False, verbose: bool = False, out: str = None, defines=(
     return lib
 
 
+def host_path() -> str:
+    """The extension module is compiled against the C++ ABI of one torch and one Python, which its name says: with another of
+    either it is another file."""
+    import torch
+    return os.path.join(HERE, "_host.%s-torch%s.so" % (sys.implementation.cache_tag, torch.__version__))
+
+
 def build_host(force: bool = False) -> str:
-    """Compile the extension module that marshals torch tensors into the C ABI, if it is missing or older than its source;
-    return its path.  It links libbf1.so from its own folder, which has to be there already."""
+    """Compile the extension module that marshals torch tensors into the C ABI, if there is none for this torch and Python or it
+    is older than its source; return its path.  It links libbf1.so from its own folder, which has to be there already."""
     deps = [HOST_SOURCE, os.path.join(CSRC, HEADERS[1])]
-    if not force and os.path.exists(HOST) and all(os.path.getmtime(d) <= os.path.getmtime(HOST) for d in deps):
-        return HOST
+    host = host_path()
+    if not force and os.path.exists(host) and all(os.path.getmtime(d) <= os.path.getmtime(host) for d in deps):
+        return host
     import torch
     root = os.path.dirname(torch.__file__)
     cuda = os.path.join(os.path.dirname(os.path.dirname(_nvcc())) or "/usr/local/cuda", "include")
-    tmp = HOST + ".tmp.%d" % os.getpid()
+    tmp = host + ".tmp.%d" % os.getpid()
     cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI,
            "-I" + sysconfig.get_paths()["include"], "-I" + os.path.join(root, "include"),
            "-I" + os.path.join(root, "include", "torch", "csrc", "api", "include"), "-I" + cuda, HOST_SOURCE, "-o", tmp,
@@ -69,9 +76,9 @@ def build_host(force: bool = False) -> str:
            "-L" + HERE, "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN"]
     res = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
     if res.returncode != 0:
-        raise RuntimeError("g++ failed building _host.so:\n" + res.stdout)
-    os.replace(tmp, HOST)
-    return HOST
+        raise RuntimeError("g++ failed building _host:\n" + res.stdout)
+    os.replace(tmp, host)
+    return host
 
 
 if __name__ == "__main__":

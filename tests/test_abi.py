@@ -78,3 +78,25 @@ def test_route_capacity_is_the_longest_list(kw):
     for nblk in range(1, 301):
         longest = max(longest, int(count[nblk - 1]))
         assert bf1.route_capacity(1, 64 * nblk, 64 * nblk, bf1.RouteCfg(**kw))[1] == longest, nblk
+
+
+def test_the_call_path_is_built_for_the_torch_and_python_at_hand(monkeypatch):
+    """It is compiled against torch's C++ ABI: with another torch in the same tree the module that is there is not used."""
+    import sys
+
+    import torch
+
+    from paper_2608_20427_b200 import build
+    path = build.host_path()
+    assert torch.__version__ in path and sys.implementation.cache_tag in path
+    build.build_host()
+    commands = []
+
+    class Done:
+        returncode, stdout = 0, ""
+
+    monkeypatch.setattr(build.subprocess, "run", lambda cmd, **kw: commands.append(cmd) or Done)
+    monkeypatch.setattr(build.os, "replace", lambda *a: None)
+    assert build.build_host() == path and not commands          # fresh
+    monkeypatch.setattr(torch, "__version__", "0.0.1+other")
+    assert build.build_host() != path and len(commands) == 1
