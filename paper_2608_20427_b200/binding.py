@@ -246,6 +246,8 @@ def attn_fwd_noalloc(q, k, v, cu_seqlens, max_seqlen: int, out, lse, cfg: Option
     For callers that must not allocate device memory, so `out` and `lse` are required here and
     the call itself allocates nothing (neither through torch nor through CUDA).  Up to 4096
     query blocks per batch; calls sharing a GPU must not overlap in time."""
+    if out is None or lse is None:
+        raise TypeError("attn_fwd_noalloc allocates nothing: out and lse are required")
     cfg = cfg or RouteCfg()
     return _host().forward(2, q, k, v, cu_seqlens, max_seqlen, scale, out, lse, _stream_ptr(stream),
                            getattr(cu_seqlens, "_bf1_total", None), ctypes.addressof(cfg), status)

@@ -100,3 +100,12 @@ def test_the_call_path_is_built_for_the_torch_and_python_at_hand(monkeypatch):
     assert build.build_host() == path and not commands          # fresh
     monkeypatch.setattr(torch, "__version__", "0.0.1+other")
     assert build.build_host() != path and len(commands) == 1
+
+
+def test_the_call_without_allocation_wants_its_outputs():
+    import torch
+    q, kv = torch.zeros(64, 2, 64, dtype=torch.bfloat16), torch.zeros(64, 1, 64, dtype=torch.bfloat16)
+    cu, lse = torch.tensor([0, 64], dtype=torch.int32), torch.zeros(2, 64)
+    for out, l in ((None, lse), (torch.zeros_like(q), None), (None, None)):
+        with pytest.raises(TypeError, match="out and lse"):
+            bf1.attn_fwd_noalloc(q, kv, kv, cu, 64, out, l)
