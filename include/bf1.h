@@ -208,8 +208,8 @@ int bf1_plan_decode(const int32_t *seqlens_dev, const int32_t *page_table_dev,
                     int32_t max_pages_per_seq, int32_t batch, const bf1_route_cfg *cfg /* host */,
                     const bf1_decode_plan *out /* host struct, device arrays */, void *stream);
 
-/* Bytes of device scratch bf1_decode_fwd may use.  Host only; -1 on bad arguments.  (The present kernels keep
- * the partial results of the split over pages on the chip and leave the scratch alone.) */
+/* Bytes of device scratch bf1_decode_fwd may use.  Host only; -1 on bad arguments.  (16: the partial results of the split
+ * over pages stay on the chip, and the scratch is left alone.) */
 int64_t bf1_decode_workspace_bytes(int32_t batch, int32_t hq, int32_t hkv, int32_t max_degree,
                                    int32_t d);
 
@@ -217,8 +217,7 @@ int64_t bf1_decode_workspace_bytes(int32_t batch, int32_t hq, int32_t hkv, int32
  *   q            device bf16 [batch, hq, d]: the newest token's queries
  *   seqlens_dev  [batch] current cached lengths INCLUDING the newest token; must lie in the block
  *                the plan was made for, otherwise BF1_DEV_BAD_ROUTE is set and the sequence skipped
- *   workspace    device, 16-byte aligned, bf1_decode_workspace_bytes() bytes, all zero before the
- *                first call; can be reused by calls that do not overlap on the GPU
+ *   workspace    device, 16-byte aligned, bf1_decode_workspace_bytes() bytes, whatever they hold
  *   o            device bf16 [batch, hq, d];  lse  device fp32 [hq, batch]
  * Rows of empty sequences are not written.  Geometry limits as for bf1_attn_fwd. */
 int bf1_decode_fwd(const void *q, const void *k_pages, const void *v_pages, int32_t num_pages,

@@ -285,7 +285,7 @@ def plan_decode(seqlens: torch.Tensor, page_table: torch.Tensor, cfg: Optional[R
 
 
 def decode_workspace(batch: int, hq: int, hkv: int, max_degree: int, d: int, device) -> torch.Tensor:
-    """Zero-initialised scratch for decode_fwd (reusable across calls that do not overlap)."""
+    """Scratch for decode_fwd (reusable; its contents do not matter)."""
     nbytes = int(load().bf1_decode_workspace_bytes(batch, hq, hkv, max_degree, d))
     return torch.zeros(max(nbytes, 16), dtype=torch.uint8, device=device)
 

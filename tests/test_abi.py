@@ -109,3 +109,12 @@ def test_the_call_without_allocation_wants_its_outputs():
     for out, l in ((None, lse), (torch.zeros_like(q), None), (None, None)):
         with pytest.raises(TypeError, match="out and lse"):
             bf1.attn_fwd_noalloc(q, kv, kv, cu, 64, out, l)
+
+
+def test_decode_scratch_is_no_larger_than_what_is_used():
+    """Partial results stay on the chip: nothing grows with the batch, its heads or its lists."""
+    lib = bf1.load()
+    for args in ((1, 16, 8, 11, 128), (0, 2, 1, 1, 64), (65535, 64, 16, 64, 128)):
+        assert lib.bf1_decode_workspace_bytes(*args) == 16
+    for args in ((-1, 16, 8, 11, 128), (1, 0, 8, 11, 128), (1, 16, 0, 11, 128), (1, 15, 8, 11, 128), (1, 16, 8, 0, 128), (1, 16, 8, 11, 0)):
+        assert lib.bf1_decode_workspace_bytes(*args) == -1
