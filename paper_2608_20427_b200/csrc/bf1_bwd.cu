@@ -30,7 +30,7 @@
 // 1.02 -> 0.944 ms at 32K.
 // A route whose dS would not fit (kDsMost for one KV head) is run by bwd_dq_recompute_kernel instead.
 //
-// The compute kernels are persistent: one CTA of 10 to 16 warps per SM that walks through its share of the units, with
+// The compute kernels are persistent: one CTA of 11 or 16 warps per SM that walks through its share of the units, with
 // warps for copies, for issuing MMAs, for the arithmetic on S and dP and for reading finished sums out, so that copies,
 // MMAs and arithmetic of neighbouring entries and units overlap (see the comment in front of each kernel).  P is rounded
 // to bf16 before the MMAs, as in the forward.  With d = 64 the transposed products still run as M = 128 MMAs:
@@ -48,7 +48,11 @@ constexpr int kBlock64 = 64;     // b: tokens per block
 constexpr int kMinChunk = 16;    // readers per dK/dV unit, at least
 constexpr int kDsTile = 128 * 64 * 2;          // bytes of one dS tile: [128 q rows][64 kv], 128-byte rows, swizzled
 constexpr int64_t kDsGroup = 1LL << 30;        // dS kept at a time: as many KV heads as fit this (at least one)
-constexpr int64_t kDsMost = 8LL << 30;         // one KV head's dS larger than this is not kept but computed again
+// One KV head's dS larger than this is not kept but computed again.  Keeping it is faster at every size that was measured, so
+// the line is drawn by what a caller may be asked for.  Kept against computed again (a backward with one KV head, two
+// query heads, d = 128): 4K tokens 41 / 54 us, 32K 107 / 136, 262K (0.9 GB) 953 / 1114, 1M (4.3 GB) 4895 / 5450; 64K
+// tokens with windows of 63 blocks (1.1 GB) 880 / 1041, of 500 (8.4 GB) 5240 / 5810.
+constexpr int64_t kDsMost = 8LL << 30;
 
 // The inverse route and the units of bwd_dkv_kernel, all inside the caller's workspace.
 struct InvPlan {
@@ -963,8 +967,9 @@ __device__ __forceinline__ void inverse_route_in_cta(const BwdArgs& a, int32_t* 
 
 // D_i = <dO_i, O_i> of every row, and (kInverse) in the first CTA the whole inverse route: a chain of a few
 // microseconds on one SM that is hidden behind the pass over dO and O on the others.  kInverse is chosen while the
-// entries fit shared memory beside the counters (kInvInts words): up to about 64K tokens with the
-// paper's route; beyond, several launches share the work.
+// entries fit shared memory beside the counters (kInvInts words): up to 945 query blocks of one sequence with
+// the paper's route, 60,480 tokens; beyond, several launches share the work.  Where the two meet they cost the same: a backward of
+// 60,480 tokens 197.7 us, of 60,500 196.9 (2 query heads, d = 64).
 // Measured: 7 us at 4K tokens (16 query heads, d = 128), of which the pass over dO and O alone takes 5.1 and the inverse
 // route alone 6.9, and 48 us at 32K, where the inverse route alone takes 21.  (With more dependent steps in the
 // inverse route, a scan for each of its sums, a search for every unit and everything behind the number of query blocks: 8.2
@@ -1035,8 +1040,8 @@ __global__ void __launch_bounds__(1024, 1) bwd_prep_kernel(const BwdArgs a) {
 //               the workspace, as it lies in shared memory: its own MMAs read the tile at the same time
 //     warps 4-11   the arithmetic on S and dP (two threads per tile row), P and dS as bf16 tiles to shared memory
 //     warps 12-15  the finished sums of the unit before, from tensor memory to global memory
-// A step moves 304 KB through shared memory (192 KB of MMA operands, 64 KB in, P and dS written, dS read again):
-// 2375 cycles at 128 bytes per cycle, which is the bound.
+// A step moves 304 KiB through shared memory (192 of MMA operands, 64 in, P and dS written, dS read again): 2432 cycles
+// at 128 bytes per cycle, which is the bound.
 // Units described through shared memory, LSE and D_i brought there a step ahead and dynamic hand-out: 55 -> 46 us at 4K
 // tokens, 96 -> 76 us for 16K tokens in 12 sequences (four heads per KV head), 544 -> 483 us at 32K.  (Every role read the
 // unit and the rows' LSE from global memory itself before: 940 of 2900 cycles of a step in the arithmetic warps; and

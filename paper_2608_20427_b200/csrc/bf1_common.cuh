@@ -65,9 +65,10 @@ __host__ __device__ inline int list_tile(const ListShape& s, int f, int e) {
 // ---- programmatic dependent launch ---------------------------------------------------------------------------
 // The kernels of a call (and of consecutive calls on a stream) are short, and each begins with a set-up that needs
 // nothing from the one in front: barriers, tensor memory, tensor maps.  They are launched so that their start and this
-// set-up overlap the end of the kernel in front (the forward waits first and sets up beside its first loads).  pdl_wait() stands in front of a kernel's first access to global memory,
-// reads and writes alike, in every thread that makes one, and on every path out of the kernel: it returns when the kernel
-// in front is complete and its writes are visible, and through that kernel's own wait everything before it.
+// set-up overlap the end of the kernel in front (the forward waits first and sets up beside its first loads).  pdl_wait()
+// stands in front of a kernel's first access to global memory, reads and writes alike, in every thread that makes one,
+// and on every path out of the kernel: it returns when the kernel in front is complete and its writes are visible, and
+// through that kernel's own wait everything before it.
 // No kernel lets the next one start earlier than at its own end (griddepcontrol.launch_dependents): tried right behind the
 // set-up, the waiting CTAs cost the running ones more than they gained (forward and backward of 4K tokens: 106.8 us
 // without any of this, 106.6 with the early start, 99.3 as it is; 32K tokens: 892, 925, 893), started as late as a CTA's
@@ -192,13 +193,6 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const void* tmap, int 
         "[%0], [%1, {%2, %3, %4, %5}], [%6];"
         ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
         : "memory");
-}
-// TMA prefetch of a tile into L2 only (no shared-memory destination, no completion signal).
-__device__ __forceinline__ void tma_prefetch_l2_4d(const void* tmap, int c0, int c1, int c2, int c3) {
-    asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile [%0, {%1, %2, %3, %4}];" ::"l"(
-                     reinterpret_cast<uint64_t>(tmap)),
-                 "r"(c0), "r"(c1), "r"(c2), "r"(c3)
-                 : "memory");
 }
 // TMA: 3-D tiled store shared -> global (bulk async group), and the group bookkeeping.
 __device__ __forceinline__ void tma_store_3d(const void* tmap, int c0, int c1, int c2, uint32_t src) {
