@@ -970,8 +970,9 @@ __device__ __forceinline__ void inverse_route_in_cta(const BwdArgs& a, int32_t* 
 // entries fit shared memory beside the counters (kInvInts words): up to 945 query blocks of one sequence with
 // the paper's route, 60,480 tokens; beyond, several launches share the work.  Where the two meet they cost the same: a backward of
 // 60,480 tokens 197.7 us, of 60,500 196.9 (2 query heads, d = 64).
-// Measured: 7 us at 4K tokens (16 query heads, d = 128), of which the pass over dO and O alone takes 5.1 and the inverse
-// route alone 6.9, and 48 us at 32K, where the inverse route alone takes 21.  (With more dependent steps in the
+// Measured: 8 us at 4K tokens (16 query heads, d = 128), of which the pass over dO and O alone takes 5.1 and the inverse
+// route alone 7.8 (7.5 without looking at the slot that an entry names; looking at four entries' slots without a branch, all
+// at once: 9.7), and 48 us at 32K, where the inverse route alone takes 22.  (With more dependent steps in the
 // inverse route, a scan for each of its sums, a search for every unit and everything behind the number of query blocks: 8.2
 // and 28 us of its own, a forward and backward of 4K tokens 97.6 us, 95.4 as it is; 16K tokens in 12 sequences 163.7 and
 // 162.8.  As launches of their own: 12 and 28 us, with D_i in the dQ kernel.)
