@@ -52,7 +52,7 @@ def run_decode(w, q, k_pages, v_pages, table, seqlens=None, plan=None):
     ws = bf1.decode_workspace(len(w.seqlens), w.hq, w.hkv, plan.max_degree, w.d, dev)
     out = torch.full((len(w.seqlens), w.hq, w.d), float("nan"), dtype=torch.bfloat16, device=dev)
     lse = torch.full((w.hq, len(w.seqlens)), float("nan"), dtype=torch.float32, device=dev)
-    for _ in range(2):   # twice: the second call finds the ticket words the first one left
+    for _ in range(2):   # twice: a call leaves nothing behind (the scratch is looked at below)
         bf1.decode_fwd(qd, k_pages.to(dev), v_pages.to(dev), sl, plan, ws, out=out, lse=lse)
     torch.cuda.synchronize()
     pairs = (w.hq // w.hkv + 1) // 2
