@@ -181,6 +181,49 @@ __device__ __forceinline__ void decode_slot(const AttnArgs& a, const Place& pl, 
     un.tok0 = un.seq0 + un.j * kBlock + pl.tok_off;
 }
 
+// ---- pieces of the softmax: one thread per row of a 128 x 64 tile of scores in tensor memory ----
+// The tile's 64 exponentials are what bounds a warp: 550 cycles of special-function unit if it does nothing else, 560 to 600 with
+// all of this (two to four warps on a scheduler; without the exponentials 190).
+__device__ __forceinline__ void load_scores(uint32_t t_s, uint32_t (&s)[64]) {
+    uint32_t (&lo)[32] = *reinterpret_cast<uint32_t (*)[32]>(&s[0]);
+    uint32_t (&hi)[32] = *reinterpret_cast<uint32_t (*)[32]>(&s[32]);
+    tmem_ld32(t_s, lo);
+    tmem_ld32(t_s + 32, hi);
+    tmem_wait_ld();
+}
+__device__ __forceinline__ void mask_behind(uint32_t (&s)[64], int last) {   // columns behind `last` do not exist for this row
+#pragma unroll
+    for (int c = 0; c < 64; ++c)
+        if (c > last) s[c] = 0xff800000u;   // -inf
+}
+__device__ __forceinline__ float row_max(const uint32_t (&s)[64]) {
+    float a = -INFINITY, b = -INFINITY;
+#pragma unroll
+    for (int c = 0; c < 64; c += 4) {
+        a = fmax3(a, __uint_as_float(s[c]), __uint_as_float(s[c + 1]));
+        b = fmax3(b, __uint_as_float(s[c + 2]), __uint_as_float(s[c + 3]));
+    }
+    return fmaxf(a, b);
+}
+// p = exp2((s - m) * c2) as bf16 pairs; returns the sum of the unrounded weights.
+__device__ __forceinline__ float weights(const uint32_t (&s)[64], float m, float c2, uint32_t (&p)[32]) {
+    const float msc = m * c2;
+    const uint64_t c2p = pack2(c2, c2), mscp = pack2(-msc, -msc);
+    uint64_t sum_a = pack2(0.f, 0.f), sum_b = sum_a;
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {
+        const uint64_t x = fma2(pack2(__uint_as_float(s[2 * c]), __uint_as_float(s[2 * c + 1])), c2p, mscp);
+        float x0, x1;
+        unpack2(x, x0, x1);
+        const float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
+        if (c & 1) sum_b = add2(sum_b, pack2(p0, p1)); else sum_a = add2(sum_a, pack2(p0, p1));
+        p[c] = pack_bf16x2(p0, p1);
+    }
+    float r0, r1;
+    unpack2(add2(sum_a, sum_b), r0, r1);
+    return r0 + r1;
+}
+
 template <int REGS>
 __device__ __forceinline__ void setmaxnreg_inc() {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS));
@@ -604,69 +647,38 @@ __global__ void __launch_bounds__(kThreads, 2) attn_fwd_kernel(const __grid_cons
                 // values it already had, so a row's arithmetic depends on that row alone (later tokens of the
                 // block cannot change it).
                 uint32_t preg[32];
-                float tile_sum = 0.f;
-                bool tripped = false;
-#pragma unroll 1
-                for (int pass = 0; pass < 2; ++pass) {
+                float tile_sum;
+                {
                     uint32_t sreg[64];
-                    {
-                        uint32_t (&lo)[32] = *reinterpret_cast<uint32_t (*)[32]>(&sreg[0]);
-                        uint32_t (&hi)[32] = *reinterpret_cast<uint32_t (*)[32]>(&sreg[32]);
-                        tmem_ld32(t_s, lo);
-                        tmem_ld32(t_s + 32, hi);
+                    load_scores(t_s, sreg);
+                    if (i == cnt - 1) mask_behind(sreg, tl);   // self block: causal triangle (warp-uniform branch)
+                    if (i == 0) m_used = row_max(sreg);
+                    tile_sum = weights(sreg, m_used, c2, preg);
+                }
+                // (The second pass is code of its own: as a loop around one copy of it the tile cost 889 cycles at 32K tokens and 767 in
+                // dense mode, 875 and 757 as it is; 167.9 -> 165.9 us for 32K tokens once in a while, 1 % back to back.)
+                const bool tripped = i > 0 && !(tile_sum < kSumGuard);
+                if (__builtin_expect(__any_sync(0xffffffffu, tripped), 0)) {
+                    uint32_t sreg[64];
+                    load_scores(t_s, sreg);
+                    if (i == cnt - 1) mask_behind(sreg, tl);
+                    const float mx = row_max(sreg);
+                    const float alpha = tripped ? ex2_approx((m_used - mx) * c2) : 1.0f;
+                    l_run *= alpha;
+                    m_used = tripped ? mx : m_used;
+                    // O holds the sum up to tile i-1 once PV(g-1) has completed
+                    mbar_wait(bar_pv_done + 8 * ((g - 1) & 1), ((g - 1) >> 1) & 1, abort_flag, args.status);
+                    tc_fence_after();
+#pragma unroll
+                    for (int c = 0; c < D / 16; ++c) {
+                        uint32_t oreg[16];
+                        tmem_ld16(t_lane + C::kColO + c * 16, oreg);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) oreg[e] = __float_as_uint(__uint_as_float(oreg[e]) * alpha);
+                        tmem_st16(t_lane + C::kColO + c * 16, oreg);
                     }
-                    tmem_wait_ld();
-                    if (i == cnt - 1) {   // self block: causal triangle (warp-uniform branch)
-#pragma unroll
-                        for (int c = 0; c < 64; ++c)
-                            if (c > tl) sreg[c] = 0xff800000u;   // -inf
-                    }
-                    if (i == 0 || pass == 1) {
-                        float mxa = -INFINITY, mxb = -INFINITY;
-#pragma unroll
-                        for (int c = 0; c < 64; c += 4) {
-                            mxa = fmax3(mxa, __uint_as_float(sreg[c]), __uint_as_float(sreg[c + 1]));
-                            mxb = fmax3(mxb, __uint_as_float(sreg[c + 2]), __uint_as_float(sreg[c + 3]));
-                        }
-                        const float mx = fmaxf(mxa, mxb);
-                        if (i == 0) {
-                            m_used = mx;
-                        } else {
-                            const float alpha = tripped ? ex2_approx((m_used - mx) * c2) : 1.0f;
-                            l_run *= alpha;
-                            m_used = tripped ? mx : m_used;
-                            // O holds the sum up to tile i-1 once PV(g-1) has completed
-                            mbar_wait(bar_pv_done + 8 * ((g - 1) & 1), ((g - 1) >> 1) & 1, abort_flag, args.status);
-                            tc_fence_after();
-#pragma unroll
-                            for (int c = 0; c < D / 16; ++c) {
-                                uint32_t oreg[16];
-                                tmem_ld16(t_lane + C::kColO + c * 16, oreg);
-                                tmem_wait_ld();
-#pragma unroll
-                                for (int e = 0; e < 16; ++e) oreg[e] = __float_as_uint(__uint_as_float(oreg[e]) * alpha);
-                                tmem_st16(t_lane + C::kColO + c * 16, oreg);
-                            }
-                        }
-                    }
-                    const float msc = m_used * c2;
-                    const uint64_t c2p = pack2(c2, c2), mscp = pack2(-msc, -msc);
-                    uint64_t sum_a = pack2(0.f, 0.f), sum_b = sum_a;
-#pragma unroll
-                    for (int c = 0; c < 32; ++c) {
-                        const uint64_t x = fma2(pack2(__uint_as_float(sreg[2 * c]), __uint_as_float(sreg[2 * c + 1])), c2p, mscp);
-                        float x0, x1;
-                        unpack2(x, x0, x1);
-                        const float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
-                        if (c & 1) sum_b = add2(sum_b, pack2(p0, p1)); else sum_a = add2(sum_a, pack2(p0, p1));
-                        preg[c] = pack_bf16x2(p0, p1);
-                    }
-                    float r0, r1;
-                    unpack2(add2(sum_a, sum_b), r0, r1);
-                    tile_sum = r0 + r1;
-                    if (i == 0 || pass == 1) break;
-                    tripped = !(tile_sum < kSumGuard);
-                    if (!__any_sync(0xffffffffu, tripped)) break;
+                    tile_sum = weights(sreg, m_used, c2, preg);
                 }
                 l_run += tile_sum;
                 tmem_st32(t_s, preg);   // P overwrites the first 32 columns of this S buffer
