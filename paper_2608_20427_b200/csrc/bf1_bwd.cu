@@ -45,7 +45,8 @@
 namespace bf1 {
 
 constexpr int kBlock64 = 64;     // b: tokens per block
-constexpr int kMinChunk = 16;    // readers per dK/dV unit, at least
+constexpr int kLeastChunk = 2, kMostChunk = 16;   // readers per dK/dV unit (run_length() chooses)
+constexpr int kSms = 148;        // (sizes of the workspace only)
 constexpr int kDsTile = 128 * 64 * 2;          // bytes of one dS tile: [128 q rows][64 kv], 128-byte rows, swizzled
 constexpr int64_t kDsGroup = 1LL << 30;        // dS kept at a time: as many KV heads as fit this (at least one)
 // One KV head's dS larger than this is not kept but computed again.  Keeping it is faster at every size that was measured, so
@@ -68,7 +69,7 @@ struct InvPlan {
     int32_t* tickets;     // [hkv] hand-out counters of the dK/dV launches, by first KV head
     int32_t* multi;       // [cap] the KV slots whose readers were cut into more than one run
     int32_t* scalars;     // [8] number of units, total readers, chunk, partial slots, slots in `multi`
-    int32_t cap, max_units;
+    int32_t cap, max_units, max_parts;
 };
 
 struct BwdArgs {
@@ -81,6 +82,7 @@ struct BwdArgs {
     const int32_t* order;      // may be null
     int32_t batch, max_degree, capacity, total_tokens, hq, hkv, group;
     int32_t head0, nheads; // KV heads this launch works on: head0 .. head0 + nheads - 1
+    int32_t sms;           // of this GPU
     int32_t interleave;    // 1: units of all KV heads interleaved (longest first over all heads); 0: KV head by KV head
     int32_t* status;
     float scale, scale_log2;
@@ -633,10 +635,16 @@ __global__ void __launch_bounds__(256) inverse_sort_kernel(const BwdArgs a) {
     }
 }
 
-// Runs of at least kMinChunk readers, and long enough that the slots with more than one run cannot need more than `cap`
-// partial-sum slots between them (such a slot has fewer than 2 * count / chunk runs).
-__device__ __forceinline__ int run_length(const InvPlan& v, int readers_total) {
-    return max(kMinChunk, (2 * readers_total + max(v.cap, 1) - 1) / max(v.cap, 1));
+// Readers to a run: two more than what an SM gets on average, at most 16 (a unit's K, V and sums are moved once for them), and
+// never so few that the slots with more than one run need more than `max_parts` partial-sum slots between them (such a slot
+// has fewer than 2 * count / chunk runs).  With 16 everywhere the readers of block 0 were one unit of 16 steps, 1.4 us each,
+// while most SMs had less.  A backward in us with runs of 2 / 4 / 6 / 8 / 12 / 16 readers: 1000 tokens, 2 query heads, d = 64 (0.5
+// readers an SM) 20.0 / 22.6 / 24.6 / 27.1 / 31.9 / 37.3; 8 heads, d = 128 (2.1) 28.3 / 25.0 / 26.1 / 28.0 / 32.7 / 38.1; 4096 tokens,
+// 2 heads (3.0) 35.1 / 30.5 / 29.6 / 29.6 / 33.8 / 38.4; 2000 tokens, 16 heads (10) 75 / 55 / 38.3 / 37.6 / 37.3 / 41.8; 4096
+// tokens, 8 heads (12) 88 / 66 / 51.8 / 41.9 / 41.4 / 43.8; from 15 readers an SM on 10, 12 and 16 cost the same.
+__device__ __forceinline__ int run_length(const BwdArgs& a, int readers_total) {
+    const int even = (int)min((long long)readers_total * a.hkv / a.sms + kLeastChunk, (long long)kMostChunk);
+    return max(even, (2 * readers_total + a.inv.max_parts - 1) / a.inv.max_parts);
 }
 
 // One CTA: offsets of the reader lists, the run length, and the units of the dK/dV kernel.  inverse_route_kernel has
@@ -682,7 +690,7 @@ __global__ void __launch_bounds__(1024, 1) inverse_units_kernel(const BwdArgs a)
         readers_total += (int)total;
     }
     if (tid == 0) start[nqb] = readers_total;
-    const int chunk = run_length(v, readers_total);
+    const int chunk = run_length(a, readers_total);
     // pass 2: runs per slot -> unit numbers, partial-sum slots and places in `multi`: one scan, 21 bits each
     int units = 0, parts = 0, multis = 0;
     for (int b0 = 0; b0 < nqb; b0 += 1024) {
@@ -701,7 +709,7 @@ __global__ void __launch_bounds__(1024, 1) inverse_units_kernel(const BwdArgs a)
         }
         units += (int)(total & 0x1fffff), parts += (int)(total >> 21 & 0x1fffff), multis += (int)(total >> 42);
     }
-    const bool sound = __ldcg(v.count + v.cap) == 0, fits = sound && units <= v.max_units && parts <= v.cap;
+    const bool sound = __ldcg(v.count + v.cap) == 0, fits = sound && units <= v.max_units && parts <= v.max_parts;
     if (tid == 0) {
         unit0[nqb] = units;
         if (!fits && a.status) atomicOr(a.status, sound ? BF1_DEV_CAPACITY : BF1_DEV_BAD_ROUTE);
@@ -846,7 +854,7 @@ __device__ __forceinline__ void inverse_route_in_cta(const BwdArgs& a, int32_t* 
         }
         return;
     }
-    const int readers_total = s_total, chunk = run_length(v, readers_total);
+    const int readers_total = s_total, chunk = run_length(a, readers_total);
     // prefix sums over the slots of the readers, the units, the partial-sum slots and the slots cut into runs, 16 bits each
     // (there are fewer entries than that); the number of units of every length is counted beside them
     auto bin_of = [](int len) { return 1023 - min(len, 1023); };
@@ -889,7 +897,7 @@ __device__ __forceinline__ void inverse_route_in_cta(const BwdArgs& a, int32_t* 
         __syncthreads();
     }
     const int units = (int)(carry >> 16 & 0xffff), parts = (int)(carry >> 32 & 0xffff);
-    const bool fits = units > 0 && units <= v.max_units && parts <= v.cap;
+    const bool fits = units > 0 && units <= v.max_units && parts <= v.max_parts;
     if (tid == 0) {
         start[nqb] = readers_total;
         if (units > 0 && !fits && a.status) atomicOr(a.status, BF1_DEV_CAPACITY);
@@ -1446,33 +1454,43 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
     if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-// KV blocks whose readers were cut into several runs: add the runs' partial sums in run order.  Few blocks need it
-// (block 0 of a sequence, with the paper's route); a work item is (such a block, KV head, one of its key rows, dK or dV),
-// one warp each.
+// KV blocks whose readers were cut into several runs: add the runs' partial sums in run order.  A work item is (such a block,
+// KV head, kCombineRows of its key rows, dK or dV), one warp each: what is looked up for it is a chain of four loads, so
+// several rows share it and are read together.  (A row to an item, and only in the CTAs that had dQ units: 47 us for the 2048
+// rows of 1000 tokens cut into runs of 2, under 4 as it is.)
+constexpr int kCombineRows = 4;
 template <int D>
 __device__ __forceinline__ void combine_runs(const BwdArgs& a, int worker, int workers) {
-    constexpr int kVec = D / 32;
+    constexpr int kVec = D / 32, kGroups = kBlock64 / kCombineRows;
     const int lane = threadIdx.x & 31;
-    const int items = a.inv.scalars[4] * a.nheads * kBlock64 * 2;
+    const int items = a.inv.scalars[4] * a.nheads * kGroups * 2;
     for (int item = worker; item < items; item += workers) {
-        const int which = item & 1, row = (item >> 1) % kBlock64;   // which = 0: dK, 1: dV
-        const int hm = item / (2 * kBlock64), kvh = a.head0 + hm % a.nheads;
+        const int which = item & 1, row0 = (item >> 1) % kGroups * kCombineRows;   // which = 0: dK, 1: dV
+        const int hm = item / (2 * kGroups), kvh = a.head0 + hm % a.nheads;
         const int gp = a.inv.multi[hm / a.nheads];
         const int runs = a.inv.chunks[gp], q0 = a.inv.part0[gp];
         const int seq = slot_seq(a, gp), p = a.qb_block[gp];
         const int seq0 = a.cu_seqlens[seq];
-        if (row >= a.cu_seqlens[seq + 1] - seq0 - p * kBlock64) continue;   // key row outside the sequence
-        const float* pk = a.partial + (((size_t)q0 * a.hkv + kvh) * 2 + which) * (kBlock64 * D) + row * D + lane * kVec;
+        const int rows = a.cu_seqlens[seq + 1] - seq0 - p * kBlock64 - row0;       // rows behind these lie outside the sequence
+        const float* pk = a.partial + (((size_t)q0 * a.hkv + kvh) * 2 + which) * (kBlock64 * D) + row0 * D + lane * kVec;
         const size_t run_stride = (size_t)a.hkv * 2 * kBlock64 * D;
-        float sum[kVec] = {};
-#pragma unroll 8
+        if (rows <= 0) continue;
+        float sum[kCombineRows][kVec] = {};
+#pragma unroll 4
         for (int r = 0; r < runs; ++r) {
 #pragma unroll
-            for (int e = 0; e < kVec; ++e) sum[e] += pk[r * run_stride + e];
-        }
-        uint32_t* out = reinterpret_cast<uint32_t*>((which ? a.dv : a.dk) + ((size_t)(seq0 + p * kBlock64 + row) * a.hkv + kvh) * D + lane * kVec);
+            for (int i = 0; i < kCombineRows; ++i) {
 #pragma unroll
-        for (int e = 0; e < kVec; e += 2) out[e / 2] = pack_bf16x2(sum[e], sum[e + 1]);
+                for (int e = 0; e < kVec; ++e) sum[i][e] += pk[r * run_stride + min(i, rows - 1) * D + e];
+            }
+        }
+        uint32_t* out = reinterpret_cast<uint32_t*>((which ? a.dv : a.dk) + ((size_t)(seq0 + p * kBlock64 + row0) * a.hkv + kvh) * D + lane * kVec);
+#pragma unroll
+        for (int i = 0; i < kCombineRows; ++i) {
+            if (i >= rows) break;
+#pragma unroll
+            for (int e = 0; e < kVec; e += 2) out[i * (a.hkv * D / 2) + e / 2] = pack_bf16x2(sum[i][e], sum[i][e + 1]);
+        }
     }
 }
 template <int D>
@@ -1746,7 +1764,7 @@ int make_store_map(CUtensorMap* m, void* ptr, int64_t T, int H, int d);         
 struct BwdLayout {
     size_t delta, ints, partial, ds, total;
     int ds_heads;   // KV heads whose dS is kept at a time; 0: dS is computed again
-    size_t n_count, n_start, n_chunks, n_part0, n_readers, n_units, n_multi;
+    size_t n_count, n_start, n_chunks, n_part0, n_readers, n_units, n_parts, n_multi;
     BwdLayout(int64_t T, int hq, int hkv, int d, int cap, int max_degree) {
         auto up = [](size_t x) { return (x + 255) / 256 * 256; };
         n_count = (size_t)cap + 1;
@@ -1754,13 +1772,15 @@ struct BwdLayout {
         n_chunks = (size_t)cap;
         n_part0 = (size_t)cap;
         n_readers = (size_t)cap * max_degree;
-        n_units = 2 * (size_t)cap;
+        // (what run_length() can make of as many readers; a slot whose readers are not cut has one unit)
+        n_parts = std::max<size_t>(cap, std::min<size_t>(2 * (size_t)cap * max_degree / kLeastChunk, 2 * kSms / hkv + 1));
+        n_units = cap + n_parts;
         n_multi = (size_t)cap;
         delta = 0;
         ints = up((size_t)T * hq * sizeof(float));
         const size_t n_ints = n_count + 2 * n_start + n_chunks + n_part0 + n_readers + 8 * n_units + (size_t)hkv + n_multi + 8;
         partial = ints + up(n_ints * sizeof(int32_t));
-        ds = partial + up((size_t)cap * hkv * 2 * kBlock64 * d * sizeof(float));
+        ds = partial + up(n_parts * hkv * 2 * kBlock64 * d * sizeof(float));
         const int64_t per_head = (int64_t)cap * max_degree * (hq / hkv == 4 ? 2 : 1) * kDsTile;
         ds_heads = per_head > kDsMost ? 0 : (int)std::max<int64_t>(1, std::min<int64_t>(hkv, kDsGroup / per_head));
         total = ds + up((size_t)ds_heads * per_head);
@@ -1872,9 +1892,11 @@ extern "C" int bf1_attn_bwd(const void* q, const void* k, const void* v, const v
     a.inv.scalars = ip;
     a.inv.cap = cap;
     a.inv.max_units = (int32_t)lay.n_units;
+    a.inv.max_parts = (int32_t)lay.n_parts;
     cudaStream_t st = (cudaStream_t)stream;
     int sms = 0;
     BF1_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    a.sms = sms;
     // D_i of every row, and the inverse route (readers of every KV block, cut into units)
     const bool one_cta = inverse_words(cap, route->max_degree) <= kInvInts;
     // (one CTA fits an SM: with the inverse route's there must not be more than SMs, or the last one runs all by itself)
@@ -1899,7 +1921,8 @@ extern "C" int bf1_attn_bwd(const void* q, const void* k, const void* v, const v
     for (int h0 = 0; h0 < hkv; h0 += step) {
         a.head0 = h0;
         a.nheads = std::min(step, hkv - h0);
-        const int grid_q = (int)std::min<int64_t>(sms, (int64_t)cap * a.nheads * (group == 4 ? 2 : 1));   // persistent: one CTA per SM
+        const int busy_q = (int)std::min<int64_t>(sms, (int64_t)cap * a.nheads * (group == 4 ? 2 : 1));   // persistent: one CTA per SM
+        const int grid_q = a.ds ? sms : busy_q;          // (CTAs without a unit add up partial sums all the same)
         const int grid_kv = (int)std::min<int64_t>(sms, (int64_t)lay.n_units * a.nheads);
         if (d == 128) {
             BF1_CUDA_CHECK(launch_pdl(bwd_dkv_kernel<128>, grid_kv, kDkvThreads, DkvSmem<128>::kTotal, st, tq, tk, tv, tg, a));

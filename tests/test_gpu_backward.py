@@ -381,3 +381,16 @@ def test_blocks_with_many_readers_are_the_same_however_the_inverse_route_is_made
         route.check_status()
     assert all(torch.equal(x, y) for x, y in zip(*grads))
     assert all(bool(x.isfinite().all()) for x in grads[0])
+
+
+@pytest.mark.parametrize("lens,hq,hkv,d,kw", [
+    ([64 * 2 + 1], 1, 1, 64, dict()),                                     # runs of 2, none of them cut further
+    ([64 * 31 + 7], 2, 1, 128, dict(local_blocks=0, dyadic=0)),           # 16 runs of block 0, the last block short
+    ([1000], 8, 4, 128, dict()),                                          # runs of 4
+    ([700, 33, 64 * 9], 16, 4, 64, dict()),                               # two pairs of heads, short and empty tails
+    ([64 * 33], 16, 8, 64, dict())],                                      # runs of 16, and block 0 in three
+    ids=["2", "2-window", "4", "G4", "16"])
+def test_few_units_are_cut_into_short_runs(lens, hq, hkv, d, kw):
+    w = I.custom(lens, hq=hq, hkv=hkv, d=d, seed=7700 + sum(lens), **kw)
+    for name, (rms, mx) in run_case(w, seed=15).items():
+        assert rms <= REL_RMS and mx <= REL_MAX, (name, rms, mx)
