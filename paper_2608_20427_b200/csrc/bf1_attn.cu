@@ -41,10 +41,9 @@ namespace bf1 {
 constexpr int kBlock = 64;            // b: tokens per block
 constexpr int kRows = 128;            // MMA M: 2 query heads x 64 tokens
 constexpr int kThreads = 384;         // 12 warps
-// Decoded units queued between scheduler and producer.  One is enough to hide the decode, and every
+// One decoded unit is queued between scheduler and producer.  That is enough to hide the decode, and every
 // unit a CTA holds in advance is a unit another CTA cannot take at the end of the launch: with three
 // the last CTAs finished 20 us after the first at 32K, and 8K was 7 % slower.
-constexpr int kQueue = 1;
 // The next unit is taken when the producer has this many list entries of the unit at hand left to copy: late enough that
 // the CTAs that finish first get the units that are left, early enough to hide the look-ups (a tile takes about 1 us with two
 // CTAs on the SM, the look-ups 2 to 3).  Taken when the unit at hand begins: dense 8K tokens 256.3 us, 253.9 as it is (the last CTA
@@ -110,10 +109,10 @@ struct Cfg {
     static constexpr int kStageOff = kRingOff + kRing * kTileBytes;         // O staging: 4 warps x 32 rows x 64 B
     static constexpr int kStageBytes = 4 * 32 * 64;
     static constexpr int kHandOff = kStageOff + kStageBytes;                // Handoff[2]
-    static constexpr int kQueueOff = kHandOff + 2 * (int)sizeof(Handoff);   // QueueEntry[kQueue]
-    static constexpr int kInfoOff = kQueueOff + kQueue * (int)sizeof(QueueEntry);   // int4[2]
+    static constexpr int kQueueOff = kHandOff + 2 * (int)sizeof(Handoff);   // QueueEntry
+    static constexpr int kInfoOff = kQueueOff + (int)sizeof(QueueEntry);   // int4[2]
     static constexpr int kBarOff = kInfoOff + 32;
-    static constexpr int kNumBars = 2 + 2 * kRing + 2 + 2 + 2 + 1 + 2 + 2 * kQueue + 2 + 2 + 2 + 1;
+    static constexpr int kNumBars = 2 + 2 * kRing + 2 + 2 + 2 + 1 + 2 + 2 + 2 + 2 + 2 + 1;
     static constexpr int kMiscOff = kBarOff + 8 * kNumBars;
     static constexpr int kTotal = kMiscOff + 16;
     static constexpr int kTmemCols = 256;
@@ -151,9 +150,22 @@ __device__ __forceinline__ Place unit_place(const AttnArgs& a, int nqb, int u) {
     }
     return p;
 }
+// cu_seqlens of a batch of up to 31 sequences stands in the lanes of the warp (read once, beside the first look-ups; 0.4 us of
+// every launch's start when it was read for each unit behind its sequence).
+constexpr int kLaneBatch = 31;
+// Query blocks of the whole batch.
+__device__ __forceinline__ int batch_blocks(const AttnArgs& a, int cu, int lane) {
+    if (a.batch <= kLaneBatch) {
+        const int next = __shfl_down_sync(0xffffffffu, cu, 1);
+        return __reduce_add_sync(0xffffffffu, lane < a.batch ? (next - cu + kBlock - 1) / kBlock : 0);
+    }
+    int n = 0;
+    for (int s = 0; s < a.batch; ++s) n += (a.cu_seqlens[s + 1] - a.cu_seqlens[s] + kBlock - 1) / kBlock;
+    return n;
+}
 // A slot of the route (dense: a query block of the batch) -> the unit.  `kvh` carries the unit's token offset inside its
 // query block in its upper half; p: the first 32 list entries, one per lane, as the route holds them.
-__device__ __forceinline__ void decode_slot(const AttnArgs& a, const Place& pl, int slot, int lane, Unit& un, int& p) {
+__device__ __forceinline__ void decode_slot(const AttnArgs& a, const Place& pl, int slot, int cu, int lane, Unit& un, int& p) {
     un.kvh = pl.head | (pl.tok_off << 16);
     un.slot = slot;
     int seq = 0;
@@ -165,18 +177,37 @@ __device__ __forceinline__ void decode_slot(const AttnArgs& a, const Place& pl, 
         un.cnt = min(max(a.kv_count[slot], 1), a.max_degree);
         if (a.batch > 1) seq = a.qb_seq[slot];
     } else {
-        int acc = 0;
         un.j = 0;
-        for (int s = 0; s < a.batch; ++s) {
-            const int nb = (a.cu_seqlens[s + 1] - a.cu_seqlens[s] + kBlock - 1) / kBlock;
-            if (slot < acc + nb) { seq = s; un.j = slot - acc; break; }
-            acc += nb;
+        if (a.batch <= kLaneBatch) {
+            const int next = __shfl_down_sync(0xffffffffu, cu, 1), nb = lane < a.batch ? (next - cu + kBlock - 1) / kBlock : 0;
+            int incl = nb;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int up = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += up;
+            }
+            seq = __ffs(__ballot_sync(0xffffffffu, lane < a.batch && slot < incl)) - 1;      // (slot < number of blocks)
+            un.j = slot - __shfl_sync(0xffffffffu, incl - nb, seq);
+        } else {
+            int acc = 0;
+            for (int s = 0; s < a.batch; ++s) {
+                const int nb = (a.cu_seqlens[s + 1] - a.cu_seqlens[s] + kBlock - 1) / kBlock;
+                if (slot < acc + nb) { seq = s; un.j = slot - acc; break; }
+                acc += nb;
+            }
         }
         un.cnt = un.j + 1;
         p = lane;
     }
-    un.seq0 = a.cu_seqlens[seq];
-    const int seqlen = a.cu_seqlens[seq + 1] - un.seq0;
+    int end;
+    if (a.batch <= kLaneBatch) {
+        un.seq0 = __shfl_sync(0xffffffffu, cu, seq);
+        end = __shfl_sync(0xffffffffu, cu, seq + 1);
+    } else {
+        un.seq0 = a.cu_seqlens[seq];
+        end = a.cu_seqlens[seq + 1];
+    }
+    const int seqlen = end - un.seq0;
     un.rows_valid = max(0, min(1 << a.r_shift, seqlen - un.j * kBlock - pl.tok_off));   // of this unit's R tokens
     un.tok0 = un.seq0 + un.j * kBlock + pl.tok_off;
 }
@@ -246,18 +277,6 @@ __global__ void __launch_bounds__(kThreads, 2) attn_fwd_kernel(const __grid_cons
     const int warp = tid >> 5;
     const int lane = tid & 31;
 
-    // Dynamic hand-out: sched[0] is the next unit, sched[1] counts CTAs that are done; the last
-    // one to finish puts both back to zero, so the words are ready for the next launch.
-    auto retire = [&]() {
-        if (args.sched && threadIdx.x == 0) {
-            __threadfence();
-            if (atomicAdd(args.sched + 1, 1) == (int)gridDim.x - 1) {
-                args.sched[0] = 0;
-                args.sched[1] = 0;
-                __threadfence();
-            }
-        }
-    };
     const uint32_t base = smem_u32(smem);
     const uint32_t sQ = base + C::kQOff;
     const uint32_t sRing = base + C::kRingOff;
@@ -270,9 +289,9 @@ __global__ void __launch_bounds__(kThreads, 2) attn_fwd_kernel(const __grid_cons
     const uint32_t bar_pv_done = bar_p_full + 16;             // [2]
     const uint32_t bar_o_free = bar_pv_done + 16;
     const uint32_t bar_info = bar_o_free + 8;                 // [2]
-    const uint32_t bar_sq_full = bar_info + 16;               // [kQueue]
-    const uint32_t bar_sq_free = bar_sq_full + 8 * kQueue;    // [kQueue]
-    const uint32_t bar_ho_full = bar_sq_free + 8 * kQueue;    // [2]
+    const uint32_t bar_sq_full = bar_info + 16;
+    const uint32_t bar_sq_free = bar_sq_full + 8;
+    const uint32_t bar_ho_full = bar_sq_free + 8;             // [2]
     const uint32_t bar_ho_free = bar_ho_full + 16;            // [2]
     const uint32_t bar_info_free = bar_ho_free + 16;          // [2]
     const uint32_t bar_ask = bar_info_free + 16;              // the producer nears the end of a unit
@@ -289,25 +308,14 @@ __global__ void __launch_bounds__(kThreads, 2) attn_fwd_kernel(const __grid_cons
     // 24.7, 24.3; 1K 13.6, 13.5.
     pdl_wait();
     if (tid == 0) {
-        // The status word and the block count are read together (two independent loads in flight), and no other
-        // warp waits for them before its own set-up.  If an earlier launch on this status word gave up, this one
-        // raises its abort flag: every role then sees an empty queue and the CTA leaves through the normal exit.
+        // If an earlier launch on this status word gave up, this one raises its abort flag: every role then sees an empty queue and
+        // the CTA leaves through the normal exit.
         const int earlier = args.status ? *args.status : 0;
-        int nqb = 0;
-        if (!args.dense) {
-            nqb = min(*args.num_qblocks, args.capacity);
-        }
         *s_abort = (earlier & BF1_DEV_WAIT_TIMEOUT) ? 1 : 0;
         if (base & 1023u) {   // the swizzled tiles need a 1024-byte aligned window
             *s_abort = 1;
             if (args.status) atomicOr(args.status, BF1_DEV_WAIT_TIMEOUT);
         }
-        if (args.dense) {
-            for (int s = 0; s < args.batch; ++s)
-                nqb += (args.cu_seqlens[s + 1] - args.cu_seqlens[s] + kBlock - 1) / kBlock;
-        }
-        *s_nqb = nqb;
-        s_nqb[1] = 0;
         mbar_init(bar_q_full, 1);
         mbar_init(bar_q_free, 1);
         for (int s = 0; s < C::kRing; ++s) {
@@ -323,10 +331,8 @@ __global__ void __launch_bounds__(kThreads, 2) attn_fwd_kernel(const __grid_cons
             mbar_init(bar_ho_free + 8 * s, 4);   // epilogue warps
             mbar_init(bar_info_free + 8 * s, 5); // softmax warps + PV issuer have read the unit descriptor
         }
-        for (int s = 0; s < kQueue; ++s) {
-            mbar_init(bar_sq_full + 8 * s, 1);
-            mbar_init(bar_sq_free + 8 * s, 1);
-        }
+        mbar_init(bar_sq_full, 1);
+        mbar_init(bar_sq_free, 1);
         mbar_init(bar_o_free, 4);                // epilogue warps
         mbar_init(bar_ask, 1);
         fence_mbar_init();
@@ -342,9 +348,10 @@ __global__ void __launch_bounds__(kThreads, 2) attn_fwd_kernel(const __grid_cons
     auto slot_at = [&](const Place& pl, int nqb_) {
         return args.dense ? nqb_ - 1 - pl.idx : args.order ? args.order[min(pl.idx, args.capacity - 1)] : pl.idx;
     };
+    int cu = 0;                   // (see kLaneBatch)
     auto fetch_unit = [&](const Place& pl, int slot, Unit& un, int& my_p) {
         int p;
-        decode_slot(args, pl, slot, lane, un, p);
+        decode_slot(args, pl, slot, cu, lane, un, p);
         my_p = 0;
         if (lane < un.cnt) {   // entries 0..31, one per lane, made safe to use
             if (p < 0 || p > un.j || (lane == un.cnt - 1) != (p == un.j)) {
@@ -354,11 +361,24 @@ __global__ void __launch_bounds__(kThreads, 2) attn_fwd_kernel(const __grid_cons
             my_p = p;
         }
     };
-    Unit un0 = {};
-    int my_p0 = 0;
+    volatile QueueEntry* e = s_queue;
+    auto queue_unit = [&](bool have, const Unit& un, int my_p) {
+        e->p[lane] = my_p;
+        if (lane == 0) {
+            e->cnt = have ? un.cnt : 0;
+            e->rows_valid = un.rows_valid;
+            e->tok0 = un.tok0;
+            e->kvh = un.kvh;
+            e->seq0 = un.seq0;
+            e->j = un.j;
+            e->slot = un.slot;
+        }
+    };
     bool have0 = false;
     if (warp == 2) {
-        int nqb0 = 0, slot = 0;
+        if (args.batch <= kLaneBatch) cu = args.cu_seqlens[min(lane, args.batch)];
+        Unit un0 = {};
+        int nqb0 = 0, slot = 0, my_p0 = 0;
         Place pl = {};
         const bool early = !args.dense && args.tail_div == 1;   // the place does not depend on the block count
         if (early) {
@@ -368,9 +388,9 @@ __global__ void __launch_bounds__(kThreads, 2) attn_fwd_kernel(const __grid_cons
         if (!args.dense) {
             nqb0 = min(*args.num_qblocks, args.capacity);
         } else {
-            for (int s = 0; s < args.batch; ++s)
-                nqb0 += (args.cu_seqlens[s + 1] - args.cu_seqlens[s] + kBlock - 1) / kBlock;
+            nqb0 = batch_blocks(args, cu, lane);
         }
+        if (lane == 0) *s_nqb = nqb0;
         have0 = (int)blockIdx.x < nqb0 * args.hkv * (kBlock >> args.r_shift);
         if (have0) {
             if (!early) {
@@ -379,6 +399,7 @@ __global__ void __launch_bounds__(kThreads, 2) attn_fwd_kernel(const __grid_cons
             }
             fetch_unit(pl, slot, un0, my_p0);
         }
+        queue_unit(have0, un0, my_p0);      // (the producer finds the first unit there behind the CTA's barrier)
     }
     if (warp == 1) {
         tmem_alloc(smem_u32(s_tmem_base), C::kTmemCols);
@@ -405,47 +426,44 @@ __global__ void __launch_bounds__(kThreads, 2) attn_fwd_kernel(const __grid_cons
         setmaxnreg_dec<kRegsCtl>();
         if (warp == 2) {
             // ================================ scheduler =======================================
-            for (int n = 0;; ++n) {
-                Unit un = un0;
-                int my_p = my_p0;
-                bool have = have0 && !*abort_flag;
-                if (n > 0) {
-                    mbar_wait(bar_ask, (n - 1) & 1, abort_flag, args.status);
-                    int u = 0;
-                    if (lane == 0)
-                        u = (args.sched ? atomicAdd(args.sched, 1) + (int)gridDim.x : (int)(blockIdx.x + n * gridDim.x));
-                    u = __shfl_sync(0xffffffffu, u, 0);
-                    have = u < total_units && !*abort_flag;
-                    if (have) {
-                        const Place pl = unit_place(args, nqb, u);
-                        fetch_unit(pl, slot_at(pl, nqb), un, my_p);
-                    }
+            for (int n = 1; have0 && !*abort_flag; ++n) {
+                mbar_wait(bar_ask, (n - 1) & 1, abort_flag, args.status);
+                int u = 0;
+                if (lane == 0)
+                    u = (args.sched ? atomicAdd(args.sched, 1) + (int)gridDim.x : (int)(blockIdx.x + n * gridDim.x));
+                u = __shfl_sync(0xffffffffu, u, 0);
+                const bool have = u < total_units && !*abort_flag;
+                Unit un = {};
+                int my_p = 0;
+                if (have) {
+                    const Place pl = unit_place(args, nqb, u);
+                    fetch_unit(pl, slot_at(pl, nqb), un, my_p);
                 }
-                const int qs = n % kQueue;
-                if (n >= kQueue) mbar_wait(bar_sq_free + 8 * qs, ((n / kQueue) - 1) & 1, abort_flag, args.status);
-                volatile QueueEntry* e = s_queue + qs;
-                e->p[lane] = my_p;
-                if (lane == 0) {
-                    e->cnt = have ? un.cnt : 0;
-                    e->rows_valid = un.rows_valid;
-                    e->tok0 = un.tok0;
-                    e->kvh = un.kvh;
-                    e->seq0 = un.seq0;
-                    e->j = un.j;
-                    e->slot = un.slot;
-                }
+                mbar_wait(bar_sq_free, (n - 1) & 1, abort_flag, args.status);
+                queue_unit(have, un, my_p);
                 __syncwarp();
-                if (lane == 0) mbar_arrive(bar_sq_full + 8 * qs);
+                if (lane == 0) mbar_arrive(bar_sq_full);
                 if (!have) break;
+            }
+            // Dynamic hand-out: sched[0] is the next unit, sched[1] counts the CTAs that will take no more; the last one puts
+            // both back to zero, so the words are ready for the next launch.  Here and not at the CTA's end, where the fence and the
+            // atomic's round trip were the last microsecond of every launch (with cu_seqlens in the lanes, the first unit queued in
+            // front of the set-up barrier and the stores not waited for: forward of 137 / 1000 / 4096 tokens in 1, 2 and 16
+            // heads 8.2 / 9.9 / 22.3 -> 6.9 / 8.4 / 20.2 us).
+            if (args.sched && lane == 0) {
+                __threadfence();
+                if (atomicAdd(args.sched + 1, 1) == (int)gridDim.x - 1) {
+                    args.sched[0] = 0;
+                    args.sched[1] = 0;
+                    __threadfence();
+                }
             }
         } else if (warp == 0) {
             // ================================ TMA producer ====================================
             // The whole warp walks the loop; one elected lane issues the copies.
             int slot = 0, pass = 0;
             for (int n = 0;; ++n) {
-                const int qs = n % kQueue;
-                mbar_wait(bar_sq_full + 8 * qs, (n / kQueue) & 1, abort_flag, args.status);
-                volatile QueueEntry* e = s_queue + qs;
+                if (n > 0) mbar_wait(bar_sq_full, (n - 1) & 1, abort_flag, args.status);
                 int cnt = e->cnt;
                 const int rows_valid = e->rows_valid, tok0 = e->tok0, kvh_packed = e->kvh, seq0 = e->seq0, j = e->j;
                 const int kvh = kvh_packed & 0xffff;
@@ -526,7 +544,7 @@ __global__ void __launch_bounds__(kThreads, 2) attn_fwd_kernel(const __grid_cons
                     p_prev = p_cur;
                 }
                 if (cnt == 0) break;
-                if (elect_one()) mbar_arrive(bar_sq_free + 8 * qs);
+                if (elect_one()) mbar_arrive(bar_sq_free);
                 __syncwarp();
             }
         } else if (warp == 1) {
@@ -784,11 +802,12 @@ __global__ void __launch_bounds__(kThreads, 2) attn_fwd_kernel(const __grid_cons
         }
     }
 
-    if (warp >= 8 && lane == 0) bulk_wait0();   // this thread's output stores have landed
+    // This thread's output stores have read the staging tiles.  That they land is waited for by the end of the grid, as for any
+    // other store.
+    if (warp >= 8 && lane == 0) bulk_wait_read0();
     tc_fence_before();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem, C::kTmemCols);
-    retire();
 }
 
 // ---- host side ---------------------------------------------------------------------------
