@@ -66,6 +66,8 @@ struct InvPlan {
     int32_t* readers;     // [cap * max_degree] list entries (query slot * max_degree + place), ascending per KV slot
     int4* units;          // [max_units][2] longest first: {KV slot, first reader, readers, partial-sum slot or -1 (it
                           // writes the final bf16 rows)}, {first token of the sequence, block, tokens of the sequence, -}
+    int4* ranked;         // [cap][2] the query blocks in the order of the dQ units: {slot, list entries, block, first token of the
+                          // sequence}, {tokens of the sequence, -, -, -}
     int32_t* tickets;     // [hkv] hand-out counters of the dK/dV launches, by first KV head
     int32_t* multi;       // [cap] the KV slots whose readers were cut into more than one run
     int32_t* scalars;     // [8] number of units, total readers, chunk, partial slots, slots in `multi`
@@ -236,6 +238,14 @@ struct DqUnit {
     int ok, slot, kvh, pair, cnt, seq0, seqlen, j, tok0, rows_valid;
 };
 
+// The query block of rank r in the hand-out order, looked up for the dQ kernel (by the preparation, beside the pass over dO and O): a
+// chain of three loads that would stand in front of its first copy (backward of 1000 and 4096 tokens 0.4 and 1 us shorter for it).
+__device__ __forceinline__ void rank_query_block(const BwdArgs& a, int r, int nqb) {
+    const int slot = min(max(a.order ? a.order[r] : r, 0), nqb - 1), seq = min(max(slot_seq(a, slot), 0), a.batch - 1);
+    const int seq0 = a.cu_seqlens[seq];
+    a.inv.ranked[2 * r] = make_int4(slot, min(max(a.kv_count[slot], 1), a.max_degree), a.qb_block[slot], seq0);
+    a.inv.ranked[2 * r + 1] = make_int4(a.cu_seqlens[seq + 1] - seq0, 0, 0, 0);
+}
 // Unit n of this CTA (see above for the order).
 __device__ __forceinline__ DqUnit dq_unit(const BwdArgs& a, int n, int nqb, int pairs) {
     DqUnit u;
@@ -261,14 +271,12 @@ __device__ __forceinline__ DqUnit dq_unit(const BwdArgs& a, int n, int nqb, int 
             u.pair = rem - rank * pairs;
         }
         u.kvh += a.head0;
-        int slot = a.order ? a.order[rank] : rank;
-        slot = min(max(slot, 0), nqb - 1);
-        u.slot = slot;
-        const int seq = slot_seq(a, slot);
-        u.j = a.qb_block[slot];
-        u.cnt = min(max(a.kv_count[slot], 1), a.max_degree);
-        u.seq0 = a.cu_seqlens[seq];
-        u.seqlen = a.cu_seqlens[seq + 1] - u.seq0;
+        const int4 x = a.inv.ranked[2 * rank];
+        u.slot = x.x;
+        u.cnt = x.y;
+        u.j = x.z;
+        u.seq0 = x.w;
+        u.seqlen = a.inv.ranked[2 * rank + 1].x;
         u.rows_valid = min(kBlock64, u.seqlen - u.j * kBlock64);
         u.tok0 = u.seq0 + u.j * kBlock64;
     }
@@ -1032,6 +1040,8 @@ __global__ void __launch_bounds__(1024, 1) bwd_prep_kernel(const BwdArgs a) {
         const int tok = t0 + sub * kRowsAtOnce + r0;
         if (sub < kTokens / kRowsAtOnce && tok < a.total_tokens) a.delta[(size_t)h * a.total_tokens + tok] = mine;
     }
+    const int nqb = min(*a.num_qblocks, a.capacity);
+    for (int r = (ctas - 1 - cta) * 1024 + threadIdx.x; r < nqb; r += ctas * 1024) rank_query_block(a, r, nqb);
 }
 
 // ---- dK, dV ----------------------------------------------------------------------------------------------------
@@ -1367,7 +1377,6 @@ __global__ void __launch_bounds__(kDkvThreads, 1) bwd_dkv_kernel(const __grid_co
                 }
             }
         }
-        bulk_wait0();   // (this thread's copies of dS have landed; nothing to wait for in the other lanes and warp 2)
     } else if (warp < 12) {
         // ---- arithmetic on S and dP: two threads per tile row (head hl, token tl of the reader), warps 4-7 on key
         // columns 0..31 and warps 8-11 on columns 32..63 ----
@@ -1747,7 +1756,7 @@ __global__ void __launch_bounds__(kDqThreads, 1) bwd_dq_kernel(const __grid_cons
                     *reinterpret_cast<uint4*>(dqrow + c * 8) = make_uint4(pk[c * 4], pk[c * 4 + 1], pk[c * 4 + 2], pk[c * 4 + 3]);
             }
         }
-        if (lane == 0) bulk_wait0();
+        if (lane == 0) bulk_wait_read0();     // (that the stores land is waited for by the end of the grid)
         __syncwarp();
     } else {
         combine_runs<D>(a, blockIdx.x * 4 + (warp - 6), gridDim.x * 4);
@@ -1764,7 +1773,7 @@ int make_store_map(CUtensorMap* m, void* ptr, int64_t T, int H, int d);         
 struct BwdLayout {
     size_t delta, ints, partial, ds, total;
     int ds_heads;   // KV heads whose dS is kept at a time; 0: dS is computed again
-    size_t n_count, n_start, n_chunks, n_part0, n_readers, n_units, n_parts, n_multi;
+    size_t n_count, n_start, n_chunks, n_part0, n_readers, n_units, n_parts, n_multi, n_ranked;
     BwdLayout(int64_t T, int hq, int hkv, int d, int cap, int max_degree) {
         auto up = [](size_t x) { return (x + 255) / 256 * 256; };
         n_count = (size_t)cap + 1;
@@ -1776,9 +1785,10 @@ struct BwdLayout {
         n_parts = std::max<size_t>(cap, std::min<size_t>(2 * (size_t)cap * max_degree / kLeastChunk, 2 * kSms / hkv + 1));
         n_units = cap + n_parts;
         n_multi = (size_t)cap;
+        n_ranked = 2 * (size_t)cap;
         delta = 0;
         ints = up((size_t)T * hq * sizeof(float));
-        const size_t n_ints = n_count + 2 * n_start + n_chunks + n_part0 + n_readers + 8 * n_units + (size_t)hkv + n_multi + 8;
+        const size_t n_ints = n_count + 2 * n_start + n_chunks + n_part0 + n_readers + 8 * n_units + 4 * n_ranked + (size_t)hkv + n_multi + 8;
         partial = ints + up(n_ints * sizeof(int32_t));
         ds = partial + up(n_parts * hkv * 2 * kBlock64 * d * sizeof(float));
         const int64_t per_head = (int64_t)cap * max_degree * (hq / hkv == 4 ? 2 : 1) * kDsTile;
@@ -1880,7 +1890,8 @@ extern "C" int bf1_attn_bwd(const void* q, const void* k, const void* v, const v
     a.dv = (__nv_bfloat16*)dv;
     a.partial = (float*)(ws + lay.partial);
     a.inv.units = (int4*)(ws + lay.ints);   // (16-byte entries first)
-    int32_t* ip = (int32_t*)(ws + lay.ints) + 8 * lay.n_units;
+    a.inv.ranked = a.inv.units + 2 * lay.n_units;
+    int32_t* ip = (int32_t*)(a.inv.ranked + lay.n_ranked);
     a.inv.count = ip;            ip += lay.n_count;
     a.inv.start = ip;            ip += lay.n_start;
     a.inv.unit0 = ip;            ip += lay.n_start;
