@@ -28,6 +28,7 @@
 // pages 23.6 -> 13.9 us, 40 lists 9.5 -> 6.0.
 #include <algorithm>
 #include <atomic>
+#include <cfloat>
 
 #include "bf1_common.cuh"
 
@@ -103,6 +104,10 @@ __device__ __forceinline__ void st_cluster(uint32_t addr, const float (&v)[N]) {
 }
 // x / y for small whole numbers (below 2^20: half a step from a whole quotient is more than the division's error)
 __device__ __forceinline__ int small_div(int x, int y) { return (int)__fdividef((float)x + 0.5f, (float)y); }
+
+// A sum over the rounded weights and the one over what rounding left of them.  Where V is not finite the first says it all, as in a
+// whole list: the rest of a weight is zero or has the other sign half of the time, and would make NaN of an infinity.
+__device__ __forceinline__ float with_rest(float sum, float rest) { return fabsf(sum) <= FLT_MAX ? sum + rest : sum; }
 
 // One CTA per (sequence, KV head[, part of the list]).  Pages stream in through a kDecStages-deep cp.async ring with ONE
 // block-wide synchronisation per page; inside a page each of the four warps owns 16 keys and keeps its own online-softmax
@@ -275,7 +280,7 @@ __global__ void __launch_bounds__(kDecThreads, D == 64 ? 4 : 2) decode_fused_ker
         if (tig == 0) { st.m[warp][gid] = m_run; st.l[warp][gid] = l_run; }
 #pragma unroll
         for (int dn = 0; dn < D / 8; ++dn)
-            *reinterpret_cast<float2*>(&st.o[warp][gid][dn * 8 + 2 * tig]) = kSplit ? make_float2(acc[dn][0] + acc[dn][2], acc[dn][1] + acc[dn][3]) : make_float2(acc[dn][0], acc[dn][1]);
+            *reinterpret_cast<float2*>(&st.o[warp][gid][dn * 8 + 2 * tig]) = kSplit ? make_float2(with_rest(acc[dn][0], acc[dn][2]), with_rest(acc[dn][1], acc[dn][3])) : make_float2(acc[dn][0], acc[dn][1]);
     }
     __syncthreads();
     // ---- merge the four warps' states -------------------------------------------------------------------

@@ -300,3 +300,38 @@ def test_parts_of_a_list_lose_nothing_but_the_rounding_of_the_result(hq, hkv, d,
     off = np.linalg.norm(out - o_ref) / np.linalg.norm(o_ref)
     if (hq, hkv, d, batch) != (16, 4, 128, 19):
         assert off <= 2.0 ** -9 + 1e-5, off
+
+
+@pytest.mark.parametrize("hq,hkv,d", [(1, 1, 128), (4, 2, 64), (4, 2, 128), (8, 2, 64), (8, 2, 128)], ids=["G1", "G2-d64", "G2", "G4-d64", "G4"])
+def test_what_is_not_finite_in_v_comes_out_the_same_however_the_lists_are_walked(hq, hkv, d):
+    """One sequence alone, whose list is cut (eleven parts of a page, and longer ones), and a batch of it that fills the GPU, whose
+    lists are walked whole.  Every column but the last 8 has an infinity at one selected key, with a weight that is not zero:
+    the result is that infinity.  Of the others some have both infinities or a NaN at a key: NaN."""
+    n = 64 * 520
+    w = I.custom([n], hq=hq, hkv=hkv, d=d, seed=4400 + d + hq)
+    q, k, v = I.draw_qkv(w)
+    idx, c, _, _ = O.route(O.cfg(), n, 16)
+    listed = [int(b) for b in idx[n // 64 - 1, :c[n // 64 - 1]]]
+    want = torch.zeros(d)
+    for col in range(d - 8):
+        key = 64 * listed[col % len(listed)] + (col * 29) % 64
+        want[col] = float("inf") if col % 2 else float("-inf")
+        v[key, :, col] = want[col]
+    for col in (d - 8, d - 7):
+        v[64 * listed[0] + col % 64, :, col] = float("inf")
+        v[64 * listed[-1], :, col] = float("-inf")
+        v[64 * listed[-1] + 1, :, col + 2] = float("nan")
+        want[col] = want[col + 2] = float("nan")
+    k_pages, v_pages, table = (t.to(DEV) for t in paged_cache(w, k, v, seed=15))
+    last = None
+    for batch in (1, 30 // hkv, 60 // hkv, 160 // hkv):
+        sl = torch.full((batch,), n, dtype=torch.int32, device=DEV)
+        plan = bf1.plan_decode(sl, table.repeat(batch, 1))
+        ws = bf1.decode_workspace(batch, hq, hkv, plan.max_degree, d, torch.device(DEV))
+        out, _ = bf1.decode_fwd(q[-1].to(DEV).repeat(batch, 1, 1), k_pages, v_pages, sl, plan, ws)
+        out = out.float().cpu()
+        assert torch.equal(out.isnan(), want.isnan().expand_as(out)), batch
+        assert torch.equal(torch.where(out.isinf(), out, 0.0), torch.where(want.isinf(), want, 0.0).expand_as(out)), batch
+        if last is not None:
+            assert (out - last)[..., d - 4:].abs().max() <= O_MAX_ABS
+        last = out[:1]
