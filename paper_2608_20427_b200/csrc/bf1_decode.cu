@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(kDecThreads, D == 64 ? 4 : 2) decode_fused_ker
     // ---- add the parts up in list order (fixed and data-independent): every CTA of the cluster its share of the columns, 32
     //      to a warp, and every warp the maxima and sums of its head, a part to a lane
     cluster_wait();                                      // the other CTAs of the cluster have started
-    if (e_lo < e_hi) {
+    {                                                    // (a part without entries: zeros, under a weight of zero)
         const int v = h * D + c0, rank = small_div(v, a.share);
         const uint32_t to = map_cluster(smem_u32(dsmem) + a.gather + (blockIdx.z * a.share + v - rank * a.share) * 4, rank);
         st_cluster(to, out);
@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(kDecThreads, D == 64 ? 4 : 2) decode_fused_ker
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i)
-                if (wi[i] > 0.f) o = fmaf(wi[i], p[i], o);       // (a part without entries left no columns)
+                if (i0 + i < a.nctas) o = fmaf(wi[i], p[i], o);  // (a weight of zero counts too: times an infinity it is NaN)
         }
         if (hv < a.group) {                              // (G = 1: the second head does not exist)
             a.o[((size_t)s * a.hq + hbase + hv) * D + col] = __float2bfloat16_rn(o * (1.f / l));

@@ -335,3 +335,25 @@ def test_what_is_not_finite_in_v_comes_out_the_same_however_the_lists_are_walked
         if last is not None:
             assert (out - last)[..., d - 4:].abs().max() <= O_MAX_ABS
         last = out[:1]
+
+
+@pytest.mark.parametrize("hq,hkv,d", [(4, 2, 64), (4, 2, 128), (8, 2, 128)], ids=["G2-d64", "G2", "G4"])
+def test_an_infinity_under_a_weight_of_zero_is_nan_however_the_lists_are_walked(hq, hkv, d):
+    """The keys of one listed page have scores some 300 below the others', a weight of 0 in fp32, and an infinity in the first
+    column: 0 times infinity.  Where the page is a part by itself the part is fine and its weight among the parts is 0."""
+    n = 64 * 520
+    w = I.custom([n], hq=hq, hkv=hkv, d=d, seed=4500 + d + hq)
+    q, k, v = I.draw_qkv(w)
+    idx, c, _, _ = O.route(O.cfg(), n, 16)
+    low = int(idx[n // 64 - 1, 4])
+    q[..., 0] = 8.0
+    k[..., 0] = 0.0
+    k[64 * low:64 * low + 64, :, 0] = -448.0
+    v[64 * low + 5, :, 0] = float("inf")
+    k_pages, v_pages, table = (t.to(DEV) for t in paged_cache(w, k, v, seed=16))
+    for batch in (1, 30 // hkv, 60 // hkv, 160 // hkv):
+        sl = torch.full((batch,), n, dtype=torch.int32, device=DEV)
+        plan = bf1.plan_decode(sl, table.repeat(batch, 1))
+        ws = bf1.decode_workspace(batch, hq, hkv, plan.max_degree, d, torch.device(DEV))
+        out, _ = bf1.decode_fwd(q[-1].to(DEV).repeat(batch, 1, 1), k_pages, v_pages, sl, plan, ws)
+        assert bool(out[..., 0].isnan().all()) and bool(out[..., 1:].isfinite().all()), batch
