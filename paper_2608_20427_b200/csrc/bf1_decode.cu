@@ -474,8 +474,8 @@ extern "C" int bf1_decode_fwd(const void* q, const void* k_pages, const void* v_
     if (d != 64 && d != 128) return fail(BF1_ERR_UNSUPPORTED, "head dimension %d: only 64 and 128 are supported", d);
     if (((uintptr_t)q | (uintptr_t)k_pages | (uintptr_t)v_pages | (uintptr_t)o | (uintptr_t)workspace) & 15)
         return fail(BF1_ERR_INVALID_ARG, "q, k_pages, v_pages, o and workspace must be 16-byte aligned");
-    if (plan->max_degree < 1 || plan->max_degree > 64 || hkv > 65535 || batch > 65535)
-        return fail(BF1_ERR_UNSUPPORTED, "max_degree must be <= 64; hkv and batch must fit the grid (<= 65535)");
+    if (plan->max_degree < 1 || plan->max_degree > 64 || hkv * ((group + 1) / 2) > 65535 || batch > 65535)
+        return fail(BF1_ERR_UNSUPPORTED, "max_degree must be <= 64; pairs of query heads and batch <= 65535");
     if (batch == 0) return BF1_OK;
     DecodeArgs a;
     a.q = (const __nv_bfloat16*)q;

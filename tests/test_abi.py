@@ -118,3 +118,13 @@ def test_decode_scratch_is_no_larger_than_what_is_used():
         assert lib.bf1_decode_workspace_bytes(*args) == 16
     for args in ((-1, 16, 8, 11, 128), (1, 0, 8, 11, 128), (1, 16, 0, 11, 128), (1, 15, 8, 11, 128), (1, 16, 8, 0, 128), (1, 16, 8, 11, 0)):
         assert lib.bf1_decode_workspace_bytes(*args) == -1
+
+
+def test_decode_refuses_more_kv_heads_than_pairs_of_query_heads_fit_a_grid_dimension():
+    """65535 pairs of query heads: with four to a KV head half as many KV heads."""
+    lib = bf1.load()
+    fake = ctypes.c_void_p(0x1000)
+    plan = binding._DecodePlanC(11, 0x1000, 0x1000, 0x1000, 0x1000)
+    for group, hkv, code in ((1, 65535, 0), (1, 65536, -2), (2, 65535, 0), (2, 65536, -2), (4, 32767, 0), (4, 32768, -2), (4, 65535, -2)):
+        rc = lib.bf1_decode_fwd(fake, fake, fake, 1, fake, 0, group * hkv, hkv, 64, 0.0, ctypes.byref(plan), fake, fake, fake, None)
+        assert rc == code, (group, hkv, lib.bf1_last_error())
