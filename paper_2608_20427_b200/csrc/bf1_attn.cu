@@ -426,13 +426,15 @@ __global__ void __launch_bounds__(kThreads, 2) attn_fwd_kernel(const __grid_cons
         setmaxnreg_dec<kRegsCtl>();
         if (warp == 2) {
             // ================================ scheduler =======================================
-            for (int n = 1; have0 && !*abort_flag; ++n) {
+            // (The lanes agree on whether a role has given up: the look-ups are made by the whole warp together, and lanes that read
+            // the flag on either side of its being raised would wait for one another in them without end.)
+            for (int n = 1; have0 && !__any_sync(0xffffffffu, *abort_flag); ++n) {
                 mbar_wait(bar_ask, (n - 1) & 1, abort_flag, args.status);
-                int u = 0;
-                if (lane == 0)
+                int u = total_units;
+                if (lane == 0 && !*abort_flag)
                     u = (args.sched ? atomicAdd(args.sched, 1) + (int)gridDim.x : (int)(blockIdx.x + n * gridDim.x));
                 u = __shfl_sync(0xffffffffu, u, 0);
-                const bool have = u < total_units && !*abort_flag;
+                const bool have = u < total_units;
                 Unit un = {};
                 int my_p = 0;
                 if (have) {
