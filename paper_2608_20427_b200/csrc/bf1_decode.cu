@@ -174,13 +174,12 @@ __global__ void __launch_bounds__(kDecThreads, D == 64 ? 4 : 2) decode_fused_ker
             cp_async16_zfill(vb + off, vp + rr * row_stride + c * 8, nbytes);
         }
     };
-    // Few pages: all stages are asked for at once, and the first is filled again when page e_lo + 1 is in use.  A whole list
-    // begins with one page less (batch 32, 256 lists of 11 and 12 pages, with its plan: 19.4 us, 20.0 with three), and asks for a
-    // third when the first has landed.
-    constexpr int kAhead = kSplit ? kDecStages : kDecStages - 1;
+    // Two pages are asked for at the start and the third when the first has landed.  With three at once the first lands later: 64
+    // lists of 11 / 26 pages that no cache holds 8.7 / 12.9 us in parts, 8.1 / 12.0 as it is (16 query / 8 KV heads, d = 128); 256 whole
+    // lists of 11 and 12 pages, with their plan, 20.0 and 19.4.
 #pragma unroll
-    for (int i = 0; i < kDecStages; ++i) {
-        if (i < kAhead && e_lo + i < e_hi) issue_page(e_lo + i, i);
+    for (int i = 0; i < kDecStages - 1; ++i) {
+        if (e_lo + i < e_hi) issue_page(e_lo + i, i);
         cp_async_commit();                               // possibly empty: keeps the group count uniform
     }
     if (kSplit) cluster_arrive_relaxed();                        // (waited for in front of the first store to another CTA)
@@ -201,14 +200,10 @@ __global__ void __launch_bounds__(kDecThreads, D == 64 ? 4 : 2) decode_fused_ker
     const int key0 = warp * 16;                          // this warp's 16 keys of every page
 
     for (int e = e_lo, stage = 0; e < e_hi; ++e) {
-        // page e has landed (for this thread's copies): behind it e_lo + 1 and + 2 are in flight at first, then one page
-        if (e == e_lo) cp_async_wait<kDecStages - 1>();
-        else cp_async_wait<kDecStages - 2>();
+        cp_async_wait<kDecStages - 2>();                 // page e has landed (for this thread's copies)
         __syncthreads();                                 // ... for everybody's; and page e-1 is no longer read
-        if (e > e_lo || kAhead < kDecStages) {
-            if (e + kDecStages - 1 < e_hi) issue_page(e + kDecStages - 1, stage == 0 ? kDecStages - 1 : stage - 1);
-            cp_async_commit();
-        }
+        if (e + kDecStages - 1 < e_hi) issue_page(e + kDecStages - 1, stage == 0 ? kDecStages - 1 : stage - 1);
+        cp_async_commit();
         const int valid = (e == cnt - 1) ? tail : kPage;
         const uint32_t kb = ring + stage * 2 * kPageBytes, vb = kb + kPageBytes;
         if (++stage == kDecStages) stage = 0;
