@@ -119,7 +119,9 @@ template <int D, int kHeads>
 struct RunState {                                       // the four warps' states at the end of the CTA's part
     float o[4][kHeads][D + 8], m[4][kHeads], l[4][kHeads];   // (rows 8 banks apart)
 };
-template <int D, int kHeads, bool kSplit>
+// kSplit: the list is cut, and the CTAs of a cluster add the parts up.  kRest: what rounding takes from P is multiplied with V too (always
+// where the list is cut).
+template <int D, int kHeads, bool kSplit, bool kRest>
 __global__ void __launch_bounds__(kDecThreads, D == 64 ? 4 : 2) decode_fused_kernel(const DecodeArgs a) {
     constexpr int kRowBytes = D * 2;
     constexpr int kVecPerRow = D / 8;                   // 16-byte chunks per row
@@ -252,7 +254,7 @@ __global__ void __launch_bounds__(kDecThreads, D == 64 ? 4 : 2) decode_fused_ker
 #pragma unroll
         for (int i = 0; i < 2; ++i) {                    // keys 2*tig, +1 and 8 + 2*tig, +1
             hi[i] = pack_bf16x2(pv[2 * i], pv[2 * i + 1]);
-            lo[i] = !kSplit ? 0u : pack_bf16x2(pv[2 * i] - __uint_as_float(hi[i] << 16), pv[2 * i + 1] - __uint_as_float(hi[i] & 0xffff0000u));
+            lo[i] = !kRest ? 0u : pack_bf16x2(pv[2 * i] - __uint_as_float(hi[i] << 16), pv[2 * i + 1] - __uint_as_float(hi[i] & 0xffff0000u));
             if (gid >= kHeads) hi[i] = lo[i] = 0u;
         }
         // ---- O = alpha * O + P V: D / 8 n-tiles of 8 columns, V fragments by ldmatrix.trans ---------
@@ -262,7 +264,7 @@ __global__ void __launch_bounds__(kDecThreads, D == 64 ? 4 : 2) decode_fused_ker
         for (int dn = 0; dn < D / 8; dn += 2) {
             if (rescale) {
 #pragma unroll
-                for (int i = 0; i < (kSplit ? 4 : 2); ++i) acc[dn][i] *= alpha, acc[dn + 1][i] *= alpha;
+                for (int i = 0; i < (kRest ? 4 : 2); ++i) acc[dn][i] *= alpha, acc[dn + 1][i] *= alpha;
             }
             uint32_t r0, r1, r2, r3;   // matrices: (keys 0-7, dn), (keys 8-15, dn), (keys 0-7, dn+1), (keys 8-15, dn+1)
             ldmatrix_x4_trans(vrow + (((dn + (lane >> 4)) ^ (lrow & 7)) << 4), r0, r1, r2, r3);
@@ -275,7 +277,7 @@ __global__ void __launch_bounds__(kDecThreads, D == 64 ? 4 : 2) decode_fused_ker
         if (tig == 0) { st.m[warp][gid] = m_run; st.l[warp][gid] = l_run; }
 #pragma unroll
         for (int dn = 0; dn < D / 8; ++dn)
-            *reinterpret_cast<float2*>(&st.o[warp][gid][dn * 8 + 2 * tig]) = kSplit ? make_float2(with_rest(acc[dn][0], acc[dn][2]), with_rest(acc[dn][1], acc[dn][3])) : make_float2(acc[dn][0], acc[dn][1]);
+            *reinterpret_cast<float2*>(&st.o[warp][gid][dn * 8 + 2 * tig]) = kRest ? make_float2(with_rest(acc[dn][0], acc[dn][2]), with_rest(acc[dn][1], acc[dn][3])) : make_float2(acc[dn][0], acc[dn][1]);
     }
     __syncthreads();
     // ---- merge the four warps' states -------------------------------------------------------------------
@@ -415,11 +417,15 @@ static int clusters_that_fit(void (*kernel)(DecodeArgs), int dev, int which, int
 typedef void (*DecodeKernel)(DecodeArgs);
 struct DecodeVariant {
     DecodeKernel whole, split;
+    DecodeKernel brief;               // a whole list with unrounded P (four heads only)
     int page_bytes, state_bytes;      // of a page pair, of a RunState
 };
 template <int D, int kHeads>
 static DecodeVariant decode_variant() {
-    return {decode_fused_kernel<D, kHeads, false>, decode_fused_kernel<D, kHeads, true>, 2 * kPage * D * 2, (int)sizeof(RunState<D, kHeads>)};
+    DecodeKernel brief = nullptr;
+    if constexpr (kHeads == 4) brief = decode_fused_kernel<D, kHeads, false, true>;
+    return {decode_fused_kernel<D, kHeads, false, false>, decode_fused_kernel<D, kHeads, true, true>, brief, 2 * kPage * D * 2,
+            (int)sizeof(RunState<D, kHeads>)};
 }
 
 int check_cfg(const bf1_route_cfg* cfg);   // bf1_plan.cu
@@ -512,6 +518,7 @@ extern "C" int bf1_decode_fwd(const void* q, const void* k_pages, const void* v_
             const DecodeVariant& v = variants[i];
             const int most = v.state_bytes + v.page_bytes * kDecStages + 16 * 1024;    // (exchange: kMaxCtas * (32 + 128) * 4 and less)
             BF1_CUDA_CHECK(cudaFuncSetAttribute(v.whole, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+            if (v.brief) BF1_CUDA_CHECK(cudaFuncSetAttribute(v.brief, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
             BF1_CUDA_CHECK(cudaFuncSetAttribute(v.split, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
             BF1_CUDA_CHECK(cudaFuncSetAttribute(v.split, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         }
@@ -521,14 +528,23 @@ extern "C" int bf1_decode_fwd(const void* q, const void* k_pages, const void* v_
     const int64_t lists = (int64_t)batch * hkv;
     const int heads = group == 4 ? 4 : 2, which = (group == 4 ? 2 : 0) + (d == 128);
     const DecodeVariant& variant = variants[which];
-    // Enough lists to fill the GPU: one CTA walks a whole list.  With four heads and d = 128, where a part costs the most to
-    // exchange, half as many are enough: 96 / 128 / 144 lists of 11 pages 9.7 / 10.5 / 11.0 us whole, 11.3 / 12.6 / 13.6 in parts
-    // (two heads: 10.0 in parts and 9.6 with 96, but 18.1 and 19.4 with 26 pages; d = 64: 6.1 and 7.2).
-    if ((group == 4 && d == 128 ? 2 : 1) * lists >= sms) {
+    // Enough lists to fill the GPU: one CTA walks a whole list.  With four heads, where a part costs the most to exchange, there are
+    // two more cases of it (us on pages that no cache holds):
+    //   d = 128, lists for half of the SMs: 96 / 128 / 144 lists of 11 pages 9.6 / 10.4 / 11.1 whole, 10.7 / 11.6 / 12.3 in parts, of
+    //     4 pages 5.4 / 5.8 / 6.0 and 7.2 / 7.8 / 8.1.  Long lists lose by it while some SMs have none: 74 / 112 / 144 lists of 26
+    //     pages 18.1 / 19.4 / 21.9 whole, 14.2 / 18.8 / 22.3 in parts.
+    //   brief lists, walked with what rounding takes from P, as their parts would be.  A page is 0.47 us of one CTA's time; cut, a list
+    //     pays for the exchange and, with many lists, for the wait for an SM.  d = 64, whole / in parts: 48 lists of 4 pages 4.2 /
+    //     4.3, 80 of 4 / 6 / 8 4.4 / 4.9, 5.4 / 5.4, 6.3 / 6.1, 112 of 4 / 8 / 11 4.6 / 5.3, 6.5 / 6.7, 8.0 / 7.9, 144 of 4 / 8 / 11
+    //     4.8 / 5.8, 6.8 / 7.5, 8.2 / 8.5.  Up to three pages never pay for a cluster: 8 lists of 1 / 2 / 3 2.1 / 2.5 / 2.9 whole, 3.2 /
+    //     3.3 / 3.3 in parts, with d = 128 2.5 / 3.0 / 3.5 and 4.4 / 4.0 / 4.0; of 4 (d = 64, 16 lists) 3.4 and 3.3.
+    const bool half = group == 4 && d == 128 && 2 * lists >= sms;
+    const bool brief = group == 4 && !half && lists < sms && (plan->max_degree <= 3 || (d == 64 && plan->max_degree * (int64_t)sms <= 12 * lists));
+    if (lists >= sms || half || brief) {
         a.nctas = 1;
         a.ring = up(variant.state_bytes);
-        BF1_CUDA_CHECK(launch_pdl(variant.whole, dim3(hkv, batch), kDecThreads, (size_t)a.ring + (size_t)variant.page_bytes * kDecStages,
-                                  (cudaStream_t)stream, a));
+        BF1_CUDA_CHECK(launch_pdl(brief ? variant.brief : variant.whole, dim3(hkv, batch), kDecThreads,
+                                  (size_t)a.ring + (size_t)variant.page_bytes * kDecStages, (cudaStream_t)stream, a));
         return BF1_OK;
     }
     // A list goes to as many CTAs as still let all clusters run at once (a cluster's CTAs share a GPC, so this is less than

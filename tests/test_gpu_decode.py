@@ -282,6 +282,36 @@ def test_a_plan_that_changes_between_the_ctas_of_a_list_stays_in_bounds():
     assert np.isfinite(out[3]).all()
 
 
+def distances_from_64_bits(w, q, k, v, out, last):
+    """Relative distance from 64 bits, over the sequences of more than ten blocks (in a short one the first keys' V fills the norm, and the
+    rounding of P does not show), of `out` and of a result whose weights are rounded to bf16 where that costs least: every weight
+    against the maximum of its own 16 keys."""
+    off = planted = norm = 0.0
+    cu, bf16 = w.cu_seqlens(), lambda x: x.to(torch.bfloat16).double()
+    for s, n in enumerate(w.seqlens):
+        if n <= 64 * 10:
+            continue
+        j = (n - 1) // 64
+        idx, c, _, _ = O.route(O.cfg(), n)
+        blocks = [torch.arange(64 * b, min(64 * b + 64, n)) + cu[s] for b in idx[j, :c[j]]]
+        rows = torch.cat(blocks)
+        kk, vv = (t[rows].double().repeat_interleave(w.hq // w.hkv, 1) for t in (k, v))
+        score = torch.einsum("hd,nhd->hn", q[last[s]].double(), kk) * w.d ** -0.5
+        p = torch.exp(score - score.max(1, keepdim=True).values)
+        piece = torch.cat([(torch.arange(len(b)) // 16) + 4 * i for i, b in enumerate(blocks)]).expand_as(p)
+        top = torch.zeros(w.hq, 4 * len(blocks), dtype=torch.float64).scatter_reduce(1, piece, p, "amax").gather(1, piece)
+        want, rounded = (torch.einsum("hn,nhd->hd", x, vv) / p.sum(1, keepdim=True) for x in (p, bf16(p / top) * top))
+        off += float(((torch.from_numpy(out[s]).double() - want) ** 2).sum())
+        planted += float(((bf16(rounded) - want) ** 2).sum())
+        norm += float((want ** 2).sum())
+    return (off / norm) ** 0.5, (planted / norm) ** 0.5
+
+
+# The rounding of a result to bf16 is 1.64e-3 to 1.69e-3 of its norm in the cases below, computed in 64 bits, and with rounded
+# weights, page by page, 1.9e-3 and more.
+UNROUNDED = 1.78e-3
+
+
 @pytest.mark.parametrize("hq,hkv,d,batch", [(16, 4, 128, 18), (16, 4, 128, 19), (8, 2, 64, 70), (8, 8, 64, 3), (4, 2, 128, 37)],
                          ids=["G4-parts", "G4-whole", "G4-d64", "G1", "G2"])
 def test_parts_of_a_list_lose_nothing_but_the_rounding_of_the_result(hq, hkv, d, batch):
@@ -302,12 +332,13 @@ def test_parts_of_a_list_lose_nothing_but_the_rounding_of_the_result(hq, hkv, d,
         assert off <= 2.0 ** -9 + 1e-5, off
 
 
-@pytest.mark.parametrize("hq,hkv,d", [(1, 1, 128), (4, 2, 64), (4, 2, 128), (8, 2, 64), (8, 2, 128)], ids=["G1", "G2-d64", "G2", "G4-d64", "G4"])
-def test_what_is_not_finite_in_v_comes_out_the_same_however_the_lists_are_walked(hq, hkv, d):
-    """One sequence alone, whose list is cut (eleven parts of a page, and longer ones), and a batch of it that fills the GPU, whose
+@pytest.mark.parametrize("hq,hkv,d,blocks", [(1, 1, 128, 520), (4, 2, 64, 520), (4, 2, 128, 520), (8, 2, 64, 520), (8, 2, 64, 32), (8, 2, 128, 520)],
+                         ids=["G1", "G2-d64", "G2", "G4-d64", "G4-d64-brief", "G4"])
+def test_what_is_not_finite_in_v_comes_out_the_same_however_the_lists_are_walked(hq, hkv, d, blocks):
+    """One sequence alone, whose list is cut (into parts of a page, and longer ones), and batches of it that fill the GPU, whose
     lists are walked whole.  Every column but the last 8 has an infinity at one selected key, with a weight that is not zero:
     the result is that infinity.  Of the others some have both infinities or a NaN at a key: NaN."""
-    n = 64 * 520
+    n = 64 * blocks
     w = I.custom([n], hq=hq, hkv=hkv, d=d, seed=4400 + d + hq)
     q, k, v = I.draw_qkv(w)
     idx, c, _, _ = O.route(O.cfg(), n, 16)
@@ -324,7 +355,7 @@ def test_what_is_not_finite_in_v_comes_out_the_same_however_the_lists_are_walked
         want[col] = want[col + 2] = float("nan")
     k_pages, v_pages, table = (t.to(DEV) for t in paged_cache(w, k, v, seed=15))
     last = None
-    for batch in (1, 30 // hkv, 60 // hkv, 160 // hkv):
+    for batch in (1, 30 // hkv, 60 // hkv, 100 // hkv, 160 // hkv):
         sl = torch.full((batch,), n, dtype=torch.int32, device=DEV)
         plan = bf1.plan_decode(sl, table.repeat(batch, 1))
         ws = bf1.decode_workspace(batch, hq, hkv, plan.max_degree, d, torch.device(DEV))
@@ -357,3 +388,22 @@ def test_an_infinity_under_a_weight_of_zero_is_nan_however_the_lists_are_walked(
         ws = bf1.decode_workspace(batch, hq, hkv, plan.max_degree, d, torch.device(DEV))
         out, _ = bf1.decode_fwd(q[-1].to(DEV).repeat(batch, 1, 1), k_pages, v_pages, sl, plan, ws)
         assert bool(out[..., 0].isnan().all()) and bool(out[..., 1:].isfinite().all()), batch
+
+
+@pytest.mark.parametrize("d,blocks,batch", [(64, 32, 86), (64, 32, 87), (64, 32, 147), (64, 32, 148), (64, 3, 3), (64, 4, 3), (128, 3, 3),
+                                            (128, 4, 3), (128, 3, 73), (128, 3, 74), (128, 1, 5)])
+def test_brief_lists_of_four_heads_are_walked_whole_and_unrounded(d, blocks, batch):
+    """One KV head, 148 SMs.  Seven pages (32 blocks): cut up to 86 lists, whole and unrounded from 87, whole and rounded from 148.  Up to
+    three pages: whole and unrounded however many lists there are, with d = 128 rounded from 74.  Four pages: cut."""
+    rng = np.random.default_rng(blocks + batch)
+    lens = [int(x) for x in rng.integers(64 * 12 if blocks == 32 else 1, 64 * blocks, size=batch)]
+    lens[:3] = [64 * blocks, 1, 64 * (blocks // 2) + 1]
+    w = I.custom(lens, hq=4, hkv=1, d=d, seed=4600 + batch)
+    q, k, v = I.draw_qkv(w)
+    k_pages, v_pages, table = paged_cache(w, k, v, seed=17)
+    out, lse, plan, last = run_decode(w, q, k_pages, v_pages, table)
+    assert int(plan.status.item()) == 0 and plan.max_degree == {32: 7, 4: 4, 3: 3, 1: 1}[blocks]
+    check(w, q, k, v, out, lse, last)
+    if blocks == 32:
+        off, planted = distances_from_64_bits(w, q, k, v, out, last)
+        assert planted > UNROUNDED and (batch == 148 or off <= UNROUNDED), (off, planted)
