@@ -383,14 +383,39 @@ def test_blocks_with_many_readers_are_the_same_however_the_inverse_route_is_made
     assert all(bool(x.isfinite().all()) for x in grads[0])
 
 
-@pytest.mark.parametrize("lens,hq,hkv,d,kw", [
-    ([64 * 2 + 1], 1, 1, 64, dict()),                                     # runs of 2, none of them cut further
-    ([64 * 31 + 7], 2, 1, 128, dict(local_blocks=0, dyadic=0)),           # 16 runs of block 0, the last block short
-    ([1000], 8, 4, 128, dict()),                                          # runs of 4
-    ([700, 33, 64 * 9], 16, 4, 64, dict()),                               # two pairs of heads, short and empty tails
-    ([64 * 33], 16, 8, 64, dict())],                                      # runs of 16, and block 0 in three
-    ids=["2", "2-window", "4", "G4", "16"])
-def test_few_units_are_cut_into_short_runs(lens, hq, hkv, d, kw):
+def runs_of_readers(w):
+    """(units, readers, run length, partial sums, blocks cut) that a backward leaves in its workspace: the last words of its
+    integers, which lie behind one float per row and head."""
+    dev = torch.device("cuda:0")
+    q, k, v = (t.to(dev) for t in I.draw_qkv(w))
+    cu = bf1.cu_seqlens_tensor(w.seqlens, dev)
+    route = bf1.plan_route(cu, w.max_seqlen, lib_cfg(w))
+    o, lse = bf1.attn_fwd(q, k, v, cu, w.max_seqlen, route)
+    ws = bf1.bwd_workspace(route, w.total_tokens, w.hq, w.hkv, w.d, dev)
+    bf1.attn_bwd(q, k, v, o, lse, torch.ones_like(q), cu, w.max_seqlen, route, workspace=ws)
+    cap, deg = route.capacity_qblocks, route.max_degree
+    parts = max(cap, min(cap * deg, 2 * 148 // w.hkv + 1))
+    ints = 3 * (cap + 1) + 3 * cap + cap * deg + 8 * (cap + parts) + 8 * cap + w.hkv + 8
+    at = (w.total_tokens * w.hq * 4 + 255) // 256 * 256 + 4 * (ints - 8)
+    return ws[at:at + 20].view(torch.int32).tolist()
+
+
+@pytest.mark.parametrize("lens,hq,hkv,d,kw,chunk", [
+    ([64 * 2 + 1], 1, 1, 64, dict(), 2),
+    ([64 * 31 + 7], 2, 1, 128, dict(local_blocks=0, dyadic=0), 2),        # 16 runs of block 0, the last block short
+    ([1000], 8, 4, 128, dict(), 4),
+    ([700, 33, 64 * 9], 16, 4, 64, dict(), 4),                            # two pairs of heads, short and empty tails
+    ([64 * 33], 16, 8, 64, dict(), 12),
+    ([64 * 64], 8, 8, 64, dict(), 16)],                                   # the longest; block 0 in four
+    ids=["2", "2-window", "4", "G4", "12", "16"])
+def test_few_units_are_cut_into_short_runs(lens, hq, hkv, d, kw, chunk):
     w = I.custom(lens, hq=hq, hkv=hkv, d=d, seed=7700 + sum(lens), **kw)
+    readers = []
+    for n in lens:
+        idx, count, _, _ = O.route(oracle_cfg(w), n)
+        readers += list(np.bincount(np.concatenate([row[:c] for row, c in zip(idx, count)]), minlength=len(count)))
+    cut = [-(-int(r) // chunk) for r in readers]
+    assert chunk == min(sum(readers) * hkv // 148 + 2, 16)
+    assert runs_of_readers(w) == [sum(cut), sum(readers), chunk, sum(c for c in cut if c > 1), sum(c > 1 for c in cut)]
     for name, (rms, mx) in run_case(w, seed=15).items():
         assert rms <= REL_RMS and mx <= REL_MAX, (name, rms, mx)
