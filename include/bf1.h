@@ -234,8 +234,10 @@ int bf1_decode_fwd(const void *q, const void *k_pages, const void *v_pages, int3
  * at a time over the query blocks that read it), which the call derives from the lists itself: no
  * floating-point atomics anywhere, so all three gradients come out bit-identical on every run.
  * `workspace` (bf1_attn_bwd_workspace_bytes() bytes, 256-byte aligned, contents irrelevant on entry)
- * holds the row terms <d_o, o>, the inverse route, the partial sums of KV blocks with very many readers
- * and, 16 KB per list entry and pair of query heads, the terms dS that dk, dv and dq share (for as many KV
+ * holds the row terms <d_o, o>, the inverse route, what dq looks up of every query block (32 bytes each), the partial
+ * sums of KV blocks whose readers are cut into runs (hkv * 2 * 64 * d floats each, for as many as there are query blocks and
+ * for some 300 / hkv where there are fewer: in short problems runs are short, 75 of them or 20 MB for 1000 tokens, hkv = 4,
+ * d = 128) and, 16 KB per list entry and pair of query heads, the terms dS that dk, dv and dq share (for as many KV
  * heads at a time as fit 1 GiB, at least one; none when one alone would take more than 8 GiB: they are
  * then computed twice).  Geometry limits as bf1_attn_fwd.  `route` must be the forward's (host struct; only its
  * capacities are used by the size helper), and more is asked of it than by the forward: the block p that an entry of slot

@@ -18,8 +18,8 @@
 //                        dV^T += dO^T P  (d x 64 x 128)    A = dO MN-major, B = P MN-major ([q][kv] tile)
 //                        dK^T += Q^T  dS (d x 64 x 128)    A = Q MN-major,  B = dS MN-major
 //                    accumulating in tensor memory across all readers (head dimension on the lanes), and
-//                    one store at the end.  A block with very many readers (block 0: every query block)
-//                    is cut into runs of `chunk` readers handled by different CTAs that leave fp32 partial sums.
+//                    one store at the end.  A block with more readers than a run (2 to 16 of them, by the size of the problem)
+//                    is cut into runs handled by different CTAs that leave fp32 partial sums.
 //                    The dS tiles (bf16, 16 KB each) also go to the workspace, one per list entry.
 //   bwd_dq_kernel    unit = (query block, KV head, pair of query heads): dQ += dS K_p over the list, dS as the
 //                    dK/dV kernel left it; and, in warps of their own, the partial sums added up in run order.
@@ -1516,8 +1516,9 @@ __global__ void __launch_bounds__(256) bwd_combine_kernel(const BwdArgs a) {
 // both cases, whether dS lies in L2 or comes from HBM, which is what bounds it now.
 // One persistent CTA of 11 warps per SM; units are dealt out statically, longest list first (KV head by KV head, or all
 // heads together: BwdArgs::interleave), back and forth over the CTAs:
-//     warp 10   describes the units to the other roles.  What it looks up is a chain of four loads; it does so for 32 units
-//               at a time, one per lane.  (With every role looking its units up itself 4K tokens took 0.6 us more.)
+//     warp 10   describes the units to the other roles: what the preparation wrote down of the query block, then its list, two
+//               dependent loads, for 32 units at a time, one per lane.  (With every role looking its units up itself, in what was
+//               a chain of four loads before the preparation made it, 4K tokens took 0.6 us more.)
 //     warp 0    copies: the dS tile (as the dK/dV kernel left it: the K-major layout of an A operand) and the K tile of
 //               every list entry, through a ring of kDqStages
 //     warp 1    issues the MMAs; dQ accumulates in one of two buffers in tensor memory

@@ -22,8 +22,9 @@
 // at all).  Where a list is cut, what the rounding takes away is therefore multiplied with V as well: it stands in rows of the
 // mma's operand that were zero, so that it costs no mma.  The relative error against 64 bits is then 1.6e-3 (the rounding of
 // the result) whatever the parts are, 1.95e-3 page by page without it and 1.99e-3 in parts of two pages, and
-// the parts are free to be what is fastest: eight sequences of 65 to 32768 tokens 7.2 -> 6.4 us against runs that were
-// kept short for their precision and dealt to the CTAs.  A whole list (lists for every SM) is rounded as it was.
+// the parts are free to be what is fastest: eight sequences of 65 to 32768 tokens 7.2 -> 6.1 us against runs that were
+// kept short for their precision and dealt to the CTAs.  Where there are lists for every SM (four
+// heads, d = 128: for half of them), P is rounded.
 // Four query heads share a CTA and with it one reading of K and V (a CTA for each pair of heads before): 192 lists of 11
 // pages 23.6 -> 13.9 us, 40 lists 9.5 -> 6.0.
 #include <algorithm>
@@ -37,7 +38,8 @@ namespace bf1 {
 constexpr int kPage = 64;             // tokens per page = block width b
 constexpr int kDecThreads = 128;
 constexpr int kDecStages = 3;          // page-pair buffers per CTA
-constexpr int kDecCtasPerSm = 4;       // CTAs asked for, at most, while there are few lists (how many fit decides)
+// CTAs asked for, at most, while there are few lists (how many fit decides): over 645 shapes 0.3 % faster than two, on average.
+constexpr int kDecCtasPerSm = 4;
 // CTAs of a cluster at most.  Above 8 a cluster may find fewer places (bf1_decode_fwd asks), but a CTA with one page instead
 // of two or more wins whatever it costs: one list of 11 / 41 / 64 pages takes 5.1 / 9.4 / 11.6 us with eight CTAs, 4.0 /
 // 6.7 / 8.1 with up to sixteen.
@@ -548,7 +550,9 @@ extern "C" int bf1_decode_fwd(const void* q, const void* k_pages, const void* v_
         return BF1_OK;
     }
     // A list goes to as many CTAs as still let all clusters run at once (a cluster's CTAs share a GPC, so this is less than
-    // what the SMs hold: 48 lists of 11 pages over six CTAs each took 12.0 us, a second wave of clusters; with four 8.8).
+    // what the SMs hold: 48 lists of 11 pages over six CTAs each took 12.0 us, a second wave of clusters; with four 8.8).  Against the
+    // best of eleven numbers, over 645 shapes (8 to 144 lists of 2 to 64 pages, cold and cached) this one takes 0.6 % longer on
+    // average with two heads and d = 128, 6.7 % at most; with d = 64 1.1 and 7.4 %, with four heads 1.3 and 9 %.
     auto ceil_div = [](int x, int y) { return (x + y - 1) / y; };
     const int most = plan->max_degree;
     size_t smem = 0;
